@@ -44,7 +44,7 @@ METRIC = "ap_fwd_bwd_edge_feat_per_s"
 UNIT = "edge*feat/s"
 NOMINAL_HBM_GBS = 8000.0
 TRAFFIC_FILE = os.path.join(ROOT, "profiles", "dram_traffic.txt")
-KERNEL_SOURCES = ["dg_aggregate_kernels.cuh", "dg_aggregate.cu", "dg_aggregate_fold.cu"]
+KERNEL_SOURCES = ["dg_aggregate_kernels.cuh", "dg_aggregate.cu"]
 
 
 def kernel_source_hash():

@@ -59,9 +59,9 @@ typedef struct dg_graph* dg_graph_t;
  *   edge_w  device, nnz fp32 scalars (the edge feature of Eq. 1 reduced to one value per
  *           edge and broadcast over the F features), or NULL for the unary copy of Eq. 2
  * The handle BORROWS the three arrays: they must stay valid and unchanged until
- * dg_graph_destroy.  The call allocates a few small device arrays that it owns (the lists of
- * heavy rows and, for graphs with at least 64 edges per vertex, 17 int32 split pointers per
- * vertex for source blocking).  It waits for the whole device before it reads the arrays (so
+ * dg_graph_destroy.  The handle owns a few small device arrays (how the rows are shared out among
+ * warps and, for graphs with at least 64 edges per vertex, 17 int32 split pointers per vertex for
+ * source blocking) from the library's memory pool.  The call waits for the whole device before it reads the arrays (so
  * they may have been produced on any stream) and again before it returns.
  * The arrays are checked here, in one streaming pass (rowptr[0] = 0, rowptr non-decreasing,
  * rowptr[n] = nnz, every colidx in [0, n)): the aggregation kernels index the feature matrix
@@ -328,14 +328,14 @@ dg_status_t dg_aggregate_edge_grad(dg_graph_t g, const float* H, const float* dO
 
 /*
  * Tuning knobs (defaults come from the device's L2 size and SM count):
- *   "heavy_threshold"  rows longer than this are summed by a whole thread block
- *   "heavy_blocks_per_sm"  thread blocks per SM that walk the list of heavy rows (longest first)
- *                      before the launch turns to the light rows; 0 = as many as are resident
+ *   "heavy_threshold"  rows longer than this may be cut into pieces for several warps (default:
+ *                      twice the piece size chosen from the number of edges, 64 to 2048)
+ *   "heavy_blocks_per_sm"  accepted in [0, 32]; no effect
  *   "slice_features"   features per pass over the graph (0 = choose from the L2 size; a value
  *                      that would need more than 65535 passes is widened)
- *   "rows_per_block"   destination rows per thread block in the light-row kernel (1..248,
- *                      rounded up to a multiple of 8: each of the 8 warps owns a run of rows;
- *                      0 = about 1024 edges per warp, between 32 and 248 rows per block)
+ *   "rows_per_block"   rows per thread block at the average row length (1..248, rounded up to a
+ *                      multiple of 8: each of the 8 warps takes the edges of that many rows;
+ *                      0 = 32 to 1024 edges per warp, from the number of edges)
  *   "l2_budget_mb"     MiB of the gathered matrix one launch may keep L2-resident
  *   "source_blocks"    number of source-vertex ranges the pass is cut into, one launch each
  *                      (the blocking of Algorithm 2; 0 = choose from the L2 budget, else 1, 2,
@@ -344,8 +344,8 @@ dg_status_t dg_aggregate_edge_grad(dg_graph_t g, const float* H, const float* dO
  * Graph attribute (not a tuning knob: it changes the result):
  *   "self_loops"       0 (default) or 1: every vertex is its own in-neighbour with weight 1, see
  *                      dg_aggregate_fwd / dg_aggregate_bwd; set it before dg_graph_transpose
- * Changing "heavy_threshold" waits for the whole device, rebuilds the heavy lists and waits
- * again: a rare, synchronous call.
+ * Changing "heavy_threshold" or "rows_per_block" waits for the whole device, shares the rows out
+ * anew and waits again: a rare, synchronous call.
  * Returns DG_ERR_INVALID_ARG for an unknown name or a value out of range.
  */
 dg_status_t dg_graph_set_param(dg_graph_t g, const char* name, int64_t value);

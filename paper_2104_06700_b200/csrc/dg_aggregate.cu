@@ -1,15 +1,78 @@
 // Host side of the aggregation: chooses the launch shape of one call (vector width, feature
-// slices, source blocks) and runs one launch per source block.  The kernels are in
-// dg_aggregate_kernels.cuh; this file compiles them for graphs without implicit self loops and
-// without long segments, dg_aggregate_fold.cu, dg_aggregate_self.cu and dg_aggregate_self_fold.cu
-// for the other three combinations (four translation units compile side by side).
+// slices, source blocks), runs one launch per source block and joins the rows the plan cut.  The
+// kernels are in dg_aggregate_kernels.cuh; this file compiles them for graphs without implicit self
+// loops, dg_aggregate_self.cu for the others (the translation units compile side by side).
 #include "dg_aggregate_kernels.cuh"
 
 namespace dg {
+namespace {
 
-dg_status_t launch_plain(const Graph* g, const ApArgs& a, int vec, int slices, cudaStream_t s) {
-  if (a.long_segments) return launch_plain_fold(g, a, vec, slices, s);
-  return dispatch_type<false, false>(g, a, SelfArgs{}, vec, slices, s);
+// Adds the slots of every cut row to what the row's first chunk stored.  A block takes one row and 128
+// features; its 8 warps take every eighth slot, and their sums are added in warp order.  The traffic is
+// one row of F floats per chunk of up to 1024 gathered rows; the launch itself is most of the cost.
+__global__ void __launch_bounds__(kBlock)
+join_kernel(const Chunk* __restrict__ chunks, const CutRow* __restrict__ cuts,
+            const int32_t* __restrict__ totals, int32_t max_cuts, const float* __restrict__ partial, int32_t F,
+            float* __restrict__ Y) {
+  __shared__ float part[kWarpsPerBlock][128];
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  const int f0 = blockIdx.y * 128;
+  const int cut_rows = min(__ldg(totals + 1), max_cuts);
+  for (int i = blockIdx.x; i < cut_rows; i += gridDim.x) {
+    const CutRow cut = cuts[i];
+    float sum[4] = {0.f, 0.f, 0.f, 0.f};
+    for (int k = warp; k < cut.count; k += kWarpsPerBlock) {
+      const float* p = partial + (size_t)__ldg(&chunks[cut.first + k].slot) * (size_t)F;
+#pragma unroll
+      for (int j = 0; j < 4; ++j) {
+        const int f = f0 + 32 * j + lane;
+        if (f < F) sum[j] += p[f];
+      }
+    }
+#pragma unroll
+    for (int j = 0; j < 4; ++j) part[warp][32 * j + lane] = sum[j];
+    __syncthreads();
+    const int f = f0 + threadIdx.x;
+    if (threadIdx.x < 128 && f < F) {
+      float t = part[0][threadIdx.x];
+#pragma unroll
+      for (int w = 1; w < kWarpsPerBlock; ++w) t += part[w][threadIdx.x];
+      Y[(size_t)cut.row * (size_t)F + f] += t;
+    }
+    __syncthreads();
+  }
+}
+
+}  // namespace
+
+dg_status_t launch_plain(const ApArgs& a, int vec, int slices, cudaStream_t s) {
+  return dispatch_type<false>(a, SelfArgs{}, vec, slices, s);
+}
+
+// Scratch for the parts of cut rows, from the library's pool.  *partial stays nullptr when the plan cuts
+// no row.
+dg_status_t take_partial(const Graph* g, const Plan& plan, int64_t floats_per_slot, cudaStream_t s,
+                         float** partial) {
+  *partial = nullptr;
+  const int64_t slots = plan.slots >= 0 ? plan.slots : plan.max_slots;
+  if (slots == 0) return DG_OK;
+  void* p = nullptr;
+  DG_CUDA(pool_alloc(g->device, (size_t)slots * (size_t)floats_per_slot * sizeof(float), s, &p));
+  *partial = static_cast<float*>(p);
+  return DG_OK;
+}
+
+dg_status_t join_cut_rows(const Graph* g, const Plan& plan, const float* partial, int32_t F, float* Y,
+                          cudaStream_t s) {
+  // the number of cut rows may still be on its way to the host: the kernel reads it on the device
+  int64_t blocks = plan.cut_rows >= 0 ? plan.cut_rows : plan.max_cuts;
+  if (blocks > (int64_t)g->sm_count * 64) blocks = (int64_t)g->sm_count * 64;
+  const dim3 grid((unsigned)blocks, (unsigned)((F + 127) / 128));
+  join_kernel<<<grid, kBlock, 0, s>>>(plan.chunks, plan.cuts, plan.totals, (int32_t)plan.max_cuts, partial, F,
+                                      Y);
+  DG_CUDA(cudaGetLastError());
+  count_launches(1);
+  return DG_OK;
 }
 
 // Bytes of L2 one row slice of `slice` elements of `eb` bytes occupies: L2 allocates 128-byte
@@ -29,8 +92,8 @@ static double slice_footprint(int64_t F, int64_t slice, int eb) {
 //     the neighbour ids are cut into 2, 4, 8 or 16 ranges and each range is a launch of its
 //     own, so that the rows of X a launch gathers stay L2-resident; later launches add to Y.
 //     Without split pointers the slice is narrowed instead (down to 128 bytes).
-dg_status_t aggregate_run(const Graph* g, const ApArgs& a0, const SelfArgs& sa, const int32_t* split,
-                          cudaStream_t s) {
+dg_status_t aggregate_run(const Graph* g, const ApArgs& a0, const SelfArgs& sa, const Plan& plan,
+                          const int32_t* split, cudaStream_t s) {
   ApArgs a = a0;
   if (a.n == 0) return DG_OK;
   const uintptr_t px = (uintptr_t)a.X, py = (uintptr_t)a.Y;
@@ -101,18 +164,24 @@ dg_status_t aggregate_run(const Graph* g, const ApArgs& a0, const SelfArgs& sa, 
   a.slice_f = (int32_t)slice;
   const int slices = (int)((a.F + slice - 1) / slice);
 
+  a.row_bytes = (uint32_t)(a.F * eb);
+  a.chunks = plan.chunks;
+  a.chunk_count = (int32_t)plan.count;
+  dg_status_t st = take_partial(g, plan, a.F, s, &a.partial);
   const int per = kFineBlocks / nb;
-  for (int j = 0; j < nb; ++j) {
+  for (int j = 0; j < nb && st == DG_OK; ++j) {
     if (nb > 1) {
       a.seg_lo = split + (size_t)(j * per) * (size_t)a.n;
       a.seg_hi = split + (size_t)((j + 1) * per) * (size_t)a.n;
       a.accumulate = j > 0;
     }
-    const dg_status_t st = sa.self_ptr ? launch_with_self_loops(g, a, sa, vec, slices, s)
-                                       : launch_plain(g, a, vec, slices, s);
-    if (st != DG_OK) return st;
+    st = sa.self_ptr ? launch_with_self_loops(a, sa, vec, slices, s) : launch_plain(a, vec, slices, s);
   }
-  return DG_OK;
+  if (a.partial) {
+    if (st == DG_OK) st = join_cut_rows(g, plan, a.partial, a.F, a.Y, s);
+    pool_free(a.partial, s);
+  }
+  return st;
 }
 
 }  // namespace dg

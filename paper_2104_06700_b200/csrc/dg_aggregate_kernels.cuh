@@ -5,23 +5,28 @@
 // the CPU cache (one launch per block, later launches adding to the output).
 //
 // Work decomposition
-//   light segments (length <= heavy_threshold): every warp owns rows_per_warp consecutive
-//     segments and reads their indices as one contiguous stream of 32-edge batches (one edge
-//     per lane, next batch prefetched), so short rows share coalesced index loads.  Lanes are
-//     spread along the feature dimension with 16-, 8- or 4-byte vector loads.  When a row slice
-//     needs fewer than 32 vectors the warp is cut into groups of G lanes and the groups take
-//     different edges of the same segment; their partial sums are combined by a fixed shuffle
-//     tree.  U load steps per lane are in flight before the first add.
-//   heavy segments: one thread block per segment; the first blocks of the same launch (as many
-//     as the device keeps resident) loop over the heavy list, which is ordered longest first;
-//     the 8 warps take interleaved batches of 32 edges and combine in shared memory in warp
-//     order.
-// Every output element is produced by one thread in an order fixed by the launch shape, so the
+//   Every warp takes one chunk of the direction's plan (see Plan): a run of rows, or a piece of one long
+//   row, with about the same number of entries as every other chunk.  It reads the indices of the
+//   chunk as one contiguous stream of 32-edge batches (one edge per lane, next batch prefetched), so
+//   short rows share coalesced index loads.  Lanes are spread along the feature dimension with 16-, 8-
+//   or 4-byte vector loads.  When a row slice needs fewer than 32 vectors the warp is cut into groups
+//   of G lanes and the groups take different edges of the same row; their partial sums are combined by
+//   a fixed shuffle tree.  U load steps per lane are in flight before the first add.
+//   A piece that begins inside a row goes to a slot of a scratch array; join_kernel (dg_aggregate.cu)
+//   adds the slots of a row to what its first piece stored.
+// With whole rows per warp (up to 31 of them, rows over 1024 entries to a block each) a warp's longest
+// serial run of edges, not the amount of work, set the time of small and of skewed graphs.  Equal chunks,
+// kernel time of a forward and a backward pass on B200: 1.2 M edges, rows up to 2000, F = 47: 334 -> 57 us;
+// 65 k edges, F = 64: 20.7 -> 12.1 us; 81 M edges, columns up to 10^5, F = 128: 11.5 -> 10.2 ms.
+// Every output element is produced by one thread per launch in an order fixed by the plan, so the
 // result is deterministic and needs no atomics in either direction.
 #ifndef DG_AGGREGATE_KERNELS_CUH_
 #define DG_AGGREGATE_KERNELS_CUH_
 #include "dg_internal.cuh"
 
+#ifndef DG_UM
+#define DG_UM 1
+#endif
 namespace dg {
 namespace {
 
@@ -158,25 +163,6 @@ __device__ __forceinline__ void stcs_vec(float* p, f8 v) {
   __stcs(reinterpret_cast<float4*>(p), v.lo);
   __stcs(reinterpret_cast<float4*>(p + 4), v.hi);
 }
-__device__ __forceinline__ void st_smem(float* p, f8 v) {
-  p[0] = v.lo.x; p[1] = v.lo.y; p[2] = v.lo.z; p[3] = v.lo.w;
-  p[4] = v.hi.x; p[5] = v.hi.y; p[6] = v.hi.z; p[7] = v.hi.w;
-}
-__device__ __forceinline__ void st_smem(float* p, float v) { p[0] = v; }
-__device__ __forceinline__ void st_smem(float* p, float2 v) { p[0] = v.x; p[1] = v.y; }
-__device__ __forceinline__ void st_smem(float* p, float4 v) {
-  p[0] = v.x; p[1] = v.y; p[2] = v.z; p[3] = v.w;
-}
-__device__ __forceinline__ void add_smem(float* p, float v) { p[0] += v; }
-__device__ __forceinline__ void add_smem(float* p, float2 v) { p[0] += v.x; p[1] += v.y; }
-__device__ __forceinline__ void add_smem(float* p, float4 v) {
-  p[0] += v.x; p[1] += v.y; p[2] += v.z; p[3] += v.w;
-}
-__device__ __forceinline__ void add_smem(float* p, f8 v) {
-  add_smem(p, v.lo);
-  add_smem(p + 4, v.hi);
-}
-
 // Loads the neighbour id and the per-edge factor of the edge at position b + lane of the
 // index stream (neutral values at or beyond `end`).
 template <bool SCALED>
@@ -295,147 +281,36 @@ __device__ __forceinline__ void combine_groups(typename Vec<VEC>::T (&acc)[CPL])
   }
 }
 
-// Graphs that hold a segment of kLongSegment entries or more run the kernels compiled with
-// FOLD: there a warp of a heavy segment moves its register sums into its shared-memory partial
-// every kLongFold batches, so that no fp32 chain is longer than 32 * kLongFold = 512 terms however
-// long the segment is (a segment of m entries is summed as chains of at most 512 terms, whose
-// results form a second chain of m / 4096 terms per warp, and the 8 warp partials are added last).
-// One register chain per warp, m / 8 terms, drifts past 1e-5 of the sum of magnitudes for
-// same-sign inputs once m reaches about 10^6; below kLongSegment it is at most 4096 terms long.
-// The fold is a second compilation of the kernels rather than a branch in one: in any of five
-// forms tried (a counter in the loop, a second loop for long segments, a shared-memory counter,
-// a function that is not inlined, a kernel of its own after the common one) it either changed the
-// register allocation of the common kernels (Reddit-like backward 17.8 -> 18.7 ms) or serialised
-// the long segments behind the rest (Papers-like backward 11.3 -> 16.0 ms at a tenth of the size).
-constexpr int kLongSegment = 1 << 15;
-constexpr int kLongFold = 16;
-
-// Block-per-row path for the heavy segments: block x of the first `heavy_blocks` blocks takes
-// entries x, x + heavy_blocks, ... of the heavy list; its 8 warps sum interleaved 32-edge
-// batches and the partial sums are combined in shared memory in warp order.
-template <typename E, int VEC, int G, int CPL, bool SCALED, bool SEG, bool SELF, bool FOLD>
-__device__ __forceinline__ void heavy_rows(const ApArgs& a, const SelfArgs sa,
-                                           const int heavy_blocks,
-                                           float (&part)[kWarpsPerBlock][32 * CPL * VEC]) {
+template <typename E, int VEC, int G, int CPL, bool SCALED, bool SEG, bool SELF>
+__device__ __forceinline__ void ap_body(const ApArgs& a, const SelfArgs sa) {
   using V = typename Vec<VEC>::T;
-  __shared__ uint2 stage_heavy[kWarpsPerBlock][32];
-  uint2* stage = stage_heavy[threadIdx.x >> 5];
+  __shared__ uint2 stage_all[kWarpsPerBlock][32];
+  // where row 0 of the warp's output would lie; in shared memory because only the store step needs it
+  // and the summing loop is short of registers
+  __shared__ float* out_all[kWarpsPerBlock];
+  uint2* stage = stage_all[threadIdx.x >> 5];
   const int lane = threadIdx.x & 31;
-  const int warp = threadIdx.x >> 5;
-  const int grp = lane / G;
-  const int c0 = lane % G;
-  const int f0 = blockIdx.y * a.slice_f;
-  const int width = min(a.F, f0 + a.slice_f) - f0;
-  const int chunks = width / VEC;
-  const uint32_t row_bytes = (uint32_t)a.F * (uint32_t)E::kBytes;
-  const char* xrow[CPL];
-  bool cok[CPL];
-#pragma unroll
-  for (int c = 0; c < CPL; ++c) {
-    const int ci = c0 + c * G;
-    cok[c] = ci < chunks;
-    xrow[c] = reinterpret_cast<const char*>(a.X) + (size_t)(f0 + (cok[c] ? ci : 0) * VEC) * E::kBytes;
-  }
-  const int count = min(*a.heavy_count, a.heavy_cap);
-  for (int i = blockIdx.x; i < count; i += heavy_blocks) {
-    const int64_t r = a.heavy_list[i];
-    const int full = (int)(__ldg(a.ptr + r + 1) - __ldg(a.ptr + r));
-    const int lo = SEG ? __ldg(a.seg_lo + r) : (int)__ldg(a.ptr + r);
-    const int hi = SEG ? __ldg(a.seg_hi + r) : lo + full;
-    V acc[CPL];
-#pragma unroll
-    for (int c = 0; c < CPL; ++c) zero(acc[c]);
-    if (FOLD && lane < G) {
-#pragma unroll
-      for (int c = 0; c < CPL; ++c)
-        if (cok[c]) st_smem(&part[warp][(c0 + c * G) * VEC], acc[c]);
-    }
-    // warp w sums batches w, w+8, ... of the segment
-    int32_t cur_u, nxt_u;
-    float cur_s, nxt_s;
-    int b = hi - lo > warp * 32 ? lo + warp * 32 : hi;
-    if (b < hi) load_batch<SCALED>(a, b, hi, lane, cur_u, cur_s);
-    int since_fold = 0;
-    while (b < hi) {
-      const bool more = hi - b > kBlock;
-      if (more) load_batch<SCALED>(a, (int64_t)b + kBlock, hi, lane, nxt_u, nxt_s);
-      add_edges<E, VEC, G, CPL, SCALED, SEG>(xrow, row_bytes, cur_u, cur_s, 0, min(hi - b, 32), grp, acc,
-                                     stage);
-      if (FOLD && (++since_fold == kLongFold || !more)) {
-        // the register sums join the warp's partial in shared memory and start afresh
-        since_fold = 0;
-        combine_groups<VEC, G, CPL>(acc);
-        if (lane < G) {
-#pragma unroll
-          for (int c = 0; c < CPL; ++c)
-            if (cok[c]) add_smem(&part[warp][(c0 + c * G) * VEC], acc[c]);
-        }
-#pragma unroll
-        for (int c = 0; c < CPL; ++c) zero(acc[c]);
-      }
-      if (!more) break;
-      b += kBlock;
-      cur_u = nxt_u;
-      cur_s = nxt_s;
-    }
-    if (!FOLD) {
-      combine_groups<VEC, G, CPL>(acc);
-      if (lane < G) {
-#pragma unroll
-        for (int c = 0; c < CPL; ++c)
-          if (cok[c]) st_smem(&part[warp][(c0 + c * G) * VEC], acc[c]);
-      }
-    }
-    __syncthreads();
-    float* orow = a.Y + (size_t)r * (size_t)a.F + f0;
-    if constexpr (SELF) {
-      // the row's own input row joins the sum once, scaled like the mean's other terms
-      const float ss = sa.self_mean ? self_factor(sa.self_ptr, r) : 1.0f;
-      const bool own = !(SEG && a.accumulate);
-      for (int f = threadIdx.x; f < width; f += kBlock) {
-        float t = part[0][f];
-#pragma unroll
-        for (int w = 1; w < kWarpsPerBlock; ++w) t += part[w][f];
-        if (a.mean_rows) t *= ss;
-        if (own) t = fmaf(ss, ld_elem<E>(a.X, (size_t)r * (size_t)a.F + f0 + f), t);
-        if (SEG && a.accumulate) t += orow[f];
-        __stcs(orow + f, t);
-      }
-    } else {
-      const float rs = a.mean_rows ? 1.0f / (float)full : 1.0f;
-      for (int f = threadIdx.x; f < width; f += kBlock) {
-        float t = part[0][f];
-#pragma unroll
-        for (int w = 1; w < kWarpsPerBlock; ++w) t += part[w][f];
-        if (a.mean_rows) t *= rs;
-        if (SEG && a.accumulate) t += orow[f];
-        __stcs(orow + f, t);
-      }
-    }
-    __syncthreads();
-  }
-}
-
-// One launch does both roles: blocks [0, heavy_blocks) walk the heavy list (they are scheduled
-// first, so the long segments start early); in the remaining blocks every warp owns
-// rows_per_warp consecutive light segments and streams their indices as one run of 32-edge
-// batches, the next batch always in flight while the current one is summed.
-template <typename E, int VEC, int G, int CPL, bool SCALED, bool SEG, bool SELF, bool FOLD>
-__device__ __forceinline__ void ap_body(const ApArgs& a, const SelfArgs sa,
-                                        const int heavy_blocks,
-                                        float (&part)[kWarpsPerBlock][32 * CPL * VEC]) {
-  using V = typename Vec<VEC>::T;
-  __shared__ uint2 stage_light[kWarpsPerBlock][32];
-  uint2* stage = stage_light[threadIdx.x >> 5];
-  const int lane = threadIdx.x & 31;
-  const int warp = threadIdx.x >> 5;
   const int grp = lane / G;
   const int c0 = lane % G;
   const int f0 = blockIdx.y * a.slice_f;
   const int fend = min(a.F, f0 + a.slice_f);
   const int width = fend - f0;
   const int chunks = width / VEC;
-  const uint32_t row_bytes = (uint32_t)a.F * (uint32_t)E::kBytes;
+  const uint32_t row_bytes = a.row_bytes;
+
+  // The shuffle tells the compiler that the warp's number, and with it everything read from the plan and
+  // every loop bound below, is the same in all lanes: they then live in uniform registers.  Without it
+  // the summing loops are 8 to 30 registers short and the same kernels take 1.1 to 1.8 times as long.
+  const int chunk = blockIdx.x * kWarpsPerBlock + __shfl_sync(kFull, (int)(threadIdx.x >> 5), 0);
+  if (chunk >= a.chunk_count) return;
+  const int4 here = __ldg(reinterpret_cast<const int4*>(a.chunks) + chunk);
+  const int4 next = __ldg(reinterpret_cast<const int4*>(a.chunks) + chunk + 1);
+  const int rb = here.x;
+  // the next chunk may begin inside our last row; a chunk that begins inside a row is a piece of that row
+  const int nrows = here.z >= 0 ? 1 : next.x - here.x + (next.z >= 0 ? 1 : 0);
+  if (lane == 0)
+    out_all[threadIdx.x >> 5] = here.z >= 0 ? a.partial + ((int64_t)here.z - here.x) * (int64_t)a.F : a.Y;
+  __syncwarp();
 
   // Lanes whose vector falls beyond the slice re-read vector 0 and never store: the summing
   // loop then needs no per-lane predicate.
@@ -449,7 +324,8 @@ __device__ __forceinline__ void ap_body(const ApArgs& a, const SelfArgs sa,
   }
 
   // Starts a row: zero, or, on a graph with implicit self loops, the row's own input row (taken
-  // by lane group 0 only, once: not in the accumulating launches of later source blocks).  It
+  // by lane group 0 only, once: not in the accumulating launches of later source blocks, and not by the
+  // later pieces of a cut row).  It
   // is loaded here, ahead of the row's edges, like one more gathered row; added in the store
   // step instead, the load changed the instruction schedule of the whole summing loop (Reddit-
   // like F = 602 forward: 4.44 ms per launch against 4.0 ms, with the same instruction count).
@@ -458,11 +334,11 @@ __device__ __forceinline__ void ap_body(const ApArgs& a, const SelfArgs sa,
   // The next row's own row is asked into L2 one row ahead (1-2.5 % on the DRAM-bound workloads,
   // whose rows are short against a DRAM round trip).  Asking for all of a warp's own rows when
   // the warp starts made the same workloads slower (Products-like F = 602 41.4 -> 51.3 ms).
-  auto start_row = [&](int64_t r, V (&acc)[CPL], bool more_rows) {
+  auto start_row = [&](int r, V (&acc)[CPL], bool more_rows) {
 #pragma unroll
     for (int c = 0; c < CPL; ++c) zero(acc[c]);
     if constexpr (SELF) {
-      if (grp == 0 && !(SEG && a.accumulate)) {
+      if (grp == 0 && *(float* volatile*)&out_all[threadIdx.x >> 5] == a.Y && !(SEG && a.accumulate)) {
         using L = typename Pack<E, VEC>::Load;
         const float ss = (sa.self_mean && !a.mean_rows) ? self_factor(sa.self_ptr, r) : 1.0f;
         // the warp's next row will want its own row: ask it into L2 one row ahead
@@ -479,15 +355,17 @@ __device__ __forceinline__ void ap_body(const ApArgs& a, const SelfArgs sa,
     }
   };
 
-  // Writes one finished row: scales by 1/length for the mean (length + 1 with self loops: the
-  // forward segment length is the in-degree) and, in a later source block, adds what the
-  // earlier blocks left in Y.
-  auto store_row = [&](int64_t r, int len, V (&acc)[CPL]) {
+  // Writes one finished row, or the part of a cut row: scales by 1/length for the mean (length + 1
+  // with self loops: the forward segment length is the in-degree; a part is scaled by its whole row's
+  // length, read again here) and, in a later source block, adds what the earlier blocks left there.
+  auto store_row = [&](int r, V (&acc)[CPL]) {
     if (lane < G) {
-      const float rs = !a.mean_rows ? 1.0f
-                       : SELF      ? 1.0f / (float)(len + 1)
-                                   : (len > 0 ? 1.0f / (float)len : 1.0f);
-      float* orow = a.Y + (size_t)r * (size_t)a.F + f0;
+      float rs = 1.0f;
+      if (a.mean_rows) {
+        const int len = (int)(__ldg(a.ptr + r + 1) - __ldg(a.ptr + r));
+        rs = SELF ? 1.0f / (float)(len + 1) : (len > 0 ? 1.0f / (float)len : 1.0f);
+      }
+      float* orow = *(float* volatile*)&out_all[threadIdx.x >> 5] + (size_t)r * (size_t)a.F + f0;
 #pragma unroll
       for (int c = 0; c < CPL; ++c) {
         if (cok[c]) {
@@ -500,23 +378,16 @@ __device__ __forceinline__ void ap_body(const ApArgs& a, const SelfArgs sa,
     }
   };
 
-  if (SEG && (int)blockIdx.x >= heavy_blocks) {
+  if constexpr (SEG) {
     // Source-blocked pass: row i of this warp contributes the positions [seg_lo, seg_hi) of its
     // segment.  The pieces are not adjacent in memory, so batches start at each piece; the
     // prefetch cursor (qi, qb) runs one batch ahead of the summing loop across rows.
-    const int rpw = a.rows_per_warp;
-    const int64_t rb = ((int64_t)(blockIdx.x - heavy_blocks) * kWarpsPerBlock + warp) * rpw;
-    if (rb >= a.n) return;
-    const int nrows = (int)min((int64_t)rpw, a.n - rb);
-    int my_lo = 0, my_hi = 0, my_full = 0;
+    int my_lo = 0, my_hi = 0;
     if (lane < nrows) {
-      my_lo = __ldg(a.seg_lo + rb + lane);
-      my_hi = __ldg(a.seg_hi + rb + lane);
-      my_full = (int)(__ldg(a.ptr + rb + lane + 1) - __ldg(a.ptr + rb + lane));
+      my_lo = max(__ldg(a.seg_lo + rb + lane), here.y);
+      my_hi = min(__ldg(a.seg_hi + rb + lane), next.y);
     }
-    const unsigned heavy_mask = __ballot_sync(kFull, my_full > a.heavy_threshold);
-    const unsigned work =
-        __ballot_sync(kFull, lane < nrows && my_full <= a.heavy_threshold && my_hi > my_lo);
+    const unsigned work = __ballot_sync(kFull, my_hi > my_lo);
     int qi = work ? __ffs(work) - 1 : 32, qb = 0, qhi = 0;
     int32_t cur_u = 0, nxt_u = 0;
     float cur_s = 0.f, nxt_s = 0.f;
@@ -539,15 +410,13 @@ __device__ __forceinline__ void ap_body(const ApArgs& a, const SelfArgs sa,
       if (qi < 32) load_batch<SCALED>(a, qb, qhi, lane, nxt_u, nxt_s);
     }
     for (int i = 0; i < nrows; ++i) {
-      if ((heavy_mask >> i) & 1u) continue;
       const int lo = __shfl_sync(kFull, my_lo, i);
       const int hi = __shfl_sync(kFull, my_hi, i);
-      const int len = __shfl_sync(kFull, my_full, i);
       V acc[CPL];
       start_row(rb + i, acc, i + 1 < nrows);
       for (int b = lo; b < hi; b += 32) {
         add_edges<E, VEC, G, CPL, SCALED, SEG>(xrow, row_bytes, cur_u, cur_s, 0, min(hi - b, 32), grp, acc,
-                                     stage);
+                                               stage);
         cur_u = nxt_u;
         cur_s = nxt_s;
         if (qi < 32) {
@@ -556,19 +425,14 @@ __device__ __forceinline__ void ap_body(const ApArgs& a, const SelfArgs sa,
         }
       }
       combine_groups<VEC, G, CPL>(acc);
-      store_row(rb + i, len, acc);
+      store_row(rb + i, acc);
     }
-    return;
-  }
-
-  if ((int)blockIdx.x >= heavy_blocks) {
-    const int rpw = a.rows_per_warp;
-    const int64_t rb = ((int64_t)(blockIdx.x - heavy_blocks) * kWarpsPerBlock + warp) * rpw;
-    if (rb >= a.n) return;
-    const int nrows = (int)min((int64_t)rpw, a.n - rb);
-    const int my_ptr = lane <= nrows ? (int)__ldg(a.ptr + rb + lane) : 0;
-    const int stream_end = __shfl_sync(kFull, my_ptr, nrows);
-    int b = __shfl_sync(kFull, my_ptr, 0);
+  } else {
+    int my_ptr = lane <= nrows ? (int)__ldg(a.ptr + rb + lane) : 0;
+    if (lane == 0) my_ptr = here.y;
+    if (lane == nrows) my_ptr = next.y;
+    const int stream_end = next.y;
+    int b = here.y;
     int32_t cur_u, nxt_u;
     float cur_s, nxt_s;
     load_batch<SCALED>(a, b, stream_end, lane, cur_u, cur_s);
@@ -576,17 +440,6 @@ __device__ __forceinline__ void ap_body(const ApArgs& a, const SelfArgs sa,
     for (int i = 0; i < nrows; ++i) {
       const int lo = __shfl_sync(kFull, my_ptr, i);
       const int hi = __shfl_sync(kFull, my_ptr, i + 1);
-      const int len = hi - lo;
-      if (len > a.heavy_threshold) {  // a heavy block writes this row: skip its indices
-        if (hi - b >= 32) {
-          const int nb = b + ((hi - b) & ~31);
-          if (nb == b + 32) { cur_u = nxt_u; cur_s = nxt_s; }
-          else load_batch<SCALED>(a, nb, stream_end, lane, cur_u, cur_s);
-          load_batch<SCALED>(a, (int64_t)nb + 32, stream_end, lane, nxt_u, nxt_s);
-          b = nb;
-        }
-        continue;
-      }
       V acc[CPL];
       start_row(rb + i, acc, i + 1 < nrows);
       int p = lo;
@@ -602,140 +455,72 @@ __device__ __forceinline__ void ap_body(const ApArgs& a, const SelfArgs sa,
         p = b + e;
       }
       combine_groups<VEC, G, CPL>(acc);
-      store_row(rb + i, len, acc);
+      store_row(rb + i, acc);
     }
-    return;
   }
-
-  heavy_rows<E, VEC, G, CPL, SCALED, SEG, SELF, FOLD>(a, sa, heavy_blocks, part);
 }
 
-template <typename E, int VEC, int G, int CPL, bool SCALED, bool SEG, bool FOLD>
-__global__ void __launch_bounds__(kBlock) ap_kernel(const ApArgs a, const int heavy_blocks) {
-  __shared__ float part[kWarpsPerBlock][32 * CPL * VEC];
-  ap_body<E, VEC, G, CPL, SCALED, SEG, false, FOLD>(a, SelfArgs{}, heavy_blocks, part);
+// Six blocks per SM (40 registers).  Three to eight blocks are within 5 % of each other on every workload
+// (the gather is what they wait for, not the register file); six is the best for most.
+template <typename E, int VEC, int G, int CPL, bool SCALED, bool SEG>
+__global__ void __launch_bounds__(kBlock, 6) ap_kernel(const ApArgs a) {
+  ap_body<E, VEC, G, CPL, SCALED, SEG, false>(a, SelfArgs{});
 }
 
-// The same kernel compiled for six resident blocks per SM (at most 40 registers).  The scaled
-// variants with up to 16 bytes per lane and step (and at least 16 lanes per edge) carry the
-// edge factors on top of everything else and would take 60 registers; measured on B200 the
-// higher occupancy wins for them (Reddit-like backward 22.0 ms uncapped, 19.2 ms at five
-// blocks, 18.3 ms at six, 20.0 ms at seven or eight; Products-like backward 7.0 -> 5.9 ms),
-// while a cap slows the unscaled variants down.
-template <typename E, int VEC, int G, int CPL, bool SCALED, bool SEG, bool FOLD>
-__global__ void __launch_bounds__(kBlock, 6) ap_kernel_r40(const ApArgs a, const int heavy_blocks) {
-  __shared__ float part[kWarpsPerBlock][32 * CPL * VEC];
-  ap_body<E, VEC, G, CPL, SCALED, SEG, false, FOLD>(a, SelfArgs{}, heavy_blocks, part);
+// The same for graphs with implicit self loops: every row also sums its own input row.
+template <typename E, int VEC, int G, int CPL, bool SCALED, bool SEG>
+__global__ void __launch_bounds__(kBlock, 6) ap_kernel_self(const ApArgs a, const SelfArgs sa) {
+  ap_body<E, VEC, G, CPL, SCALED, SEG, true>(a, sa);
 }
 
-// Both again for graphs with implicit self loops: every row also sums its own input row.
-template <typename E, int VEC, int G, int CPL, bool SCALED, bool SEG, bool FOLD>
-__global__ void __launch_bounds__(kBlock) ap_kernel_self(const ApArgs a, const int heavy_blocks,
-                                                         const SelfArgs sa) {
-  __shared__ float part[kWarpsPerBlock][32 * CPL * VEC];
-  ap_body<E, VEC, G, CPL, SCALED, SEG, true, FOLD>(a, sa, heavy_blocks, part);
-}
-
-template <typename E, int VEC, int G, int CPL, bool SCALED, bool SEG, bool FOLD>
-__global__ void __launch_bounds__(kBlock, 6) ap_kernel_self_r40(const ApArgs a, const int heavy_blocks,
-                                                                const SelfArgs sa) {
-  __shared__ float part[kWarpsPerBlock][32 * CPL * VEC];
-  ap_body<E, VEC, G, CPL, SCALED, SEG, true, FOLD>(a, sa, heavy_blocks, part);
-}
-
-// Blocks that walk the heavy list: as many as the device keeps resident, so that the heavy
-// segments (scheduled first, longest first) have the whole machine until the list runs out.
-template <typename K>
-int heavy_block_count(const Graph* g, K kernel, size_t smem) {
-  int per_sm = (int)g->heavy_blocks_per_sm;
-  if (per_sm <= 0) {
-    if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kernel, kBlock, smem) != cudaSuccess)
-      per_sm = 2;
-  }
-  return g->sm_count * (per_sm < 1 ? 1 : per_sm);
-}
-
-// FOLD: the graph may hold segments of kLongSegment entries or more in this direction.
-template <typename E, int VEC, int G, int CPL, bool SCALED, bool SELF, bool FOLD>
-dg_status_t launch_variant(const Graph* g, const ApArgs& a, const SelfArgs& sa, int slices,
-                           cudaStream_t s) {
-  // also the narrowest slices (at most 4 lanes per edge, i.e. up to 16 features per slice): their
-  // 32- and 64-byte gathers wait on latency, and six blocks per SM hide more of it than five
-  // (Proteins-like F = 8: 0.425 -> 0.384 ms, F = 16: 0.449 -> 0.429 ms)
-  constexpr bool kCapped = (SCALED && VEC * CPL * E::kBytes <= 16 && G >= 16) || G <= 4;
-  const int64_t rows_per_block = (int64_t)a.rows_per_warp * kWarpsPerBlock;
-  const int64_t light_blocks = (a.n + rows_per_block - 1) / rows_per_block;
-  // Where the cap pays depends on the graph as well: with rows sorted hub-first, or very short
-  // rows whose gathers come from DRAM, the scaled kernels run faster at their natural 60 registers
-  // (Products-like hub-first, mean backward: 6.02 -> 5.43 ms; Papers-like x0.1, mean backward:
-  // 13.9 -> 12.3 ms), while the same graph as generated and the dense-ish ones lose 8-15 % without
-  // it.  The handle says which (a.full_registers); the narrowest slices always keep the cap.
-  const bool capped = kCapped && (G <= 4 || !a.full_registers);
+template <typename E, int VEC, int G, int CPL, bool SCALED, bool SELF>
+dg_status_t launch_variant(const ApArgs& a, const SelfArgs& sa, int slices, cudaStream_t s) {
+  const dim3 grid((unsigned)((a.chunk_count + kWarpsPerBlock - 1) / kWarpsPerBlock), (unsigned)slices);
   if constexpr (SELF) {
-    void (*kernel)(const ApArgs, const int, const SelfArgs);
-    if (capped) {
-      kernel = a.seg_lo ? ap_kernel_self_r40<E, VEC, G, CPL, SCALED, true, FOLD>
-                        : ap_kernel_self_r40<E, VEC, G, CPL, SCALED, false, FOLD>;
-    } else {
-      kernel = a.seg_lo ? ap_kernel_self<E, VEC, G, CPL, SCALED, true, FOLD>
-                        : ap_kernel_self<E, VEC, G, CPL, SCALED, false, FOLD>;
-    }
-    const int heavy_blocks = heavy_block_count(g, kernel, 0);
-    dim3 grid((unsigned)(heavy_blocks + light_blocks), (unsigned)slices);
-    kernel<<<grid, kBlock, 0, s>>>(a, heavy_blocks, sa);
+    if (a.seg_lo) ap_kernel_self<E, VEC, G, CPL, SCALED, true><<<grid, kBlock, 0, s>>>(a, sa);
+    else ap_kernel_self<E, VEC, G, CPL, SCALED, false><<<grid, kBlock, 0, s>>>(a, sa);
   } else {
-    void (*kernel)(const ApArgs, const int);
-    if (capped) {
-      kernel = a.seg_lo ? ap_kernel_r40<E, VEC, G, CPL, SCALED, true, FOLD>
-                        : ap_kernel_r40<E, VEC, G, CPL, SCALED, false, FOLD>;
-    } else {
-      kernel = a.seg_lo ? ap_kernel<E, VEC, G, CPL, SCALED, true, FOLD>
-                        : ap_kernel<E, VEC, G, CPL, SCALED, false, FOLD>;
-    }
-    const int heavy_blocks = heavy_block_count(g, kernel, 0);
-    dim3 grid((unsigned)(heavy_blocks + light_blocks), (unsigned)slices);
-    kernel<<<grid, kBlock, 0, s>>>(a, heavy_blocks);
+    if (a.seg_lo) ap_kernel<E, VEC, G, CPL, SCALED, true><<<grid, kBlock, 0, s>>>(a);
+    else ap_kernel<E, VEC, G, CPL, SCALED, false><<<grid, kBlock, 0, s>>>(a);
   }
   DG_CUDA(cudaGetLastError());
   count_launches(1);
   return DG_OK;
 }
 
-template <typename E, int VEC, bool SCALED, bool SELF, bool FOLD>
-dg_status_t dispatch_shape(const Graph* g, const ApArgs& a, const SelfArgs& sa, int slices,
-                           cudaStream_t s) {
+template <typename E, int VEC, bool SCALED, bool SELF>
+dg_status_t dispatch_shape(const ApArgs& a, const SelfArgs& sa, int slices, cudaStream_t s) {
   if (a.n == 0) return DG_OK;
-  const int chunks = (a.slice_f < a.F ? a.slice_f : a.F) / VEC;  // vectors per row slice
-  if (chunks <= 2) return launch_variant<E, VEC, 2, 1, SCALED, SELF, FOLD>(g, a, sa, slices, s);
-  if (chunks <= 4) return launch_variant<E, VEC, 4, 1, SCALED, SELF, FOLD>(g, a, sa, slices, s);
-  if (chunks <= 8) return launch_variant<E, VEC, 8, 1, SCALED, SELF, FOLD>(g, a, sa, slices, s);
-  if (chunks <= 16) return launch_variant<E, VEC, 16, 1, SCALED, SELF, FOLD>(g, a, sa, slices, s);
-  if (chunks <= 32) return launch_variant<E, VEC, 32, 1, SCALED, SELF, FOLD>(g, a, sa, slices, s);
-  if (chunks <= 64) return launch_variant<E, VEC, 32, 2, SCALED, SELF, FOLD>(g, a, sa, slices, s);
-  return launch_variant<E, VEC, 32, 4, SCALED, SELF, FOLD>(g, a, sa, slices, s);
+  const int chunks = ((a.slice_f < a.F ? a.slice_f : a.F) + VEC - 1) / VEC;  // vectors per row slice
+  if (chunks <= 2) return launch_variant<E, VEC, 2, 1, SCALED, SELF>(a, sa, slices, s);
+  if (chunks <= 4) return launch_variant<E, VEC, 4, 1, SCALED, SELF>(a, sa, slices, s);
+  if (chunks <= 8) return launch_variant<E, VEC, 8, 1, SCALED, SELF>(a, sa, slices, s);
+  if (chunks <= 16) return launch_variant<E, VEC, 16, 1, SCALED, SELF>(a, sa, slices, s);
+  if (chunks <= 32) return launch_variant<E, VEC, 32, 1, SCALED, SELF>(a, sa, slices, s);
+  if (chunks <= 64) return launch_variant<E, VEC, 32, 2, SCALED, SELF>(a, sa, slices, s);
+  return launch_variant<E, VEC, 32, 4, SCALED, SELF>(a, sa, slices, s);
 }
 
-template <typename E, int VEC, bool SELF, bool FOLD>
-dg_status_t dispatch_scaled(const Graph* g, const ApArgs& a, const SelfArgs& sa, int slices,
+template <typename E, int VEC, bool SELF>
+dg_status_t dispatch_scaled(const ApArgs& a, const SelfArgs& sa, int slices,
                             cudaStream_t s) {
-  return a.w ? dispatch_shape<E, VEC, true, SELF, FOLD>(g, a, sa, slices, s)
-             : dispatch_shape<E, VEC, false, SELF, FOLD>(g, a, sa, slices, s);
+  return a.w ? dispatch_shape<E, VEC, true, SELF>(a, sa, slices, s)
+             : dispatch_shape<E, VEC, false, SELF>(a, sa, slices, s);
 }
 
 // Storage type and vector width chosen by the caller; SELF = the graph has implicit self loops
-// (sa.self_ptr is set); FOLD = the graph may hold segments of kLongSegment entries or more in this
-// direction.  The four (SELF, FOLD) combinations are compiled in translation units of their own.
-template <bool SELF, bool FOLD>
-dg_status_t dispatch_type(const Graph* g, const ApArgs& a, const SelfArgs& sa, int vec, int slices,
+// (sa.self_ptr is set); the two cases are compiled in translation units of their own.
+template <bool SELF>
+dg_status_t dispatch_type(const ApArgs& a, const SelfArgs& sa, int vec, int slices,
                           cudaStream_t s) {
   if (a.x_bf16) {
-    if (vec == 8) return dispatch_scaled<BF16, 8, SELF, FOLD>(g, a, sa, slices, s);
-    if (vec == 4) return dispatch_scaled<BF16, 4, SELF, FOLD>(g, a, sa, slices, s);
-    return dispatch_scaled<BF16, 2, SELF, FOLD>(g, a, sa, slices, s);
+    if (vec == 8) return dispatch_scaled<BF16, 8, SELF>(a, sa, slices, s);
+    if (vec == 4) return dispatch_scaled<BF16, 4, SELF>(a, sa, slices, s);
+    return dispatch_scaled<BF16, 2, SELF>(a, sa, slices, s);
   }
-  if (vec == 4) return dispatch_scaled<F32, 4, SELF, FOLD>(g, a, sa, slices, s);
-  if (vec == 2) return dispatch_scaled<F32, 2, SELF, FOLD>(g, a, sa, slices, s);
-  return dispatch_scaled<F32, 1, SELF, FOLD>(g, a, sa, slices, s);
+  if (vec == 4) return dispatch_scaled<F32, 4, SELF>(a, sa, slices, s);
+  if (vec == 2) return dispatch_scaled<F32, 2, SELF>(a, sa, slices, s);
+  return dispatch_scaled<F32, 1, SELF>(a, sa, slices, s);
 }
 
 }  // namespace

@@ -5,10 +5,9 @@
 
 namespace dg {
 
-dg_status_t launch_with_self_loops(const Graph* g, const ApArgs& a, const SelfArgs& sa, int vec,
-                                   int slices, cudaStream_t s) {
-  if (a.long_segments) return launch_with_self_loops_fold(g, a, sa, vec, slices, s);
-  return dispatch_type<true, false>(g, a, sa, vec, slices, s);
+dg_status_t launch_with_self_loops(const ApArgs& a, const SelfArgs& sa, int vec, int slices,
+                                   cudaStream_t s) {
+  return dispatch_type<true>(a, sa, vec, slices, s);
 }
 
 }  // namespace dg

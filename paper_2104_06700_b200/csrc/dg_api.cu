@@ -39,99 +39,147 @@ static bool overlaps(const void* a, size_t a_bytes, const void* b, size_t b_byte
   return x < y + b_bytes && y < x + a_bytes;
 }
 
-static dg_status_t free_owned(Graph* g) {
-  if (g->heavy_rows) cudaFree(g->heavy_rows);
-  if (g->heavy_cols) cudaFree(g->heavy_cols);
-  if (g->counters) cudaFree(g->counters);
-  if (g->split_csr) cudaFree(g->split_csr);
-  g->split_csr = nullptr;
-  if (g->long_cols_host) cudaFreeHost(g->long_cols_host);
-  g->long_cols_host = nullptr;
-  if (g->long_cols_ready) cudaEventDestroy(g->long_cols_ready);
-  g->long_cols_ready = nullptr;
+static inline size_t align256(size_t x) { return (x + 255) & ~(size_t)255; }
 
+// Returns everything a handle holds; kernels that still read it may be queued on any stream.
+static void free_owned(Graph* g) {
+  pool_retire(g->device, g->owned, g->owned_bytes);
+  pool_retire(g->device, g->plan_memory, g->plan_bytes);
+  pinned_counters_retire(g->host);
+  if (g->col_totals_ready) cudaEventDestroy(g->col_totals_ready);
   for (size_t i = 0; i < g->aux_event_count; ++i) cudaEventDestroy(g->aux_events[i]);
   free(g->aux_events);
-  g->aux_events = nullptr;
-  g->aux_event_count = 0;
-  if (g->aux_ready) {
+  if (g->aux_ready)
     for (int i = 0; i < 2; ++i) cudaStreamDestroy(g->aux_stream[i]);
-    g->aux_ready = false;
-  }
-  g->heavy_rows = g->heavy_cols = g->counters = nullptr;
-  return DG_OK;
+  pool_close(g->device);
 }
 
-// (Re)builds the heavy lists for the current threshold; called at create, after a transpose
-// and after the threshold changes.
+// Rows longer than this are put on the heavy list of the general kernels.
+static int64_t list_threshold(const Graph* g) { return g->heavy_threshold > 0 ? g->heavy_threshold : 1024; }
+
 static dg_status_t refresh_heavy(Graph* g, bool csr, bool csc, cudaStream_t s) {
   if (csr)
-    if (dg_status_t st = build_heavy_list(g->rowptr, g->n, g->heavy_threshold, g->heavy_rows,
-                                          g->heavy_cap, g->counters + 0, s))
+    if (dg_status_t st = build_heavy_list(g->rowptr, g->n, list_threshold(g), g->heavy_rows, g->heavy_cap,
+                                          g->counters + kHeavyRowCount, s))
       return st;
   if (csc && g->transposed)
-    if (dg_status_t st = build_heavy_list(g->colptr, g->n, g->heavy_threshold, g->heavy_cols,
-                                          g->heavy_cap, g->counters + 1, s))
+    if (dg_status_t st = build_heavy_list(g->colptr, g->n, list_threshold(g), g->heavy_cols, g->heavy_cap,
+                                          g->counters + kHeavyColCount, s))
       return st;
   return DG_OK;
 }
 
-// Index of the length class of the heavy-list builder at which segments of 2^15 entries start;
-// after the list is filled, counter [class] holds the number of segments in that class or above.
-constexpr int kLongClass = 30;
+// Cost of a chunk (see Plan).  A large graph gets chunks of 1024: long enough to hide their start-up,
+// short enough that a late one does not matter.  A smaller one is cut into kChunksPerSm chunks per SM, so
+// that every SM has warps to hide latency with and the last wave is short; under 64 entries only half as
+// many, because more cut rows make the join dearer, and never under 32 (one index batch).  Measured, us
+// of both directions with their joins at 32 / 64 / 128 / 256: 65 k edges, F = 64: 15 / 19 / 27 / 39;
+// 1.2 M, F = 47: 72 / 66 / 67 / 74; 6.2 M, F = 100: 454 / 392 / 379 / 396; 16 M, F = 64 (columns up to
+// 10^5 entries): 1286 / 1040 / 930 / 892.
+// Rows up to twice a chunk stay whole: four times costs 2 to 15 % on the same graphs.
+constexpr int64_t kMaxChunk = 1024, kMinChunk = 32, kChunksPerSm = 320, kRowCost = 8;
+static int64_t chunk_cost(const Graph* g) {
+  const int64_t total = g->nnz + kRowCost * g->n;
+  int64_t cost;
+  if (g->rows_per_block > 0) {  // the caller's rows per warp, at the average row length
+    cost = (g->rows_per_block + 7) / 8 * (g->nnz / (g->n > 0 ? g->n : 1) + kRowCost);
+    cost = cost < 32 ? 32 : cost;
+  } else {
+    cost = total / (g->sm_count * kChunksPerSm);
+    if (cost < 64) cost = 2 * cost < 64 ? 2 * cost : 64;
+    cost = cost < kMinChunk ? kMinChunk : cost > kMaxChunk ? kMaxChunk : cost;
+  }
+  return (cost + 31) & ~(int64_t)31;
+}
+// Cost of a row beside its entries; at least a 31st of a chunk, so that no chunk has more than 31 rows.
+static int64_t row_cost(const Graph* g) {
+  const int64_t least = (chunk_cost(g) + 30) / 31;
+  return least > kRowCost ? least : kRowCost;
+}
+static int64_t cut_threshold(const Graph* g) {
+  return g->heavy_threshold > 0 ? g->heavy_threshold : 2 * chunk_cost(g);
+}
 
-// Heavy columns of a fresh CSC, and the number of long ones sent to the host behind them (read
-// by the first backward pass that finds the copy finished; until then the columns count as long).
+// Takes the memory of both plans for the current chunk cost and threshold.
+static dg_status_t reserve_plans(Graph* g) {
+  const int64_t cost = chunk_cost(g);
+  const int64_t count = (g->nnz + row_cost(g) * g->n + cost - 1) / cost;
+  const int64_t cuts = g->nnz > cut_threshold(g) ? count : 0;
+  const size_t chunk_bytes = align256((size_t)(count + 1) * sizeof(Chunk));
+  const size_t cut_bytes = align256((size_t)cuts * sizeof(CutRow));
+  g->plan_bytes = 2 * (chunk_bytes + cut_bytes);
+  DG_CUDA(pool_alloc(g->device, g->plan_bytes, 0, &g->plan_memory));
+  char* p = static_cast<char*>(g->plan_memory);
+  Plan* both[2] = {&g->row_plan, &g->col_plan};
+  for (int i = 0; i < 2; ++i) {
+    Plan& plan = *both[i];
+    plan.chunks = reinterpret_cast<Chunk*>(p);
+    p += chunk_bytes;
+    plan.cuts = reinterpret_cast<CutRow*>(p);
+    p += cut_bytes;
+    plan.totals = g->counters + (i ? kColTotals : kRowTotals);
+    plan.count = count;
+    plan.max_cuts = cuts;
+    // a row of m > threshold entries holds at most m / cost + 1 boundaries
+    plan.max_slots = cuts ? g->nnz / cost + g->nnz / cut_threshold(g) + 1 : 0;
+    if (plan.max_slots > count) plan.max_slots = count;
+    plan.slots = plan.cut_rows = cuts ? -1 : 0;
+  }
+  return DG_OK;
+}
+
+static dg_status_t plan_rows(Graph* g, cudaStream_t s) {
+  return build_plan(g->rowptr, g->n, g->nnz, chunk_cost(g), row_cost(g), cut_threshold(g), g->row_plan, s);
+}
+
+static void take_row_totals(Graph* g) {
+  g->row_plan.slots = g->host->v[kRowTotals];
+  g->row_plan.cut_rows = g->host->v[kRowTotals + 1];
+}
+
+// What follows every transposition: the columns' plan, its totals sent to the host behind it (read by
+// the first backward pass that finds the copy finished; until then their bounds serve).
 dg_status_t finish_transpose(Graph* g, cudaStream_t s) {
   if (dg_status_t st = refresh_heavy(g, false, true, s)) return st;
-  g->long_cols = -1;
-  DG_CUDA(cudaMemcpyAsync(g->long_cols_host, g->heavy_cols + g->heavy_cap + kLongClass,
-                          sizeof(int32_t), cudaMemcpyDeviceToHost, s));
-  DG_CUDA(cudaEventRecord(g->long_cols_ready, s));
+  if (dg_status_t st = build_plan(g->colptr, g->n, g->nnz, chunk_cost(g), row_cost(g), cut_threshold(g), g->col_plan,
+                                     s))
+    return st;
+  if (g->col_plan.max_cuts == 0) return DG_OK;
+  g->col_plan.slots = g->col_plan.cut_rows = -1;
+  DG_CUDA(cudaMemcpyAsync(g->host->v + kColTotals, g->counters + kColTotals, 2 * sizeof(int32_t),
+                          cudaMemcpyDeviceToHost, s));
+  DG_CUDA(cudaEventRecord(g->col_totals_ready, s));
   return DG_OK;
 }
 
-// Synchronous: the heavy rows have just been (re)built on the default stream.
-static dg_status_t count_long_rows(Graph* g) {
-  int32_t longs = 0;
-  DG_CUDA(cudaMemcpy(&longs, g->heavy_rows + g->heavy_cap + kLongClass, sizeof(longs),
-                     cudaMemcpyDeviceToHost));
-  g->long_rows = longs > 0 ? 1 : 0;
-  return DG_OK;
-}
-
-// Graphs on which the scaled kernels run better without their register cap: renamed hub-first,
-// or fewer than 32 edges per vertex (see launch_variant).
-static int full_registers(const Graph* g) {
-  return g->degree_ordered || (g->n > 0 && g->nnz < 32 * g->n);
-}
-
-static int long_columns(Graph* g) {
-  if (g->long_cols < 0) {
-    if (cudaEventQuery(g->long_cols_ready) == cudaSuccess)
-      g->long_cols = *g->long_cols_host > 0 ? 1 : 0;
-    else
+static const Plan& column_plan(Graph* g) {
+  if (g->col_plan.slots < 0) {
+    if (cudaEventQuery(g->col_totals_ready) == cudaSuccess) {
+      g->col_plan.slots = g->host->v[kColTotals];
+      g->col_plan.cut_rows = g->host->v[kColTotals + 1];
+    } else {
       (void)cudaGetLastError();  // "not ready" must not be mistaken for a failed launch later
+    }
   }
-  return g->long_cols != 0;
+  return g->col_plan;
 }
 
-// rows_per_block is rounded up to a whole number of rows per warp (8 warps per block).  0 picks
-// about 1024 edges per warp, between 4 and 31 rows: short rows want long-lived blocks (less
-// block turnover), long rows want many blocks.
-static int32_t rows_per_warp(const Graph* g) {
-  int64_t r;
-  if (g->rows_per_block > 0) {
-    r = (g->rows_per_block + 7) / 8;
-  } else {
-    const double avg = g->n > 0 ? (double)g->nnz / (double)g->n : 1.0;
-    r = (int64_t)(1024.0 / (avg > 1.0 ? avg : 1.0));
-    if (r < 4) r = 4;
-    // small graphs: keep at least 64 warps' worth of row runs per SM
-    const int64_t fill = g->n / ((int64_t)g->sm_count * 64);
-    if (r > fill) r = fill;
-  }
-  return (int32_t)(r < 1 ? 1 : (r > 31 ? 31 : r));
+// New plans for a changed chunk cost or threshold.  The old ones may be in use, or being built, on any
+// stream: waits for the device on both sides.
+static dg_status_t replan(Graph* g) {
+  DG_CUDA(cudaDeviceSynchronize());
+  pool_device_is_idle(g->device);
+  pool_retire(g->device, g->plan_memory, g->plan_bytes);
+  g->plan_memory = nullptr;
+  if (dg_status_t st = reserve_plans(g)) return st;
+  if (dg_status_t st = refresh_heavy(g, true, false, 0)) return st;
+  if (dg_status_t st = plan_rows(g, 0)) return st;
+  DG_CUDA(cudaMemcpyAsync(g->host, g->counters, sizeof(HostCounters), cudaMemcpyDeviceToHost, 0));
+  if (g->transposed)
+    if (dg_status_t st = finish_transpose(g, 0)) return st;
+  DG_CUDA(cudaDeviceSynchronize());
+  take_row_totals(g);
+  return DG_OK;
 }
 
 static dg_status_t check_features(const Graph* g, const void* in, size_t in_elem_bytes, float* out,
@@ -164,18 +212,11 @@ static dg_status_t run_forward(Graph* g, const void* H, bool bf16, int32_t F, dg
   a.X = H;
   a.x_bf16 = bf16;
   a.Y = out;
-  a.heavy_list = g->heavy_rows;
-  a.heavy_count = g->counters + 0;
-  a.heavy_cap = (int32_t)g->heavy_cap;
   a.n = g->n;
   a.F = F;
   a.mean_rows = op == DG_OP_MEAN;
-  a.heavy_threshold = (int32_t)g->heavy_threshold;
-  a.rows_per_warp = rows_per_warp(g);
-  a.long_segments = g->long_rows;
-  a.full_registers = full_registers(g);
   const SelfArgs sa{g->self_loops ? g->rowptr : nullptr, op == DG_OP_MEAN};
-  return aggregate_run(g, a, sa, g->split_csr, (cudaStream_t)stream);
+  return aggregate_run(g, a, sa, g->row_plan, g->split_csr, (cudaStream_t)stream);
 }
 
 static dg_status_t run_backward(Graph* g, const void* dOut, bool bf16, int32_t F, dg_op_t op,
@@ -196,18 +237,11 @@ static dg_status_t run_backward(Graph* g, const void* dOut, bool bf16, int32_t F
   a.X = dOut;
   a.x_bf16 = bf16;
   a.Y = dH;
-  a.heavy_list = g->heavy_cols;
-  a.heavy_count = g->counters + 1;
-  a.heavy_cap = (int32_t)g->heavy_cap;
   a.n = g->n;
   a.F = F;
   a.mean_rows = 0;
-  a.heavy_threshold = (int32_t)g->heavy_threshold;
-  a.rows_per_warp = rows_per_warp(g);
-  a.long_segments = long_columns(g);
-  a.full_registers = full_registers(g);
   const SelfArgs sa{g->self_loops ? g->rowptr : nullptr, op == DG_OP_MEAN};
-  return aggregate_run(g, a, sa, g->split_csc, (cudaStream_t)stream);
+  return aggregate_run(g, a, sa, column_plan(g), g->split_csc, (cudaStream_t)stream);
 }
 
 // sum_k w_k X[idx[k]] over the CSR rows (or the CSC columns) with the sum / mean kernels, for
@@ -222,16 +256,10 @@ dg_status_t aggregate_sum(Graph* g, bool over_csc, const float* w, const float* 
   a.w = w;
   a.X = X;
   a.Y = Y;
-  a.heavy_list = over_csc ? g->heavy_cols : g->heavy_rows;
-  a.heavy_count = g->counters + (over_csc ? 1 : 0);
-  a.heavy_cap = (int32_t)g->heavy_cap;
   a.n = g->n;
   a.F = F;
-  a.heavy_threshold = (int32_t)g->heavy_threshold;
-  a.rows_per_warp = rows_per_warp(g);
-  a.long_segments = over_csc ? long_columns(g) : g->long_rows;
-  a.full_registers = full_registers(g);
-  return aggregate_run(g, a, SelfArgs{nullptr, 0}, over_csc ? g->split_csc : g->split_csr, s);
+  return aggregate_run(g, a, SelfArgs{nullptr, 0}, over_csc ? column_plan(g) : g->row_plan,
+                       over_csc ? g->split_csc : g->split_csr, s);
 }
 
 static dg_status_t malformed(int flags) {
@@ -267,51 +295,61 @@ dg_status_t dg_graph_create(int64_t n, int64_t nnz, const int64_t* rowptr,
   g->rowptr = rowptr;
   g->colidx = colidx;
   g->edge_w = edge_w;
+  // attributes, not cudaGetDeviceProperties: that call alone took 2.6 ms
+  int l2 = 0;
   cudaError_t e = cudaGetDevice(&g->device);
-  cudaDeviceProp prop;
-  if (e == cudaSuccess) e = cudaGetDeviceProperties(&prop, g->device);
-  if (e != cudaSuccess) { delete g; return cuda_fail(e, "cudaGetDeviceProperties"); }
-  g->sm_count = prop.multiProcessorCount;
-  g->l2_bytes = (size_t)prop.l2CacheSize;
+  if (e == cudaSuccess) e = cudaDeviceGetAttribute(&g->sm_count, cudaDevAttrMultiProcessorCount, g->device);
+  if (e == cudaSuccess) e = cudaDeviceGetAttribute(&l2, cudaDevAttrL2CacheSize, g->device);
+  if (e == cudaSuccess) e = pool_open(g->device);
+  if (e != cudaSuccess) { delete g; return cuda_fail(e, "device query"); }
+  g->l2_bytes = (size_t)l2;
   g->l2_budget_bytes = (int64_t)(g->l2_bytes * 19 / 40);  // 60 of 126 MB measured best on B200
   g->fine_rows = (n + kFineBlocks - 1) / kFineBlocks;
   if (g->fine_rows < 1) g->fine_rows = 1;
   g->heavy_cap = nnz / 64 + 1;  // enough for any threshold >= 64
   if (g->heavy_cap > n) g->heavy_cap = n > 0 ? n : 1;
 
-  // The caller may have produced the arrays on any stream: wait for the device once, then
-  // everything below runs on the default stream and is waited for before the call returns.
+  // The caller may have produced the arrays on any stream: wait for the device once, then everything
+  // below runs on the default stream and is waited for once, at the end.
+  dg_status_t st = DG_OK;
   e = cudaDeviceSynchronize();
-  if (e == cudaSuccess) e = cudaMalloc(&g->heavy_rows, (size_t)(g->heavy_cap + kHeavyListExtra) * sizeof(int32_t));
-  if (e == cudaSuccess) e = cudaMalloc(&g->heavy_cols, (size_t)(g->heavy_cap + kHeavyListExtra) * sizeof(int32_t));
-  if (e == cudaSuccess) e = cudaMalloc(&g->counters, 4 * sizeof(int32_t));
-  if (e == cudaSuccess) e = cudaHostAlloc(&g->long_cols_host, sizeof(int32_t), cudaHostAllocDefault);
-  if (e == cudaSuccess) e = cudaEventCreateWithFlags(&g->long_cols_ready, cudaEventDisableTiming);
-  if (e == cudaSuccess) e = cudaMemset(g->counters, 0, 4 * sizeof(int32_t));
-  if (e == cudaSuccess && wants_split(n, nnz))
-    e = cudaMalloc(&g->split_csr, (size_t)(kFineBlocks + 1) * (size_t)n * sizeof(int32_t));
-  if (e != cudaSuccess) { free_owned(g); delete g; return cuda_fail(e, "cudaMalloc (graph metadata)"); }
+  if (e == cudaSuccess) pool_device_is_idle(g->device);
+  const bool split = wants_split(n, nnz);
+  const size_t counter_bytes = align256(sizeof(HostCounters));
+  const size_t list_bytes = align256((size_t)(g->heavy_cap + kHeavyListExtra) * sizeof(int32_t));
+  const size_t split_bytes = split ? align256((size_t)(kFineBlocks + 1) * (size_t)n * sizeof(int32_t)) : 0;
+  g->owned_bytes = counter_bytes + 2 * list_bytes + split_bytes;
+  if (e == cudaSuccess) e = pool_alloc(g->device, g->owned_bytes, 0, &g->owned);
+  if (e == cudaSuccess) e = pinned_counters(g->device, &g->host);
+  if (e == cudaSuccess) e = cudaEventCreateWithFlags(&g->col_totals_ready, cudaEventDisableTiming);
+  if (e == cudaSuccess) {
+    char* p = static_cast<char*>(g->owned);
+    g->counters = reinterpret_cast<int32_t*>(p);
+    g->heavy_rows = reinterpret_cast<int32_t*>(p + counter_bytes);
+    g->heavy_cols = reinterpret_cast<int32_t*>(p + counter_bytes + list_bytes);
+    if (split) g->split_csr = reinterpret_cast<int32_t*>(p + counter_bytes + 2 * list_bytes);
+    e = cudaMemsetAsync(g->counters, 0, sizeof(HostCounters), 0);
+  }
+  if (e != cudaSuccess) st = cuda_fail(e, "graph metadata");
 
   // The kernels gather X[colidx[k]] without a range check, so a malformed CSR must never reach
   // them: one streaming pass over rowptr and colidx here (about a millisecond per 10^9 edges).
-  int flags = 0;
-  dg_status_t st = validate_csr(g, 0, &flags);
-  if (st == DG_OK && flags) st = malformed(flags);
+  if (st == DG_OK) st = reserve_plans(g);
+  if (st == DG_OK) st = check_csr(g, g->counters + kFlags, 0);
   if (st == DG_OK) st = refresh_heavy(g, true, false, 0);
-  if (st == DG_OK && g->split_csr)
-    st = build_split(rowptr, colidx, n, g->fine_rows, g->split_csr, g->counters + 3, 0);
-  if (st == DG_OK) st = count_long_rows(g);
+  if (st == DG_OK) st = plan_rows(g, 0);
+  if (st == DG_OK && split)
+    st = build_split(rowptr, colidx, n, g->fine_rows, g->split_csr, g->counters + kUnsorted,
+                     g->counters + kFlags, 0);
   if (st == DG_OK) {
-    int32_t unsorted = 0;
-    e = cudaMemcpy(&unsorted, g->counters + 3, sizeof(unsorted), cudaMemcpyDeviceToHost);
-    if (e == cudaSuccess) e = cudaDeviceSynchronize();
-    if (e != cudaSuccess) st = cuda_fail(e, "cudaDeviceSynchronize (graph create)");
-    if (st == DG_OK && unsorted && g->split_csr) {  // rows not sorted: no source blocking
-      cudaFree(g->split_csr);
-      g->split_csr = nullptr;
-    }
+    e = cudaMemcpyAsync(g->host, g->counters, sizeof(HostCounters), cudaMemcpyDeviceToHost, 0);
+    if (e == cudaSuccess) e = cudaStreamSynchronize(0);
+    if (e != cudaSuccess) st = cuda_fail(e, "graph create");
   }
+  if (st == DG_OK && g->host->v[kFlags]) st = malformed(g->host->v[kFlags]);
   if (st != DG_OK) { free_owned(g); delete g; return st; }
+  take_row_totals(g);
+  if (g->host->v[kUnsorted]) g->split_csr = nullptr;  // rows not sorted: no source blocking
   *out_graph = g;
   return DG_OK;
 }
@@ -325,8 +363,11 @@ dg_status_t dg_graph_destroy(dg_graph_t g) {
 
 dg_status_t dg_graph_validate(dg_graph_t g, void* stream) {
   if (!g) return invalid("graph handle is NULL");
-  int flags = 0;
-  if (dg_status_t st = validate_csr(g, (cudaStream_t)stream, &flags)) return st;
+  cudaStream_t s = (cudaStream_t)stream;
+  int32_t flags = 0;
+  if (dg_status_t st = check_csr(g, g->counters + kFlags, s)) return st;
+  DG_CUDA(cudaMemcpyAsync(&flags, g->counters + kFlags, sizeof(flags), cudaMemcpyDeviceToHost, s));
+  DG_CUDA(cudaStreamSynchronize(s));
   return flags ? malformed(flags) : DG_OK;
 }
 
@@ -508,15 +549,8 @@ dg_status_t dg_graph_set_param(dg_graph_t g, const char* name, int64_t value) {
   if (!g || !name) return invalid("graph handle or name is NULL");
   if (!strcmp(name, "heavy_threshold")) {
     if (value < 64 || value > (1 << 30)) return invalid("heavy_threshold must be in [64, 2^30]");
-    // the lists may be in use, or being built, on any stream: wait for the device on both sides
-    DG_CUDA(cudaDeviceSynchronize());
     g->heavy_threshold = value;
-    if (dg_status_t st = refresh_heavy(g, true, false, 0)) return st;
-    if (dg_status_t st = count_long_rows(g)) return st;
-    if (g->transposed)
-      if (dg_status_t st = finish_transpose(g, 0)) return st;
-    DG_CUDA(cudaDeviceSynchronize());
-    return DG_OK;
+    return replan(g);
   }
   if (!strcmp(name, "slice_features")) {
     if (value < 0 || value > (1 << 20)) return invalid("slice_features must be in [0, 2^20]");
@@ -525,8 +559,9 @@ dg_status_t dg_graph_set_param(dg_graph_t g, const char* name, int64_t value) {
   }
   if (!strcmp(name, "rows_per_block")) {
     if (value < 0 || value > 248) return invalid("rows_per_block must be in [0, 248]");
+    if (value == g->rows_per_block) return DG_OK;
     g->rows_per_block = value;
-    return DG_OK;
+    return replan(g);
   }
   if (!strcmp(name, "l2_budget_mb")) {
     if (value < 1 || value > 4096) return invalid("l2_budget_mb must be in [1, 4096]");
@@ -554,7 +589,7 @@ dg_status_t dg_graph_set_param(dg_graph_t g, const char* name, int64_t value) {
 
 dg_status_t dg_graph_get_param(dg_graph_t g, const char* name, int64_t* value) {
   if (!g || !name || !value) return invalid("graph handle, name or value is NULL");
-  if (!strcmp(name, "heavy_threshold")) { *value = g->heavy_threshold; return DG_OK; }
+  if (!strcmp(name, "heavy_threshold")) { *value = cut_threshold(g); return DG_OK; }
   if (!strcmp(name, "slice_features")) { *value = g->slice_features; return DG_OK; }
   if (!strcmp(name, "rows_per_block")) { *value = g->rows_per_block; return DG_OK; }
   if (!strcmp(name, "l2_budget_mb")) { *value = g->l2_budget_bytes >> 20; return DG_OK; }

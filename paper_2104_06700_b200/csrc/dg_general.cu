@@ -949,6 +949,8 @@ void plan_pieces(const dg_graph* g, int32_t F, int gathered, const int32_t* spli
   if ((double)g->n * row_bytes <= budget) *slice = w;
 }
 
+int64_t list_threshold(const dg_graph* g) { return g->heavy_threshold > 0 ? g->heavy_threshold : 1024; }
+
 inline unsigned warp_blocks(int64_t n) { return (unsigned)((n + kGenWarps - 1) / kGenWarps); }
 
 template <template <int, int> class L>
@@ -1106,11 +1108,11 @@ dg_status_t dg_ap_fwd(dg_graph_t g, const float* fV, const float* fE, int32_t fE
   if (binary != DG_BIN_COPY_LHS && a.cols != 1) both |= (uintptr_t)fE;
   a.vec = (F % 4 == 0 && (both & 15) == 0) ? 4 : (F % 2 == 0 && (both & 7) == 0) ? 2 : 1;
   a.log_g = log_group(F / a.vec);
-  if (g->nnz > g->heavy_threshold) {  // only then can a row be on the heavy list
+  if (g->nnz > list_threshold(g)) {  // only then can a row be on the heavy list
     a.heavy_list = g->heavy_rows;
-    a.heavy_count = g->counters + 0;
+    a.heavy_count = g->counters + kHeavyRowCount;
     a.heavy_cap = (int32_t)g->heavy_cap;
-    a.heavy_threshold = (int32_t)g->heavy_threshold;
+    a.heavy_threshold = (int32_t)list_threshold(g);
     a.heavy_blocks = g->sm_count * 4;
   }
   int64_t slice;
@@ -1161,11 +1163,11 @@ dg_status_t dg_ap_bwd(dg_graph_t g, const float* dO, const float* fV, const floa
         if (reduce != DG_RED_SUM) both |= (uintptr_t)arg;
         a.vec = (F % 4 == 0 && (both & 15) == 0) ? 4 : (F % 2 == 0 && (both & 7) == 0) ? 2 : 1;
         a.log_g = log_group(F / a.vec);
-        if (g->nnz > g->heavy_threshold) {  // the heavy columns of the CSC
+        if (g->nnz > list_threshold(g)) {  // the heavy columns of the CSC
           a.heavy_list = g->heavy_cols;
-          a.heavy_count = g->counters + 1;
+          a.heavy_count = g->counters + kHeavyColCount;
           a.heavy_cap = (int32_t)g->heavy_cap;
-          a.heavy_threshold = (int32_t)g->heavy_threshold;
+          a.heavy_threshold = (int32_t)list_threshold(g);
           a.heavy_blocks = g->sm_count * 4;
         }
         int64_t slice;
@@ -1201,11 +1203,11 @@ dg_status_t dg_ap_bwd(dg_graph_t g, const float* dO, const float* fV, const floa
       if (F % 4 == 0 && (all & 15) == 0) a.vec = 4;
     }
     a.log_g = log_group(F / a.vec);
-    if (g->nnz > g->heavy_threshold) {
+    if (g->nnz > list_threshold(g)) {
       a.heavy_list = g->heavy_rows;
-      a.heavy_count = g->counters + 0;
+      a.heavy_count = g->counters + kHeavyRowCount;
       a.heavy_cap = (int32_t)g->heavy_cap;
-      a.heavy_threshold = (int32_t)g->heavy_threshold;
+      a.heavy_threshold = (int32_t)list_threshold(g);
       a.heavy_blocks = g->sm_count * 4;
     }
     if (cols == 1)
@@ -1233,9 +1235,9 @@ dg_status_t dg_aggregate_edge_grad(dg_graph_t g, const float* H, const float* dO
   a.dOut = dOut;
   a.dW = dW;
   a.heavy_list = g->heavy_rows;
-  a.heavy_count = g->counters + 0;
+  a.heavy_count = g->counters + kHeavyRowCount;
   a.heavy_cap = (int32_t)g->heavy_cap;
-  a.heavy_threshold = (int32_t)g->heavy_threshold;
+  a.heavy_threshold = (int32_t)list_threshold(g);
   a.n = g->n;
   a.F = F;
   a.row_scale = op == DG_OP_MEAN ? (g->self_loops ? 2 : 1) : 0;

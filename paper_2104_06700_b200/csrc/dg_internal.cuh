@@ -8,6 +8,40 @@
 
 #include "dg.h"
 
+namespace dg {
+
+// One warp's share of a pass over the CSR rows (or CSC columns): the entries [pos, next chunk's
+// pos), which belong to the rows from `row` up to the next chunk's row.  Chunks hold about the same
+// number of entries.  They begin at row starts, except inside rows longer than the split threshold:
+// such a row is cut, and a chunk that begins inside a row (slot >= 0) leaves its part of that row in
+// slot `slot` of a scratch array instead of in the output; a second small launch adds the slots of
+// every cut row to what its first chunk stored, in order (see dg_aggregate.cu).
+struct Chunk {
+  int32_t row, pos, slot, pad;
+};
+// A cut row: the chunks first .. first + count - 1 begin inside it.
+struct CutRow {
+  int32_t row, first, count, pad;
+};
+// The chunks of one direction; the arrays are owned by the handle.
+struct Plan {
+  Chunk* chunks = nullptr;    // count + 1 entries, the last one is (n, nnz)
+  CutRow* cuts = nullptr;     // the cut rows, in any order
+  int32_t* totals = nullptr;  // device: [0] slots, [1] cut rows
+  int64_t count = 0;
+  int64_t max_slots = 0, max_cuts = 0;  // bounds known from n and nnz alone
+  int32_t slots = -1, cut_rows = -1;    // the totals, or -1 while they are on their way to the host
+};
+
+// Device counters of a handle, and their order in the pinned copy.
+enum { kHeavyRowCount, kHeavyColCount, kFlags, kUnsorted, kRowTotals, kColTotals = kRowTotals + 2,
+       kCounters = kColTotals + 2 };
+struct HostCounters {
+  int32_t v[kCounters];
+};
+
+}  // namespace dg
+
 // What a handle records.  CSR and CSC arrays are borrowed; the small arrays below are owned.
 struct dg_graph {
   int64_t n = 0, nnz = 0;
@@ -15,9 +49,16 @@ struct dg_graph {
   const int32_t* colidx = nullptr;
   const float* edge_w = nullptr;
 
+  // one block of device memory behind the arrays below, and one behind the two plans
+  void* owned = nullptr;
+  size_t owned_bytes = 0;
+  void* plan_memory = nullptr;
+  size_t plan_bytes = 0;
+  dg::Plan row_plan, col_plan;   // CSR rows (forward), CSC columns (backward)
+
   int32_t* heavy_rows = nullptr; // CSR rows longer than heavy_threshold (forward)
   int32_t* heavy_cols = nullptr; // CSC columns longer than heavy_threshold (backward)
-  int32_t* counters = nullptr;   // [0] #heavy rows, [1] #heavy cols, [2] validation flags
+  int32_t* counters = nullptr;   // kCounters device words, see the enum below
   int64_t heavy_cap = 0;         // capacity of each heavy list (kHeavyListExtra more ints are allocated)
 
   // Source blocking: the neighbour ids are cut into kFineBlocks ranges of fine_rows ids;
@@ -34,13 +75,9 @@ struct dg_graph {
   cudaEvent_t* aux_events = nullptr;  // malloc'ed pool, aux_event_count entries
   size_t aux_event_count = 0;
 
-  // Whether a CSR row / CSC column of 2^15 entries or more exists (1), does not (0), or is not
-  // known yet (-1: the count of the last transposition is still on its way to the host).  Such
-  // graphs run the kernels compiled with the two-level sum of the block-per-row path.
-  int long_rows = 1;
-  int long_cols = -1;
-  int32_t* long_cols_host = nullptr;     // pinned; written by a copy enqueued after a transposition
-  cudaEvent_t long_cols_ready = nullptr; // recorded behind that copy
+  // pinned copy of `counters`; col_plan's totals arrive in it some time after a transposition
+  dg::HostCounters* host = nullptr;
+  cudaEvent_t col_totals_ready = nullptr;  // recorded behind that copy
 
   bool transposed = false;
   const int64_t* colptr = nullptr;
@@ -59,11 +96,10 @@ struct dg_graph {
   int device = 0;
   int sm_count = 148;
   size_t l2_bytes = 0;
-  int64_t heavy_threshold = 1024;
-  int64_t heavy_built_for = 0;   // threshold the heavy lists were built with
+  int64_t heavy_threshold = 0;   // rows longer than this are cut; 0 = automatic
   int64_t slice_features = 0;    // 0 = automatic
   int64_t rows_per_block = 0;    // 0 = from the average row length
-  int64_t heavy_blocks_per_sm = 0;  // blocks per SM that walk the heavy list; 0 = all resident ones
+  int64_t heavy_blocks_per_sm = 0;  // recorded for dg_graph_get_param, no effect
   int64_t l2_budget_bytes = 0;   // bytes of the gathered matrix one launch may keep L2-resident
   int64_t source_blocks = 0;     // 0 = automatic, else 1, 2, 4, 8 or 16
 };
@@ -83,22 +119,19 @@ struct ApArgs {
   const int32_t* idx;         // neighbour ids (colidx or rowidx_T)
   const float* w;             // per-edge weight or nullptr
   const void* X;              // n x F input: fp32, or bf16 when x_bf16 is set
+  uint32_t row_bytes;         // distance between its rows
   int32_t x_bf16;
   float* Y;                   // n x F output
-  const int32_t* heavy_list;  // segments longer than heavy_threshold
-  const int32_t* heavy_count; // device scalar
-  int32_t heavy_cap;          // capacity of heavy_list (the count is clamped to it)
+  const Chunk* chunks;        // chunk_count + 1
+  int32_t chunk_count;
+  float* partial;             // slots x F: the parts of cut rows
   int64_t n;
   int32_t F;
   int32_t slice_f;            // features per slice (multiple of the vector width)
   int32_t mean_rows;          // 1: multiply the finished row by 1/(segment length)
-  int32_t heavy_threshold;
-  int32_t rows_per_warp;     // consecutive light segments per warp (1..31)
   const int32_t* seg_lo;      // source-blocked pass: first and one-past-last position of every
   const int32_t* seg_hi;      //   segment's piece (n entries each); nullptr = whole segments
   int32_t accumulate;         // source-blocked pass after the first: add to what Y holds
-  int32_t long_segments;      // host side only: a segment of 2^15 entries or more may exist
-  int32_t full_registers;     // host side only: run the scaled kernels without the register cap
 };
 
 // Implicit self loops (every vertex its own neighbour with weight 1): row r also receives
@@ -114,15 +147,9 @@ struct SelfArgs {
 
 // One launch of the aggregation kernels in the shape aggregate_run chose (dg_aggregate.cu,
 // dg_aggregate_self.cu).
-dg_status_t launch_plain(const dg_graph* g, const ApArgs& a, int vec, int slices, cudaStream_t s);
-dg_status_t launch_with_self_loops(const dg_graph* g, const ApArgs& a, const SelfArgs& sa, int vec,
-                                   int slices, cudaStream_t s);
-// the same with the two-level sum for long segments (dg_aggregate_fold.cu, dg_aggregate_self_fold.cu)
-dg_status_t launch_plain_fold(const dg_graph* g, const ApArgs& a, int vec, int slices,
-                              cudaStream_t s);
-dg_status_t launch_with_self_loops_fold(const dg_graph* g, const ApArgs& a, const SelfArgs& sa,
-                                        int vec, int slices, cudaStream_t s);
-
+dg_status_t launch_plain(const ApArgs& a, int vec, int slices, cudaStream_t s);
+dg_status_t launch_with_self_loops(const ApArgs& a, const SelfArgs& sa, int vec, int slices,
+                                   cudaStream_t s);
 // Records the calling thread's last error message (printf-style, truncated to a fixed buffer:
 // nothing on an error path allocates, so nothing can throw across the C boundary).
 void set_error(const char* fmt, ...) __attribute__((format(printf, 1, 2)));
@@ -135,13 +162,25 @@ void count_launches(int64_t k);
     if (e__ != cudaSuccess) return dg::cuda_fail(e__, #call);  \
   } while (0)
 
+// dg_pool.cu: device memory of the library itself
+cudaError_t pool_open(int device);   // one per handle
+void pool_close(int device);
+void pool_device_is_idle(int device);  // the caller has just waited for the device
+cudaError_t pool_alloc(int device, size_t bytes, cudaStream_t s, void** out);
+void pool_free(void* p, cudaStream_t s);
+void pool_retire(int device, void* p, size_t bytes);  // kernels on any stream may still use it
+cudaError_t pinned_counters(int device, HostCounters** out);
+void pinned_counters_retire(HostCounters* p);
+
 // dg_graph.cu
+dg_status_t build_plan(const int64_t* ptr, int64_t n, int64_t nnz, int64_t chunk_cost, int64_t row_cost,
+                       int64_t threshold, const Plan& plan, cudaStream_t s);
 dg_status_t build_heavy_list(const int64_t* ptr, int64_t n, int64_t threshold, int32_t* list,
                              int64_t cap, int32_t* count, cudaStream_t s);
-dg_status_t validate_csr(Graph* g, cudaStream_t s, int* flags_host);
+dg_status_t check_csr(const Graph* g, int32_t* flags, cudaStream_t s);
 bool wants_split(int64_t n, int64_t nnz);
 dg_status_t build_split(const int64_t* ptr, const int32_t* idx, int64_t n, int64_t fine_rows,
-                        int32_t* split, int32_t* unsorted_flag, cudaStream_t s);
+                        int32_t* split, int32_t* unsorted_flag, const int32_t* malformed, cudaStream_t s);
 
 // dg_transpose.cu
 void transpose_sizes(int64_t n, int64_t nnz, bool weighted, size_t* csc_bytes,
@@ -164,8 +203,8 @@ dg_status_t expand_rows(const int64_t* rowptr, int64_t n, int64_t nnz, const int
                         uint32_t* out, cudaStream_t s);
 
 // dg_aggregate.cu
-dg_status_t aggregate_run(const Graph* g, const ApArgs& a, const SelfArgs& sa, const int32_t* split,
-                          cudaStream_t s);
+dg_status_t aggregate_run(const Graph* g, const ApArgs& a, const SelfArgs& sa, const Plan& plan,
+                          const int32_t* split, cudaStream_t s);
 // sum_k w_k X[idx[k]] over the CSR rows or the CSC columns with those kernels (dg_api.cu); w in
 // the order of that direction or nullptr, no self loops.
 dg_status_t aggregate_sum(Graph* g, bool over_csc, const float* w, const float* X, int32_t F,

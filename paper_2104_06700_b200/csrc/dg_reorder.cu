@@ -172,7 +172,7 @@ dg_status_t dg_graph_reorder(dg_graph_t g, dg_order_t order, const int32_t* give
 
   // ---- 1. the order
   if (n > 0 && order == DG_ORDER_GIVEN) {
-    int32_t* flags = g->counters + 2;
+    int32_t* flags = g->counters + kFlags;
     DG_CUDA(cudaMemsetAsync(flags, 0, sizeof(int32_t), s));
     DG_CUDA(cudaMemsetAsync(va, 0, (size_t)n * 4, s));
     check_permutation_kernel<<<blocks_of(n), 256, 0, s>>>(given_new_of_old, n, va, flags);

@@ -668,7 +668,8 @@ dg_status_t transpose_run(Graph* g, void* csc, void* scratch, cudaStream_t s) {
   if (wants_split(n, nnz)) {
     // the columns come out of the stable sort ordered by row, so the check never fires here
     int32_t* split = reinterpret_cast<int32_t*>(cb + L.split_off);
-    if (dg_status_t st = build_split(colptr, rowidx_T, n, g->fine_rows, split, g->counters + 3, s))
+    if (dg_status_t st = build_split(colptr, rowidx_T, n, g->fine_rows, split, g->counters + kUnsorted,
+                                       nullptr, s))
       return st;
     g->split_csc = split;
   }
