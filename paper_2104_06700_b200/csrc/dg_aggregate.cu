@@ -43,6 +43,24 @@ join_kernel(const Chunk* __restrict__ chunks, const CutRow* __restrict__ cuts,
   }
 }
 
+// out[r][0..ld) = in[r][0..F) followed by zeros, elements of T; a thread writes 16 bytes.  Reads and
+// writes are streams: bound by DRAM where the matrix exceeds L2 (561 MB of fp32 in 185 us, 6.1 TB/s read + written).
+template <typename T>
+__global__ void __launch_bounds__(256)
+pad_rows_kernel(const T* __restrict__ in, int32_t F, int32_t ld, int64_t n, uint4* __restrict__ out) {
+  constexpr int kPer = 16 / sizeof(T);
+  const uint32_t per_row = (uint32_t)ld / kPer;
+  const int64_t i = (int64_t)blockIdx.x * 256 + threadIdx.x;
+  const int64_t r = i / per_row;
+  if (r >= n) return;
+  const int f = (int)(i - r * per_row) * kPer;
+  const T* src = in + r * F + f;
+  union { T t[kPer]; uint4 v; } u;
+#pragma unroll
+  for (int q = 0; q < kPer; ++q) u.t[q] = f + q < F ? src[q] : T(0);
+  out[i] = u.v;
+}
+
 }  // namespace
 
 dg_status_t launch_plain(const ApArgs& a, int vec, int slices, cudaStream_t s) {
@@ -83,9 +101,18 @@ static double slice_footprint(int64_t F, int64_t slice, int eb) {
   return (double)(((bytes + 127) / 128) * 128 + (aligned ? 0 : 128));
 }
 
+// Whether a call first copies X into padded rows: 16-byte loads need rows that start on 16 bytes, and a
+// width like 47 or 602 (8-byte rows, or 4-byte rows in bf16) otherwise gathers every row with two to
+// four times as many, narrower loads.  The copy costs about two passes over X against nnz / n gathers of
+// every row, so it wants a mean degree of 8; rows of up to 4 elements gain nothing.  Measured
+// (kernels of a forward and a backward pass): F = 47, 1.2 M edges: 79 -> 62 us with the two copies of
+// 2.5 us; F = 602, 114.6 M edges: 34.9 -> 32.8 ms; F = 602 in bf16, 28.7 M edges: 7.5 -> 5.0 ms.
+constexpr int64_t kPadMinDegree = 8;
+constexpr size_t kPadMaxBytes = (size_t)1 << 30;  // the pool keeps this much between calls
+
 // Chooses the launch shape, then runs one launch per source block.
-//   vector width: the widest both matrices allow (16-byte loads of the gathered matrix when
-//     its rows and its base are 16-byte aligned, else 8 or 4 bytes);
+//   vector width: 16-byte loads of the gathered matrix when its rows and its base are 16-byte aligned,
+//     or of its padded copy; else 8 or 4 bytes;
 //   slice: at most 128 vectors per row slice (4 per lane);
 //   source blocks (Algorithm 2 of the paper, with L2 in the role of the CPU cache): when one
 //     slice of X over all n rows exceeds the L2 budget and the segments carry split pointers,
@@ -99,19 +126,38 @@ dg_status_t aggregate_run(const Graph* g, const ApArgs& a0, const SelfArgs& sa, 
   const uintptr_t px = (uintptr_t)a.X, py = (uintptr_t)a.Y;
   const bool bf16 = a.x_bf16 != 0;
   const int eb = bf16 ? 2 : 4;
-  int vec = 1;  // elements per lane and vector
-  if (bf16) {
-    if (a.F % 8 == 0 && px % 16 == 0 && py % 16 == 0) vec = 8;
-    else if (a.F % 4 == 0 && px % 8 == 0 && py % 16 == 0) vec = 4;
-    else if (a.F % 2 == 0 && px % 4 == 0 && py % 8 == 0) vec = 2;
-    else {
-      set_error("bf16 feature matrices need an even F and 4-byte (input) / 8-byte (output) alignment");
-      return DG_ERR_UNSUPPORTED;
-    }
-  } else {
-    if (a.F % 4 == 0 && px % 16 == 0 && py % 16 == 0) vec = 4;
-    else if (a.F % 2 == 0 && px % 8 == 0 && py % 8 == 0) vec = 2;
+  const int wide = 16 / eb;  // elements of a 16-byte load
+  if (bf16 && (a.F % 2 != 0 || px % 4 != 0 || py % 8 != 0)) {
+    set_error("bf16 feature matrices need an even F and 4-byte (input) / 8-byte (output) alignment");
+    return DG_ERR_UNSUPPORTED;
   }
+  int vec = 1;  // elements per lane and vector
+  if (a.F % wide == 0 && px % 16 == 0 && py % 16 == 0) vec = wide;
+  else if (bf16 && a.F % 4 == 0 && px % 8 == 0 && py % 16 == 0) vec = 4;
+  else if (bf16 || (a.F % 2 == 0 && px % 8 == 0 && py % 8 == 0)) vec = 2;
+  int64_t ld = a.F;
+  void* padded = nullptr;
+  if (vec < wide && a.F > 4 && g->nnz >= kPadMinDegree * a.n) {
+    // rows of whole 32-byte sectors, of whole 128-byte lines where a row has several
+    const int64_t unit = (a.F * eb > 512 ? 128 : 32) / eb;
+    const int64_t to = (a.F + unit - 1) / unit * unit;
+    const size_t bytes = (size_t)a.n * (size_t)to * (size_t)eb;
+    if (bytes <= kPadMaxBytes && pool_alloc(g->device, bytes, s, &padded) == cudaSuccess) {
+      ld = to;
+      vec = wide;
+      a.narrow_store = a.F % 4 != 0 || py % 16 != 0 || (bf16 && a.F % 8 != 0);
+      const unsigned blocks = (unsigned)((bytes / 16 + 255) / 256);
+      if (bf16)
+        pad_rows_kernel<uint16_t><<<blocks, 256, 0, s>>>(static_cast<const uint16_t*>(a.X), a.F, (int32_t)ld,
+                                                         a.n, static_cast<uint4*>(padded));
+      else
+        pad_rows_kernel<uint32_t><<<blocks, 256, 0, s>>>(static_cast<const uint32_t*>(a.X), a.F, (int32_t)ld,
+                                                         a.n, static_cast<uint4*>(padded));
+      count_launches(1);
+      a.X = padded;
+    }
+  }
+  a.row_bytes = (uint32_t)(ld * eb);
 
   const double budget = (double)g->l2_budget_bytes;
   const double avg_len = (double)g->nnz / (double)a.n;
@@ -122,23 +168,29 @@ dg_status_t aggregate_run(const Graph* g, const ApArgs& a0, const SelfArgs& sa, 
   int nb = 1;
   if (g->source_blocks > 0) {
     nb = split ? (int)g->source_blocks : 1;
-  } else if (g->slice_features <= 0 && (double)a.n * slice_footprint(a.F, slice, eb) > budget) {
+  } else if (g->slice_features <= 0 && (double)a.n * slice_footprint(ld, slice, eb) > budget) {
     if (split) {
-      // widest slice first; a candidate is feasible when some block count keeps one block of
-      // the slice inside the budget and leaves a row at least 32 edges per block on average
+      // A width is feasible when some block count keeps one block of the slice inside the budget and
+      // leaves a row at least 32 edges per block on average.  Among those, the least traffic beside the
+      // gather: every slice reads the index stream again, every block after the first reads and writes
+      // the output again.
       const int64_t widths[4] = {64LL * vec, 32LL * vec, 16LL * vec, 8LL * vec};
+      const double stream = (double)g->nnz * (a.w ? 8.0 : 4.0), output = (double)a.n * a.F * 4.0;
+      const int64_t widest = slice;
+      double best = 0.0;
       bool found = false;
-      for (int t = 0; t < 4 && !found; ++t) {
-        int64_t w = widths[t];
-        if (w > slice) w = slice;
+      for (int t = 0; t < 4; ++t) {
+        const int64_t w = widths[t] < widest ? widths[t] : widest;
         int cand = 1;
-        while (cand < kFineBlocks && (double)a.n / cand * slice_footprint(a.F, w, eb) > budget)
-          cand *= 2;
-        if ((double)a.n / cand * slice_footprint(a.F, w, eb) <= budget && avg_len / cand >= 32.0) {
+        while (cand < kFineBlocks && (double)a.n / cand * slice_footprint(ld, w, eb) > budget) cand *= 2;
+        if ((double)a.n / cand * slice_footprint(ld, w, eb) > budget || avg_len / cand < 32.0) continue;
+        const double cost = stream * (double)((a.F + w - 1) / w) + output * (2 * cand - 1);
+        if (!found || cost < best) {
+          best = cost;
           slice = w;
           nb = cand;
-          found = true;
         }
+        found = true;
       }
       if (!found) {  // as many blocks as the row length allows, narrowest slice
         nb = 1;
@@ -150,21 +202,21 @@ dg_status_t aggregate_run(const Graph* g, const ApArgs& a0, const SelfArgs& sa, 
       if (w * eb >= 128) slice = w < slice ? w : slice;  // under 128 bytes is not worth a pass
     }
   }
-  slice = (slice / vec) * vec;
+  slice = slice < a.F ? (slice / vec) * vec : ld;  // a padded row ends in a vector that reaches beyond F
   if (slice < vec) slice = vec;
   if ((a.F + slice - 1) / slice > 65535) {  // grid.y limit: widen a (requested) tiny slice
     slice = (a.F + 65534) / 65535;
     slice = ((slice + vec - 1) / vec) * vec;
   }
-  // even out the slices: same count, smallest width that covers F
+  // even out the slices: same count, smallest width that covers F (in whole lines when X is padded)
   const int64_t nsl = (a.F + slice - 1) / slice;
+  const int64_t unit = padded && nsl > 1 ? 128 / eb : vec;
   int64_t even = (a.F + nsl - 1) / nsl;
-  even = ((even + vec - 1) / vec) * vec;
+  even = ((even + unit - 1) / unit) * unit;
   if (even <= slice) slice = even;
   a.slice_f = (int32_t)slice;
   const int slices = (int)((a.F + slice - 1) / slice);
 
-  a.row_bytes = (uint32_t)(a.F * eb);
   a.chunks = plan.chunks;
   a.chunk_count = (int32_t)plan.count;
   dg_status_t st = take_partial(g, plan, a.F, s, &a.partial);
@@ -181,6 +233,7 @@ dg_status_t aggregate_run(const Graph* g, const ApArgs& a0, const SelfArgs& sa, 
     if (st == DG_OK) st = join_cut_rows(g, plan, a.partial, a.F, a.Y, s);
     pool_free(a.partial, s);
   }
+  pool_free(padded, s);
   return st;
 }
 

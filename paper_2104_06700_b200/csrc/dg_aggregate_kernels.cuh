@@ -156,6 +156,15 @@ __device__ __forceinline__ f8 shfl_xor(f8 a, int m) {
   r.hi = shfl_xor(a.hi, m);
   return r;
 }
+__device__ __forceinline__ void unpack(float (&t)[1], float v) { t[0] = v; }
+__device__ __forceinline__ void unpack(float (&t)[2], float2 v) { t[0] = v.x; t[1] = v.y; }
+__device__ __forceinline__ void unpack(float (&t)[4], float4 v) {
+  t[0] = v.x; t[1] = v.y; t[2] = v.z; t[3] = v.w;
+}
+__device__ __forceinline__ void unpack(float (&t)[8], f8 v) {
+  t[0] = v.lo.x; t[1] = v.lo.y; t[2] = v.lo.z; t[3] = v.lo.w;
+  t[4] = v.hi.x; t[5] = v.hi.y; t[6] = v.hi.z; t[7] = v.hi.w;
+}
 __device__ __forceinline__ void stcs_vec(float* p, float v) { __stcs(p, v); }
 __device__ __forceinline__ void stcs_vec(float* p, float2 v) { __stcs(reinterpret_cast<float2*>(p), v); }
 __device__ __forceinline__ void stcs_vec(float* p, float4 v) { __stcs(reinterpret_cast<float4*>(p), v); }
@@ -295,7 +304,7 @@ __device__ __forceinline__ void ap_body(const ApArgs& a, const SelfArgs sa) {
   const int f0 = blockIdx.y * a.slice_f;
   const int fend = min(a.F, f0 + a.slice_f);
   const int width = fend - f0;
-  const int chunks = width / VEC;
+  const int chunks = (width + VEC - 1) / VEC;  // the last vector of a padded X may reach beyond F
   const uint32_t row_bytes = a.row_bytes;
 
   // The shuffle tells the compiler that the warp's number, and with it everything read from the plan and
@@ -371,8 +380,17 @@ __device__ __forceinline__ void ap_body(const ApArgs& a, const SelfArgs sa) {
         if (cok[c]) {
           float* dst = orow + (c0 + c * G) * VEC;
           if (a.mean_rows) scale(acc[c], rs);
-          if (SEG && a.accumulate) add(acc[c], ld_vec(dst, V()));
-          stcs_vec(dst, acc[c]);
+          if (VEC > 1 && a.narrow_store) {  // X is a padded copy, the output is not padded
+            const int room = min(VEC, fend - f0 - (c0 + c * G) * VEC);
+            float t[VEC];
+            unpack(t, acc[c]);
+#pragma unroll
+            for (int q = 0; q < VEC; ++q)
+              if (q < room) __stcs(dst + q, SEG && a.accumulate ? dst[q] + t[q] : t[q]);
+          } else {
+            if (SEG && a.accumulate) add(acc[c], ld_vec(dst, V()));
+            stcs_vec(dst, acc[c]);
+          }
         }
       }
     }

@@ -122,6 +122,7 @@ struct ApArgs {
   uint32_t row_bytes;         // distance between its rows
   int32_t x_bf16;
   float* Y;                   // n x F output
+  int32_t narrow_store;       // 1: the rows of Y cannot take the vector width that X is read with
   const Chunk* chunks;        // chunk_count + 1
   int32_t chunk_count;
   float* partial;             // slots x F: the parts of cut rows
