@@ -108,7 +108,30 @@ static double slice_footprint(int64_t F, int64_t slice, int eb) {
 // (kernels of a forward and a backward pass): F = 47, 1.2 M edges: 79 -> 62 us with the two copies of
 // 2.5 us; F = 602, 114.6 M edges: 34.9 -> 32.8 ms; F = 602 in bf16, 28.7 M edges: 7.5 -> 5.0 ms.
 constexpr int64_t kPadMinDegree = 8;
-constexpr size_t kPadMaxBytes = (size_t)1 << 30;  // the pool keeps this much between calls
+constexpr size_t kPadMaxBytes = (size_t)1 << 30;
+bool worth_padding(const Graph* g, int32_t F, int elem_bytes) {
+  return F > 4 && g->nnz >= kPadMinDegree * g->n &&
+         (size_t)g->n * (size_t)(F + 128 / elem_bytes) * (size_t)elem_bytes <= kPadMaxBytes;
+}
+
+// Makes the copy; false when there is no memory for it (the caller then uses X as it is).
+bool pad_rows(const Graph* g, const void* X, int32_t F, int elem_bytes, cudaStream_t s, void** copy, int64_t* ld) {
+  // rows of whole 32-byte sectors, of whole 128-byte lines where a row has several
+  const int64_t unit = (F * elem_bytes > 512 ? 128 : 32) / elem_bytes;
+  const int64_t to = (F + unit - 1) / unit * unit;
+  const size_t bytes = (size_t)g->n * (size_t)to * (size_t)elem_bytes;
+  if (pool_alloc(g->device, bytes, s, copy) != cudaSuccess) return false;
+  *ld = to;
+  const unsigned blocks = (unsigned)((bytes / 16 + 255) / 256);
+  if (elem_bytes == 2)
+    pad_rows_kernel<uint16_t><<<blocks, 256, 0, s>>>(static_cast<const uint16_t*>(X), F, (int32_t)to, g->n,
+                                                     static_cast<uint4*>(*copy));
+  else
+    pad_rows_kernel<uint32_t><<<blocks, 256, 0, s>>>(static_cast<const uint32_t*>(X), F, (int32_t)to, g->n,
+                                                     static_cast<uint4*>(*copy));
+  count_launches(1);
+  return true;
+}
 
 // Chooses the launch shape, then runs one launch per source block.
 //   vector width: 16-byte loads of the gathered matrix when its rows and its base are 16-byte aligned,
@@ -137,25 +160,10 @@ dg_status_t aggregate_run(const Graph* g, const ApArgs& a0, const SelfArgs& sa, 
   else if (bf16 || (a.F % 2 == 0 && px % 8 == 0 && py % 8 == 0)) vec = 2;
   int64_t ld = a.F;
   void* padded = nullptr;
-  if (vec < wide && a.F > 4 && g->nnz >= kPadMinDegree * a.n) {
-    // rows of whole 32-byte sectors, of whole 128-byte lines where a row has several
-    const int64_t unit = (a.F * eb > 512 ? 128 : 32) / eb;
-    const int64_t to = (a.F + unit - 1) / unit * unit;
-    const size_t bytes = (size_t)a.n * (size_t)to * (size_t)eb;
-    if (bytes <= kPadMaxBytes && pool_alloc(g->device, bytes, s, &padded) == cudaSuccess) {
-      ld = to;
-      vec = wide;
-      a.narrow_store = a.F % 4 != 0 || py % 16 != 0 || (bf16 && a.F % 8 != 0);
-      const unsigned blocks = (unsigned)((bytes / 16 + 255) / 256);
-      if (bf16)
-        pad_rows_kernel<uint16_t><<<blocks, 256, 0, s>>>(static_cast<const uint16_t*>(a.X), a.F, (int32_t)ld,
-                                                         a.n, static_cast<uint4*>(padded));
-      else
-        pad_rows_kernel<uint32_t><<<blocks, 256, 0, s>>>(static_cast<const uint32_t*>(a.X), a.F, (int32_t)ld,
-                                                         a.n, static_cast<uint4*>(padded));
-      count_launches(1);
-      a.X = padded;
-    }
+  if (vec < wide && worth_padding(g, a.F, eb) && pad_rows(g, a.X, a.F, eb, s, &padded, &ld)) {
+    a.X = padded;
+    vec = wide;
+    a.narrow_store = a.F % 4 != 0 || py % 16 != 0 || (bf16 && a.F % 8 != 0);
   }
   a.row_bytes = (uint32_t)(ld * eb);
 

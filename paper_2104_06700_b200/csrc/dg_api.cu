@@ -54,21 +54,6 @@ static void free_owned(Graph* g) {
   pool_close(g->device);
 }
 
-// Rows longer than this are put on the heavy list of the general kernels.
-static int64_t list_threshold(const Graph* g) { return g->heavy_threshold > 0 ? g->heavy_threshold : 1024; }
-
-static dg_status_t refresh_heavy(Graph* g, bool csr, bool csc, cudaStream_t s) {
-  if (csr)
-    if (dg_status_t st = build_heavy_list(g->rowptr, g->n, list_threshold(g), g->heavy_rows, g->heavy_cap,
-                                          g->counters + kHeavyRowCount, s))
-      return st;
-  if (csc && g->transposed)
-    if (dg_status_t st = build_heavy_list(g->colptr, g->n, list_threshold(g), g->heavy_cols, g->heavy_cap,
-                                          g->counters + kHeavyColCount, s))
-      return st;
-  return DG_OK;
-}
-
 // Cost of a chunk (see Plan).  A large graph gets chunks of 1024: long enough to hide their start-up,
 // short enough that a late one does not matter.  A smaller one is cut into kChunksPerSm chunks per SM, so
 // that every SM has warps to hide latency with and the last wave is short; under 64 entries only half as
@@ -140,7 +125,6 @@ static void take_row_totals(Graph* g) {
 // What follows every transposition: the columns' plan, its totals sent to the host behind it (read by
 // the first backward pass that finds the copy finished; until then their bounds serve).
 dg_status_t finish_transpose(Graph* g, cudaStream_t s) {
-  if (dg_status_t st = refresh_heavy(g, false, true, s)) return st;
   if (dg_status_t st = build_plan(g->colptr, g->n, g->nnz, chunk_cost(g), row_cost(g), cut_threshold(g), g->col_plan,
                                      s))
     return st;
@@ -152,7 +136,7 @@ dg_status_t finish_transpose(Graph* g, cudaStream_t s) {
   return DG_OK;
 }
 
-static const Plan& column_plan(Graph* g) {
+const Plan& column_plan(Graph* g) {
   if (g->col_plan.slots < 0) {
     if (cudaEventQuery(g->col_totals_ready) == cudaSuccess) {
       g->col_plan.slots = g->host->v[kColTotals];
@@ -172,7 +156,6 @@ static dg_status_t replan(Graph* g) {
   pool_retire(g->device, g->plan_memory, g->plan_bytes);
   g->plan_memory = nullptr;
   if (dg_status_t st = reserve_plans(g)) return st;
-  if (dg_status_t st = refresh_heavy(g, true, false, 0)) return st;
   if (dg_status_t st = plan_rows(g, 0)) return st;
   DG_CUDA(cudaMemcpyAsync(g->host, g->counters, sizeof(HostCounters), cudaMemcpyDeviceToHost, 0));
   if (g->transposed)
@@ -306,8 +289,6 @@ dg_status_t dg_graph_create(int64_t n, int64_t nnz, const int64_t* rowptr,
   g->l2_budget_bytes = (int64_t)(g->l2_bytes * 3 / 8);  // 47 of 126 MB: see aggregate_run
   g->fine_rows = (n + kFineBlocks - 1) / kFineBlocks;
   if (g->fine_rows < 1) g->fine_rows = 1;
-  g->heavy_cap = nnz / 64 + 1;  // enough for any threshold >= 64
-  if (g->heavy_cap > n) g->heavy_cap = n > 0 ? n : 1;
 
   // The caller may have produced the arrays on any stream: wait for the device once, then everything
   // below runs on the default stream and is waited for once, at the end.
@@ -316,18 +297,15 @@ dg_status_t dg_graph_create(int64_t n, int64_t nnz, const int64_t* rowptr,
   if (e == cudaSuccess) pool_device_is_idle(g->device);
   const bool split = wants_split(n, nnz);
   const size_t counter_bytes = align256(sizeof(HostCounters));
-  const size_t list_bytes = align256((size_t)(g->heavy_cap + kHeavyListExtra) * sizeof(int32_t));
   const size_t split_bytes = split ? align256((size_t)(kFineBlocks + 1) * (size_t)n * sizeof(int32_t)) : 0;
-  g->owned_bytes = counter_bytes + 2 * list_bytes + split_bytes;
+  g->owned_bytes = counter_bytes + split_bytes;
   if (e == cudaSuccess) e = pool_alloc(g->device, g->owned_bytes, 0, &g->owned);
   if (e == cudaSuccess) e = pinned_counters(g->device, &g->host);
   if (e == cudaSuccess) e = cudaEventCreateWithFlags(&g->col_totals_ready, cudaEventDisableTiming);
   if (e == cudaSuccess) {
     char* p = static_cast<char*>(g->owned);
     g->counters = reinterpret_cast<int32_t*>(p);
-    g->heavy_rows = reinterpret_cast<int32_t*>(p + counter_bytes);
-    g->heavy_cols = reinterpret_cast<int32_t*>(p + counter_bytes + list_bytes);
-    if (split) g->split_csr = reinterpret_cast<int32_t*>(p + counter_bytes + 2 * list_bytes);
+    if (split) g->split_csr = reinterpret_cast<int32_t*>(p + counter_bytes);
     e = cudaMemsetAsync(g->counters, 0, sizeof(HostCounters), 0);
   }
   if (e != cudaSuccess) st = cuda_fail(e, "graph metadata");
@@ -336,7 +314,6 @@ dg_status_t dg_graph_create(int64_t n, int64_t nnz, const int64_t* rowptr,
   // them: one streaming pass over rowptr and colidx here (about a millisecond per 10^9 edges).
   if (st == DG_OK) st = reserve_plans(g);
   if (st == DG_OK) st = check_csr(g, g->counters + kFlags, 0);
-  if (st == DG_OK) st = refresh_heavy(g, true, false, 0);
   if (st == DG_OK) st = plan_rows(g, 0);
   if (st == DG_OK && split)
     st = build_split(rowptr, colidx, n, g->fine_rows, g->split_csr, g->counters + kUnsorted,

@@ -1,4 +1,4 @@
-// Graph ingest kernels: the lists of heavy segments, split pointers, CSR validation.
+// Graph ingest kernels: how rows are shared out among warps, split pointers, CSR validation.
 // All integer work; nothing here waits on another block.
 #include "dg_internal.cuh"
 
@@ -6,52 +6,6 @@ namespace dg {
 namespace {
 
 constexpr int kBlock = 256;
-
-// The heavy list holds every segment longer than `threshold`, longest first (in 64 length
-// classes, two per power of two): the blocks that walk it take entries x, x + B, x + 2B, ...,
-// so starting with the long ones evens out their finishing times.  The order of the list does
-// not influence any result: each heavy segment is summed by one block on its own.  The 64
-// class counters sit behind the list's `cap` entries.
-__device__ __forceinline__ int length_class(int64_t len) {
-  const int lg = 63 - __clzll(len);                     // len >= 1
-  const int half = lg > 0 ? (int)((len >> (lg - 1)) & 1) : 0;
-  const int c = 2 * lg + half;
-  return c > 63 ? 63 : c;
-}
-
-__global__ void heavy_count_kernel(const int64_t* __restrict__ ptr, int64_t n, int64_t threshold,
-                                   int32_t* __restrict__ classes, int32_t* __restrict__ count) {
-  const int64_t v = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-  if (v >= n) return;
-  const int64_t len = ptr[v + 1] - ptr[v];
-  if (len > threshold) {
-    atomicAdd(&classes[length_class(len)], 1);
-    atomicAdd(count, 1);
-  }
-}
-
-// One warp: classes[c] becomes the list position where class c starts (longest class first).
-__global__ void heavy_offsets_kernel(int32_t* __restrict__ classes) {
-  if (threadIdx.x != 0) return;
-  int32_t run = 0;
-  for (int c = 63; c >= 0; --c) {
-    const int32_t k = classes[c];
-    classes[c] = run;
-    run += k;
-  }
-}
-
-__global__ void heavy_fill_kernel(const int64_t* __restrict__ ptr, int64_t n, int64_t threshold,
-                                  int32_t* __restrict__ list, int64_t cap,
-                                  int32_t* __restrict__ classes) {
-  const int64_t v = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-  if (v >= n) return;
-  const int64_t len = ptr[v + 1] - ptr[v];
-  if (len > threshold) {
-    const int32_t slot = atomicAdd(&classes[length_class(len)], 1);
-    if (slot < cap) list[slot] = (int32_t)v;
-  }
-}
 
 // Boundary c of a plan lies at cost c * chunk_cost, where reaching entry k of row r has cost
 // k + row_cost * r: a row costs its entries and row_cost for its pointer, its index batch and its store,
@@ -166,22 +120,6 @@ __global__ void sorted_check_kernel(const int64_t* __restrict__ ptr,
 inline unsigned blocks_for(int64_t items) { return (unsigned)((items + kBlock - 1) / kBlock); }
 
 }  // namespace
-
-dg_status_t build_heavy_list(const int64_t* ptr, int64_t n, int64_t threshold, int32_t* list,
-                             int64_t cap, int32_t* count, cudaStream_t s) {
-  int32_t* classes = list + cap;  // 64 counters behind the list (see kHeavyListExtra)
-  DG_CUDA(cudaMemsetAsync(count, 0, sizeof(int32_t), s));
-  DG_CUDA(cudaMemsetAsync(classes, 0, kHeavyListExtra * sizeof(int32_t), s));
-  if (n == 0) return DG_OK;
-  heavy_count_kernel<<<blocks_for(n), kBlock, 0, s>>>(ptr, n, threshold, classes, count);
-  DG_CUDA(cudaGetLastError());
-  heavy_offsets_kernel<<<1, 32, 0, s>>>(classes);
-  DG_CUDA(cudaGetLastError());
-  heavy_fill_kernel<<<blocks_for(n), kBlock, 0, s>>>(ptr, n, threshold, list, cap, classes);
-  DG_CUDA(cudaGetLastError());
-  count_launches(3);
-  return DG_OK;
-}
 
 bool wants_split(int64_t n, int64_t nnz) {
   return n >= 4096 && nnz >= kBlockingMinAvgLen * n &&

@@ -34,8 +34,7 @@ struct Plan {
 };
 
 // Device counters of a handle, and their order in the pinned copy.
-enum { kHeavyRowCount, kHeavyColCount, kFlags, kUnsorted, kRowTotals, kColTotals = kRowTotals + 2,
-       kCounters = kColTotals + 2 };
+enum { kFlags, kUnsorted, kRowTotals, kColTotals = kRowTotals + 2, kCounters = kColTotals + 2 };
 struct HostCounters {
   int32_t v[kCounters];
 };
@@ -56,10 +55,7 @@ struct dg_graph {
   size_t plan_bytes = 0;
   dg::Plan row_plan, col_plan;   // CSR rows (forward), CSC columns (backward)
 
-  int32_t* heavy_rows = nullptr; // CSR rows longer than heavy_threshold (forward)
-  int32_t* heavy_cols = nullptr; // CSC columns longer than heavy_threshold (backward)
   int32_t* counters = nullptr;   // kCounters device words, see the enum below
-  int64_t heavy_cap = 0;         // capacity of each heavy list (kHeavyListExtra more ints are allocated)
 
   // Source blocking: the neighbour ids are cut into kFineBlocks ranges of fine_rows ids;
   // split[b * n + v] is the first position of segment v whose neighbour id is >= b * fine_rows
@@ -108,7 +104,6 @@ namespace dg {
 
 using Graph = ::dg_graph;
 
-constexpr int kHeavyListExtra = 64;      // counters of the length classes, stored behind a heavy list
 constexpr int kFineBlocks = 16;          // finest cut of the neighbour ids for source blocking
 constexpr int64_t kBlockingMinAvgLen = 64;  // split pointers are built when nnz >= 64 n
 
@@ -176,8 +171,6 @@ void pinned_counters_retire(HostCounters* p);
 // dg_graph.cu
 dg_status_t build_plan(const int64_t* ptr, int64_t n, int64_t nnz, int64_t chunk_cost, int64_t row_cost,
                        int64_t threshold, const Plan& plan, cudaStream_t s);
-dg_status_t build_heavy_list(const int64_t* ptr, int64_t n, int64_t threshold, int32_t* list,
-                             int64_t cap, int32_t* count, cudaStream_t s);
 dg_status_t check_csr(const Graph* g, int32_t* flags, cudaStream_t s);
 bool wants_split(int64_t n, int64_t nnz);
 dg_status_t build_split(const int64_t* ptr, const int32_t* idx, int64_t n, int64_t fine_rows,
@@ -202,6 +195,20 @@ dg_status_t pointers_from_sorted_keys(const uint32_t* sorted, int64_t count, int
                                       int64_t* ptr, cudaStream_t s);
 dg_status_t expand_rows(const int64_t* rowptr, int64_t n, int64_t nnz, const int32_t* map,
                         uint32_t* out, cudaStream_t s);
+
+// Whether a call first copies a gathered matrix into padded rows, and the copy (dg_aggregate.cu).
+bool worth_padding(const Graph* g, int32_t F, int elem_bytes);
+bool pad_rows(const Graph* g, const void* X, int32_t F, int elem_bytes, cudaStream_t s, void** copy, int64_t* ld);
+// Scratch for the parts of cut rows (nullptr when the plan cuts none), and their join.
+dg_status_t take_partial(const Graph* g, const Plan& plan, int64_t floats_per_slot, cudaStream_t s,
+                         float** partial);
+dg_status_t join_cut_rows(const Graph* g, const Plan& plan, const float* partial, int32_t F, float* Y,
+                          cudaStream_t s);
+// dg_edge_grad.cu
+dg_status_t edge_grad_run(const Graph* g, const float* H, const float* dOut, int32_t F, int row_scale,
+                          float* dW, cudaStream_t s);
+// dg_api.cu: the plan of the CSC, with its totals if they have arrived
+const Plan& column_plan(Graph* g);
 
 // dg_aggregate.cu
 dg_status_t aggregate_run(const Graph* g, const ApArgs& a, const SelfArgs& sa, const Plan& plan,
