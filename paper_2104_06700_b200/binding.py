@@ -103,18 +103,22 @@ def _check(status: int) -> None:
 def _dev_ptr(t: Optional[torch.Tensor], dtype, name: str):
     if t is None:
         return None
+    if t.is_cuda and t.dtype is dtype and t.is_contiguous():
+        return t.data_ptr()
     if not t.is_cuda:
         raise ValueError(f"{name} must be a CUDA tensor")
     if t.dtype != dtype:
         raise TypeError(f"{name} must be {dtype}, got {t.dtype}")
-    if not t.is_contiguous():
-        raise ValueError(f"{name} must be contiguous")
-    return ctypes.c_void_p(t.data_ptr())
+    raise ValueError(f"{name} must be contiguous")
+
+
+# The handle of the current stream of the current device.  torch.cuda.current_stream() builds two
+# Python objects on the way to it: 3.2 us, a third of what a call on a small graph took on the host.
+_raw_stream, _device = torch._C._cuda_getCurrentRawStream, torch._C._cuda_getDevice
 
 
 def _stream(stream=None):
-    s = torch.cuda.current_stream() if stream is None else stream
-    return ctypes.c_void_p(s.cuda_stream)
+    return _raw_stream(_device()) if stream is None else stream.cuda_stream
 
 
 def dg_version() -> str:

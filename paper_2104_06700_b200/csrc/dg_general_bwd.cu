@@ -88,7 +88,10 @@ __global__ void __launch_bounds__(kGenBlock, 4) general_dv_sum_kernel(const GenA
 // is feature f_lo + 32 w + j's extremum (arg is read once, nnz * words * 4 bytes are written); then
 // general_dv_mask_kernel walks the CSC, reads the words of every edge, one random sector of 32 bytes, and of
 // dO only the values that are selected.
-// @@DVMASK@@
+// Bound by instruction issue and DRAM together (68 % and 58 % busy at F = 100): about 20 instructions per
+// edge with a selected feature, and a random sector per edge for its words beside the selected values.
+// Both kernels, B200: 31 M edges F = 100 3.71 -> 1.59 ms; 16 M edges, columns up to 10^5, F = 128
+// 4.28 -> 1.63 ms; 24 M edges F = 64 0.69 -> 0.41 ms; 5.7 M edges F = 602 5.73 -> 1.30 ms.
 
 constexpr int kWindowWords = 1024;  // words of the mask a warp builds at a time
 
@@ -108,25 +111,34 @@ __global__ void __launch_bounds__(kGenBlock) arg_mask_kernel(const GenArgs a) {
     my_lo = max((int)__ldg(a.ptr + here.x + lane), here.y);
     my_hi = min((int)__ldg(a.ptr + here.x + lane + 1), next.y);
   }
-  const int width = min(32 * WORDS, a.F - a.f_lo);
-  int i0 = 0;
+  const int32_t* lane_arg = a.arg + (int64_t)here.x * a.F + a.f_lo + lane;
+  const int width = min(32 * WORDS, a.F - a.f_lo) - lane;
+  // the positions that row i selects, feature lane + 32 w in [w]; those of the next row are in flight
+  auto load = [&](int i, int32_t (&k)[WORDS]) {
+#pragma unroll
+    for (int w = 0; w < WORDS; ++w)
+      k[w] = i < nrows && 32 * w < width ? __ldg(lane_arg + (int64_t)i * a.F + 32 * w) : -1;
+  };
+  int32_t cur[WORDS], nxt[WORDS];
+  load(0, cur);
+  load(1, nxt);
+  int i = 0;
   for (int p0 = here.y; p0 < next.y; p0 += kEdges) {
     const int p1 = min(next.y, p0 + kEdges);
     for (int t = lane; t < (p1 - p0) * WORDS; t += 32) window[t] = 0;
     __syncwarp();
-    for (int i = i0; i < nrows; ++i) {
+    while (i < nrows) {
       const int lo = max(__shfl_sync(kAll, my_lo, i), p0), end = __shfl_sync(kAll, my_hi, i);
       if (lo >= p1) break;
       const int hi = min(end, p1);
-      const int32_t* row = a.arg + (int64_t)(here.x + i) * a.F + a.f_lo;
-      if (lo < hi) {
-#pragma unroll 4
-        for (int j = lane; j < width; j += 32) {
-          const int32_t k = __ldg(row + j);
-          if (k >= lo && k < hi) atomicOr(&window[(k - p0) * WORDS + (j >> 5)], 1u << (j & 31));
-        }
-      }
-      if (end <= p1) i0 = i + 1;
+#pragma unroll
+      for (int w = 0; w < WORDS; ++w)
+        if (cur[w] >= lo && cur[w] < hi) atomicOr(&window[(cur[w] - p0) * WORDS + w], 1u << lane);
+      if (end > p1) break;  // the rest of this row lies in the next window
+      ++i;
+#pragma unroll
+      for (int w = 0; w < WORDS; ++w) cur[w] = nxt[w];
+      load(i + 1, nxt);
     }
     __syncwarp();
     uint32_t* out = a.mask + (int64_t)p0 * WORDS;
@@ -165,7 +177,7 @@ __device__ __forceinline__ float selected(const GenArgs& a, bool on, int64_t id,
 // More than 16 features: lane L holds the features f_lo + 32 w + L.  Edges without a selected feature are
 // skipped, U of the others are in flight.
 template <int BIN, int YM, int WORDS>
-__global__ void __launch_bounds__(kGenBlock, WORDS > 4 ? 4 : 6) general_dv_mask_kernel(const GenArgs a) {
+__global__ void __launch_bounds__(kGenBlock, WORDS > 4 ? 5 : 6) general_dv_mask_kernel(const GenArgs a) {
   constexpr int U = WORDS > 4 ? 2 : 4;
   const int lane = threadIdx.x & 31;
   const int f = a.f_lo + lane;
