@@ -108,7 +108,7 @@ static double slice_footprint(int64_t F, int64_t slice, int eb) {
 // (kernels of a forward and a backward pass): F = 47, 1.2 M edges: 79 -> 62 us with the two copies of
 // 2.5 us; F = 602, 114.6 M edges: 34.9 -> 32.8 ms; F = 602 in bf16, 28.7 M edges: 7.5 -> 5.0 ms.
 constexpr int64_t kPadMinDegree = 8;
-constexpr size_t kPadMaxBytes = (size_t)1 << 30;
+constexpr size_t kPadMaxBytes = (size_t)4 << 30;  // the pool keeps this much
 bool worth_padding(const Graph* g, int32_t F, int elem_bytes) {
   return F > 4 && g->nnz >= kPadMinDegree * g->n &&
          (size_t)g->n * (size_t)(F + 128 / elem_bytes) * (size_t)elem_bytes <= kPadMaxBytes;
@@ -136,12 +136,17 @@ bool pad_rows(const Graph* g, const void* X, int32_t F, int elem_bytes, cudaStre
 // Chooses the launch shape, then runs one launch per source block.
 //   vector width: 16-byte loads of the gathered matrix when its rows and its base are 16-byte aligned,
 //     or of its padded copy; else 8 or 4 bytes;
-//   slice: at most 128 vectors per row slice (4 per lane);
+//   slice: 32 vectors, one per lane (512 bytes of a row), where the rows are long enough (24 entries) to
+//     pay for reading the indices once per slice and F fills the slices, else 64.  Several rows of a
+//     gather then cover few L2 sets' worth of one matrix at a time, and a lane keeps more edges in
+//     flight.  Forward sum, F = 256, widths 256 / 128 / 64 / 32: 25 M edges, mean degree 50: 1.91 / 1.67 /
+//     1.76 / 2.67 ms; 8 M edges, degree 14.5: 366 / 466 / 746 / 1354 us.  Slices narrow enough to keep
+//     a graph of short rows in L2 were slower on every graph tried (12 M edges, degree 50, F = 256,
+//     245 MB: 44 floats a slice 1.22 ms, 128 floats 0.73);
 //   source blocks (Algorithm 2 of the paper, with L2 in the role of the CPU cache): when one
 //     slice of X over all n rows exceeds the L2 budget and the segments carry split pointers,
 //     the neighbour ids are cut into 2, 4, 8 or 16 ranges and each range is a launch of its
 //     own, so that the rows of X a launch gathers stay L2-resident; later launches add to Y.
-//     Without split pointers the slice is narrowed instead (down to 128 bytes).
 dg_status_t aggregate_run(const Graph* g, const ApArgs& a0, const SelfArgs& sa, const Plan& plan,
                           const int32_t* split, cudaStream_t s) {
   ApArgs a = a0;
@@ -170,44 +175,35 @@ dg_status_t aggregate_run(const Graph* g, const ApArgs& a0, const SelfArgs& sa, 
   const double budget = (double)g->l2_budget_bytes;
   const double avg_len = (double)g->nnz / (double)a.n;
   const int64_t cap = 128LL * vec;
-  int64_t slice = g->slice_features > 0 ? g->slice_features : (a.F < cap ? (int64_t)a.F : cap);
-  if (slice > cap) slice = cap;
-  if (slice > a.F) slice = a.F;
+  int64_t slice;
   int nb = 1;
+  if (g->slice_features > 0) {
+    slice = g->slice_features < cap ? g->slice_features : cap;
+    if (slice > a.F) slice = a.F;
+  } else {
+    slice = avg_len >= 24.0 && 2 * a.F >= 96LL * vec ? 32LL * vec : 64LL * vec;
+    if (slice > a.F) slice = a.F;
+  }
   if (g->source_blocks > 0) {
     nb = split ? (int)g->source_blocks : 1;
-  } else if (g->slice_features <= 0 && (double)a.n * slice_footprint(ld, slice, eb) > budget) {
-    if (split) {
-      // A width is feasible when some block count keeps one block of the slice inside the budget and
-      // leaves a row at least 32 edges per block on average.  Among those, the least traffic beside the
-      // gather: every slice reads the index stream again, every block after the first reads and writes
-      // the output again.
-      const int64_t widths[4] = {64LL * vec, 32LL * vec, 16LL * vec, 8LL * vec};
-      const double stream = (double)g->nnz * (a.w ? 8.0 : 4.0), output = (double)a.n * a.F * 4.0;
-      const int64_t widest = slice;
-      double best = 0.0;
-      bool found = false;
-      for (int t = 0; t < 4; ++t) {
-        const int64_t w = widths[t] < widest ? widths[t] : widest;
-        int cand = 1;
-        while (cand < kFineBlocks && (double)a.n / cand * slice_footprint(ld, w, eb) > budget) cand *= 2;
-        if ((double)a.n / cand * slice_footprint(ld, w, eb) > budget || avg_len / cand < 32.0) continue;
-        const double cost = stream * (double)((a.F + w - 1) / w) + output * (2 * cand - 1);
-        if (!found || cost < best) {
-          best = cost;
-          slice = w;
-          nb = cand;
-        }
-        found = true;
+  } else if (split && g->slice_features <= 0 && (double)a.n * slice_footprint(ld, a.F, eb) > budget) {
+    // A width is feasible when some block count keeps one block of the slice inside the budget and
+    // leaves a row at least 32 edges per block on average.  Among those, the least traffic beside the
+    // gather: every slice reads the index stream again, every block after the first reads and writes
+    // the output again.
+    const double stream = (double)g->nnz * (a.w ? 8.0 : 4.0), output = (double)a.n * a.F * 4.0;
+    double best = 0.0;
+    for (int64_t wide = 64LL * vec; wide >= 8LL * vec; wide /= 2) {
+      const int64_t w = wide < a.F ? wide : a.F;
+      int cand = 1;
+      while (cand < kFineBlocks && (double)a.n / cand * slice_footprint(ld, w, eb) > budget) cand *= 2;
+      if ((double)a.n / cand * slice_footprint(ld, w, eb) > budget || avg_len / cand < 32.0) continue;
+      const double cost = stream * (double)((a.F + w - 1) / w) + output * (2 * cand - 1);
+      if (best == 0.0 || cost < best) {
+        best = cost;
+        slice = w;
+        nb = cand;
       }
-      if (!found) {  // as many blocks as the row length allows, narrowest slice
-        nb = 1;
-        while (nb < kFineBlocks && avg_len / (nb * 2) >= 32.0) nb *= 2;
-        if (slice > 8LL * vec) slice = 8LL * vec;
-      }
-    } else {
-      int64_t w = (int64_t)(budget / ((double)a.n * eb));
-      if (w * eb >= 128) slice = w < slice ? w : slice;  // under 128 bytes is not worth a pass
     }
   }
   slice = slice < a.F ? (slice / vec) * vec : ld;  // a padded row ends in a vector that reaches beyond F

@@ -16,7 +16,7 @@ namespace dg {
 namespace {
 
 constexpr int kMaxDevices = 64;
-constexpr size_t kKeepInUse = (size_t)2 << 30;
+constexpr size_t kKeepInUse = (size_t)4 << 30;
 constexpr size_t kKeepIdle = (size_t)32 << 20;
 constexpr int kMaxPendingBlocks = 64;
 constexpr size_t kMaxPending = kKeepIdle;
