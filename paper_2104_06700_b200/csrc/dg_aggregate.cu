@@ -93,9 +93,11 @@ dg_status_t join_cut_rows(const Graph* g, const Plan& plan, const float* partial
   return DG_OK;
 }
 
-// Bytes of L2 one row slice of `slice` elements of `eb` bytes occupies: L2 allocates 128-byte
-// lines, and a slice that does not start on a line boundary in every row touches one more line.
+// Bytes of L2 one row slice of `slice` elements of `eb` bytes occupies (`F` from one row to the next): L2
+// allocates 128-byte lines, and a slice that does not start on a line boundary in every row touches one
+// more line; whole rows follow one another without gaps.
 static double slice_footprint(int64_t F, int64_t slice, int eb) {
+  if (slice >= F) return (double)(F * eb);
   const int64_t bytes = slice * eb;
   const bool aligned = (F * eb) % 128 == 0 && bytes % 128 == 0;
   return (double)(((bytes + 127) / 128) * 128 + (aligned ? 0 : 128));
@@ -104,13 +106,18 @@ static double slice_footprint(int64_t F, int64_t slice, int eb) {
 // Whether a call first copies X into padded rows: 16-byte loads need rows that start on 16 bytes, and a
 // width like 47 or 602 (8-byte rows, or 4-byte rows in bf16) otherwise gathers every row with two to
 // four times as many, narrower loads.  The copy costs about two passes over X against nnz / n gathers of
-// every row, so it wants a mean degree of 8; rows of up to 4 elements gain nothing.  Measured
-// (kernels of a forward and a backward pass): F = 47, 1.2 M edges: 79 -> 62 us with the two copies of
-// 2.5 us; F = 602, 114.6 M edges: 34.9 -> 32.8 ms; F = 602 in bf16, 28.7 M edges: 7.5 -> 5.0 ms.
-constexpr int64_t kPadMinDegree = 8;
+// every row.  It pays from a mean degree of about 20 on, and from 8 on where it is the odd rows of over
+// 128 floats that would take several times the slices (`vec` is the width X allows); rows of up to 4
+// elements gain nothing, and its launch and its scratch cost more than the narrow loads of a call that
+// gathers fewer than kPadMinWork elements.  Measured, us of a forward and a backward pass with / without:
+// degree 50, 0.6 M edges, F = 47 57 / 58, 225 113 / 191, 602 250 / 300, 602 in bf16 215 / 287; degree
+// 14.5, 1.6 M edges, F = 47 132 / 120, 110 197 / 156, 225 336 / 406, 602 849 / 672; 10 k edges, F = 41
+// 27 / 19.  At degree 492, F = 602: 32.8 / 34.9 ms.
+constexpr int64_t kPadMinDegree = 20, kPadMinDegreeOdd = 8, kPadMinWork = 1 << 24;
 constexpr size_t kPadMaxBytes = (size_t)4 << 30;  // the pool keeps this much
-bool worth_padding(const Graph* g, int32_t F, int elem_bytes) {
-  return F > 4 && g->nnz >= kPadMinDegree * g->n &&
+bool worth_padding(const Graph* g, int32_t F, int elem_bytes, int vec) {
+  const int64_t degree = vec == 1 && F > 128 ? kPadMinDegreeOdd : kPadMinDegree;
+  return vec * elem_bytes < 16 && F > 4 && g->nnz >= degree * g->n && g->nnz * F >= kPadMinWork &&
          (size_t)g->n * (size_t)(F + 128 / elem_bytes) * (size_t)elem_bytes <= kPadMaxBytes;
 }
 
@@ -165,7 +172,7 @@ dg_status_t aggregate_run(const Graph* g, const ApArgs& a0, const SelfArgs& sa, 
   else if (bf16 || (a.F % 2 == 0 && px % 8 == 0 && py % 8 == 0)) vec = 2;
   int64_t ld = a.F;
   void* padded = nullptr;
-  if (vec < wide && worth_padding(g, a.F, eb) && pad_rows(g, a.X, a.F, eb, s, &padded, &ld)) {
+  if (worth_padding(g, a.F, eb, vec) && pad_rows(g, a.X, a.F, eb, s, &padded, &ld)) {
     a.X = padded;
     vec = wide;
     a.narrow_store = a.F % 4 != 0 || py % 16 != 0 || (bf16 && a.F % 8 != 0);
@@ -186,7 +193,7 @@ dg_status_t aggregate_run(const Graph* g, const ApArgs& a0, const SelfArgs& sa, 
   }
   if (g->source_blocks > 0) {
     nb = split ? (int)g->source_blocks : 1;
-  } else if (split && g->slice_features <= 0 && (double)a.n * slice_footprint(ld, a.F, eb) > budget) {
+  } else if (split && g->slice_features <= 0 && (double)a.n * slice_footprint(ld, ld, eb) > budget) {
     // A width is feasible when some block count keeps one block of the slice inside the budget and
     // leaves a row at least 32 edges per block on average.  Among those, the least traffic beside the
     // gather: every slice reads the index stream again, every block after the first reads and writes
@@ -194,7 +201,7 @@ dg_status_t aggregate_run(const Graph* g, const ApArgs& a0, const SelfArgs& sa, 
     const double stream = (double)g->nnz * (a.w ? 8.0 : 4.0), output = (double)a.n * a.F * 4.0;
     double best = 0.0;
     for (int64_t wide = 64LL * vec; wide >= 8LL * vec; wide /= 2) {
-      const int64_t w = wide < a.F ? wide : a.F;
+      const int64_t w = wide < a.F ? wide : ld;
       int cand = 1;
       while (cand < kFineBlocks && (double)a.n / cand * slice_footprint(ld, w, eb) > budget) cand *= 2;
       if ((double)a.n / cand * slice_footprint(ld, w, eb) > budget || avg_len / cand < 32.0) continue;

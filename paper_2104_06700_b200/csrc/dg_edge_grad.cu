@@ -132,7 +132,7 @@ dg_status_t edge_grad_run(const Graph* g, const float* H, const float* dOut, int
   int vec = (F % 4 == 0 && (both & 15) == 0) ? 4 : (F % 2 == 0 && (both & 7) == 0) ? 2 : 1;
   void *padded_h = nullptr, *padded_g = nullptr;
   dg_status_t st = DG_OK;
-  if (vec < 4 && worth_padding(g, F, 4)) {
+  if (worth_padding(g, F, 4, vec)) {
     // both rows of a dot product in the same padded layout; the padding multiplies to zero
     int64_t ld = 0;
     if (pad_rows(g, H, F, 4, s, &padded_h, &ld) && pad_rows(g, dOut, F, 4, s, &padded_g, &ld)) {
