@@ -478,16 +478,19 @@ __device__ __forceinline__ void ap_body(const ApArgs& a, const SelfArgs sa) {
   }
 }
 
-// Six blocks per SM (40 registers).  Three to eight blocks are within 5 % of each other on every workload
-// (the gather is what they wait for, not the register file); six is the best for most.
-template <typename E, int VEC, int G, int CPL, bool SCALED, bool SEG>
-__global__ void __launch_bounds__(kBlock, 6) ap_kernel(const ApArgs a) {
+// BLOCKS blocks per SM.  Six (40 registers): three to eight blocks are within 5 % of each other on every large
+// workload (the gather is what they wait for, not the register file), six is the best for most.  Four (64
+// registers) on grids that fit in one wave of those: occupancy is no limit there, and with 40 registers
+// not all of a lane's eight loads are in flight (forward + backward, 40 k edges, F = 256: 38.2 -> 30.7 us; 74 k
+// edges, F = 100: 36.9 -> 32.6 us).
+template <typename E, int VEC, int G, int CPL, bool SCALED, bool SEG, int BLOCKS>
+__global__ void __launch_bounds__(kBlock, BLOCKS) ap_kernel(const ApArgs a) {
   ap_body<E, VEC, G, CPL, SCALED, SEG, false>(a, SelfArgs{});
 }
 
 // The same for graphs with implicit self loops: every row also sums its own input row.
-template <typename E, int VEC, int G, int CPL, bool SCALED, bool SEG>
-__global__ void __launch_bounds__(kBlock, 6) ap_kernel_self(const ApArgs a, const SelfArgs sa) {
+template <typename E, int VEC, int G, int CPL, bool SCALED, bool SEG, int BLOCKS>
+__global__ void __launch_bounds__(kBlock, BLOCKS) ap_kernel_self(const ApArgs a, const SelfArgs sa) {
   ap_body<E, VEC, G, CPL, SCALED, SEG, true>(a, sa);
 }
 
@@ -495,11 +498,13 @@ template <typename E, int VEC, int G, int CPL, bool SCALED, bool SELF>
 dg_status_t launch_variant(const ApArgs& a, const SelfArgs& sa, int slices, cudaStream_t s) {
   const dim3 grid((unsigned)((a.chunk_count + kWarpsPerBlock - 1) / kWarpsPerBlock), (unsigned)slices);
   if constexpr (SELF) {
-    if (a.seg_lo) ap_kernel_self<E, VEC, G, CPL, SCALED, true><<<grid, kBlock, 0, s>>>(a, sa);
-    else ap_kernel_self<E, VEC, G, CPL, SCALED, false><<<grid, kBlock, 0, s>>>(a, sa);
+    if (a.seg_lo) ap_kernel_self<E, VEC, G, CPL, SCALED, true, 6><<<grid, kBlock, 0, s>>>(a, sa);
+    else if (a.few_blocks) ap_kernel_self<E, VEC, G, CPL, SCALED, false, 4><<<grid, kBlock, 0, s>>>(a, sa);
+    else ap_kernel_self<E, VEC, G, CPL, SCALED, false, 6><<<grid, kBlock, 0, s>>>(a, sa);
   } else {
-    if (a.seg_lo) ap_kernel<E, VEC, G, CPL, SCALED, true><<<grid, kBlock, 0, s>>>(a);
-    else ap_kernel<E, VEC, G, CPL, SCALED, false><<<grid, kBlock, 0, s>>>(a);
+    if (a.seg_lo) ap_kernel<E, VEC, G, CPL, SCALED, true, 6><<<grid, kBlock, 0, s>>>(a);
+    else if (a.few_blocks) ap_kernel<E, VEC, G, CPL, SCALED, false, 4><<<grid, kBlock, 0, s>>>(a);
+    else ap_kernel<E, VEC, G, CPL, SCALED, false, 6><<<grid, kBlock, 0, s>>>(a);
   }
   DG_CUDA(cudaGetLastError());
   count_launches(1);

@@ -56,13 +56,19 @@ static void free_owned(Graph* g) {
 
 // Cost of a chunk (see Plan).  A large graph gets chunks of 1024: long enough to hide their start-up,
 // short enough that a late one does not matter.  A smaller one is cut into kChunksPerSm chunks per SM, so
-// that every SM has warps to hide latency with and the last wave is short; under 64 entries only half as
-// many, because more cut rows make the join dearer, and never under 32 (one index batch).  Measured, us
+// that every SM has warps to hide latency with and the last wave is short, down to 64 entries, because
+// more cut rows make the join dearer; and into chunks of 32 (one index batch) where there are at most
+// kShortChunksPerSm of those (396 k edges, rows of 42, F = 64: 24.6 us at 32, 28.7 at 64; 619 k edges, rows up
+// to 1400, F = 100: 76 / 69).  Measured, us
 // of both directions with their joins at 32 / 64 / 128 / 256: 65 k edges, F = 64: 15 / 19 / 27 / 39;
 // 1.2 M, F = 47: 72 / 66 / 67 / 74; 6.2 M, F = 100: 454 / 392 / 379 / 396; 16 M, F = 64 (columns up to
 // 10^5 entries): 1286 / 1040 / 930 / 892.
-// Rows up to twice a chunk stay whole: four times costs 2 to 15 % on the same graphs.
+// Rows up to twice a chunk stay whole: four times costs 2 to 15 % on the same graphs.  With the smallest
+// chunks rows up to kFewEdgesRow entries do: such a call is short against its launches, and the join of
+// cut rows is one more launch with scratch of its own, 4.5 us of host time and 3.5 us on the device (125 k
+// edges, rows up to 157, forward + backward: 31.4 us cut at 64, 20.5 whole).
 constexpr int64_t kMaxChunk = 1024, kMinChunk = 32, kChunksPerSm = 320, kRowCost = 8;
+constexpr int64_t kShortChunksPerSm = 108, kFewEdgesRow = 160;
 static int64_t chunk_cost(const Graph* g) {
   const int64_t total = g->nnz + kRowCost * g->n;
   int64_t cost;
@@ -71,8 +77,8 @@ static int64_t chunk_cost(const Graph* g) {
     cost = cost < 32 ? 32 : cost;
   } else {
     cost = total / (g->sm_count * kChunksPerSm);
-    if (cost < 64) cost = 2 * cost < 64 ? 2 * cost : 64;
-    cost = cost < kMinChunk ? kMinChunk : cost > kMaxChunk ? kMaxChunk : cost;
+    if (cost < 64) cost = total <= g->sm_count * kShortChunksPerSm * kMinChunk ? kMinChunk : 64;
+    if (cost > kMaxChunk) cost = kMaxChunk;
   }
   return (cost + 31) & ~(int64_t)31;
 }
@@ -82,7 +88,8 @@ static int64_t row_cost(const Graph* g) {
   return least > kRowCost ? least : kRowCost;
 }
 static int64_t cut_threshold(const Graph* g) {
-  return g->heavy_threshold > 0 ? g->heavy_threshold : 2 * chunk_cost(g);
+  if (g->heavy_threshold > 0) return g->heavy_threshold;
+  return g->rows_per_block == 0 && chunk_cost(g) == kMinChunk ? kFewEdgesRow : 2 * chunk_cost(g);
 }
 
 // Takes the memory of both plans for the current chunk cost and threshold.

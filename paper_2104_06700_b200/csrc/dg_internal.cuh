@@ -128,6 +128,7 @@ struct ApArgs {
   const int32_t* seg_lo;      // source-blocked pass: first and one-past-last position of every
   const int32_t* seg_hi;      //   segment's piece (n entries each); nullptr = whole segments
   int32_t accumulate;         // source-blocked pass after the first: add to what Y holds
+  int32_t few_blocks;         // host side: the grid is small, see ap_kernel
 };
 
 // Implicit self loops (every vertex its own neighbour with weight 1): row r also receives
