@@ -162,11 +162,11 @@ __device__ __forceinline__ unsigned digit_peers(uint32_t d, bool valid) {
 }
 
 // ---- stable scatter of one tile ----
-// vals_in == nullptr means "the value of key k is k" (first pass).  keys_out may be nullptr when
-// the sorted keys are not needed (never the case for the last pass, which feeds colptr).
-// Four blocks per SM (64 registers a thread): the ranking is a chain of shared-memory and
-// ballot latencies, and the fourth block hides more of it than the few spilled words cost
-// (three blocks at 80 registers were 10 % slower, five with the values read late 3 % slower).
+// vals_in == nullptr means "the value of key k is k" (first pass).
+// The tile is staged in shared memory sorted by digit, one array after the other in the same 16 KB.
+// Four blocks per SM (64 registers a thread): the ranking is a chain of shared-memory and ballot latencies.
+// Values are read only when the keys have left their registers, and two places share one: nothing spills
+// (0.78 -> 0.68 ms per pass over 124 M pairs; three blocks at 80 registers 1.02, five at 48 0.73).
 template <int BITS>
 __global__ void __launch_bounds__(kSortBlock, 4)
 digit_scatter(const uint32_t* __restrict__ keys_in, const uint32_t* __restrict__ vals_in,
@@ -176,15 +176,13 @@ digit_scatter(const uint32_t* __restrict__ keys_in, const uint32_t* __restrict__
   constexpr int DPT = R / kSortBlock;  // digits a thread owns (consecutive ones): 1 or 2
   // A warp ranks its 512 keys as two streams of 256 (rounds 0..7 and 8..15), each with its own
   // counters, so that two independent chains of counter updates are in flight at a time.
-  // Dynamic shared memory (52 KB with 9-bit digits): cnt_a, cnt_b, digit_base, global_base,
-  // skeys, svals.
+  // Dynamic shared memory (36 KB with 9-bit digits): cnt_a, cnt_b, digit_base, global_base, stage.
   extern __shared__ __align__(16) unsigned char scatter_smem[];
   uint16_t (*cnt_a)[R] = reinterpret_cast<uint16_t (*)[R]>(scatter_smem);
   uint16_t (*cnt_b)[R] = cnt_a + kSortWarps;
   uint32_t* digit_base = reinterpret_cast<uint32_t*>(cnt_b + kSortWarps);
   uint32_t* global_base = digit_base + R;
-  uint32_t* skeys = global_base + R;
-  uint32_t* svals = skeys + kTile;
+  uint32_t* stage = global_base + R;
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   const unsigned lt_mask = (1u << lane) - 1u;
   const int64_t tile_base = (int64_t)blockIdx.x * kTile;
@@ -208,16 +206,14 @@ digit_scatter(const uint32_t* __restrict__ keys_in, const uint32_t* __restrict__
   // Warp `warp` owns keys [warp*512, warp*512+512) of the tile, 32 consecutive keys per round,
   // so (warp, round, lane) order is input order.
   uint32_t key[kItems];
-  uint32_t val[kItems];
-  uint16_t rank[kItems];
+  constexpr int kHalf = kItems / 2;
+  uint32_t place[kHalf];  // rank, later the place in the sorted tile: of key r low, of key r + kHalf high
+  auto place_of = [&](int r) { return r < kHalf ? place[r] & 0xffffu : place[r - kHalf] >> 16; };
 #pragma unroll
   for (int r = 0; r < kItems; ++r) {
     const int local = warp * (32 * kItems) + r * 32 + lane;
-    const bool valid = local < tile_count;
-    key[r] = valid ? keys_in[tile_base + local] : 0u;
-    val[r] = valid ? (vals_in ? vals_in[tile_base + local] : (uint32_t)(tile_base + local)) : 0u;
+    key[r] = local < tile_count ? keys_in[tile_base + local] : 0u;
   }
-  constexpr int kHalf = kItems / 2;
 #pragma unroll
   for (int r = 0; r < kHalf; ++r) {
 #pragma unroll
@@ -234,7 +230,8 @@ digit_scatter(const uint32_t* __restrict__ keys_in, const uint32_t* __restrict__
         cnt[d] = (uint16_t)(before + __popc(peers));
       }
       before = __shfl_sync(kFull, before, leader);
-      rank[rr] = (uint16_t)(before + __popc(peers & lt_mask));
+      const uint32_t rank = before + __popc(peers & lt_mask);
+      place[r] = stream ? place[r] | rank << 16 : rank;
     }
     __syncwarp();
   }
@@ -277,27 +274,45 @@ digit_scatter(const uint32_t* __restrict__ keys_in, const uint32_t* __restrict__
     const int local = warp * (32 * kItems) + r * 32 + lane;
     if (local < tile_count) {
       const uint32_t d = digit_of<BITS>(key[r], shift);
-      const uint32_t in_digit = r < kHalf ? cnt_a[warp][d] : cnt_b[warp][d];
-      const uint32_t pos = digit_base[d] + in_digit + rank[r];
-      skeys[pos] = key[r];
-      svals[pos] = val[r];
+      const uint32_t add = digit_base[d] + (r < kHalf ? cnt_a[warp][d] : cnt_b[warp][d]);
+      place[r % kHalf] += r < kHalf ? add : add << 16;  // places are below 4096: no carry into the high half
+      stage[place_of(r)] = key[r];
+      // the key has been staged: its register takes the value, on its way while the keys are written
+      key[r] = vals_in ? vals_in[tile_base + local] : (uint32_t)(tile_base + local);
     }
   }
   __syncthreads();
-
-  for (int i = threadIdx.x; i < tile_count; i += kSortBlock) {
-    const uint32_t k = skeys[i];
-    const uint32_t d = digit_of<BITS>(k, shift);
-    const uint32_t dst = global_base[d] + ((uint32_t)i - digit_base[d]);
-    if (keys_out) keys_out[dst] = k;
-    vals_out[dst] = svals[i];
+  uint32_t dst[kItems];
+#pragma unroll
+  for (int j = 0; j < kItems; ++j) {
+    const int i = j * kSortBlock + threadIdx.x;
+    if (i < tile_count) {
+      const uint32_t k = stage[i];
+      const uint32_t d = digit_of<BITS>(k, shift);
+      dst[j] = global_base[d] + ((uint32_t)i - digit_base[d]);
+      keys_out[dst[j]] = k;
+    }
+  }
+  __syncthreads();
+#pragma unroll
+  for (int r = 0; r < kItems; ++r) {
+    const int local = warp * (32 * kItems) + r * 32 + lane;
+    if (local < tile_count) {
+      stage[place_of(r)] = key[r];
+    }
+  }
+  __syncthreads();
+#pragma unroll
+  for (int j = 0; j < kItems; ++j) {
+    const int i = j * kSortBlock + threadIdx.x;
+    if (i < tile_count) vals_out[dst[j]] = stage[i];
   }
 }
 
 template <int BITS>
 constexpr size_t scatter_smem_bytes() {
   return (size_t)2 * kSortWarps * (1 << BITS) * sizeof(uint16_t) + (size_t)2 * (1 << BITS) * sizeof(uint32_t) +
-         (size_t)2 * kTile * sizeof(uint32_t);
+         (size_t)kTile * sizeof(uint32_t);
 }
 
 // colptr[u] = first position q whose sorted key is >= u.  Position q fills the ids between the
@@ -350,50 +365,39 @@ __global__ void fill_long_gaps(const uint32_t* __restrict__ sorted, int64_t nnz,
   colptr[u] = lo;
 }
 
-// row_info[k] = (row r with rowptr[r] <= k < rowptr[r+1], bits of 1/(deg(r) + self)) for every
-// CSR position k; self = 1 when the graph has implicit self loops, else 0.  A thread takes kRowItems consecutive positions: one binary search for the first, then a
-// galloping search forward from the previous row for each of the others (rows are usually a few
-// positions long, empty rows are skipped in doubling strides).  Searching once per perm[q] in
-// CSC order instead, with random access to rowptr, took 218 ms of the 296 ms transpose of the
-// 1.6 G-edge graph.
-constexpr int kRowItems = 8;
-__global__ void row_info_kernel(const int64_t* __restrict__ rowptr, int self, int64_t n,
-                                int64_t nnz, uint2* __restrict__ row_info) {
-  const int64_t k0 = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) * kRowItems;
-  if (k0 >= nnz) return;
-  int64_t lo = 0, hi = n;  // invariant: rowptr[lo] <= k0 < rowptr[hi]
-  while (hi - lo > 1) {
-    const int64_t mid = (lo + hi) >> 1;
-    if (__ldg(rowptr + mid) <= k0) lo = mid; else hi = mid;
+// row_info[k] = (row r that holds CSR position k, bits of 1/(deg(r) + self)); self = 1 when the graph has
+// implicit self loops, else 0.  A warp takes one chunk of the rows' plan (see Plan) and writes its rows'
+// pairs over their entries: bound by the 8 bytes written per edge.  A search for the row of every eighth
+// position, and a walk from there, took 0.58 ms for 124 M edges, this 0.16.
+__global__ void __launch_bounds__(256)
+row_info_kernel(const Chunk* __restrict__ chunks, int32_t chunk_count, const int64_t* __restrict__ rowptr,
+                int self, uint2* __restrict__ row_info) {
+  const int lane = threadIdx.x & 31;
+  const int chunk = blockIdx.x * 8 + __shfl_sync(kFull, (int)(threadIdx.x >> 5), 0);
+  if (chunk >= chunk_count) return;
+  const int4 here = __ldg(reinterpret_cast<const int4*>(chunks) + chunk);
+  const int4 next = __ldg(reinterpret_cast<const int4*>(chunks) + chunk + 1);
+  const int nrows = here.z >= 0 ? 1 : next.x - here.x + (next.z >= 0 ? 1 : 0);
+  int end = next.y;
+  uint32_t inv = 0;
+  if (lane < nrows) {
+    const int64_t row_end = __ldg(rowptr + here.x + lane + 1);
+    end = min((int)row_end, next.y);
+    inv = __float_as_uint(1.0f / (float)(row_end - __ldg(rowptr + here.x + lane) + self));
   }
-  int64_t r = lo;
-  int64_t r_end = __ldg(rowptr + r + 1);  // first position after row r
-#pragma unroll 1
-  for (int i = 0; i < kRowItems; ++i) {
-    const int64_t k = k0 + i;
-    if (k >= nnz) break;
-    if (k >= r_end) {
-      // gallop: find a row `hi2` with rowptr[hi2] > k, then bisect (r, hi2]
-      int64_t step = 1, lo2 = r, hi2 = r + 1;
-      while (hi2 < n && __ldg(rowptr + hi2) <= k) {
-        lo2 = hi2;
-        step <<= 1;
-        hi2 = hi2 + step < n ? hi2 + step : n;
-      }
-      while (hi2 - lo2 > 1) {
-        const int64_t mid = (lo2 + hi2) >> 1;
-        if (__ldg(rowptr + mid) <= k) lo2 = mid; else hi2 = mid;
-      }
-      r = lo2;
-      r_end = __ldg(rowptr + r + 1);
-    }
-    // k lies in row r, so deg(r) >= 1
-    const float inv = 1.0f / (float)(r_end - __ldg(rowptr + r) + self);
-    row_info[k] = make_uint2((uint32_t)r, __float_as_uint(inv));
+  int p = here.y;
+  for (int i = 0; i < nrows; ++i) {
+    const int hi = __shfl_sync(kFull, end, i);
+    const uint2 info = make_uint2((uint32_t)(here.x + i), __shfl_sync(kFull, inv, i));
+    for (int k = p + lane; k < hi; k += 32) row_info[k] = info;
+    p = hi;
   }
 }
 
-// The same walk with another payload: out[k] = map[r] (or r) for the row r that holds position k.
+constexpr int kRowItems = 8;
+// out[k] = map[r] (or r) for the row r that holds position k.  A thread takes kRowItems consecutive
+// positions: one binary search for the first, then a galloping search forward from the previous row for
+// each of the others (rows are usually a few positions long, empty rows are skipped in doubling strides).
 __global__ void expand_rows_kernel(const int64_t* __restrict__ rowptr, int64_t n, int64_t nnz,
                                    const int32_t* __restrict__ map, uint32_t* __restrict__ out) {
   const int64_t k0 = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) * kRowItems;
@@ -431,7 +435,10 @@ __global__ void expand_rows_kernel(const int64_t* __restrict__ rowptr, int64_t n
 
 // rowidx_T[q] = row of perm[q];  w_T[q] = edge_w[perm[q]];  mean_scale_T[q] = w_T[q] (1 if
 // unweighted) / (deg(row) + self), the factor of edge q in the backward pass of the mean, so that
-// the backward kernel streams it instead of gathering 1/deg.  One 8-byte gather per edge.
+// the backward kernel streams it instead of gathering 1/deg.  Bound by the random reads, one of 8 bytes per
+// edge (two if weighted): 4-byte reads of the row alone and the degree from its row pointers, three random
+// reads, took 2.06 ms instead of 1.52 for 124 M edges; the row carried through the sort instead took 2.5 ms
+// more in the scatters.
 __global__ void gather_rows_and_weights(const uint32_t* __restrict__ perm, int64_t nnz,
                                         const uint2* __restrict__ row_info,
                                         const float* __restrict__ edge_w,
@@ -451,18 +458,33 @@ __global__ void gather_rows_and_weights(const uint32_t* __restrict__ perm, int64
 }
 
 // After the caller changed edge_w in place (learnable edge weights): the two weight arrays of the
-// CSC again, from perm.  The in-degree comes from the CSR row pointer.
-__global__ void regather_weights_kernel(const uint32_t* __restrict__ perm, int64_t nnz,
-                                        const float* __restrict__ edge_w,
-                                        const int32_t* __restrict__ rowidx_T,
-                                        const int64_t* __restrict__ rowptr, int self,
-                                        float* __restrict__ w_T, float* __restrict__ mean_scale_T) {
-  const int64_t q = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-  if (q >= nnz) return;
-  const float w = edge_w[perm[q]];
-  const int64_t v = rowidx_T[q];
-  w_T[q] = w;
-  mean_scale_T[q] = w * (1.0f / (float)(__ldg(rowptr + v + 1) - __ldg(rowptr + v) + self));
+// CSC again, from perm.  The in-degree comes from the CSR row pointer.  A thread takes four edges: their
+// random reads are in flight together.
+__global__ void __launch_bounds__(256)
+regather_weights_kernel(const uint32_t* __restrict__ perm, int64_t nnz, const float* __restrict__ edge_w,
+                        const int32_t* __restrict__ rowidx_T, const int64_t* __restrict__ rowptr, int self,
+                        float* __restrict__ w_T, float* __restrict__ mean_scale_T) {
+  const int64_t q0 = ((int64_t)blockIdx.x * 256 + threadIdx.x) * 4;
+  if (q0 >= nnz) return;
+  if (nnz - q0 >= 4) {  // the arrays of the CSC are 256-byte aligned
+    const int4 v = *reinterpret_cast<const int4*>(rowidx_T + q0);
+    const uint4 k = *reinterpret_cast<const uint4*>(perm + q0);
+    const float w[4] = {__ldg(edge_w + k.x), __ldg(edge_w + k.y), __ldg(edge_w + k.z), __ldg(edge_w + k.w)};
+    const int32_t r[4] = {v.x, v.y, v.z, v.w};
+    float t[4];
+#pragma unroll
+    for (int i = 0; i < 4; ++i)
+      t[i] = w[i] * (1.0f / (float)(__ldg(rowptr + r[i] + 1) - __ldg(rowptr + r[i]) + self));
+    *reinterpret_cast<float4*>(w_T + q0) = make_float4(w[0], w[1], w[2], w[3]);
+    *reinterpret_cast<float4*>(mean_scale_T + q0) = make_float4(t[0], t[1], t[2], t[3]);
+    return;
+  }
+  for (int64_t q = q0; q < nnz; ++q) {
+    const float w = edge_w[perm[q]];
+    const int64_t v = rowidx_T[q];
+    w_T[q] = w;
+    mean_scale_T[q] = w * (1.0f / (float)(__ldg(rowptr + v + 1) - __ldg(rowptr + v) + self));
+  }
 }
 
 inline size_t align256(size_t x) { return (x + 255) & ~(size_t)255; }
@@ -532,14 +554,12 @@ void sort_scratch_sizes(int64_t count, size_t* hist_bytes, size_t* sums_bytes) {
 template <int BITS>
 static dg_status_t sort_passes_run(const uint32_t* keys_in, const uint32_t* vals_in, int64_t count,
                                    int passes, uint32_t* const keys_buf[2], uint32_t* vals_final,
-                                   uint32_t* vals_tmp, uint32_t* hist, uint32_t* sums,
-                                   const uint32_t** sorted_keys, cudaStream_t s) {
+                                   uint32_t* vals_tmp, uint32_t* hist,
+                                   uint32_t* sums, const uint32_t** sorted_keys, cudaStream_t s) {
   const int64_t tiles = (count + kTile - 1) / kTile;
   const int64_t hist_len = tiles * (1 << BITS);
   const int64_t chunks = (hist_len + kScanChunk - 1) / kScanChunk;
   constexpr size_t smem = scatter_smem_bytes<BITS>();
-  DG_CUDA(cudaFuncSetAttribute(digit_scatter<BITS>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                               (int)smem));
   for (int p = 0; p < passes; ++p) {
     const int shift = p * BITS;
     // value buffers alternate so that the last pass lands in vals_final
@@ -613,7 +633,7 @@ void transpose_sizes(int64_t n, int64_t nnz, bool weighted, size_t* csc_bytes,
 
 dg_status_t refresh_csc_weights(Graph* g, cudaStream_t s) {
   if (g->nnz == 0 || !g->edge_w) return DG_OK;
-  regather_weights_kernel<<<(unsigned)((g->nnz + 255) / 256), 256, 0, s>>>(
+  regather_weights_kernel<<<(unsigned)((g->nnz + 1023) / 1024), 256, 0, s>>>(
       reinterpret_cast<const uint32_t*>(g->perm), g->nnz, g->edge_w, g->rowidx_T, g->rowptr,
       g->self_loops_in_csc ? 1 : 0, const_cast<float*>(g->w_T), const_cast<float*>(g->mean_scale_T));
   DG_CUDA(cudaGetLastError());
@@ -646,15 +666,14 @@ dg_status_t transpose_run(Graph* g, void* csc, void* scratch, cudaStream_t s) {
                                     sort_plan(n), keys_buf, perm, vals_tmp, hist, sums, &keys_in, s))
       return st;
     if (dg_status_t st = pointers_from_sorted_keys(keys_in, nnz, n, colptr, s)) return st;
-    const unsigned b2 = (unsigned)((nnz + 255) / 256);
     // colptr has been derived from the sorted keys (stream order), so both key buffers, which
     // are adjacent in the scratch, are free: they hold the nnz (row, 1/deg) pairs
     uint2* row_info = reinterpret_cast<uint2*>(sb + L.keys_a_off);
-    const unsigned b3 = (unsigned)(((nnz + kRowItems - 1) / kRowItems + 255) / 256);
-    row_info_kernel<<<b3, 256, 0, s>>>(g->rowptr, g->self_loops ? 1 : 0, n, nnz, row_info);
+    row_info_kernel<<<(unsigned)((g->row_plan.count + 7) / 8), 256, 0, s>>>(
+        g->row_plan.chunks, (int32_t)g->row_plan.count, g->rowptr, g->self_loops ? 1 : 0, row_info);
     DG_CUDA(cudaGetLastError());
-    gather_rows_and_weights<<<b2, 256, 0, s>>>(perm, nnz, row_info, g->edge_w, rowidx_T, w_T,
-                                               mean_scale_T);
+    gather_rows_and_weights<<<(unsigned)((nnz + 255) / 256), 256, 0, s>>>(perm, nnz, row_info, g->edge_w, rowidx_T,
+                                                                          w_T, mean_scale_T);
     DG_CUDA(cudaGetLastError());
     count_launches(2);
   }
