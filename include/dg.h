@@ -182,6 +182,18 @@ dg_status_t dg_aggregate_bwd(dg_graph_t g, const float* dOut, int32_t F, dg_op_t
                              void* stream);
 
 /*
+ * dg_aggregate_fwd / dg_aggregate_bwd as with the graph attribute "self_loops" = 1, whatever its value:
+ * one handle then serves the plain aggregation and the GCN aggregator (own row added, mean over
+ * in-degree + 1).  The backward pass of DG_OP_MEAN still needs the factors of a CSC built with
+ * "self_loops" = 1 (DG_ERR_NOT_TRANSPOSED otherwise); that of DG_OP_SUM takes any CSC.
+ * Asynchronous on `stream`.
+ */
+dg_status_t dg_aggregate_fwd_self(dg_graph_t g, const float* H, int32_t F, dg_op_t op, float* out,
+                                  void* stream);
+dg_status_t dg_aggregate_bwd_self(dg_graph_t g, const float* dOut, int32_t F, dg_op_t op, float* dH,
+                                  void* stream);
+
+/*
  * The same two passes with the gathered matrix stored as bf16 (two bytes per element, the
  * upper half of an fp32; the paper's Conclusion names reduced precision as future work).  Every
  * gathered byte is halved; products and sums are fp32 (a bf16 value converts to fp32 exactly)

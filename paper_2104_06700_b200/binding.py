@@ -29,6 +29,7 @@ DG_ORDER_GIVEN, DG_ORDER_OUT_DEGREE, DG_ORDER_IN_DEGREE = range(3)
 EXPORTS = [
     "dg_graph_create", "dg_graph_destroy", "dg_graph_validate", "dg_graph_transpose_workspace",
     "dg_graph_transpose", "dg_graph_transpose_static", "dg_graph_update_weights", "dg_graph_get_csc", "dg_aggregate_fwd", "dg_aggregate_bwd",
+    "dg_aggregate_fwd_self", "dg_aggregate_bwd_self",
     "dg_aggregate_fwd_bf16", "dg_aggregate_bwd_bf16",
     "dg_ap_fwd", "dg_ap_bwd", "dg_aggregate_edge_grad",
     "dg_graph_reorder_workspace", "dg_graph_reorder", "dg_graph_get_order", "dg_permute_rows",
@@ -68,6 +69,8 @@ def lib() -> ctypes.CDLL:
         L.dg_graph_get_csc.argtypes = [p, pp, pp, pp, pp]
         L.dg_aggregate_fwd.argtypes = [p, p, i32, ctypes.c_int, p, p]
         L.dg_aggregate_bwd.argtypes = [p, p, i32, ctypes.c_int, p, p]
+        L.dg_aggregate_fwd_self.argtypes = [p, p, i32, ctypes.c_int, p, p]
+        L.dg_aggregate_bwd_self.argtypes = [p, p, i32, ctypes.c_int, p, p]
         L.dg_aggregate_fwd_bf16.argtypes = [p, p, i32, ctypes.c_int, p, p]
         L.dg_aggregate_bwd_bf16.argtypes = [p, p, i32, ctypes.c_int, p, p]
         L.dg_ap_fwd.argtypes = [p, p, p, i32, i32, ctypes.c_int, ctypes.c_int, p, p, p]
@@ -309,6 +312,24 @@ class Graph:
             dH = torch.empty_like(dOut)
         _check(lib().dg_aggregate_bwd(self._h, _dev_ptr(dOut, torch.float32, "dOut"), F, int(op),
                                       _dev_ptr(dH, torch.float32, "dH"), _stream(stream)))
+        return dH
+
+    def dg_aggregate_fwd_self(self, H: torch.Tensor, op: int, out: Optional[torch.Tensor] = None,
+                              stream=None) -> torch.Tensor:
+        if out is None:
+            out = torch.empty_like(H)
+        _check(lib().dg_aggregate_fwd_self(self._h, _dev_ptr(H, torch.float32, "H"), H.shape[1],
+                                           int(op), _dev_ptr(out, torch.float32, "out"),
+                                           _stream(stream)))
+        return out
+
+    def dg_aggregate_bwd_self(self, dOut: torch.Tensor, op: int,
+                              dH: Optional[torch.Tensor] = None, stream=None) -> torch.Tensor:
+        if dH is None:
+            dH = torch.empty_like(dOut)
+        _check(lib().dg_aggregate_bwd_self(self._h, _dev_ptr(dOut, torch.float32, "dOut"),
+                                           dOut.shape[1], int(op),
+                                           _dev_ptr(dH, torch.float32, "dH"), _stream(stream)))
         return dH
 
     def dg_aggregate_fwd_bf16(self, H: torch.Tensor, op: int, out: Optional[torch.Tensor] = None,

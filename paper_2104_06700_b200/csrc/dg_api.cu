@@ -192,7 +192,8 @@ static dg_status_t check_features(const Graph* g, const void* in, size_t in_elem
 }
 
 // Forward / backward AP for either storage type of the gathered matrix.
-static dg_status_t run_forward(Graph* g, const void* H, bool bf16, int32_t F, dg_op_t op,
+// `loops`: implicit self loops in this call.
+static dg_status_t run_forward(Graph* g, const void* H, bool bf16, int32_t F, dg_op_t op, bool loops,
                                float* out, void* stream) {
   if (dg_status_t st = check_features(g, H, bf16 ? 2 : 4, out, F, op)) return st;
   ApArgs a{};
@@ -205,19 +206,19 @@ static dg_status_t run_forward(Graph* g, const void* H, bool bf16, int32_t F, dg
   a.n = g->n;
   a.F = F;
   a.mean_rows = op == DG_OP_MEAN;
-  const SelfArgs sa{g->self_loops ? g->rowptr : nullptr, op == DG_OP_MEAN};
+  const SelfArgs sa{loops ? g->rowptr : nullptr, op == DG_OP_MEAN};
   return aggregate_run(g, a, sa, g->row_plan, g->split_csr, (cudaStream_t)stream);
 }
 
-static dg_status_t run_backward(Graph* g, const void* dOut, bool bf16, int32_t F, dg_op_t op,
+static dg_status_t run_backward(Graph* g, const void* dOut, bool bf16, int32_t F, dg_op_t op, bool loops,
                                 float* dH, void* stream) {
   if (dg_status_t st = check_features(g, dOut, bf16 ? 2 : 4, dH, F, op)) return st;
   if (!g->transposed) {
     set_error("the backward pass needs dg_graph_transpose first");
     return DG_ERR_NOT_TRANSPOSED;
   }
-  if (op == DG_OP_MEAN && g->self_loops != g->self_loops_in_csc) {
-    set_error("self_loops was changed after dg_graph_transpose: transpose again");
+  if (op == DG_OP_MEAN && loops != (g->self_loops_in_csc != 0)) {
+    set_error("the CSC was built with another value of self_loops: transpose again");
     return DG_ERR_NOT_TRANSPOSED;
   }
   ApArgs a{};
@@ -230,7 +231,7 @@ static dg_status_t run_backward(Graph* g, const void* dOut, bool bf16, int32_t F
   a.n = g->n;
   a.F = F;
   a.mean_rows = 0;
-  const SelfArgs sa{g->self_loops ? g->rowptr : nullptr, op == DG_OP_MEAN};
+  const SelfArgs sa{loops ? g->rowptr : nullptr, op == DG_OP_MEAN};
   return aggregate_run(g, a, sa, column_plan(g), g->split_csc, (cudaStream_t)stream);
 }
 
@@ -405,22 +406,32 @@ dg_status_t dg_graph_get_csc(dg_graph_t g, const int64_t** colptr, const int32_t
 
 dg_status_t dg_aggregate_fwd(dg_graph_t g, const float* H, int32_t F, dg_op_t op, float* out,
                              void* stream) {
-  return run_forward(g, H, false, F, op, out, stream);
+  return run_forward(g, H, false, F, op, g && g->self_loops, out, stream);
+}
+
+dg_status_t dg_aggregate_fwd_self(dg_graph_t g, const float* H, int32_t F, dg_op_t op, float* out,
+                                  void* stream) {
+  return run_forward(g, H, false, F, op, true, out, stream);
+}
+
+dg_status_t dg_aggregate_bwd_self(dg_graph_t g, const float* dOut, int32_t F, dg_op_t op, float* dH,
+                                  void* stream) {
+  return run_backward(g, dOut, false, F, op, true, dH, stream);
 }
 
 dg_status_t dg_aggregate_bwd(dg_graph_t g, const float* dOut, int32_t F, dg_op_t op, float* dH,
                              void* stream) {
-  return run_backward(g, dOut, false, F, op, dH, stream);
+  return run_backward(g, dOut, false, F, op, g && g->self_loops, dH, stream);
 }
 
 dg_status_t dg_aggregate_fwd_bf16(dg_graph_t g, const uint16_t* H, int32_t F, dg_op_t op,
                                   float* out, void* stream) {
-  return run_forward(g, H, true, F, op, out, stream);
+  return run_forward(g, H, true, F, op, g && g->self_loops, out, stream);
 }
 
 dg_status_t dg_aggregate_bwd_bf16(dg_graph_t g, const uint16_t* dOut, int32_t F, dg_op_t op,
                                   float* dH, void* stream) {
-  return run_backward(g, dOut, true, F, op, dH, stream);
+  return run_backward(g, dOut, true, F, op, g && g->self_loops, dH, stream);
 }
 
 size_t dg_aggregate_host_workspace(dg_graph_t g, int32_t F) {
