@@ -45,9 +45,11 @@ join_kernel(const Chunk* __restrict__ chunks, const CutRow* __restrict__ cuts,
 
 // out[r][0..ld) = in[r][0..F) followed by zeros, elements of T; a thread writes 16 bytes.  Reads and
 // writes are streams: bound by DRAM where the matrix exceeds L2 (561 MB of fp32 in 185 us, 6.1 TB/s read + written).
+// With mean_ptr (T = float) the rows are divided by their lengths there (+ mean_self).
 template <typename T>
 __global__ void __launch_bounds__(256)
-pad_rows_kernel(const T* __restrict__ in, int32_t F, int32_t ld, int64_t n, uint4* __restrict__ out) {
+pad_rows_kernel(const T* __restrict__ in, int32_t F, int32_t ld, int64_t n, const int64_t* __restrict__ mean_ptr,
+                int mean_self, uint4* __restrict__ out) {
   constexpr int kPer = 16 / sizeof(T);
   const uint32_t per_row = (uint32_t)ld / kPer;
   const int64_t i = (int64_t)blockIdx.x * 256 + threadIdx.x;
@@ -58,6 +60,14 @@ pad_rows_kernel(const T* __restrict__ in, int32_t F, int32_t ld, int64_t n, uint
   union { T t[kPer]; uint4 v; } u;
 #pragma unroll
   for (int q = 0; q < kPer; ++q) u.t[q] = f + q < F ? src[q] : T(0);
+  if constexpr (sizeof(T) == 4) {
+    if (mean_ptr) {
+      const int64_t len = __ldg(mean_ptr + r + 1) - __ldg(mean_ptr + r) + mean_self;
+      const float inv = len > 0 ? 1.0f / (float)len : 0.f;
+#pragma unroll
+      for (int q = 0; q < kPer; ++q) u.t[q] *= inv;
+    }
+  }
   out[i] = u.v;
 }
 
@@ -121,8 +131,20 @@ bool worth_padding(const Graph* g, int32_t F, int elem_bytes, int vec) {
          (size_t)g->n * (size_t)(F + 128 / elem_bytes) * (size_t)elem_bytes <= kPadMaxBytes;
 }
 
+// Whether the backward pass of the mean on an unweighted graph divides the rows of dOut in such a copy (also
+// when they need no padding) and runs the kernel without edge factors.  That kernel reads 4 bytes less per
+// edge and takes about 10 % less time; the copy is 8 bytes per element against nnz / n gathers of 4, so it
+// wants long rows.  Copy and kernel: degree 492, F = 602 16.9 -> 14.9 ms, F = 256 6.7 -> 5.9 ms; degree 422,
+// F = 64 565 -> 513 us; degree 85, 3.4 M edges, F = 128 162 -> 125 us.
+constexpr int64_t kDivideMinDegree = 64;
+static bool worth_dividing(const Graph* g, int32_t F) {
+  return g->nnz >= kDivideMinDegree * g->n && g->nnz * F >= kPadMinWork &&
+         (size_t)g->n * (size_t)(F + 32) * 4 <= kPadMaxBytes;
+}
+
 // Makes the copy; false when there is no memory for it (the caller then uses X as it is).
-bool pad_rows(const Graph* g, const void* X, int32_t F, int elem_bytes, cudaStream_t s, void** copy, int64_t* ld) {
+bool pad_rows(const Graph* g, const void* X, int32_t F, int elem_bytes, const int64_t* mean_ptr, int mean_self,
+              cudaStream_t s, void** copy, int64_t* ld) {
   // rows of whole 32-byte sectors, of whole 128-byte lines where a row has several
   const int64_t unit = (F * elem_bytes > 512 ? 128 : 32) / elem_bytes;
   const int64_t to = (F + unit - 1) / unit * unit;
@@ -131,11 +153,11 @@ bool pad_rows(const Graph* g, const void* X, int32_t F, int elem_bytes, cudaStre
   *ld = to;
   const unsigned blocks = (unsigned)((bytes / 16 + 255) / 256);
   if (elem_bytes == 2)
-    pad_rows_kernel<uint16_t><<<blocks, 256, 0, s>>>(static_cast<const uint16_t*>(X), F, (int32_t)to, g->n,
+    pad_rows_kernel<uint16_t><<<blocks, 256, 0, s>>>(static_cast<const uint16_t*>(X), F, (int32_t)to, g->n, nullptr, 0,
                                                      static_cast<uint4*>(*copy));
   else
-    pad_rows_kernel<uint32_t><<<blocks, 256, 0, s>>>(static_cast<const uint32_t*>(X), F, (int32_t)to, g->n,
-                                                     static_cast<uint4*>(*copy));
+    pad_rows_kernel<float><<<blocks, 256, 0, s>>>(static_cast<const float*>(X), F, (int32_t)to, g->n, mean_ptr,
+                                                  mean_self, static_cast<uint4*>(*copy));
   count_launches(1);
   return true;
 }
@@ -154,9 +176,10 @@ bool pad_rows(const Graph* g, const void* X, int32_t F, int elem_bytes, cudaStre
 //     slice of X over all n rows exceeds the L2 budget and the segments carry split pointers,
 //     the neighbour ids are cut into 2, 4, 8 or 16 ranges and each range is a launch of its
 //     own, so that the rows of X a launch gathers stay L2-resident; later launches add to Y.
-dg_status_t aggregate_run(const Graph* g, const ApArgs& a0, const SelfArgs& sa, const Plan& plan,
+dg_status_t aggregate_run(const Graph* g, const ApArgs& a0, const SelfArgs& sa0, const Plan& plan,
                           const int32_t* split, cudaStream_t s) {
   ApArgs a = a0;
+  SelfArgs sa = sa0;
   if (a.n == 0) return DG_OK;
   const uintptr_t px = (uintptr_t)a.X, py = (uintptr_t)a.Y;
   const bool bf16 = a.x_bf16 != 0;
@@ -172,7 +195,13 @@ dg_status_t aggregate_run(const Graph* g, const ApArgs& a0, const SelfArgs& sa, 
   else if (bf16 || (a.F % 2 == 0 && px % 8 == 0 && py % 8 == 0)) vec = 2;
   int64_t ld = a.F;
   void* padded = nullptr;
-  if (worth_padding(g, a.F, eb, vec) && pad_rows(g, a.X, a.F, eb, s, &padded, &ld)) {
+  const bool divide = worth_dividing(g, a.F) && a.mean_factors && !bf16;
+  if ((divide || worth_padding(g, a.F, eb, vec)) &&
+      pad_rows(g, a.X, a.F, eb, divide ? g->rowptr : nullptr, sa.self_ptr != nullptr, s, &padded, &ld)) {
+    if (divide) {  // the factors are in the copy, the own rows' too
+      a.w = nullptr;
+      sa.self_mean = 0;
+    }
     a.X = padded;
     vec = wide;
     a.narrow_store = a.F % 4 != 0 || py % 16 != 0 || (bf16 && a.F % 8 != 0);

@@ -225,6 +225,7 @@ static dg_status_t run_backward(Graph* g, const void* dOut, bool bf16, int32_t F
   a.ptr = g->colptr;
   a.idx = g->rowidx_T;
   a.w = op == DG_OP_MEAN ? g->mean_scale_T : g->w_T;
+  a.mean_factors = op == DG_OP_MEAN && !g->edge_w;
   a.X = dOut;
   a.x_bf16 = bf16;
   a.Y = dH;

@@ -135,7 +135,8 @@ dg_status_t edge_grad_run(const Graph* g, const float* H, const float* dOut, int
   if (worth_padding(g, F, 4, vec)) {
     // both rows of a dot product in the same padded layout; the padding multiplies to zero
     int64_t ld = 0;
-    if (pad_rows(g, H, F, 4, s, &padded_h, &ld) && pad_rows(g, dOut, F, 4, s, &padded_g, &ld)) {
+    if (pad_rows(g, H, F, 4, nullptr, 0, s, &padded_h, &ld) &&
+        pad_rows(g, dOut, F, 4, nullptr, 0, s, &padded_g, &ld)) {
       a.H = static_cast<const float*>(padded_h);
       a.dOut = static_cast<const float*>(padded_g);
       a.ld = ld;

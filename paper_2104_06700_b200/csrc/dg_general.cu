@@ -77,7 +77,7 @@ int vector_width(int32_t F, uintptr_t pointers) {
 // 16-byte loads of a gathered matrix whose rows forbid them, through a padded copy (returned for pool_free)
 void* widen(const dg_graph* g, GenArgs* a, cudaStream_t s) {
   void* copy = nullptr;
-  if (worth_padding(g, a->F, 4, a->vec) && pad_rows(g, a->X, a->F, 4, s, &copy, &a->ldx)) {
+  if (worth_padding(g, a->F, 4, a->vec) && pad_rows(g, a->X, a->F, 4, nullptr, 0, s, &copy, &a->ldx)) {
     a->X = static_cast<const float*>(copy);
     a->vec = 4;
   }

@@ -129,6 +129,7 @@ struct ApArgs {
   const int32_t* seg_hi;      //   segment's piece (n entries each); nullptr = whole segments
   int32_t accumulate;         // source-blocked pass after the first: add to what Y holds
   int32_t few_blocks;         // host side: the grid is small, see ap_kernel
+  int32_t mean_factors;       // host side: w are the factors 1 / deg (+ 1) of the mean's backward pass alone
 };
 
 // Implicit self loops (every vertex its own neighbour with weight 1): row r also receives
@@ -199,7 +200,8 @@ dg_status_t expand_rows(const int64_t* rowptr, int64_t n, int64_t nnz, const int
 
 // Whether a call first copies a gathered matrix into padded rows, and the copy (dg_aggregate.cu).
 bool worth_padding(const Graph* g, int32_t F, int elem_bytes, int vec);
-bool pad_rows(const Graph* g, const void* X, int32_t F, int elem_bytes, cudaStream_t s, void** copy, int64_t* ld);
+bool pad_rows(const Graph* g, const void* X, int32_t F, int elem_bytes, const int64_t* mean_ptr, int mean_self,
+              cudaStream_t s, void** copy, int64_t* ld);
 // Scratch for the parts of cut rows (nullptr when the plan cuts none), and their join.
 dg_status_t take_partial(const Graph* g, const Plan& plan, int64_t floats_per_slot, cudaStream_t s,
                          float** partial);
