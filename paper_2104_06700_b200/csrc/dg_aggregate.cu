@@ -259,7 +259,7 @@ dg_status_t aggregate_run(const Graph* g, const ApArgs& a0, const SelfArgs& sa0,
 
   a.chunks = plan.chunks;
   a.chunk_count = (int32_t)plan.count;
-  a.few_blocks = plan.count * slices <= (int64_t)g->sm_count * 4 * kWarpsPerBlock;
+  a.few_blocks = plan.count * slices <= 4 * (int64_t)g->sm_count * 4 * kWarpsPerBlock;  // four waves
   dg_status_t st = take_partial(g, plan, a.F, s, &a.partial);
   const int per = kFineBlocks / nb;
   for (int j = 0; j < nb && st == DG_OK; ++j) {
