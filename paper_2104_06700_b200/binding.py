@@ -337,7 +337,7 @@ class Graph:
         """H is a torch.bfloat16 matrix; the result is fp32."""
         F = H.shape[1]
         if out is None:
-            out = torch.empty(H.shape, dtype=torch.float32, device=H.device)
+            out = torch.empty_like(H, dtype=torch.float32)
         _check(lib().dg_aggregate_fwd_bf16(self._h, _dev_ptr(H, torch.bfloat16, "H"), F, int(op),
                                            _dev_ptr(out, torch.float32, "out"), _stream(stream)))
         return out
@@ -346,7 +346,7 @@ class Graph:
                               dH: Optional[torch.Tensor] = None, stream=None) -> torch.Tensor:
         F = dOut.shape[1]
         if dH is None:
-            dH = torch.empty(dOut.shape, dtype=torch.float32, device=dOut.device)
+            dH = torch.empty_like(dOut, dtype=torch.float32)
         _check(lib().dg_aggregate_bwd_bf16(self._h, _dev_ptr(dOut, torch.bfloat16, "dOut"), F,
                                            int(op), _dev_ptr(dH, torch.float32, "dH"),
                                            _stream(stream)))
