@@ -480,9 +480,10 @@ __device__ __forceinline__ void ap_body(const ApArgs& a, const SelfArgs sa) {
 
 // BLOCKS blocks per SM.  Six (40 registers): three to eight blocks are within 5 % of each other on every large
 // workload (the gather is what they wait for, not the register file), six is the best for most.  Four (64
-// registers) on grids that fit in one wave of those: occupancy is no limit there, and with 40 registers
-// not all of a lane's eight loads are in flight (forward + backward, 40 k edges, F = 256: 38.2 -> 30.7 us; 74 k
-// edges, F = 100: 36.9 -> 32.6 us).
+// registers) on grids of up to four waves of those: latency is the limit there, and with 40 registers not all
+// of a lane's eight loads are in flight (forward + backward, kernels: 40 k edges, F = 256: 29.1 -> 21.3 us; 184 k,
+// F = 256, bf16: 27.2 -> 24.7; 619 k, F = 100: 42.7 -> 39.1 of two waves or more; but 125 k, F = 48, bf16:
+// 17.9 -> 20.6).  At eight waves the two are equal.
 template <typename E, int VEC, int G, int CPL, bool SCALED, bool SEG, int BLOCKS>
 __global__ void __launch_bounds__(kBlock, BLOCKS) ap_kernel(const ApArgs a) {
   ap_body<E, VEC, G, CPL, SCALED, SEG, false>(a, SelfArgs{});
