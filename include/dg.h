@@ -194,7 +194,22 @@ dg_status_t dg_aggregate_bwd_self(dg_graph_t g, const float* dOut, int32_t F, dg
                                   void* stream);
 
 /*
- * The same two passes with the gathered matrix stored as bf16 (two bytes per element, the
+ * The elementwise passes of a GraphSAGE layer  out = act(D Z + b)  around its GEMM, on n x F fp32 matrices
+ * (rows = the handle's vertices), D = diag(row_scale).
+ *
+ *   fwd:  Y[v,f] = act(row_scale[v] * Y[v,f] + bias[f]) in place; act = ReLU if `relu`, else the identity.
+ *   bwd:  d[v,f] = out[v,f] <= 0 ? 0 : dOut[v,f]  (`out` NULL: d = dOut);
+ *         G[v,f] = row_scale[v] * d[v,f];  dbias[f] = sum over v of d[v,f], always in the same order.
+ *         G may be dOut itself.
+ * Asynchronous on `stream`.
+ */
+dg_status_t dg_layer_fwd(dg_graph_t g, float* Y, int32_t F, const float* row_scale, const float* bias,
+                         int32_t relu, void* stream);
+dg_status_t dg_layer_bwd(dg_graph_t g, const float* dOut, const float* out, int32_t F, const float* row_scale,
+                         float* G, float* dbias, void* stream);
+
+/*
+ * dg_aggregate_fwd / dg_aggregate_bwd with the gathered matrix stored as bf16 (two bytes per element, the
  * upper half of an fp32; the paper's Conclusion names reduced precision as future work).  Every
  * gathered byte is halved; products and sums are fp32 (a bf16 value converts to fp32 exactly)
  * and the output is fp32, so the result equals the fp32 entry point's on the same values and

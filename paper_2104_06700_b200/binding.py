@@ -29,7 +29,7 @@ DG_ORDER_GIVEN, DG_ORDER_OUT_DEGREE, DG_ORDER_IN_DEGREE = range(3)
 EXPORTS = [
     "dg_graph_create", "dg_graph_destroy", "dg_graph_validate", "dg_graph_transpose_workspace",
     "dg_graph_transpose", "dg_graph_transpose_static", "dg_graph_update_weights", "dg_graph_get_csc", "dg_aggregate_fwd", "dg_aggregate_bwd",
-    "dg_aggregate_fwd_self", "dg_aggregate_bwd_self",
+    "dg_aggregate_fwd_self", "dg_aggregate_bwd_self", "dg_layer_fwd", "dg_layer_bwd",
     "dg_aggregate_fwd_bf16", "dg_aggregate_bwd_bf16",
     "dg_ap_fwd", "dg_ap_bwd", "dg_aggregate_edge_grad",
     "dg_graph_reorder_workspace", "dg_graph_reorder", "dg_graph_get_order", "dg_permute_rows",
@@ -71,6 +71,8 @@ def lib() -> ctypes.CDLL:
         L.dg_aggregate_bwd.argtypes = [p, p, i32, ctypes.c_int, p, p]
         L.dg_aggregate_fwd_self.argtypes = [p, p, i32, ctypes.c_int, p, p]
         L.dg_aggregate_bwd_self.argtypes = [p, p, i32, ctypes.c_int, p, p]
+        L.dg_layer_fwd.argtypes = [p, p, i32, p, p, i32, p]
+        L.dg_layer_bwd.argtypes = [p, p, p, i32, p, p, p, p]
         L.dg_aggregate_fwd_bf16.argtypes = [p, p, i32, ctypes.c_int, p, p]
         L.dg_aggregate_bwd_bf16.argtypes = [p, p, i32, ctypes.c_int, p, p]
         L.dg_ap_fwd.argtypes = [p, p, p, i32, i32, ctypes.c_int, ctypes.c_int, p, p, p]
@@ -331,6 +333,26 @@ class Graph:
                                            dOut.shape[1], int(op),
                                            _dev_ptr(dH, torch.float32, "dH"), _stream(stream)))
         return dH
+
+    def dg_layer_fwd(self, Y: torch.Tensor, row_scale: torch.Tensor, bias: torch.Tensor, relu: bool,
+                     stream=None) -> torch.Tensor:
+        """Y = act(row_scale * Y + bias), in place."""
+        _check(lib().dg_layer_fwd(self._h, _dev_ptr(Y, torch.float32, "Y"), Y.shape[1],
+                                  _dev_ptr(row_scale, torch.float32, "row_scale"),
+                                  _dev_ptr(bias, torch.float32, "bias"), bool(relu), _stream(stream)))
+        return Y
+
+    def dg_layer_bwd(self, dOut: torch.Tensor, out: Optional[torch.Tensor], row_scale: torch.Tensor,
+                     stream=None):
+        """(row_scale * d, column sums of d) with d = dOut where out > 0 (out None: dOut)."""
+        G = torch.empty_like(dOut)
+        dbias = dOut.new_empty(dOut.shape[1])
+        _check(lib().dg_layer_bwd(self._h, _dev_ptr(dOut, torch.float32, "dOut"),
+                                  _dev_ptr(out, torch.float32, "out"), dOut.shape[1],
+                                  _dev_ptr(row_scale, torch.float32, "row_scale"),
+                                  _dev_ptr(G, torch.float32, "G"), _dev_ptr(dbias, torch.float32, "dbias"),
+                                  _stream(stream)))
+        return G, dbias
 
     def dg_aggregate_fwd_bf16(self, H: torch.Tensor, op: int, out: Optional[torch.Tensor] = None,
                               stream=None) -> torch.Tensor:

@@ -420,6 +420,23 @@ dg_status_t dg_aggregate_bwd_self(dg_graph_t g, const float* dOut, int32_t F, dg
   return run_backward(g, dOut, false, F, op, true, dH, stream);
 }
 
+dg_status_t dg_layer_fwd(dg_graph_t g, float* Y, int32_t F, const float* row_scale, const float* bias,
+                         int32_t relu, void* stream) {
+  if (!g) return invalid("graph handle is NULL");
+  if (F < 1 || F > (1 << 20)) return invalid("F must be from 1 to 2^20");
+  if (g->n == 0) return DG_OK;
+  if (!Y || !row_scale || !bias) return invalid("a pointer is NULL");
+  return layer_fwd(g, Y, F, row_scale, bias, relu != 0, (cudaStream_t)stream);
+}
+
+dg_status_t dg_layer_bwd(dg_graph_t g, const float* dOut, const float* out, int32_t F, const float* row_scale,
+                         float* G, float* dbias, void* stream) {
+  if (!g) return invalid("graph handle is NULL");
+  if (F < 1 || F > (1 << 20)) return invalid("F must be from 1 to 2^20");
+  if (!dbias || (g->n > 0 && (!dOut || !row_scale || !G))) return invalid("a pointer is NULL");
+  return layer_bwd(g, dOut, out, F, row_scale, G, dbias, (cudaStream_t)stream);
+}
+
 dg_status_t dg_aggregate_bwd(dg_graph_t g, const float* dOut, int32_t F, dg_op_t op, float* dH,
                              void* stream) {
   return run_backward(g, dOut, false, F, op, g && g->self_loops, dH, stream);

@@ -178,6 +178,12 @@ bool wants_split(int64_t n, int64_t nnz);
 dg_status_t build_split(const int64_t* ptr, const int32_t* idx, int64_t n, int64_t fine_rows,
                         int32_t* split, int32_t* unsorted_flag, const int32_t* malformed, cudaStream_t s);
 
+// dg_layer.cu
+dg_status_t layer_fwd(const Graph* g, float* Y, int32_t F, const float* scale, const float* bias, bool relu,
+                      cudaStream_t s);
+dg_status_t layer_bwd(const Graph* g, const float* dOut, const float* out, int32_t F, const float* scale,
+                      float* G, float* dbias, cudaStream_t s);
+
 // dg_transpose.cu
 void transpose_sizes(int64_t n, int64_t nnz, bool weighted, size_t* csc_bytes,
                      size_t* scratch_bytes);
