@@ -4,7 +4,7 @@ columns, one row, and more rows than the grid holds at once."""
 import pytest
 import torch
 
-from paper_2104_06700_b200 import binding
+from paper_2104_06700_b200 import binding, graphsage
 
 pytestmark = pytest.mark.gpu
 DEV = "cuda"
@@ -52,3 +52,12 @@ def test_nan_passes_through_and_arguments_are_checked():
     for bad in (dict(row_scale=None), dict(bias=None)):
         with pytest.raises(binding.DgError):
             g.dg_layer_fwd(out, **{"row_scale": scale, "bias": bias, "relu": True, **bad})
+
+
+@pytest.mark.parametrize("n", [8191, 8192, 8257, 20000])
+def test_weight_gradient_in_slices(n):
+    gen = torch.Generator(device=DEV).manual_seed(n)
+    G, X = torch.randn(n, 130, device=DEV, generator=gen), torch.randn(n, 128, device=DEV, generator=gen)
+    want = G.double().t() @ X.double()
+    bound = n * EPS * (G.double().abs().t() @ X.double().abs())
+    assert bool(((graphsage._weight_grad(G, X).double() - want).abs() <= bound).all())
