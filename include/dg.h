@@ -209,6 +209,23 @@ dg_status_t dg_layer_bwd(dg_graph_t g, const float* dOut, const float* out, int3
                          float* G, float* dbias, void* stream);
 
 /*
+ * Mean softmax cross-entropy of the rows index[0..count) of the n x C matrix `logits` against
+ * labels[index[t]] (n labels; -100: the row does not count), and its gradient.
+ *
+ *   fwd:  result[0] = the mean loss (NaN if no row counts or an index or a label is out of range),
+ *         result[1] = 1 / rows that count, stats = 2 * count floats, 8-byte aligned, for the backward pass.
+ *   bwd:  dLogits (n x C, all rows written) = grad[0] * d result[0] / d logits; rows that do not count and
+ *         rows out of range add nothing.
+ * Negative indices count from the end.  Results are the same in every run.  Asynchronous on `stream`.
+ */
+dg_status_t dg_cross_entropy_fwd(dg_graph_t g, const float* logits, int32_t C, const int64_t* index,
+                                 int64_t count, const int64_t* labels, float* stats, float* result,
+                                 void* stream);
+dg_status_t dg_cross_entropy_bwd(dg_graph_t g, const float* logits, int32_t C, const int64_t* index,
+                                 int64_t count, const int64_t* labels, const float* stats,
+                                 const float* result, const float* grad, float* dLogits, void* stream);
+
+/*
  * dg_aggregate_fwd / dg_aggregate_bwd with the gathered matrix stored as bf16 (two bytes per element, the
  * upper half of an fp32; the paper's Conclusion names reduced precision as future work).  Every
  * gathered byte is halved; products and sums are fp32 (a bf16 value converts to fp32 exactly)

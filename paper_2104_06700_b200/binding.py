@@ -30,6 +30,7 @@ EXPORTS = [
     "dg_graph_create", "dg_graph_destroy", "dg_graph_validate", "dg_graph_transpose_workspace",
     "dg_graph_transpose", "dg_graph_transpose_static", "dg_graph_update_weights", "dg_graph_get_csc", "dg_aggregate_fwd", "dg_aggregate_bwd",
     "dg_aggregate_fwd_self", "dg_aggregate_bwd_self", "dg_layer_fwd", "dg_layer_bwd",
+    "dg_cross_entropy_fwd", "dg_cross_entropy_bwd",
     "dg_aggregate_fwd_bf16", "dg_aggregate_bwd_bf16",
     "dg_ap_fwd", "dg_ap_bwd", "dg_aggregate_edge_grad",
     "dg_graph_reorder_workspace", "dg_graph_reorder", "dg_graph_get_order", "dg_permute_rows",
@@ -73,6 +74,8 @@ def lib() -> ctypes.CDLL:
         L.dg_aggregate_bwd_self.argtypes = [p, p, i32, ctypes.c_int, p, p]
         L.dg_layer_fwd.argtypes = [p, p, i32, p, p, i32, p]
         L.dg_layer_bwd.argtypes = [p, p, p, i32, p, p, p, p]
+        L.dg_cross_entropy_fwd.argtypes = [p, p, i32, p, i64, p, p, p, p]
+        L.dg_cross_entropy_bwd.argtypes = [p, p, i32, p, i64, p, p, p, p, p, p]
         L.dg_aggregate_fwd_bf16.argtypes = [p, p, i32, ctypes.c_int, p, p]
         L.dg_aggregate_bwd_bf16.argtypes = [p, p, i32, ctypes.c_int, p, p]
         L.dg_ap_fwd.argtypes = [p, p, p, i32, i32, ctypes.c_int, ctypes.c_int, p, p, p]
@@ -353,6 +356,28 @@ class Graph:
                                   _dev_ptr(G, torch.float32, "G"), _dev_ptr(dbias, torch.float32, "dbias"),
                                   _stream(stream)))
         return G, dbias
+
+    def dg_cross_entropy_fwd(self, logits: torch.Tensor, index: torch.Tensor, labels: torch.Tensor, stream=None):
+        """(result, stats): result[0] is the mean loss of logits[index] against labels[index]."""
+        result, stats = logits.new_empty(2), logits.new_empty((index.shape[0], 2))
+        _check(lib().dg_cross_entropy_fwd(self._h, _dev_ptr(logits, torch.float32, "logits"), logits.shape[1],
+                                          _dev_ptr(index, torch.int64, "index"), index.shape[0],
+                                          _dev_ptr(labels, torch.int64, "labels"), stats.data_ptr(),
+                                          result.data_ptr(), _stream(stream)))
+        return result, stats
+
+    def dg_cross_entropy_bwd(self, logits: torch.Tensor, index: torch.Tensor, labels: torch.Tensor,
+                             result: torch.Tensor, stats: torch.Tensor, grad: torch.Tensor,
+                             stream=None) -> torch.Tensor:
+        d = torch.empty_like(logits)
+        _check(lib().dg_cross_entropy_bwd(self._h, _dev_ptr(logits, torch.float32, "logits"), logits.shape[1],
+                                          _dev_ptr(index, torch.int64, "index"), index.shape[0],
+                                          _dev_ptr(labels, torch.int64, "labels"),
+                                          _dev_ptr(stats, torch.float32, "stats"),
+                                          _dev_ptr(result, torch.float32, "result"),
+                                          _dev_ptr(grad, torch.float32, "grad"), d.data_ptr(),
+                                          _stream(stream)))
+        return d
 
     def dg_aggregate_fwd_bf16(self, H: torch.Tensor, op: int, out: Optional[torch.Tensor] = None,
                               stream=None) -> torch.Tensor:

@@ -184,6 +184,13 @@ dg_status_t layer_fwd(const Graph* g, float* Y, int32_t F, const float* scale, c
 dg_status_t layer_bwd(const Graph* g, const float* dOut, const float* out, int32_t F, const float* scale,
                       float* G, float* dbias, cudaStream_t s);
 
+// dg_loss.cu
+dg_status_t loss_fwd(const Graph* g, const float* logits, int32_t C, const int64_t* index, int64_t count,
+                     const int64_t* labels, float* stats, float* result, cudaStream_t s);
+dg_status_t loss_bwd(const Graph* g, const float* logits, int32_t C, const int64_t* index, int64_t count,
+                     const int64_t* labels, const float* stats, const float* result, const float* grad,
+                     float* d, cudaStream_t s);
+
 // dg_transpose.cu
 void transpose_sizes(int64_t n, int64_t nnz, bool weighted, size_t* csc_bytes,
                      size_t* scratch_bytes);

@@ -112,6 +112,22 @@ class _GcnLayer(torch.autograd.Function):
         return dM, dW, db if needs[2] else None, None, None, None, None
 
 
+class _CrossEntropy(torch.autograd.Function):
+    """torch's cross_entropy(logits[index], labels[index]) in two kernels forward and one backward."""
+
+    @staticmethod
+    def forward(ctx, logits, index, labels, graph):
+        result, stats = graph.dg_cross_entropy_fwd(logits, index, labels)
+        ctx.graph = graph
+        ctx.save_for_backward(logits, index, labels, result, stats)
+        return result[0].clone()
+
+    @staticmethod
+    def backward(ctx, grad: torch.Tensor):
+        logits, index, labels, result, stats = ctx.saved_tensors
+        return ctx.graph.dg_cross_entropy_bwd(logits, index, labels, result, stats, grad), None, None, None
+
+
 def aggregate(graph: "binding.Graph", H: torch.Tensor, op: int = binding.DG_OP_SUM,
               bf16: bool = False, row_scale=None, edge_w=None) -> torch.Tensor:
     """Differentiable aggregation primitive (the graph must have been transposed).
@@ -190,10 +206,25 @@ def make_epoch(model: GraphSAGE, X: torch.Tensor, labels: torch.Tensor, train_id
     opt = torch.optim.Adam(model.parameters(), lr=lr, weight_decay=weight_decay,
                            fused=all(p.is_cuda for p in model.parameters()))
 
+    n = model.graph.n
+    # vertex indices and class indices, one row of logits each; masks, probabilities and the like are torch's
+    plain = (train_idx.dtype == labels.dtype == torch.int64 and train_idx.dim() == labels.dim() == 1
+             and train_idx.is_contiguous() and labels.is_contiguous() and labels.shape[0] == n
+             and train_idx.is_cuda and labels.is_cuda)
+    if plain and train_idx.numel():     # the kernel has no way to raise: it returns NaN
+        if int(train_idx.min()) < -n or int(train_idx.max()) >= n:
+            raise IndexError("train_idx holds an index outside the graph")
+        y = labels[train_idx]
+        if bool(((y != -100) & ((y < 0) | (y >= model.lin[-1].out_features))).any()):
+            raise IndexError("labels holds a class outside the model's last layer")
+
     def epoch() -> torch.Tensor:
         opt.zero_grad(set_to_none=True)
         logits = model(X)
-        loss = torch.nn.functional.cross_entropy(logits[train_idx], labels[train_idx])
+        if plain:
+            loss = _CrossEntropy.apply(logits, train_idx, labels, model.graph)
+        else:
+            loss = torch.nn.functional.cross_entropy(logits[train_idx], labels[train_idx])
         loss.backward()
         opt.step()
         return loss.detach()
