@@ -1,14 +1,13 @@
 """Full-batch GraphSAGE with the GCN aggregator (Section 5.1 of the paper, Models and
 Parameters), as the composite workload the epoch-time metric is quoted on.
 
-Only the aggregation primitive runs in libdgagg; everything dense stays in torch, outside the
-hot path: per layer  z_v = (sum_{u in N(v)} h_u + h_v) / (deg(v) + 1),  h'_v = act(z_v W + b)
-(aggregate first, then the Linear: Table 8 of the paper lists the aggregation widths 100, 256,
-256 for the 3-layer model, i.e. the layers' input widths), ReLU between layers, none after the
-last, softmax cross-entropy on a training mask, Adam.  The features need no gradient, so an
-L-layer epoch runs L forward and L-1 backward aggregations.  With ``fused_aggregator`` the
-own row and the division are done by the library inside the aggregation kernels (graph
-attribute "self_loops"), which saves the elementwise passes over the n x F matrices.
+libdgagg runs the aggregation with the own row, the elementwise passes of a layer and the loss; the
+GEMMs and Adam are torch's.  Per layer  z_v = (sum_{u in N(v)} h_u + h_v) / (deg(v) + 1),
+h'_v = act(z_v W + b)  (aggregate first, then the Linear: Table 8 of the paper lists the aggregation
+widths 100, 256, 256 for the 3-layer model, i.e. the layers' input widths), ReLU between layers, none
+after the last, softmax cross-entropy on a training mask, Adam.  The features need no gradient, so an
+L-layer epoch runs L forward and L-1 backward aggregations.  ``fused_aggregator`` is for handles with
+the graph attribute "self_loops", which add the own row in every call.
 """
 from __future__ import annotations
 
@@ -75,6 +74,17 @@ def _weight_grad(G: torch.Tensor, X: torch.Tensor) -> torch.Tensor:
     return dW.addmm_(G[m:].t(), X[m:]) if m < n else dW
 
 
+def _with_own_row(graph: "binding.Graph", M: torch.Tensor, bf16: bool, transposed: bool) -> torch.Tensor:
+    """(A + I) M, or with ``transposed`` (A^T + I) M.  bf16: the gathered rows are rounded; the own row too where
+    the handle adds it itself."""
+    if not bf16:
+        call = graph.dg_aggregate_bwd_self if transposed else graph.dg_aggregate_fwd_self
+        return call(M, binding.DG_OP_SUM)
+    call = graph.dg_aggregate_bwd_bf16 if transposed else graph.dg_aggregate_fwd_bf16
+    out = call(M.to(torch.bfloat16), binding.DG_OP_SUM)
+    return out if graph.dg_graph_get_param("self_loops") else out.add_(M)
+
+
 class _GcnLayer(torch.autograd.Function):
     """One layer  act(D (A M + M) W^T + b),  D = diag(1 / (deg + 1)),  with the own row added inside the
     aggregation kernel.  D is applied after the GEMM, forward together with bias and ReLU, backward together
@@ -84,15 +94,15 @@ class _GcnLayer(torch.autograd.Function):
     ``project``: D ((A + I) (M W^T)) + b instead, the narrower product aggregated."""
 
     @staticmethod
-    def forward(ctx, M, weight, bias, graph, inv_deg1, relu: bool, project: bool):
+    def forward(ctx, M, weight, bias, graph, inv_deg1, relu: bool, project: bool, bf16: bool):
         M = M.contiguous()
         if project:
-            Z, X = graph.dg_aggregate_fwd_self(M @ weight.t(), binding.DG_OP_SUM), M
+            Z, X = _with_own_row(graph, M @ weight.t(), bf16, False), M
         else:
-            X = graph.dg_aggregate_fwd_self(M, binding.DG_OP_SUM)
+            X = _with_own_row(graph, M, bf16, False)
             Z = X @ weight.t()
         out = graph.dg_layer_fwd(Z, inv_deg1, bias.contiguous(), relu)
-        ctx.graph, ctx.project, ctx.relu = graph, project, relu
+        ctx.graph, ctx.project, ctx.bf16 = graph, project, bf16
         ctx.save_for_backward(X, weight, inv_deg1, out if relu else None)
         return out
 
@@ -102,14 +112,14 @@ class _GcnLayer(torch.autograd.Function):
         graph, needs = ctx.graph, ctx.needs_input_grad
         G, db = graph.dg_layer_bwd(dOut.contiguous(), out, inv_deg1)
         if ctx.project and (needs[0] or needs[1]):
-            G = graph.dg_aggregate_bwd_self(G, binding.DG_OP_SUM)
+            G = _with_own_row(graph, G, ctx.bf16, True)
         dW = _weight_grad(G, X) if needs[1] else None
         dM = None
         if needs[0]:
             dM = G @ weight
             if not ctx.project:
-                dM = graph.dg_aggregate_bwd_self(dM, binding.DG_OP_SUM)
-        return dM, dW, db if needs[2] else None, None, None, None, None
+                dM = _with_own_row(graph, dM, ctx.bf16, True)
+        return dM, dW, db if needs[2] else None, None, None, None, None, None
 
 
 class _CrossEntropy(torch.autograd.Function):
@@ -155,14 +165,8 @@ class GraphSAGE(torch.nn.Module):
         self.graph = graph
         self.project_first = project_first
         self.bf16_aggregate = bf16_aggregate   # aggregate bf16-rounded activations (even widths)
-        # the whole aggregator (own row added, division by in-degree + 1) inside the library's
-        # kernels, forward and backward: needs a handle whose "self_loops" attribute was set
-        # to 1 before dg_graph_transpose
+        # for a handle whose "self_loops" attribute was set to 1 before dg_graph_transpose
         self.fused_aggregator = fused_aggregator
-        # backward of the fused aggregator: per-edge factors tabulated by the transpose (short
-        # rows: the elementwise pass would cost more than the factors), or dOut scaled row by
-        # row and the sum backward (long rows)
-        self.scaled_backward = graph.nnz < 64 * graph.n
         if fused_aggregator and graph.dg_graph_get_param("self_loops") != 1:
             raise ValueError("fused_aggregator needs a graph handle with self_loops = 1")
         if not fused_aggregator and graph.dg_graph_get_param("self_loops") != 0:
@@ -172,29 +176,13 @@ class GraphSAGE(torch.nn.Module):
         deg = (graph.rowptr[1:] - graph.rowptr[:-1]).to(torch.float32)
         self.register_buffer("inv_deg1", (1.0 / (deg + 1.0)).unsqueeze(1))
 
-    def _bf16_layer(self, H: torch.Tensor, lin: torch.nn.Linear, project: bool) -> torch.Tensor:
-        P = torch.nn.functional.linear(H, lin.weight) if project else H
-        if self.fused_aggregator:
-            Z = aggregate(self.graph, P, binding.DG_OP_MEAN, True,
-                          None if self.scaled_backward else self.inv_deg1)
-        else:       # only the neighbours' rows are rounded
-            Z = (aggregate(self.graph, P, binding.DG_OP_SUM, True) + P) * self.inv_deg1
-        if project:
-            return Z + lin.bias
-        # the bias as an in-place pass of its own: as the epilogue of the fp32 GEMM it ran in a kernel that
-        # took longer (245 k vertices, 3 layers of 256, 256 and 47: 0.61 against 0.37 ms)
-        return torch.nn.functional.linear(Z, lin.weight).add_(lin.bias)
-
     def forward(self, H: torch.Tensor) -> torch.Tensor:
         for i, lin in enumerate(self.lin):
             project = self.project_first and lin.out_features < lin.in_features
             relu = i + 1 < len(self.lin)
             width = lin.out_features if project else lin.in_features
-            if self.bf16_aggregate and width % 2 == 0:
-                H = self._bf16_layer(H, lin, project)
-                H = torch.relu_(H) if relu else H
-            else:
-                H = _GcnLayer.apply(H, lin.weight, lin.bias, self.graph, self.inv_deg1, relu, project)
+            H = _GcnLayer.apply(H, lin.weight, lin.bias, self.graph, self.inv_deg1, relu, project,
+                                self.bf16_aggregate and width % 2 == 0)
         return H
 
 
