@@ -17,6 +17,7 @@ join_kernel(const Chunk* __restrict__ chunks, const CutRow* __restrict__ cuts,
   __shared__ float part[kWarpsPerBlock][128];
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   const int f0 = blockIdx.y * 128;
+  cudaGridDependencySynchronize();
   const int cut_rows = min(__ldg(totals + 1), max_cuts);
   for (int i = blockIdx.x; i < cut_rows; i += gridDim.x) {
     const CutRow cut = cuts[i];
@@ -50,6 +51,7 @@ template <typename T>
 __global__ void __launch_bounds__(256)
 pad_rows_kernel(const T* __restrict__ in, int32_t F, int32_t ld, int64_t n, const int64_t* __restrict__ mean_ptr,
                 int mean_self, uint4* __restrict__ out) {
+  cudaTriggerProgrammaticLaunchCompletion();
   constexpr int kPer = 16 / sizeof(T);
   const uint32_t per_row = (uint32_t)ld / kPer;
   const int64_t i = (int64_t)blockIdx.x * 256 + threadIdx.x;
@@ -96,9 +98,8 @@ dg_status_t join_cut_rows(const Graph* g, const Plan& plan, const float* partial
   int64_t blocks = plan.cut_rows >= 0 ? plan.cut_rows : plan.max_cuts;
   if (blocks > (int64_t)g->sm_count * 64) blocks = (int64_t)g->sm_count * 64;
   const dim3 grid((unsigned)blocks, (unsigned)((F + 127) / 128));
-  join_kernel<<<grid, kBlock, 0, s>>>(plan.chunks, plan.cuts, plan.totals, (int32_t)plan.max_cuts, partial, F,
-                                      Y);
-  DG_CUDA(cudaGetLastError());
+  DG_CUDA(launch_kernel(join_kernel, grid, kBlock, s, true, (const Chunk*)plan.chunks, (const CutRow*)plan.cuts,
+                        (const int32_t*)plan.totals, (int32_t)plan.max_cuts, partial, F, Y));
   count_launches(1);
   return DG_OK;
 }
@@ -203,6 +204,7 @@ dg_status_t aggregate_run(const Graph* g, const ApArgs& a0, const SelfArgs& sa0,
       sa.self_mean = 0;
     }
     a.X = padded;
+    a.overlap = 1;
     vec = wide;
     a.narrow_store = a.F % 4 != 0 || py % 16 != 0 || (bf16 && a.F % 8 != 0);
   }
@@ -267,6 +269,7 @@ dg_status_t aggregate_run(const Graph* g, const ApArgs& a0, const SelfArgs& sa0,
       a.seg_lo = split + (size_t)(j * per) * (size_t)a.n;
       a.seg_hi = split + (size_t)((j + 1) * per) * (size_t)a.n;
       a.accumulate = j > 0;
+      a.overlap = a.overlap && j == 0;
     }
     st = sa.self_ptr ? launch_with_self_loops(a, sa, vec, slices, s) : launch_plain(a, vec, slices, s);
   }

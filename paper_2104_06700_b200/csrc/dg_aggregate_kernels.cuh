@@ -486,28 +486,34 @@ __device__ __forceinline__ void ap_body(const ApArgs& a, const SelfArgs sa) {
 // 17.9 -> 20.6).  At eight waves the two are equal.
 template <typename E, int VEC, int G, int CPL, bool SCALED, bool SEG, int BLOCKS>
 __global__ void __launch_bounds__(kBlock, BLOCKS) ap_kernel(const ApArgs a) {
+  cudaGridDependencySynchronize();            // the padded copy
+  cudaTriggerProgrammaticLaunchCompletion();  // the join's blocks may wait beside the last of these
   ap_body<E, VEC, G, CPL, SCALED, SEG, false>(a, SelfArgs{});
 }
 
 // The same for graphs with implicit self loops: every row also sums its own input row.
 template <typename E, int VEC, int G, int CPL, bool SCALED, bool SEG, int BLOCKS>
 __global__ void __launch_bounds__(kBlock, BLOCKS) ap_kernel_self(const ApArgs a, const SelfArgs sa) {
+  cudaGridDependencySynchronize();            // the padded copy
+  cudaTriggerProgrammaticLaunchCompletion();  // the join's blocks may wait beside the last of these
   ap_body<E, VEC, G, CPL, SCALED, SEG, true>(a, sa);
 }
 
 template <typename E, int VEC, int G, int CPL, bool SCALED, bool SELF>
 dg_status_t launch_variant(const ApArgs& a, const SelfArgs& sa, int slices, cudaStream_t s) {
   const dim3 grid((unsigned)((a.chunk_count + kWarpsPerBlock - 1) / kWarpsPerBlock), (unsigned)slices);
+  const bool overlap = a.overlap;
   if constexpr (SELF) {
-    if (a.seg_lo) ap_kernel_self<E, VEC, G, CPL, SCALED, true, 6><<<grid, kBlock, 0, s>>>(a, sa);
-    else if (a.few_blocks) ap_kernel_self<E, VEC, G, CPL, SCALED, false, 4><<<grid, kBlock, 0, s>>>(a, sa);
-    else ap_kernel_self<E, VEC, G, CPL, SCALED, false, 6><<<grid, kBlock, 0, s>>>(a, sa);
+    auto kernel = a.seg_lo ? ap_kernel_self<E, VEC, G, CPL, SCALED, true, 6>
+                  : a.few_blocks ? ap_kernel_self<E, VEC, G, CPL, SCALED, false, 4>
+                                 : ap_kernel_self<E, VEC, G, CPL, SCALED, false, 6>;
+    DG_CUDA(launch_kernel(kernel, grid, kBlock, s, overlap, a, sa));
   } else {
-    if (a.seg_lo) ap_kernel<E, VEC, G, CPL, SCALED, true, 6><<<grid, kBlock, 0, s>>>(a);
-    else if (a.few_blocks) ap_kernel<E, VEC, G, CPL, SCALED, false, 4><<<grid, kBlock, 0, s>>>(a);
-    else ap_kernel<E, VEC, G, CPL, SCALED, false, 6><<<grid, kBlock, 0, s>>>(a);
+    auto kernel = a.seg_lo ? ap_kernel<E, VEC, G, CPL, SCALED, true, 6>
+                  : a.few_blocks ? ap_kernel<E, VEC, G, CPL, SCALED, false, 4>
+                                 : ap_kernel<E, VEC, G, CPL, SCALED, false, 6>;
+    DG_CUDA(launch_kernel(kernel, grid, kBlock, s, overlap, a));
   }
-  DG_CUDA(cudaGetLastError());
   count_launches(1);
   return DG_OK;
 }

@@ -128,6 +128,7 @@ struct ApArgs {
   const int32_t* seg_lo;      // source-blocked pass: first and one-past-last position of every
   const int32_t* seg_hi;      //   segment's piece (n entries each); nullptr = whole segments
   int32_t accumulate;         // source-blocked pass after the first: add to what Y holds
+  int32_t overlap;            // host side: launch while the previous kernel (the copy) drains, see launch_kernel
   int32_t few_blocks;         // host side: the grid is small, see ap_kernel
   int32_t mean_factors;       // host side: w are the factors 1 / deg (+ 1) of the mean's backward pass alone
 };
@@ -153,6 +154,25 @@ dg_status_t launch_with_self_loops(const ApArgs& a, const SelfArgs& sa, int vec,
 void set_error(const char* fmt, ...) __attribute__((format(printf, 1, 2)));
 dg_status_t cuda_fail(cudaError_t e, const char* what);
 void count_launches(int64_t k);
+
+// Launches `kernel`; with `overlap` its blocks may start while the kernel before it on the stream drains (and
+// after all of that one's blocks have started), so it must begin with cudaGridDependencySynchronize(), which
+// waits for that kernel's end and for its writes.  For kernels of a few microseconds the gap between two
+// launches is worth closing (forward + backward with copies and joins, 1.2 M edges, F = 47: 85 -> 75 us; with a
+// join, 65 k edges, F = 64: 20.5 -> 18.8 us).
+template <typename... P, typename... A>
+cudaError_t launch_kernel(void (*kernel)(P...), dim3 grid, int block, cudaStream_t s, bool overlap, const A&... args) {
+  cudaLaunchAttribute attribute{};
+  attribute.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  attribute.val.programmaticStreamSerializationAllowed = 1;
+  cudaLaunchConfig_t config{};
+  config.gridDim = grid;
+  config.blockDim = dim3((unsigned)block);
+  config.stream = s;
+  config.attrs = &attribute;
+  config.numAttrs = overlap ? 1 : 0;
+  return cudaLaunchKernelEx(&config, kernel, args...);
+}
 
 #define DG_CUDA(call)                                          \
   do {                                                         \
