@@ -10,6 +10,7 @@ _ROOT = os.path.dirname(_HERE)
 CSRC = os.path.join(_HERE, "csrc")
 INCLUDE = os.path.join(_ROOT, "include")
 LIB_PATH = os.path.join(_HERE, "libdgagg.so")
+BUILD_DIR = os.path.join(_HERE, "_build")
 SOURCES = ["dg_api.cu", "dg_graph.cu", "dg_transpose.cu", "dg_aggregate.cu", "dg_aggregate_self.cu", "dg_pool.cu",
            "dg_static.cu", "dg_probe.cu", "dg_general.cu", "dg_general_fwd.cu", "dg_general_bwd.cu", "dg_edge_grad.cu",
            "dg_layer.cu", "dg_loss.cu", "dg_reorder.cu"]
@@ -40,11 +41,10 @@ def build(force: bool = False, verbose: bool = False) -> str:
     if verbose:
         flags += ["-Xptxas", "-v"]
     objs = []
-    build_dir = os.path.join(_HERE, "_build")
-    os.makedirs(build_dir, exist_ok=True)
+    os.makedirs(BUILD_DIR, exist_ok=True)
     procs = []
     for src in _sources():
-        obj = os.path.join(build_dir, os.path.basename(src)[:-3] + ".o")
+        obj = os.path.join(BUILD_DIR, os.path.basename(src)[:-3] + ".o")
         objs.append(obj)
         cmd = [nvcc, *flags, "-I", INCLUDE, "-I", CSRC, "-c", src, "-o", obj]
         procs.append((cmd, subprocess.Popen(cmd)))

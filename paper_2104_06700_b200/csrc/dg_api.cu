@@ -45,7 +45,7 @@ static inline size_t align256(size_t x) { return (x + 255) & ~(size_t)255; }
 static void free_owned(Graph* g) {
   pool_retire(g->device, g->owned, g->owned_bytes);
   pool_retire(g->device, g->plan_memory, g->plan_bytes);
-  pinned_counters_retire(g->host);
+  pinned_counters_retire(g->device, g->host);
   if (g->col_totals_ready) cudaEventDestroy(g->col_totals_ready);
   for (size_t i = 0; i < g->aux_event_count; ++i) cudaEventDestroy(g->aux_events[i]);
   free(g->aux_events);
@@ -158,8 +158,7 @@ const Plan& column_plan(Graph* g) {
 // New plans for a changed chunk cost or threshold.  The old ones may be in use, or being built, on any
 // stream: waits for the device on both sides.
 static dg_status_t replan(Graph* g) {
-  DG_CUDA(cudaDeviceSynchronize());
-  pool_device_is_idle(g->device);
+  DG_CUDA(pool_wait(g->device));
   pool_retire(g->device, g->plan_memory, g->plan_bytes);
   g->plan_memory = nullptr;
   if (dg_status_t st = reserve_plans(g)) return st;
@@ -302,14 +301,13 @@ dg_status_t dg_graph_create(int64_t n, int64_t nnz, const int64_t* rowptr,
   // The caller may have produced the arrays on any stream: wait for the device once, then everything
   // below runs on the default stream and is waited for once, at the end.
   dg_status_t st = DG_OK;
-  e = cudaDeviceSynchronize();
-  if (e == cudaSuccess) pool_device_is_idle(g->device);
+  e = pool_wait(g->device);
   const bool split = wants_split(n, nnz);
   const size_t counter_bytes = align256(sizeof(HostCounters));
   const size_t split_bytes = split ? align256((size_t)(kFineBlocks + 1) * (size_t)n * sizeof(int32_t)) : 0;
   g->owned_bytes = counter_bytes + split_bytes;
   if (e == cudaSuccess) e = pool_alloc(g->device, g->owned_bytes, 0, &g->owned);
-  if (e == cudaSuccess) e = pinned_counters(g->device, &g->host);
+  if (e == cudaSuccess) e = pinned_counters(&g->host);
   if (e == cudaSuccess) e = cudaEventCreateWithFlags(&g->col_totals_ready, cudaEventDisableTiming);
   if (e == cudaSuccess) {
     char* p = static_cast<char*>(g->owned);

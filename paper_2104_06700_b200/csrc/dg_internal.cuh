@@ -183,12 +183,12 @@ cudaError_t launch_kernel(void (*kernel)(P...), dim3 grid, int block, cudaStream
 // dg_pool.cu: device memory of the library itself
 cudaError_t pool_open(int device);   // one per handle
 void pool_close(int device);
-void pool_device_is_idle(int device);  // the caller has just waited for the device
+cudaError_t pool_wait(int device);   // waits for the device, then frees what was retired before
 cudaError_t pool_alloc(int device, size_t bytes, cudaStream_t s, void** out);
 void pool_free(void* p, cudaStream_t s);
 void pool_retire(int device, void* p, size_t bytes);  // kernels on any stream may still use it
-cudaError_t pinned_counters(int device, HostCounters** out);
-void pinned_counters_retire(HostCounters* p);
+cudaError_t pinned_counters(HostCounters** out);
+void pinned_counters_retire(int device, HostCounters* p);
 
 // dg_graph.cu
 dg_status_t build_plan(const int64_t* ptr, int64_t n, int64_t nnz, int64_t chunk_cost, int64_t row_cost,

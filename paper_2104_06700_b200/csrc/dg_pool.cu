@@ -5,9 +5,11 @@
 //
 // The pool keeps at most kKeepInUse unused bytes while a handle is alive and kKeepIdle after the
 // last one is gone.  What a destroyed handle held may still be read by kernels queued on any stream:
-// it waits in a short list until the library next has the device idle (dg_graph_create waits for it
-// anyway), or until the list reaches kMaxPending bytes.  Everything here is safe to call from several
-// threads.
+// it waits on a list until the library next waits for the device (dg_graph_create does anyway), or
+// until the list reaches kMaxPending bytes.  A wait frees what was on the list before it began and
+// nothing that another thread adds meanwhile.  Everything here is safe to call from several threads.
+#include <stdlib.h>
+
 #include <mutex>
 
 #include "dg_internal.cuh"
@@ -18,15 +20,21 @@ namespace {
 constexpr int kMaxDevices = 64;
 constexpr size_t kKeepInUse = (size_t)4 << 30;
 constexpr size_t kKeepIdle = (size_t)32 << 20;
-constexpr int kMaxPendingBlocks = 64;
 constexpr size_t kMaxPending = kKeepIdle;
 constexpr int kPinnedWords = 128;  // one page
+
+// A device block, or a handle's pinned counters, that queued work may still use.
+struct Retired {
+  Retired* next;
+  void* block;
+  size_t bytes;
+  HostCounters* counters;
+};
 
 struct DevicePool {
   cudaMemPool_t pool = nullptr;
   int handles = 0;
-  void* pending[kMaxPendingBlocks];
-  int pending_count = 0;
+  Retired* pending = nullptr;
   size_t pending_bytes = 0;
 };
 
@@ -34,23 +42,44 @@ std::mutex g_mutex;
 DevicePool g_pools[kMaxDevices];
 // one page of host memory the device writes counters into, for the life of the process
 HostCounters* g_pinned = nullptr;
-enum : uint8_t { kWordFree = 0, kWordUsed = 1, kWordPending = 2 };  // pending: a copy may be on its way
-uint8_t g_word_state[kPinnedWords];
-uint8_t g_word_device[kPinnedWords];
+bool g_word_used[kPinnedWords];
 
-// the device must be idle with respect to everything that is pending on it
-void release_pending(DevicePool& d) {
-  for (int i = 0; i < d.pending_count; ++i) cudaFreeAsync(d.pending[i], 0);
-  d.pending_count = 0;
-  d.pending_bytes = 0;
-  const int device = (int)(&d - g_pools);
-  for (int i = 0; i < kPinnedWords; ++i)
-    if (g_word_state[i] == kWordPending && g_word_device[i] == device) g_word_state[i] = kWordFree;
-}
+bool in_page(const HostCounters* p) { return g_pinned && p >= g_pinned && p < g_pinned + kPinnedWords; }
 
 cudaError_t keep(DevicePool& d, size_t bytes) {
   uint64_t v = bytes;
   return cudaMemPoolSetAttribute(d.pool, cudaMemPoolAttrReleaseThreshold, &v);
+}
+
+// No work uses it any more.
+void release(const Retired& r) {
+  if (r.block) cudaFreeAsync(r.block, 0);
+  if (!r.counters) return;
+  if (in_page(r.counters)) {
+    std::lock_guard<std::mutex> lock(g_mutex);
+    g_word_used[r.counters - g_pinned] = false;
+  } else {
+    cudaFreeHost(r.counters);
+  }
+}
+
+void retire(int device, const Retired& what) {
+  Retired* r = static_cast<Retired*>(malloc(sizeof(Retired)));
+  if (!r) {  // no list to put it on
+    if (cudaDeviceSynchronize() == cudaSuccess) release(what);
+    return;
+  }
+  *r = what;
+  bool full;
+  {
+    std::lock_guard<std::mutex> lock(g_mutex);
+    DevicePool& d = g_pools[device];
+    r->next = d.pending;
+    d.pending = r;
+    d.pending_bytes += r->bytes;
+    full = d.pending_bytes > kMaxPending;
+  }
+  if (full) (void)pool_wait(device);
 }
 
 }  // namespace
@@ -76,24 +105,46 @@ cudaError_t pool_open(int device) {
 }
 
 void pool_close(int device) {
-  std::lock_guard<std::mutex> lock(g_mutex);
   DevicePool& d = g_pools[device];
-  if (--d.handles == 0) {
+  uint64_t reserved = 0;
+  {
+    std::lock_guard<std::mutex> lock(g_mutex);
+    if (--d.handles > 0) return;
     keep(d, kKeepIdle);
-    uint64_t reserved = 0;
     cudaMemPoolGetAttribute(d.pool, cudaMemPoolAttrReservedMemCurrent, &reserved);
-    if (reserved > kKeepIdle) {
-      cudaDeviceSynchronize();
-      release_pending(d);
-      cudaStreamSynchronize(0);
-      cudaMemPoolTrimTo(d.pool, kKeepIdle);
-    }
+  }
+  if (reserved > kKeepIdle && pool_wait(device) == cudaSuccess) {
+    cudaStreamSynchronize(0);
+    cudaMemPoolTrimTo(d.pool, kKeepIdle);
   }
 }
 
-void pool_device_is_idle(int device) {
-  std::lock_guard<std::mutex> lock(g_mutex);
-  release_pending(g_pools[device]);
+// Waits for the device and frees what had been retired before.  The list is set aside first: work that another
+// thread queues, and memory that it retires, while this one waits are not covered by the wait.
+cudaError_t pool_wait(int device) {
+  DevicePool& d = g_pools[device];
+  Retired* r;
+  {
+    std::lock_guard<std::mutex> lock(g_mutex);
+    r = d.pending;
+    d.pending = nullptr;
+    d.pending_bytes = 0;
+  }
+  const cudaError_t e = cudaDeviceSynchronize();
+  while (r) {
+    Retired* next = r->next;
+    if (e == cudaSuccess) {
+      release(*r);
+      free(r);
+    } else {  // not waited for (the calling thread captures a stream, say): back onto the list
+      std::lock_guard<std::mutex> lock(g_mutex);
+      r->next = d.pending;
+      d.pending = r;
+      d.pending_bytes += r->bytes;
+    }
+    r = next;
+  }
+  return e;
 }
 
 cudaError_t pool_alloc(int device, size_t bytes, cudaStream_t s, void** out) {
@@ -108,20 +159,10 @@ void pool_free(void* p, cudaStream_t s) {
 }
 
 void pool_retire(int device, void* p, size_t bytes) {
-  if (!p) return;
-  std::lock_guard<std::mutex> lock(g_mutex);
-  DevicePool& d = g_pools[device];
-  if (d.pending_count == kMaxPendingBlocks || d.pending_bytes + bytes > kMaxPending) {
-    cudaDeviceSynchronize();
-    release_pending(d);
-    cudaFreeAsync(p, 0);
-    return;
-  }
-  d.pending[d.pending_count++] = p;
-  d.pending_bytes += bytes;
+  if (p) retire(device, Retired{nullptr, p, bytes, nullptr});
 }
 
-cudaError_t pinned_counters(int device, HostCounters** out) {
+cudaError_t pinned_counters(HostCounters** out) {
   std::lock_guard<std::mutex> lock(g_mutex);
   if (!g_pinned)
     if (cudaError_t e = cudaHostAlloc(&g_pinned, kPinnedWords * sizeof(HostCounters), cudaHostAllocPortable)) {
@@ -129,24 +170,16 @@ cudaError_t pinned_counters(int device, HostCounters** out) {
       return e;
     }
   for (int i = 0; i < kPinnedWords; ++i) {
-    if (g_word_state[i] != kWordFree) continue;
-    g_word_state[i] = kWordUsed;
-    g_word_device[i] = (uint8_t)device;
+    if (g_word_used[i]) continue;
+    g_word_used[i] = true;
     *out = g_pinned + i;
     return cudaSuccess;
   }
   return cudaHostAlloc(out, sizeof(HostCounters), cudaHostAllocPortable);  // more handles than words
 }
 
-void pinned_counters_retire(HostCounters* p) {
-  if (!p) return;
-  std::lock_guard<std::mutex> lock(g_mutex);
-  if (p >= g_pinned && p < g_pinned + kPinnedWords) {
-    g_word_state[p - g_pinned] = kWordPending;
-  } else {
-    cudaDeviceSynchronize();
-    cudaFreeHost(p);
-  }
+void pinned_counters_retire(int device, HostCounters* p) {
+  if (p) retire(device, Retired{nullptr, nullptr, 0, p});
 }
 
 }  // namespace dg

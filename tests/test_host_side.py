@@ -1,0 +1,110 @@
+"""The host side of libdgagg on a CUDA runtime without a GPU (fake_cudart.cpp): in what order it waits, frees and
+launches, on which device, and what is left behind when an allocation or a launch fails."""
+import ctypes
+import os
+import subprocess
+
+import numpy as np
+import pytest
+
+from paper_2104_06700_b200 import binding, build
+
+HERE = os.path.dirname(os.path.abspath(__file__))
+
+
+class Fake:
+    """libdgagg linked with the fake runtime."""
+
+    def __init__(self, path):
+        self.lib = ctypes.CDLL(path)
+        self.lib.fake_event.restype = ctypes.c_char_p
+        self.lib.dg_last_error.restype = ctypes.c_char_p
+        self.lib.fake_alloc_limit.argtypes = self.lib.fake_reserved.argtypes = [ctypes.c_size_t]
+        self.lib.dg_graph_set_param.argtypes = [ctypes.c_void_p, ctypes.c_char_p, ctypes.c_int64]
+        self.lib.dg_graph_get_param.argtypes = [ctypes.c_void_p, ctypes.c_char_p, ctypes.c_void_p]
+        self.keep = []
+
+    def reset(self):
+        self.on_sync(None)
+        self.lib.fake_alloc_limit(ctypes.c_size_t(-1).value)
+        self.lib.fake_reserved(0)
+        self.lib.fake_failing_kernel(b"")
+        self.lib.fake_plan_totals(0, 0)
+        self.lib.cudaSetDevice(0)
+
+    def on_sync(self, f):
+        """f() runs in the middle of every wait for the device: what another thread does meanwhile."""
+        self.callback = ctypes.CFUNCTYPE(None)(f) if f else None
+        self.lib.fake_on_sync(self.callback)
+
+    def events(self):
+        """(what, current device, pointer) since the last call."""
+        got = []
+        for i in range(self.lib.fake_events()):
+            device, pointer, size = ctypes.c_int(), ctypes.c_void_p(), ctypes.c_size_t()
+            what = self.lib.fake_event(i, ctypes.byref(device), ctypes.byref(pointer), ctypes.byref(size))
+            got.append((what.decode(), device.value, pointer.value))
+        self.lib.fake_clear()
+        return got
+
+    def array(self, *shape, dtype=np.float32):
+        a = np.zeros(shape, dtype)
+        self.keep.append(a)
+        return ctypes.c_void_p(a.ctypes.data)
+
+    def graph(self, n=64, nnz=256):
+        h = ctypes.c_void_p()
+        st = self.lib.dg_graph_create(ctypes.c_int64(n), ctypes.c_int64(nnz), self.array(n + 1, dtype=np.int64),
+                                      self.array(nnz, dtype=np.int32), None, ctypes.byref(h))
+        assert st == binding.DG_OK, self.lib.dg_last_error()
+        return h
+
+
+@pytest.fixture(scope="module")
+def library(tmp_path_factory):
+    build.build()
+    objects = [os.path.join(build.BUILD_DIR, s[:-3] + ".o") for s in build.SOURCES]
+    if not all(os.path.exists(o) for o in objects):  # the library came without them
+        build.build(force=True)
+    path = str(tmp_path_factory.mktemp("fake") / "libdgagg_host.so")
+    cuda = os.path.join(os.environ.get("CUDA_HOME", "/usr/local/cuda"), "include")
+    subprocess.run(["g++", "-shared", "-fPIC", "-O1", "-std=c++17", "-Wl,-Bsymbolic", "-I", cuda, "-o", path,
+                    os.path.join(HERE, "fake_cudart.cpp"), *objects], check=True)
+    return Fake(path)
+
+
+@pytest.fixture
+def fake(library):
+    library.reset()
+    library.events()
+    yield library
+    library.reset()
+
+
+def test_a_handle_destroyed_during_the_wait_keeps_its_memory(fake):
+    """While dg_graph_create waits for the device another thread queues work on its own handle and destroys it:
+    that wait does not cover the work, so the memory is freed after a later wait."""
+    old = fake.graph()
+    events = fake.events()
+    blocks = {p for what, _, p in events if what == "alloc"}
+    word = [p for what, _, p in events if what == "copy"]
+    waits = []
+
+    def other_thread():
+        if not waits:
+            fake.lib.dg_graph_destroy(old)
+        waits.append(1)
+
+    fake.on_sync(other_thread)
+    new = fake.graph()
+    fake.on_sync(None)
+    events = fake.events()
+    assert waits and not blocks & {p for what, _, p in events if what == "free"}
+    assert not set(word) & {p for what, _, p in events if what == "copy"}  # nor are its counters written again
+    third = fake.graph()
+    events = fake.events()
+    order = [what for what, _, _ in events]
+    freed = [i for i, (what, _, p) in enumerate(events) if what == "free" and p in blocks]
+    assert len(freed) == len(blocks) and min(freed) > order.index("sync")
+    for h in (new, third):
+        fake.lib.dg_graph_destroy(h)
