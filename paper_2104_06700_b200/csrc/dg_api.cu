@@ -158,6 +158,7 @@ const Plan& column_plan(Graph* g) {
 // New plans for a changed chunk cost or threshold.  The old ones may be in use, or being built, on any
 // stream: waits for the device on both sides.
 static dg_status_t replan(Graph* g) {
+  const DeviceScope scope(g->device);
   DG_CUDA(pool_wait(g->device));
   pool_retire(g->device, g->plan_memory, g->plan_bytes);
   g->plan_memory = nullptr;

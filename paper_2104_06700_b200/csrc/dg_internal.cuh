@@ -180,6 +180,25 @@ cudaError_t launch_kernel(void (*kernel)(P...), dim3 grid, int block, cudaStream
     if (e__ != cudaSuccess) return dg::cuda_fail(e__, #call);  \
   } while (0)
 
+// Makes `device` current for a scope: handles are destroyed and their knobs set with any device current (a garbage
+// collector decides when), and waiting and stream-ordered calls act on the current one.
+class DeviceScope {
+ public:
+  explicit DeviceScope(int device) {
+    if (cudaGetDevice(&before_) != cudaSuccess) before_ = device;
+    if (before_ != device) cudaSetDevice(device);
+    device_ = device;
+  }
+  ~DeviceScope() {
+    if (before_ != device_) cudaSetDevice(before_);
+  }
+  DeviceScope(const DeviceScope&) = delete;
+  DeviceScope& operator=(const DeviceScope&) = delete;
+
+ private:
+  int before_ = 0, device_ = 0;
+};
+
 // dg_pool.cu: device memory of the library itself
 cudaError_t pool_open(int device);   // one per handle
 void pool_close(int device);

@@ -51,7 +51,7 @@ cudaError_t keep(DevicePool& d, size_t bytes) {
   return cudaMemPoolSetAttribute(d.pool, cudaMemPoolAttrReleaseThreshold, &v);
 }
 
-// No work uses it any more.
+// No work uses it any more; its device is current.
 void release(const Retired& r) {
   if (r.block) cudaFreeAsync(r.block, 0);
   if (!r.counters) return;
@@ -66,6 +66,7 @@ void release(const Retired& r) {
 void retire(int device, const Retired& what) {
   Retired* r = static_cast<Retired*>(malloc(sizeof(Retired)));
   if (!r) {  // no list to put it on
+    const DeviceScope scope(device);
     if (cudaDeviceSynchronize() == cudaSuccess) release(what);
     return;
   }
@@ -105,6 +106,7 @@ cudaError_t pool_open(int device) {
 }
 
 void pool_close(int device) {
+  const DeviceScope scope(device);
   DevicePool& d = g_pools[device];
   uint64_t reserved = 0;
   {
@@ -122,6 +124,7 @@ void pool_close(int device) {
 // Waits for the device and frees what had been retired before.  The list is set aside first: work that another
 // thread queues, and memory that it retires, while this one waits are not covered by the wait.
 cudaError_t pool_wait(int device) {
+  const DeviceScope scope(device);
   DevicePool& d = g_pools[device];
   Retired* r;
   {

@@ -108,3 +108,21 @@ def test_a_handle_destroyed_during_the_wait_keeps_its_memory(fake):
     assert len(freed) == len(blocks) and min(freed) > order.index("sync")
     for h in (new, third):
         fake.lib.dg_graph_destroy(h)
+
+
+@pytest.mark.parametrize("n,nnz,what", [(64, 256, "the list stays short"), (700000, 45000000, "the list is full")])
+def test_a_handle_is_destroyed_on_its_own_device(fake, n, nnz, what):
+    """Whatever device is current when a handle goes, or has a knob set: waits and frees act on the handle's, and the
+    current device is the caller's again afterwards."""
+    handle = fake.graph(n, nnz)
+    fake.lib.cudaSetDevice(1)
+    assert fake.lib.dg_graph_set_param(handle, b"rows_per_block", 64) == binding.DG_OK
+    fake.lib.fake_reserved(1 << 30)  # the pool has grown: the last handle gives memory back
+    fake.lib.dg_graph_destroy(handle)
+    device = ctypes.c_int()
+    fake.lib.cudaGetDevice(ctypes.byref(device))
+    assert device.value == 1
+    events = [e for e in fake.events() if e[0] in ("sync", "free", "free host", "trim")]
+    assert {"sync", "free", "trim"} <= {e[0] for e in events}
+    # the events up to here are the creation's, on device 0 too
+    assert {e[1] for e in events} == {0}
