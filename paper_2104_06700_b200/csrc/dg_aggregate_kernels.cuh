@@ -406,7 +406,8 @@ __device__ __forceinline__ void ap_body(const ApArgs& a, const SelfArgs sa) {
       my_hi = min(__ldg(a.seg_hi + rb + lane), next.y);
     }
     const unsigned work = __ballot_sync(kFull, my_hi > my_lo);
-    int qi = work ? __ffs(work) - 1 : 32, qb = 0, qhi = 0;
+    int qi = work ? __ffs(work) - 1 : 32;
+    Position qb = 0, qhi = 0;
     int32_t cur_u = 0, nxt_u = 0;
     float cur_s = 0.f, nxt_s = 0.f;
     auto step_q = [&]() {
@@ -428,12 +429,12 @@ __device__ __forceinline__ void ap_body(const ApArgs& a, const SelfArgs sa) {
       if (qi < 32) load_batch<SCALED>(a, qb, qhi, lane, nxt_u, nxt_s);
     }
     for (int i = 0; i < nrows; ++i) {
-      const int lo = __shfl_sync(kFull, my_lo, i);
-      const int hi = __shfl_sync(kFull, my_hi, i);
+      const Position lo = __shfl_sync(kFull, my_lo, i);
+      const Position hi = __shfl_sync(kFull, my_hi, i);
       V acc[CPL];
       start_row(rb + i, acc, i + 1 < nrows);
-      for (int b = lo; b < hi; b += 32) {
-        add_edges<E, VEC, G, CPL, SCALED, SEG>(xrow, row_bytes, cur_u, cur_s, 0, min(hi - b, 32), grp, acc,
+      for (Position b = lo; b < hi; b += 32) {
+        add_edges<E, VEC, G, CPL, SCALED, SEG>(xrow, row_bytes, cur_u, cur_s, 0, (int)min(hi - b, 32u), grp, acc,
                                                stage);
         cur_u = nxt_u;
         cur_s = nxt_s;

@@ -167,7 +167,8 @@ __device__ __forceinline__ void walk_chunk(const GenArgs& a, First first, Begin 
     my_hi = min(a.seg_hi ? __ldg(a.seg_hi + r) : (int)__ldg(a.ptr + r + 1), next.y);
   }
   const unsigned work = __ballot_sync(kAll, my_hi > my_lo);
-  int qi = work ? __ffs(work) - 1 : 32, qb = 0, qhi = 0;  // the batch that is fetched next
+  int qi = work ? __ffs(work) - 1 : 32;
+  Position qb = 0, qhi = 0;  // the batch that is fetched next
   int32_t cur_u = 0, nxt_u = 0, cur_k = 0, nxt_k = 0;
   auto fetch = [&](int32_t& u, int32_t& k) {
     const bool mine = qb + lane < qhi;
@@ -194,11 +195,11 @@ __device__ __forceinline__ void walk_chunk(const GenArgs& a, First first, Begin 
     first(cur_u, cur_k);
   }
   for (int i = 0; i < nrows; ++i) {
-    const int lo = __shfl_sync(kAll, my_lo, i);
-    const int hi = __shfl_sync(kAll, my_hi, i);
+    const Position lo = __shfl_sync(kAll, my_lo, i);
+    const Position hi = __shfl_sync(kAll, my_hi, i);
     begin(here.x + i);
-    for (int b = lo; b < hi; b += 32) {
-      batch(cur_u, cur_k, b, min(hi - b, 32), nxt_u, nxt_k);
+    for (Position b = lo; b < hi; b += 32) {
+      batch(cur_u, cur_k, (int)b, (int)min(hi - b, 32u), nxt_u, nxt_k);
       cur_u = nxt_u;
       cur_k = nxt_k;
       if (qi < 32) {

@@ -123,18 +123,18 @@ __global__ void __launch_bounds__(kGenBlock) arg_mask_kernel(const GenArgs a) {
   load(0, cur);
   load(1, nxt);
   int i = 0;
-  for (int p0 = here.y; p0 < next.y; p0 += kEdges) {
-    const int p1 = min(next.y, p0 + kEdges);
-    for (int t = lane; t < (p1 - p0) * WORDS; t += 32) window[t] = 0;
+  for (Position p0 = here.y; p0 < (Position)next.y; p0 += kEdges) {
+    const Position p1 = min((Position)next.y, p0 + kEdges);
+    for (int t = lane; t < (int)(p1 - p0) * WORDS; t += 32) window[t] = 0;
     __syncwarp();
     while (i < nrows) {
-      const int lo = max(__shfl_sync(kAll, my_lo, i), p0), end = __shfl_sync(kAll, my_hi, i);
-      if (lo >= p1) break;
-      const int hi = min(end, p1);
+      const int lo = max(__shfl_sync(kAll, my_lo, i), (int)p0), end = __shfl_sync(kAll, my_hi, i);
+      if (lo >= (int)p1) break;
+      const int hi = min(end, (int)p1);
 #pragma unroll
       for (int w = 0; w < WORDS; ++w)
-        if (cur[w] >= lo && cur[w] < hi) atomicOr(&window[(cur[w] - p0) * WORDS + w], 1u << lane);
-      if (end > p1) break;  // the rest of this row lies in the next window
+        if (cur[w] >= lo && cur[w] < hi) atomicOr(&window[(cur[w] - (int)p0) * WORDS + w], 1u << lane);
+      if (end > (int)p1) break;  // the rest of this row lies in the next window
       ++i;
 #pragma unroll
       for (int w = 0; w < WORDS; ++w) cur[w] = nxt[w];
@@ -142,7 +142,7 @@ __global__ void __launch_bounds__(kGenBlock) arg_mask_kernel(const GenArgs a) {
     }
     __syncwarp();
     uint32_t* out = a.mask + (int64_t)p0 * WORDS;
-    for (int t = lane; t < (p1 - p0) * WORDS; t += 32) out[t] = window[t];
+    for (int t = lane; t < (int)(p1 - p0) * WORDS; t += 32) out[t] = window[t];
     __syncwarp();
   }
 }

@@ -104,6 +104,10 @@ namespace dg {
 
 using Graph = ::dg_graph;
 
+// A position in the edge arrays while a kernel steps through them in batches: all are below 2^31, and a step past
+// the last one overflows a signed 32-bit number.
+using Position = uint32_t;
+
 constexpr int kFineBlocks = 16;          // finest cut of the neighbour ids for source blocking
 constexpr int64_t kBlockingMinAvgLen = 64;  // split pointers are built when nnz >= 64 n
 

@@ -393,11 +393,11 @@ row_info_kernel(const Chunk* __restrict__ chunks, int32_t chunk_count, const int
     end = min((int)row_end, next.y);
     inv = __float_as_uint(1.0f / (float)(row_end - __ldg(rowptr + here.x + lane) + self));
   }
-  int p = here.y;
+  Position p = here.y;
   for (int i = 0; i < nrows; ++i) {
-    const int hi = __shfl_sync(kFull, end, i);
+    const Position hi = __shfl_sync(kFull, end, i);
     const uint2 info = make_uint2((uint32_t)(here.x + i), __shfl_sync(kFull, inv, i));
-    for (int k = p + lane; k < hi; k += 32) row_info[k] = info;
+    for (Position k = p + lane; k < hi; k += 32) row_info[k] = info;
     p = hi;
   }
 }

@@ -147,6 +147,69 @@ def test_self_calls_are_the_attribute_for_one_call(F):
                        looped.dg_aggregate_bwd(H, binding.DG_OP_MEAN))
 
 
+@pytest.mark.parametrize("F", [8, 16])
+def test_positions_up_to_the_last(F):
+    """2^31 - 1 edges, the most a handle takes: a batch that starts in the last 32 positions ends beyond 2^31.  Rows
+    of 2048 consecutive ids, so that every result has a closed form, and integer features, so that sums are exact.
+    The wider matrix exceeds the L2 budget and takes the source-blocked kernels."""
+    torch.cuda.empty_cache()
+    n, deg, blocks = 1 << 20, 2048, 512
+    nnz = n * deg - 1
+    rowptr = (torch.arange(n + 1, device=DEV) * deg).clamp_(max=nnz)
+    colidx = torch.arange(n, dtype=torch.int32, device=DEV).repeat(deg)[:nnz]
+    g = binding.dg_graph_create(n, nnz, rowptr, colidx, None)
+    g.dg_graph_transpose()
+    _, rowidx_T, _, perm = g.dg_graph_get_csc()
+    u = torch.arange(n, device=DEV)
+    for lo in range(0, n, 1 << 15):  # column u: the rows congruent to u / 2048 modulo 512, in order
+        cols = u[lo:lo + (1 << 15)].unsqueeze(1)
+        rows = (cols // deg + blocks * torch.arange(deg, device=DEV)).flatten()[: nnz - lo * deg]
+        at = slice(lo * deg, lo * deg + rows.numel())
+        assert torch.equal(rowidx_T[at].long(), rows)
+        assert torch.equal(perm[at].long(), rows * deg + (cols % deg).expand(-1, deg).flatten()[: rows.numel()])
+    del rowidx_T, perm
+
+    H = (u.unsqueeze(1) * 5 % 7 + torch.arange(F, device=DEV)).float()
+    G = (u.unsqueeze(1) * 3 % 11 - torch.arange(F, device=DEV)).float()
+    want = H.view(blocks, deg, F).sum(1).repeat(deg, 1)
+    want[-1] -= H[-1]
+    assert torch.equal(g.dg_aggregate_fwd(H, binding.DG_OP_SUM), want)
+    want = G.view(deg, blocks, F).sum(0).repeat_interleave(deg, 0)
+    want[-1] -= G[-1]
+    assert torch.equal(g.dg_aggregate_bwd(G, binding.DG_OP_SUM), want)
+
+    # the maximum of a block lies at its last id (which the last row does not have) for even features
+    H[:, ::2] = (u % deg).float().unsqueeze(1)
+    H[:, 1::2] = -H[:, ::2]
+    fO, arg = g.dg_ap_fwd(H, None, binding.DG_BIN_COPY_LHS, binding.DG_RED_MAX)
+    best = torch.tensor([deg - 1, 0] * (F // 2), device=DEV).repeat(n, 1)
+    best[-1, ::2] = deg - 2
+    assert torch.equal(arg.long(), u.unsqueeze(1) * deg + best)
+    assert torch.equal(fO, best.float())
+    dV, _ = g.dg_ap_bwd(G, H, None, binding.DG_BIN_COPY_LHS, binding.DG_RED_MAX, arg=arg)
+    want = torch.zeros(n, F, device=DEV)
+    sums = G.view(deg, blocks, F).sum(0)
+    want.view(blocks, deg, F)[:, -1, ::2] = sums[:, ::2]
+    want.view(blocks, deg, F)[:, 0, 1::2] = sums[:, 1::2]
+    want[-1, ::2] -= G[-1, ::2]
+    want[-2, ::2] = G[-1, ::2]
+    assert torch.equal(dV, want)
+    del fO, arg, dV, want, best
+
+    H = (u.unsqueeze(1) * 5 % 7 + torch.arange(F, device=DEV)).float()
+    fE = torch.ones(nnz, 1, device=DEV)
+    for name, call in (("dot", lambda: g.dg_aggregate_edge_grad(H, G, binding.DG_OP_SUM)),
+                       ("add", lambda: g.dg_ap_bwd(G, H, fE, binding.DG_BIN_ADD, binding.DG_RED_SUM)[1])):
+        got = call().flatten()
+        for lo in (0, n - 1024):
+            X = H.view(blocks, deg, F)[u[lo:lo + 1024] % blocks] if name == "dot" else torch.ones(1024, deg, F, device=DEV)
+            want = (X * G[lo:lo + 1024].unsqueeze(1)).sum(2).flatten()
+            at = got[lo * deg:(lo + 1024) * deg]
+            assert torch.equal(at, want[: at.numel()]), name
+    del g, colidx
+    torch.cuda.empty_cache()
+
+
 def test_calls_on_two_streams_and_destroyed_handles():
     """Scratch comes from a pool shared by handles, streams and threads; a destroyed handle's memory is not
     reused while its kernels are queued."""
