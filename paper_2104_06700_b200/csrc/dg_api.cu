@@ -92,16 +92,22 @@ static int64_t cut_threshold(const Graph* g) {
   return g->rows_per_block == 0 && chunk_cost(g) == kMinChunk ? kFewEdgesRow : 2 * chunk_cost(g);
 }
 
-// Takes the memory of both plans for the current chunk cost and threshold.
+// Where the totals of the rows' (0) or the columns' (1) plan lie among the counters.
+static int totals_of(const Graph* g, int columns) { return kTotals + g->totals_set * kTotalsPerSet + 2 * columns; }
+
+// Takes the memory of both plans for the current chunk cost and threshold; on failure the plans are as they were.
 static dg_status_t reserve_plans(Graph* g) {
   const int64_t cost = chunk_cost(g);
   const int64_t count = (g->nnz + row_cost(g) * g->n + cost - 1) / cost;
   const int64_t cuts = g->nnz > cut_threshold(g) ? count : 0;
   const size_t chunk_bytes = align256((size_t)(count + 1) * sizeof(Chunk));
   const size_t cut_bytes = align256((size_t)cuts * sizeof(CutRow));
-  g->plan_bytes = 2 * (chunk_bytes + cut_bytes);
-  DG_CUDA(pool_alloc(g->device, g->plan_bytes, 0, &g->plan_memory));
-  char* p = static_cast<char*>(g->plan_memory);
+  const size_t bytes = 2 * (chunk_bytes + cut_bytes);
+  void* memory = nullptr;
+  DG_CUDA(pool_alloc(g->device, bytes, 0, &memory));
+  g->plan_memory = memory;
+  g->plan_bytes = bytes;
+  char* p = static_cast<char*>(memory);
   Plan* both[2] = {&g->row_plan, &g->col_plan};
   for (int i = 0; i < 2; ++i) {
     Plan& plan = *both[i];
@@ -109,7 +115,7 @@ static dg_status_t reserve_plans(Graph* g) {
     p += chunk_bytes;
     plan.cuts = reinterpret_cast<CutRow*>(p);
     p += cut_bytes;
-    plan.totals = g->counters + (i ? kColTotals : kRowTotals);
+    plan.totals = g->counters + totals_of(g, i);
     plan.count = count;
     plan.max_cuts = cuts;
     // a row of m > threshold entries holds at most m / cost + 1 boundaries
@@ -125,8 +131,8 @@ static dg_status_t plan_rows(Graph* g, cudaStream_t s) {
 }
 
 static void take_row_totals(Graph* g) {
-  g->row_plan.slots = g->host->v[kRowTotals];
-  g->row_plan.cut_rows = g->host->v[kRowTotals + 1];
+  g->row_plan.slots = g->host->v[totals_of(g, 0)];
+  g->row_plan.cut_rows = g->host->v[totals_of(g, 0) + 1];
 }
 
 // What follows every transposition: the columns' plan, its totals sent to the host behind it (read by
@@ -137,8 +143,8 @@ dg_status_t finish_transpose(Graph* g, cudaStream_t s) {
     return st;
   if (g->col_plan.max_cuts == 0) return DG_OK;
   g->col_plan.slots = g->col_plan.cut_rows = -1;
-  DG_CUDA(cudaMemcpyAsync(g->host->v + kColTotals, g->counters + kColTotals, 2 * sizeof(int32_t),
-                          cudaMemcpyDeviceToHost, s));
+  const int at = totals_of(g, 1);
+  DG_CUDA(cudaMemcpyAsync(g->host->v + at, g->counters + at, 2 * sizeof(int32_t), cudaMemcpyDeviceToHost, s));
   DG_CUDA(cudaEventRecord(g->col_totals_ready, s));
   return DG_OK;
 }
@@ -146,8 +152,8 @@ dg_status_t finish_transpose(Graph* g, cudaStream_t s) {
 const Plan& column_plan(Graph* g) {
   if (g->col_plan.slots < 0) {
     if (cudaEventQuery(g->col_totals_ready) == cudaSuccess) {
-      g->col_plan.slots = g->host->v[kColTotals];
-      g->col_plan.cut_rows = g->host->v[kColTotals + 1];
+      g->col_plan.slots = g->host->v[totals_of(g, 1)];
+      g->col_plan.cut_rows = g->host->v[totals_of(g, 1) + 1];
     } else {
       (void)cudaGetLastError();  // "not ready" must not be mistaken for a failed launch later
     }
@@ -155,21 +161,33 @@ const Plan& column_plan(Graph* g) {
   return g->col_plan;
 }
 
-// New plans for a changed chunk cost or threshold.  The old ones may be in use, or being built, on any
-// stream: waits for the device on both sides.
-static dg_status_t replan(Graph* g) {
-  const DeviceScope scope(g->device);
-  DG_CUDA(pool_wait(g->device));
-  pool_retire(g->device, g->plan_memory, g->plan_bytes);
-  g->plan_memory = nullptr;
-  if (dg_status_t st = reserve_plans(g)) return st;
+static dg_status_t build_plans(Graph* g) {
   if (dg_status_t st = plan_rows(g, 0)) return st;
   DG_CUDA(cudaMemcpyAsync(g->host, g->counters, sizeof(HostCounters), cudaMemcpyDeviceToHost, 0));
   if (g->transposed)
     if (dg_status_t st = finish_transpose(g, 0)) return st;
   DG_CUDA(cudaDeviceSynchronize());
-  take_row_totals(g);
   return DG_OK;
+}
+
+// Sets *knob, which the chunk cost or the cut threshold follows, and makes new plans.  The old ones may be in use,
+// or being built, on any stream: waits for the device on both sides.  If that fails, knob and plans are as before.
+static dg_status_t replan(Graph* g, int64_t* knob, int64_t value) {
+  const DeviceScope scope(g->device);
+  DG_CUDA(pool_wait(g->device));
+  const Graph before = *g;
+  *knob = value;
+  g->totals_set ^= 1;
+  dg_status_t st = reserve_plans(g);
+  if (st == DG_OK) st = build_plans(g);
+  if (st == DG_OK) {
+    take_row_totals(g);
+    pool_retire(g->device, before.plan_memory, before.plan_bytes);
+    return DG_OK;
+  }
+  if (g->plan_memory != before.plan_memory) pool_retire(g->device, g->plan_memory, g->plan_bytes);
+  *g = before;
+  return st;
 }
 
 static dg_status_t check_features(const Graph* g, const void* in, size_t in_elem_bytes, float* out,
@@ -587,8 +605,7 @@ dg_status_t dg_graph_set_param(dg_graph_t g, const char* name, int64_t value) {
   if (!g || !name) return invalid("graph handle or name is NULL");
   if (!strcmp(name, "heavy_threshold")) {
     if (value < 64 || value > (1 << 30)) return invalid("heavy_threshold must be in [64, 2^30]");
-    g->heavy_threshold = value;
-    return replan(g);
+    return replan(g, &g->heavy_threshold, value);
   }
   if (!strcmp(name, "slice_features")) {
     if (value < 0 || value > (1 << 20)) return invalid("slice_features must be in [0, 2^20]");
@@ -598,8 +615,7 @@ dg_status_t dg_graph_set_param(dg_graph_t g, const char* name, int64_t value) {
   if (!strcmp(name, "rows_per_block")) {
     if (value < 0 || value > 248) return invalid("rows_per_block must be in [0, 248]");
     if (value == g->rows_per_block) return DG_OK;
-    g->rows_per_block = value;
-    return replan(g);
+    return replan(g, &g->rows_per_block, value);
   }
   if (!strcmp(name, "l2_budget_mb")) {
     if (value < 1 || value > 4096) return invalid("l2_budget_mb must be in [1, 4096]");

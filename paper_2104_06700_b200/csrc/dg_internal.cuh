@@ -33,8 +33,9 @@ struct Plan {
   int32_t slots = -1, cut_rows = -1;    // the totals, or -1 while they are on their way to the host
 };
 
-// Device counters of a handle, and their order in the pinned copy.
-enum { kFlags, kUnsorted, kRowTotals, kColTotals = kRowTotals + 2, kCounters = kColTotals + 2 };
+// Device counters of a handle, and their order in the pinned copy.  There are two sets of plan totals, rows' then
+// columns', used in turn: until new plans are finished the old ones stay whole.
+enum { kFlags, kUnsorted, kTotals, kTotalsPerSet = 4, kCounters = kTotals + 2 * kTotalsPerSet };
 struct HostCounters {
   int32_t v[kCounters];
 };
@@ -54,6 +55,7 @@ struct dg_graph {
   void* plan_memory = nullptr;
   size_t plan_bytes = 0;
   dg::Plan row_plan, col_plan;   // CSR rows (forward), CSC columns (backward)
+  int32_t totals_set = 0;        // which totals in `counters` are theirs
 
   int32_t* counters = nullptr;   // kCounters device words, see the enum below
 

@@ -126,3 +126,30 @@ def test_a_handle_is_destroyed_on_its_own_device(fake, n, nnz, what):
     assert {"sync", "free", "trim"} <= {e[0] for e in events}
     # the events up to here are the creation's, on device 0 too
     assert {e[1] for e in events} == {0}
+
+
+@pytest.mark.parametrize("failure", ["memory", "launch"])
+def test_a_knob_that_cannot_be_set_leaves_the_handle_as_it_was(fake, failure):
+    handle = fake.graph(2000, 1 << 20)
+    blocks = {p for what, _, p in fake.events() if what == "alloc"}
+
+    def knob(name):
+        value = ctypes.c_int64()
+        assert fake.lib.dg_graph_get_param(handle, name, ctypes.byref(value)) == binding.DG_OK
+        return value.value
+
+    before = knob(b"heavy_threshold"), knob(b"rows_per_block")
+    if failure == "memory":
+        fake.lib.fake_alloc_limit(1000)
+    else:
+        fake.lib.fake_failing_kernel(b"plan_kernel")
+    assert fake.lib.dg_graph_set_param(handle, b"heavy_threshold", 4096) == binding.DG_ERR_CUDA
+    assert fake.lib.dg_graph_set_param(handle, b"rows_per_block", 64) == binding.DG_ERR_CUDA
+    assert before == (knob(b"heavy_threshold"), knob(b"rows_per_block"))
+    fake.reset()
+    other = fake.graph()  # waits for the device and frees what is not in use any more
+    assert not blocks & {p for what, _, p in fake.events() if what == "free"}
+    assert fake.lib.dg_graph_set_param(handle, b"rows_per_block", 64) == binding.DG_OK
+    assert knob(b"rows_per_block") == 64
+    for h in (handle, other):
+        fake.lib.dg_graph_destroy(h)
