@@ -143,14 +143,14 @@ static bool worth_dividing(const Graph* g, int32_t F) {
          (size_t)g->n * (size_t)(F + 32) * 4 <= kPadMaxBytes;
 }
 
-// Makes the copy; false when there is no memory for it (the caller then uses X as it is).
-bool pad_rows(const Graph* g, const void* X, int32_t F, int elem_bytes, const int64_t* mean_ptr, int mean_self,
+// Makes the copy; *copy stays nullptr when there is no memory for it (the caller then uses X as it is).
+dg_status_t pad_rows(const Graph* g, const void* X, int32_t F, int elem_bytes, const int64_t* mean_ptr, int mean_self,
               cudaStream_t s, void** copy, int64_t* ld) {
   // rows of whole 32-byte sectors, of whole 128-byte lines where a row has several
   const int64_t unit = (F * elem_bytes > 512 ? 128 : 32) / elem_bytes;
   const int64_t to = (F + unit - 1) / unit * unit;
   const size_t bytes = (size_t)g->n * (size_t)to * (size_t)elem_bytes;
-  if (pool_alloc(g->device, bytes, s, copy) != cudaSuccess) return false;
+  if (pool_alloc(g->device, bytes, s, copy) != cudaSuccess) return DG_OK;
   *ld = to;
   const unsigned blocks = (unsigned)((bytes / 16 + 255) / 256);
   if (elem_bytes == 2)
@@ -159,8 +159,13 @@ bool pad_rows(const Graph* g, const void* X, int32_t F, int elem_bytes, const in
   else
     pad_rows_kernel<float><<<blocks, 256, 0, s>>>(static_cast<const float*>(X), F, (int32_t)to, g->n, mean_ptr,
                                                   mean_self, static_cast<uint4*>(*copy));
+  if (const cudaError_t e = cudaGetLastError()) {
+    pool_free(*copy, s);
+    *copy = nullptr;
+    return cuda_fail(e, "padded copy");
+  }
   count_launches(1);
-  return true;
+  return DG_OK;
 }
 
 // Chooses the launch shape, then runs one launch per source block.
@@ -197,8 +202,11 @@ dg_status_t aggregate_run(const Graph* g, const ApArgs& a0, const SelfArgs& sa0,
   int64_t ld = a.F;
   void* padded = nullptr;
   const bool divide = worth_dividing(g, a.F) && a.mean_factors && !bf16;
-  if ((divide || worth_padding(g, a.F, eb, vec)) &&
-      pad_rows(g, a.X, a.F, eb, divide ? g->rowptr : nullptr, sa.self_ptr != nullptr, s, &padded, &ld)) {
+  if (divide || worth_padding(g, a.F, eb, vec))
+    if (dg_status_t st = pad_rows(g, a.X, a.F, eb, divide ? g->rowptr : nullptr, sa.self_ptr != nullptr, s, &padded,
+                                  &ld))
+      return st;
+  if (padded) {
     if (divide) {  // the factors are in the copy, the own rows' too
       a.w = nullptr;
       sa.self_mean = 0;

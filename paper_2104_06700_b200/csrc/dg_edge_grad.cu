@@ -135,8 +135,9 @@ dg_status_t edge_grad_run(const Graph* g, const float* H, const float* dOut, int
   if (worth_padding(g, F, 4, vec)) {
     // both rows of a dot product in the same padded layout; the padding multiplies to zero
     int64_t ld = 0;
-    if (pad_rows(g, H, F, 4, nullptr, 0, s, &padded_h, &ld) &&
-        pad_rows(g, dOut, F, 4, nullptr, 0, s, &padded_g, &ld)) {
+    st = pad_rows(g, H, F, 4, nullptr, 0, s, &padded_h, &ld);
+    if (st == DG_OK && padded_h) st = pad_rows(g, dOut, F, 4, nullptr, 0, s, &padded_g, &ld);
+    if (padded_h && padded_g) {
       a.H = static_cast<const float*>(padded_h);
       a.dOut = static_cast<const float*>(padded_g);
       a.ld = ld;

@@ -74,14 +74,15 @@ int vector_width(int32_t F, uintptr_t pointers) {
   return (F % 4 == 0 && (pointers & 15) == 0) ? 4 : (F % 2 == 0 && (pointers & 7) == 0) ? 2 : 1;
 }
 
-// 16-byte loads of a gathered matrix whose rows forbid them, through a padded copy (returned for pool_free)
-void* widen(const dg_graph* g, GenArgs* a, cudaStream_t s) {
-  void* copy = nullptr;
-  if (worth_padding(g, a->F, 4, a->vec) && pad_rows(g, a->X, a->F, 4, nullptr, 0, s, &copy, &a->ldx)) {
-    a->X = static_cast<const float*>(copy);
+// 16-byte loads of a gathered matrix whose rows forbid them, through a padded copy (*copy: for pool_free)
+dg_status_t widen(const dg_graph* g, GenArgs* a, cudaStream_t s, void** copy) {
+  if (!worth_padding(g, a->F, 4, a->vec)) return DG_OK;
+  if (dg_status_t st = pad_rows(g, a->X, a->F, 4, nullptr, 0, s, copy, &a->ldx)) return st;
+  if (*copy) {
+    a->X = static_cast<const float*>(*copy);
     a->vec = 4;
   }
-  return copy;
+  return DG_OK;
 }
 
 // dV of max / min.  The mask of the selected edges (see dg_general_bwd.cu) is made and used for up to 256
@@ -175,7 +176,8 @@ dg_status_t dg_ap_fwd(dg_graph_t g, const float* fV, const float* fE, int32_t fE
   const uintptr_t rows = (binary == DG_BIN_COPY_RHS ? 0 : (uintptr_t)fV) | (a.cols != 1 ? (uintptr_t)fE : 0);
   a.vec = vector_width(F, rows);
   void* padded = nullptr;
-  if (a.cols == 1 && binary != DG_BIN_COPY_RHS) padded = widen(g, &a, s);
+  if (a.cols == 1 && binary != DG_BIN_COPY_RHS)
+    if (dg_status_t st = widen(g, &a, s, &padded)) return st;
   a.log_g = log_group((F + a.vec - 1) / a.vec);
   // copyrhs gathers nothing: its edge rows are a stream
   const int nb = plan_blocks(g, binary == DG_BIN_COPY_RHS ? 0.0 : slice_bytes(a.ldx), g->split_csr,
@@ -236,11 +238,13 @@ dg_status_t dg_ap_bwd(dg_graph_t g, const float* dO, const float* fV, const floa
           st = extremum_dv(g, a, (int)binary, (int)reduce, s);
         } else if (st == DG_OK) {
           a.vec = vector_width(F, (uintptr_t)dO | (cols != 1 ? (uintptr_t)fE : 0));
-          void* padded = cols == 1 ? widen(g, &a, s) : nullptr;
+          void* padded = nullptr;
+          if (cols == 1) st = widen(g, &a, s, &padded);
           a.log_g = log_group((F + a.vec - 1) / a.vec);
           const int nb = plan_blocks(g, slice_bytes(a.ldx), g->split_csc, true);
-          st = run_blocks(g, a, g->split_csc, nb, a.vec,
-                          [&](const GenArgs& p) { return launch_general_dv(p, (int)binary, (int)reduce, s); });
+          if (st == DG_OK)
+            st = run_blocks(g, a, g->split_csc, nb, a.vec,
+                            [&](const GenArgs& p) { return launch_general_dv(p, (int)binary, (int)reduce, s); });
           pool_free(padded, s);
         }
         if (a.partial) {

@@ -258,8 +258,8 @@ dg_status_t expand_rows(const int64_t* rowptr, int64_t n, int64_t nnz, const int
 
 // Whether a call first copies a gathered matrix into padded rows, and the copy (dg_aggregate.cu).
 bool worth_padding(const Graph* g, int32_t F, int elem_bytes, int vec);
-bool pad_rows(const Graph* g, const void* X, int32_t F, int elem_bytes, const int64_t* mean_ptr, int mean_self,
-              cudaStream_t s, void** copy, int64_t* ld);
+dg_status_t pad_rows(const Graph* g, const void* X, int32_t F, int elem_bytes, const int64_t* mean_ptr, int mean_self,
+                     cudaStream_t s, void** copy, int64_t* ld);
 // Scratch for the parts of cut rows (nullptr when the plan cuts none), and their join.
 dg_status_t take_partial(const Graph* g, const Plan& plan, int64_t floats_per_slot, cudaStream_t s,
                          float** partial);

@@ -47,6 +47,22 @@ class Fake:
         self.lib.fake_clear()
         return got
 
+    def call(self, name, *args):
+        """A call with integers as int32, bytes as strings and None as NULL."""
+        given = [ctypes.c_int32(a) if isinstance(a, int) else a for a in args]
+        return getattr(self.lib, name)(*given, None)
+
+    def transposed(self, n, nnz):
+        g = self.graph(n, nnz)
+        storage, scratch = ctypes.c_size_t(), ctypes.c_size_t()
+        self.lib.dg_graph_transpose_workspace(g, ctypes.byref(storage), ctypes.byref(scratch))
+        buffers = []
+        for size in (storage.value, scratch.value):
+            address = self.array(size + 256, dtype=np.uint8).value
+            buffers += [ctypes.c_void_p((address + 255) // 256 * 256), ctypes.c_size_t(size)]
+        assert self.lib.dg_graph_transpose(g, *buffers, None) == binding.DG_OK
+        return g
+
     def array(self, *shape, dtype=np.float32):
         a = np.zeros(shape, dtype)
         self.keep.append(a)
@@ -153,3 +169,28 @@ def test_a_knob_that_cannot_be_set_leaves_the_handle_as_it_was(fake, failure):
     assert knob(b"rows_per_block") == 64
     for h in (handle, other):
         fake.lib.dg_graph_destroy(h)
+
+
+def aggregation_calls(fake, n, nnz, F):
+    """(name, call) of every call that gathers a matrix, on a graph of n vertices and nnz edges."""
+    g = fake.transposed(n, nnz)
+    X, Y, dV, arg = (fake.array(n, F) for _ in range(4))
+    fE, dE = fake.array(nnz), fake.array(nnz)
+    max_, sum_, copy, mul, div = (binding.DG_RED_MAX, binding.DG_RED_SUM, binding.DG_BIN_COPY_LHS, binding.DG_BIN_MUL,
+                                  binding.DG_BIN_DIV)
+    calls = [("fwd", lambda: fake.call("dg_aggregate_fwd", g, X, F, binding.DG_OP_SUM, Y)),
+             ("bwd mean", lambda: fake.call("dg_aggregate_bwd", g, X, F, binding.DG_OP_MEAN, Y)),
+             ("max", lambda: fake.call("dg_ap_fwd", g, X, None, 1, F, copy, max_, Y, arg)),
+             ("dV of div", lambda: fake.call("dg_ap_bwd", g, X, Y, fE, 1, F, div, sum_, None, dV, None)),
+             ("edge grad", lambda: fake.call("dg_aggregate_edge_grad", g, X, Y, F, binding.DG_OP_SUM, dE))]
+    return g, calls
+
+
+def test_a_padded_copy_that_does_not_launch_is_an_error(fake):
+    g, calls = aggregation_calls(fake, 5000, 200000, 101)
+    for name, call in calls:
+        assert call() == binding.DG_OK, name
+        fake.lib.fake_failing_kernel(b"pad_rows_kernel")
+        assert call() == binding.DG_ERR_CUDA, name
+        fake.lib.fake_failing_kernel(b"")
+    fake.lib.dg_graph_destroy(g)
