@@ -454,12 +454,13 @@ dg_status_t dg_layer_bwd(dg_graph_t g, const float* dOut, const float* out, int3
   return layer_bwd(g, dOut, out, F, row_scale, G, dbias, (cudaStream_t)stream);
 }
 
-static dg_status_t check_loss(const Graph* g, int32_t C, int64_t count, bool pointers) {
+static dg_status_t check_loss(const Graph* g, int32_t C, int64_t count, const void* stats, bool pointers) {
   if (!g) return invalid("graph handle is NULL");
   if (C < 1 || C > (1 << 20)) return invalid("C must be from 1 to 2^20");
   if (count < 0 || count > ((int64_t)1 << 37)) return invalid("count must be from 0 to 2^37");
   if (count > 0 && g->n == 0) return invalid("the matrix has no rows");
   if (!pointers) return invalid("a pointer is NULL");
+  if ((uintptr_t)stats & 7) return invalid("stats must be 8-byte aligned");
   return DG_OK;
 }
 
@@ -467,7 +468,7 @@ dg_status_t dg_cross_entropy_fwd(dg_graph_t g, const float* logits, int32_t C, c
                                  int64_t count, const int64_t* labels, float* stats, float* result,
                                  void* stream) {
   const bool pointers = result && (count <= 0 || (logits && index && labels && stats));
-  if (dg_status_t st = check_loss(g, C, count, pointers)) return st;
+  if (dg_status_t st = check_loss(g, C, count, stats, pointers)) return st;
   return loss_fwd(g, logits, C, index, count, labels, stats, result, (cudaStream_t)stream);
 }
 
@@ -476,7 +477,7 @@ dg_status_t dg_cross_entropy_bwd(dg_graph_t g, const float* logits, int32_t C, c
                                  const float* result, const float* grad, float* dLogits, void* stream) {
   const bool pointers = (!g || g->n == 0 || dLogits) &&
                         (count <= 0 || (logits && index && labels && stats && result && grad));
-  if (dg_status_t st = check_loss(g, C, count, pointers)) return st;
+  if (dg_status_t st = check_loss(g, C, count, stats, pointers)) return st;
   return loss_bwd(g, logits, C, index, count, labels, stats, result, grad, dLogits, (cudaStream_t)stream);
 }
 

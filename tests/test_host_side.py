@@ -194,3 +194,16 @@ def test_a_padded_copy_that_does_not_launch_is_an_error(fake):
         assert call() == binding.DG_ERR_CUDA, name
         fake.lib.fake_failing_kernel(b"")
     fake.lib.dg_graph_destroy(g)
+
+
+def test_misaligned_statistics_of_the_loss_are_refused(fake):
+    """The kernels read and write them 8 bytes at a time."""
+    g = fake.graph(8, 16)
+    logits, grads, index, labels = fake.array(8, 4), fake.array(8, 4), fake.array(4, dtype=np.int64), fake.array(8, dtype=np.int64)
+    stats, result = fake.array(12), fake.array(2)
+    for shift, want in ((0, binding.DG_OK), (4, binding.DG_ERR_INVALID_ARG)):
+        at = ctypes.c_void_p((stats.value + 7) // 8 * 8 + shift)
+        assert fake.lib.dg_cross_entropy_fwd(g, logits, 4, index, ctypes.c_int64(4), labels, at, result, None) == want
+        assert fake.lib.dg_cross_entropy_bwd(g, logits, 4, index, ctypes.c_int64(4), labels, at, result, result, grads,
+                                             None) == want
+    fake.lib.dg_graph_destroy(g)
