@@ -120,6 +120,12 @@ def _dev_ptr(t: Optional[torch.Tensor], dtype, name: str):
     raise ValueError(f"{name} must be contiguous")
 
 
+def _holds(t: torch.Tensor, count: int, name: str) -> None:
+    """The library sees pointers only: what a kernel will index has to be there."""
+    if t.numel() < count:
+        raise ValueError(f"{name} must hold {count} values, got {t.numel()}")
+
+
 # The handle of the current stream of the current device.  torch.cuda.current_stream() builds two
 # Python objects on the way to it: 3.2 us, a third of what a call on a small graph took on the host.
 _raw_stream, _device = torch._C._cuda_getCurrentRawStream, torch._C._cuda_getDevice
@@ -137,8 +143,8 @@ def dg_last_error() -> str:
     return lib().dg_last_error().decode()
 
 
-def dg_kernel_launch_count() -> int:
-    return int(lib().dg_kernel_launch_count())
+def dg_kernel_launch_holds() -> int:
+    return int(lib().dg_kernel_launch_holds())
 
 
 def dg_probe_gather(table: torch.Tensor, idx: torch.Tensor, sink: torch.Tensor, stream=None) -> None:
@@ -321,8 +327,10 @@ class Graph:
 
     def dg_aggregate_fwd_self(self, H: torch.Tensor, op: int, out: Optional[torch.Tensor] = None,
                               stream=None) -> torch.Tensor:
+        _holds(H, self.n * H.shape[1], "H")
         if out is None:
             out = torch.empty_like(H)
+        _holds(out, self.n * H.shape[1], "out")
         _check(lib().dg_aggregate_fwd_self(self._h, _dev_ptr(H, torch.float32, "H"), H.shape[1],
                                            int(op), _dev_ptr(out, torch.float32, "out"),
                                            _stream(stream)))
@@ -330,8 +338,10 @@ class Graph:
 
     def dg_aggregate_bwd_self(self, dOut: torch.Tensor, op: int,
                               dH: Optional[torch.Tensor] = None, stream=None) -> torch.Tensor:
+        _holds(dOut, self.n * dOut.shape[1], "dOut")
         if dH is None:
             dH = torch.empty_like(dOut)
+        _holds(dH, self.n * dOut.shape[1], "dH")
         _check(lib().dg_aggregate_bwd_self(self._h, _dev_ptr(dOut, torch.float32, "dOut"),
                                            dOut.shape[1], int(op),
                                            _dev_ptr(dH, torch.float32, "dH"), _stream(stream)))
@@ -340,6 +350,9 @@ class Graph:
     def dg_layer_fwd(self, Y: torch.Tensor, row_scale: torch.Tensor, bias: torch.Tensor, relu: bool,
                      stream=None) -> torch.Tensor:
         """Y = act(row_scale * Y + bias), in place."""
+        _holds(Y, self.n * Y.shape[1], "Y")
+        _holds(row_scale, self.n, "row_scale")
+        _holds(bias, Y.shape[1], "bias")
         _check(lib().dg_layer_fwd(self._h, _dev_ptr(Y, torch.float32, "Y"), Y.shape[1],
                                   _dev_ptr(row_scale, torch.float32, "row_scale"),
                                   _dev_ptr(bias, torch.float32, "bias"), bool(relu), _stream(stream)))
@@ -348,6 +361,10 @@ class Graph:
     def dg_layer_bwd(self, dOut: torch.Tensor, out: Optional[torch.Tensor], row_scale: torch.Tensor,
                      stream=None):
         """(row_scale * d, column sums of d) with d = dOut where out > 0 (out None: dOut)."""
+        _holds(dOut, self.n * dOut.shape[1], "dOut")
+        if out is not None:
+            _holds(out, self.n * dOut.shape[1], "out")
+        _holds(row_scale, self.n, "row_scale")
         G = torch.empty_like(dOut)
         dbias = dOut.new_empty(dOut.shape[1])
         _check(lib().dg_layer_bwd(self._h, _dev_ptr(dOut, torch.float32, "dOut"),
@@ -357,8 +374,13 @@ class Graph:
                                   _stream(stream)))
         return G, dbias
 
+    def _loss_shapes(self, logits, index, labels) -> None:
+        _holds(logits, self.n * logits.shape[1], "logits")
+        _holds(labels, self.n, "labels")
+
     def dg_cross_entropy_fwd(self, logits: torch.Tensor, index: torch.Tensor, labels: torch.Tensor, stream=None):
         """(result, stats): result[0] is the mean loss of logits[index] against labels[index]."""
+        self._loss_shapes(logits, index, labels)
         result, stats = logits.new_empty(2), logits.new_empty((index.shape[0], 2))
         _check(lib().dg_cross_entropy_fwd(self._h, _dev_ptr(logits, torch.float32, "logits"), logits.shape[1],
                                           _dev_ptr(index, torch.int64, "index"), index.shape[0],
@@ -369,6 +391,10 @@ class Graph:
     def dg_cross_entropy_bwd(self, logits: torch.Tensor, index: torch.Tensor, labels: torch.Tensor,
                              result: torch.Tensor, stats: torch.Tensor, grad: torch.Tensor,
                              stream=None) -> torch.Tensor:
+        self._loss_shapes(logits, index, labels)
+        _holds(stats, 2 * index.shape[0], "stats")
+        _holds(result, 2, "result")
+        _holds(grad, 1, "grad")
         d = torch.empty_like(logits)
         _check(lib().dg_cross_entropy_bwd(self._h, _dev_ptr(logits, torch.float32, "logits"), logits.shape[1],
                                           _dev_ptr(index, torch.int64, "index"), index.shape[0],

@@ -57,6 +57,42 @@ def test_host_side_argument_checks_need_no_gpu(libpath):
     assert lib.dg_graph_validate(None, None) == 1
 
 
+def test_binding_refuses_short_arguments():
+    """The layer and loss calls check what their kernels will index, before any pointer is taken."""
+    import torch
+    from paper_2104_06700_b200 import binding
+    n, F = 6, 4
+    g = binding.Graph.__new__(binding.Graph)
+    g.n, g._h = n, None
+    Y, scale, bias = torch.zeros(n, F), torch.zeros(n, 1), torch.zeros(F)
+    index, labels = torch.zeros(3, dtype=torch.int64), torch.zeros(n, dtype=torch.int64)
+    result, stats, grad = torch.zeros(2), torch.zeros(3, 2), torch.zeros(())
+    short = torch.zeros(n - 1, F)
+    calls = [
+        lambda: g.dg_layer_fwd(short, scale, bias, True),
+        lambda: g.dg_layer_fwd(Y, scale[1:], bias, True),
+        lambda: g.dg_layer_fwd(Y, scale, bias[1:], True),
+        lambda: g.dg_layer_bwd(short, None, scale),
+        lambda: g.dg_layer_bwd(Y, short, scale),
+        lambda: g.dg_layer_bwd(Y, None, scale[1:]),
+        lambda: g.dg_aggregate_fwd_self(short, 0),
+        lambda: g.dg_aggregate_fwd_self(Y, 0, out=short),
+        lambda: g.dg_aggregate_bwd_self(short, 0),
+        lambda: g.dg_aggregate_bwd_self(Y, 0, dH=short),
+        lambda: g.dg_cross_entropy_fwd(short, index, labels),
+        lambda: g.dg_cross_entropy_fwd(Y, index, labels[1:]),
+        lambda: g.dg_cross_entropy_bwd(short, index, labels, result, stats, grad),
+        lambda: g.dg_cross_entropy_bwd(Y, index, labels[1:], result, stats, grad),
+        lambda: g.dg_cross_entropy_bwd(Y, index, labels, result[1:], stats, grad),
+        lambda: g.dg_cross_entropy_bwd(Y, index, labels, result, stats[1:], grad),
+        lambda: g.dg_cross_entropy_bwd(Y, index, labels, result, stats, grad.new_zeros(0)),
+    ]
+    for i, call in enumerate(calls):
+        with pytest.raises(ValueError) as e:
+            call()
+        assert "must hold" in str(e.value), i
+
+
 def test_product_path_has_no_oracle_import():
     pkg = os.path.join(ROOT, "paper_2104_06700_b200")
     for dirpath, _, files in os.walk(pkg):
