@@ -143,8 +143,8 @@ def dg_last_error() -> str:
     return lib().dg_last_error().decode()
 
 
-def dg_kernel_launch_holds() -> int:
-    return int(lib().dg_kernel_launch_holds())
+def dg_kernel_launch_count() -> int:
+    return int(lib().dg_kernel_launch_count())
 
 
 def dg_probe_gather(table: torch.Tensor, idx: torch.Tensor, sink: torch.Tensor, stream=None) -> None:
