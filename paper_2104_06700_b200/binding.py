@@ -120,9 +120,9 @@ def _dev_ptr(t: Optional[torch.Tensor], dtype, name: str):
     raise ValueError(f"{name} must be contiguous")
 
 
-def _holds(t: torch.Tensor, count: int, name: str) -> None:
-    """The library sees pointers only: what a kernel will index has to be there."""
-    if t.numel() < count:
+def _holds(t: Optional[torch.Tensor], count: int, name: str) -> None:
+    """The library sees pointers only: what a kernel will index has to be there (it refuses NULL itself)."""
+    if t is not None and t.numel() < count:
         raise ValueError(f"{name} must hold {count} values, got {t.numel()}")
 
 
