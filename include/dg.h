@@ -19,6 +19,14 @@
  *   - feature matrices are dense, row-major, fp32, leading dimension F, 1 <= F <= 2^20;
  *   - rowptr/colptr are int64, vertex ids are int32 (n < 2^31), nnz < 2^31;
  *   - no call aborts, traps or waits without bound on the device;
+ *   - device memory: a handle owns a few arrays (see dg_graph_create), and a call that takes a stream may
+ *     use scratch between its launches (the parts of rows that several warps share, a padded copy of an
+ *     n x F matrix up to 4 GiB, the edge mask of the gradient of max / min up to 2 GiB, partial sums).  Both
+ *     come from a stream-ordered pool of the library, which keeps up to 4 GiB of unused memory per device
+ *     while a handle is alive and 32 MiB afterwards.  No call needs the scratch: without memory for it, or
+ *     beyond the handle's "scratch_mb", the call takes a slower path to the same result (sums may be added
+ *     in another order).  "scratch_mb" = 0 is for processes that gave the whole device to an allocator of
+ *     their own: then no call takes memory;
  *   - a handle may be used from any thread, by one thread at a time; different handles are
  *     independent.  Calls on one handle that are queued on different streams are not ordered
  *     against each other by the library (source-blocked passes read what the previous launch
@@ -385,11 +393,13 @@ dg_status_t dg_aggregate_edge_grad(dg_graph_t g, const float* H, const float* dO
  *                      (the blocking of Algorithm 2; 0 = choose from the L2 budget, else 1, 2,
  *                      4, 8 or 16; ignored for graphs without split pointers, i.e. with fewer
  *                      than 64 edges per vertex or unsorted rows)
+ *   "scratch_mb"       MiB one scratch block of a call may take from the library's pool (4096; 0: none)
  * Graph attribute (not a tuning knob: it changes the result):
  *   "self_loops"       0 (default) or 1: every vertex is its own in-neighbour with weight 1, see
  *                      dg_aggregate_fwd / dg_aggregate_bwd; set it before dg_graph_transpose
  * Changing "heavy_threshold" or "rows_per_block" waits for the whole device, shares the rows out
- * anew and waits again: a rare, synchronous call.
+ * anew and waits again: a rare, synchronous call.  CUDA graphs captured before it must not be launched
+ * afterwards.  If it fails the handle is as it was.
  * Returns DG_ERR_INVALID_ARG for an unknown name or a value out of range.
  */
 dg_status_t dg_graph_set_param(dg_graph_t g, const char* name, int64_t value);

@@ -79,17 +79,11 @@ dg_status_t launch_plain(const ApArgs& a, int vec, int slices, cudaStream_t s) {
   return dispatch_type<false>(a, SelfArgs{}, vec, slices, s);
 }
 
-// Scratch for the parts of cut rows, from the library's pool.  *partial stays nullptr when the plan cuts
-// no row.
-dg_status_t take_partial(const Graph* g, const Plan& plan, int64_t floats_per_slot, cudaStream_t s,
-                         float** partial) {
-  *partial = nullptr;
-  const int64_t slots = plan.slots >= 0 ? plan.slots : plan.max_slots;
-  if (slots == 0) return DG_OK;
+float* take_partial(const Graph* g, const Plan& plan, int64_t floats_per_slot, cudaStream_t s, bool* missing) {
   void* p = nullptr;
-  DG_CUDA(pool_alloc(g->device, (size_t)slots * (size_t)floats_per_slot * sizeof(float), s, &p));
-  *partial = static_cast<float*>(p);
-  return DG_OK;
+  const int64_t slots = plan.slots >= 0 ? plan.slots : plan.max_slots;
+  *missing = slots > 0 && scratch_alloc(g, (size_t)slots * (size_t)floats_per_slot * sizeof(float), s, &p) != cudaSuccess;
+  return static_cast<float*>(p);
 }
 
 dg_status_t join_cut_rows(const Graph* g, const Plan& plan, const float* partial, int32_t F, float* Y,
@@ -150,7 +144,7 @@ dg_status_t pad_rows(const Graph* g, const void* X, int32_t F, int elem_bytes, c
   const int64_t unit = (F * elem_bytes > 512 ? 128 : 32) / elem_bytes;
   const int64_t to = (F + unit - 1) / unit * unit;
   const size_t bytes = (size_t)g->n * (size_t)to * (size_t)elem_bytes;
-  if (pool_alloc(g->device, bytes, s, copy) != cudaSuccess) return DG_OK;
+  if (scratch_alloc(g, bytes, s, copy) != cudaSuccess) return DG_OK;
   *ld = to;
   const unsigned blocks = (unsigned)((bytes / 16 + 255) / 256);
   if (elem_bytes == 2)
@@ -270,7 +264,9 @@ dg_status_t aggregate_run(const Graph* g, const ApArgs& a0, const SelfArgs& sa0,
   a.chunks = plan.chunks;
   a.chunk_count = (int32_t)plan.count;
   a.few_blocks = plan.count * slices <= 4 * (int64_t)g->sm_count * 4 * kWarpsPerBlock;  // four waves
-  dg_status_t st = take_partial(g, plan, a.F, s, &a.partial);
+  bool missing = false;
+  a.partial = take_partial(g, plan, a.F, s, &missing);
+  dg_status_t st = DG_OK;
   const int per = kFineBlocks / nb;
   for (int j = 0; j < nb && st == DG_OK; ++j) {
     if (nb > 1) {
@@ -284,6 +280,20 @@ dg_status_t aggregate_run(const Graph* g, const ApArgs& a0, const SelfArgs& sa0,
   if (a.partial) {
     if (st == DG_OK) st = join_cut_rows(g, plan, a.partial, a.F, a.Y, s);
     pool_free(a.partial, s);
+  }
+  if (missing && st == DG_OK) {
+    PieceArgs p{};
+    p.idx = a.idx;
+    p.X = a.X;
+    p.ldx = ld;
+    p.bf16 = bf16;
+    p.w = a.w;
+    p.F = a.F;
+    p.red = DG_RED_SUM;
+    p.mean_ptr = a.mean_rows ? a.ptr : nullptr;
+    p.mean_self = sa.self_ptr != nullptr;
+    p.out = a.Y;
+    st = add_pieces(g, plan, p, s);
   }
   pool_free(padded, s);
   return st;

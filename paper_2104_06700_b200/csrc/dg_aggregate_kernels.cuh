@@ -314,6 +314,7 @@ __device__ __forceinline__ void ap_body(const ApArgs& a, const SelfArgs sa) {
   if (chunk >= a.chunk_count) return;
   const int4 here = __ldg(reinterpret_cast<const int4*>(a.chunks) + chunk);
   const int4 next = __ldg(reinterpret_cast<const int4*>(a.chunks) + chunk + 1);
+  if (here.z >= 0 && !a.partial) return;  // add_pieces will
   const int rb = here.x;
   // the next chunk may begin inside our last row; a chunk that begins inside a row is a piece of that row
   const int nrows = here.z >= 0 ? 1 : next.x - here.x + (next.z >= 0 ? 1 : 0);

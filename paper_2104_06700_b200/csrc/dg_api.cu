@@ -633,6 +633,11 @@ dg_status_t dg_graph_set_param(dg_graph_t g, const char* name, int64_t value) {
     g->self_loops = value;
     return DG_OK;
   }
+  if (!strcmp(name, "scratch_mb")) {
+    if (value < 0 || value > (1 << 20)) return invalid("scratch_mb must be in [0, 2^20]");
+    g->scratch_mb = value;
+    return DG_OK;
+  }
   if (!strcmp(name, "source_blocks")) {
     if (value != 0 && value != 1 && value != 2 && value != 4 && value != 8 && value != 16)
       return invalid("source_blocks must be 0 (automatic), 1, 2, 4, 8 or 16");
@@ -650,6 +655,7 @@ dg_status_t dg_graph_get_param(dg_graph_t g, const char* name, int64_t* value) {
   if (!strcmp(name, "l2_budget_mb")) { *value = g->l2_budget_bytes >> 20; return DG_OK; }
   if (!strcmp(name, "source_blocks")) { *value = g->source_blocks; return DG_OK; }
   if (!strcmp(name, "self_loops")) { *value = g->self_loops; return DG_OK; }
+  if (!strcmp(name, "scratch_mb")) { *value = g->scratch_mb; return DG_OK; }
   if (!strcmp(name, "heavy_blocks_per_sm")) { *value = g->heavy_blocks_per_sm; return DG_OK; }
   return invalid("unknown parameter name");
 }

@@ -96,7 +96,7 @@ dg_status_t extremum_dv(const dg_graph* g, GenArgs a, int bin, int red, cudaStre
   void* mask = nullptr;
   auto dv = [&](const GenArgs& p) { return launch_general_dv(p, bin, red, s); };
   if (g->nnz == 0 || (size_t)g->nnz * (size_t)words * 4 > kMaskMaxBytes ||
-      pool_alloc(g->device, (size_t)g->nnz * (size_t)words * 4, s, &mask) != cudaSuccess) {
+      scratch_alloc(g, (size_t)g->nnz * (size_t)words * 4, s, &mask) != cudaSuccess) {
     a.vec = vector_width(a.F, (uintptr_t)a.arg) == 4 ? 4 : 1;  // of arg; a lane has four features
     a.log_g = log_group((a.F + 3) / 4);
     const int nb = plan_blocks(g, 2 * slice_bytes(a.F), g->split_csc, true);  // dO and arg
@@ -117,6 +117,25 @@ dg_status_t extremum_dv(const dg_graph* g, GenArgs a, int bin, int red, cudaStre
   }
   pool_free(mask, s);
   return st;
+}
+
+// The later pieces of a call that found no memory for their results.
+PieceArgs pieces_of(const GenArgs& a, int bin, int red, bool gradient) {
+  PieceArgs p{};
+  p.idx = bin == kCopyRhs ? nullptr : a.idx;
+  p.perm = a.perm;
+  p.X = a.X;
+  p.ldx = a.ldx;
+  p.Y = bin == kCopyLhs ? nullptr : a.Y;
+  p.edge_cols = a.cols;
+  p.arg = a.arg;
+  p.F = a.F;
+  p.bin = bin;
+  p.red = red;
+  p.gradient = gradient;
+  p.out = a.out;
+  p.arg_out = a.arg_out;
+  return p;
 }
 
 dg_status_t bad(const char* msg) {
@@ -184,13 +203,16 @@ dg_status_t dg_ap_fwd(dg_graph_t g, const float* fV, const float* fE, int32_t fE
                              !extremum || arg != nullptr);
   // an extremum's parts carry their edge positions
   const Plan& plan = g->row_plan;
-  dg_status_t st = take_partial(g, plan, (int64_t)F * (extremum ? 2 : 1), s, &a.partial);
+  bool missing = false;
+  a.partial = take_partial(g, plan, (int64_t)F * (extremum ? 2 : 1), s, &missing);
+  a.skip_pieces = missing;
   if (extremum && a.partial)
     a.partial_arg =
         reinterpret_cast<int32_t*>(a.partial + (plan.slots >= 0 ? plan.slots : plan.max_slots) * (int64_t)F);
-  if (st == DG_OK)
-    st = run_blocks(g, a, g->split_csr, nb, a.vec,
-                    [&](const GenArgs& p) { return launch_general_fwd(p, (int)binary, (int)reduce, s); });
+  dg_status_t st = run_blocks(g, a, g->split_csr, nb, a.vec, [&](const GenArgs& p) {
+    return launch_general_fwd(p, (int)binary, (int)reduce, s);
+  });
+  if (missing && st == DG_OK) st = add_pieces(g, plan, pieces_of(a, (int)binary, (int)reduce, false), s);
   if (a.partial) {
     if (st == DG_OK)
       st = extremum ? join_extrema(g, plan, a, (int)reduce, s) : join_cut_rows(g, plan, a.partial, F, fO, s);
@@ -233,10 +255,14 @@ dg_status_t dg_ap_bwd(dg_graph_t g, const float* dO, const float* fV, const floa
         a.F = F;
         a.cols = cols;
         const Plan& plan = column_plan(g);
-        dg_status_t st = take_partial(g, plan, F, s, &a.partial);
-        if (st == DG_OK && reduce != DG_RED_SUM) {
+        bool missing = false;
+        a.partial = take_partial(g, plan, F, s, &missing);
+        a.skip_pieces = missing;
+        dg_status_t st = DG_OK;
+        if (reduce != DG_RED_SUM) {
           st = extremum_dv(g, a, (int)binary, (int)reduce, s);
-        } else if (st == DG_OK) {
+          if (missing && st == DG_OK) st = add_pieces(g, plan, pieces_of(a, (int)binary, (int)reduce, true), s);
+        } else {
           a.vec = vector_width(F, (uintptr_t)dO | (cols != 1 ? (uintptr_t)fE : 0));
           void* padded = nullptr;
           if (cols == 1) st = widen(g, &a, s, &padded);
@@ -245,6 +271,7 @@ dg_status_t dg_ap_bwd(dg_graph_t g, const float* dO, const float* fV, const floa
           if (st == DG_OK)
             st = run_blocks(g, a, g->split_csc, nb, a.vec,
                             [&](const GenArgs& p) { return launch_general_dv(p, (int)binary, (int)reduce, s); });
+          if (missing && st == DG_OK) st = add_pieces(g, plan, pieces_of(a, (int)binary, (int)reduce, true), s);
           pool_free(padded, s);
         }
         if (a.partial) {

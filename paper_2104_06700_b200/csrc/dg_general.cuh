@@ -43,6 +43,7 @@ struct GenArgs {
   float* out;             // n x F, or nnz x cols in the edge gradient
   int32_t* arg_out;
   float* partial;         // slots x F: the parts of cut rows
+  int32_t skip_pieces;    // no memory for them: left out, see dg_pieces.cu
   int32_t* partial_arg;   // and their edge positions (max / min)
   int32_t F, cols;
   int32_t log_g;          // lanes per edge = 1 << log_g
@@ -158,6 +159,7 @@ __device__ __forceinline__ void walk_chunk(const GenArgs& a, First first, Begin 
   const int chunk = blockIdx.x * kGenWarps + __shfl_sync(kAll, (int)(threadIdx.x >> 5), 0);
   if (chunk >= a.chunk_count) return;
   const int4 here = __ldg(reinterpret_cast<const int4*>(a.chunks) + chunk);
+  if (here.z >= 0 && a.skip_pieces) return;
   const int4 next = __ldg(reinterpret_cast<const int4*>(a.chunks) + chunk + 1);
   const int nrows = here.z >= 0 ? 1 : next.x - here.x + (next.z >= 0 ? 1 : 0);
   int my_lo = 0, my_hi = 0;

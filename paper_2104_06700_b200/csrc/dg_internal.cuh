@@ -100,6 +100,7 @@ struct dg_graph {
   int64_t heavy_blocks_per_sm = 0;  // recorded for dg_graph_get_param, no effect
   int64_t l2_budget_bytes = 0;   // bytes of the gathered matrix one launch may keep L2-resident
   int64_t source_blocks = 0;     // 0 = automatic, else 1, 2, 4, 8 or 16
+  int64_t scratch_mb = 4096;     // most MiB of a scratch block of a call; 0: calls take no memory
 };
 
 namespace dg {
@@ -126,7 +127,7 @@ struct ApArgs {
   int32_t narrow_store;       // 1: the rows of Y cannot take the vector width that X is read with
   const Chunk* chunks;        // chunk_count + 1
   int32_t chunk_count;
-  float* partial;             // slots x F: the parts of cut rows
+  float* partial;             // slots x F: the parts of cut rows; nullptr: left out, see dg_pieces.cu
   int64_t n;
   int32_t F;
   int32_t slice_f;            // features per slice (multiple of the vector width)
@@ -211,6 +212,8 @@ void pool_close(int device);
 cudaError_t pool_wait(int device);   // waits for the device, then frees what was retired before
 cudaError_t pool_alloc(int device, size_t bytes, cudaStream_t s, void** out);
 void pool_free(void* p, cudaStream_t s);
+// Scratch of a call, within the handle's limit; a call has to do without it when there is none.
+cudaError_t scratch_alloc(const Graph* g, size_t bytes, cudaStream_t s, void** out);
 void pool_retire(int device, void* p, size_t bytes);  // kernels on any stream may still use it
 cudaError_t pinned_counters(HostCounters** out);
 void pinned_counters_retire(int device, HostCounters* p);
@@ -260,9 +263,28 @@ dg_status_t expand_rows(const int64_t* rowptr, int64_t n, int64_t nnz, const int
 bool worth_padding(const Graph* g, int32_t F, int elem_bytes, int vec);
 dg_status_t pad_rows(const Graph* g, const void* X, int32_t F, int elem_bytes, const int64_t* mean_ptr, int mean_self,
                      cudaStream_t s, void** copy, int64_t* ld);
-// Scratch for the parts of cut rows (nullptr when the plan cuts none), and their join.
-dg_status_t take_partial(const Graph* g, const Plan& plan, int64_t floats_per_slot, cudaStream_t s,
-                         float** partial);
+// Scratch for the parts of cut rows, and their join.  nullptr when the plan cuts none, or when there is no memory
+// (`missing`): then the pieces are left out of the main kernels and added by add_pieces (dg_pieces.cu).
+float* take_partial(const Graph* g, const Plan& plan, int64_t floats_per_slot, cudaStream_t s, bool* missing);
+struct PieceArgs {
+  const Chunk* chunks;     // the first four come from the plan
+  const CutRow* cuts;
+  const int32_t* totals;
+  int32_t max_cuts;
+  int32_t F;
+  const int32_t* idx;      // nullptr: nothing is gathered (copyrhs)
+  const int32_t* perm;     // over the CSC: CSR position of every entry
+  const void* X;           // gathered rows, ldx elements apart
+  int64_t ldx;
+  const float* w;          // factor of the entry (sum and mean calls), in the order walked
+  const float* Y;          // edge operand, edge_cols = 1 or F columns, in CSR order
+  const int32_t* arg;      // gradient of max / min
+  const int64_t* mean_ptr; // rows divided by their length here + mean_self
+  float* out;
+  int32_t* arg_out;
+  int32_t bf16, edge_cols, bin, red, gradient, mean_self;
+};
+dg_status_t add_pieces(const Graph* g, const Plan& plan, PieceArgs a, cudaStream_t s);
 dg_status_t join_cut_rows(const Graph* g, const Plan& plan, const float* partial, int32_t F, float* Y,
                           cudaStream_t s);
 // dg_edge_grad.cu

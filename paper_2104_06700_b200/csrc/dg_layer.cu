@@ -71,8 +71,8 @@ __global__ void __launch_bounds__(kStreamBlock)
   }
 }
 
-// G = D (dOut where out > 0), and into partial[blockIdx.x] the column sums of the masked dOut over the block's
-// rows.  `out` null: no mask.
+// G = D (dOut where out > 0), and into partial[blockIdx.x] (unless null) the column sums of the masked dOut over the
+// block's rows.  `out` null: no mask.
 template <int VEC>
 __global__ void __launch_bounds__(kStreamBlock)
     layer_bwd_kernel(const float* dOut, const float* out, const float* scale, int64_t n, int32_t F, float* G,
@@ -108,6 +108,7 @@ __global__ void __launch_bounds__(kStreamBlock)
       }
     }
   }
+  if (!partial) return;
 #pragma unroll
   for (int c = 0; c < VEC; ++c) sums[(threadIdx.y * VEC + c) * blockDim.x + threadIdx.x] = total[c];
   __syncthreads();
@@ -129,6 +130,32 @@ __global__ void __launch_bounds__(1024) layer_bias_kernel(const float* partial, 
   float t = 0.f;
   if (f < F)
     for (int32_t b = threadIdx.y; b < blocks; b += 32) t += partial[(int64_t)b * F + f];
+  sums[threadIdx.y][threadIdx.x] = t;
+  __syncthreads();
+  t = sums[threadIdx.x][threadIdx.y];
+#pragma unroll
+  for (int o = 16; o > 0; o >>= 1) t += __shfl_xor_sync(0xffffffffu, t, o);
+  const int32_t column = blockIdx.x * 32 + threadIdx.y;
+  if (threadIdx.x == 0 && column < F) dbias[column] = t;
+}
+
+// dbias from dOut itself, where there is no memory for the blocks' sums: 32 columns x 32 threads per block again, the
+// sum of every 64 rows of a thread added to its total.
+__global__ void __launch_bounds__(1024) layer_bias_direct_kernel(const float* dOut, const float* out, int64_t n,
+                                                                 int32_t F, float* dbias) {
+  __shared__ float sums[32][33];
+  const int32_t f = blockIdx.x * 32 + threadIdx.x;
+  float t = 0.f;
+  if (f < F) {
+    for (int64_t r0 = threadIdx.y; r0 < n; r0 += 64 * 32) {
+      float part = 0.f;
+      for (int64_t r = r0; r < n && r < r0 + 64 * 32; r += 32) {
+        const float d = dOut[r * F + f];
+        part += out && out[r * F + f] <= 0.f ? 0.f : d;
+      }
+      t += part;
+    }
+  }
   sums[threadIdx.y][threadIdx.x] = t;
   __syncthreads();
   t = sums[threadIdx.x][threadIdx.y];
@@ -177,13 +204,16 @@ dg_status_t layer_bwd(const Graph* g, const float* dOut, const float* out, int32
   dim3 grid, block;
   stream_shape(g, F, wide ? 4 : 1, &grid, &block);
   void* partial = nullptr;
-  DG_CUDA(pool_alloc(g->device, (size_t)grid.x * (size_t)F * sizeof(float), s, &partial));
+  const unsigned columns = (unsigned)((F + 31) / 32);
+  if (scratch_alloc(g, (size_t)grid.x * (size_t)F * sizeof(float), s, &partial) != cudaSuccess)
+    // first: G may take the place of dOut
+    layer_bias_direct_kernel<<<columns, dim3(32, 32), 0, s>>>(dOut, out, g->n, F, dbias);
   float* sums = static_cast<float*>(partial);
   if (wide)
     layer_bwd_kernel<4><<<grid, block, 0, s>>>(dOut, out, scale, g->n, F, G, sums);
   else
     layer_bwd_kernel<1><<<grid, block, 0, s>>>(dOut, out, scale, g->n, F, G, sums);
-  layer_bias_kernel<<<(unsigned)((F + 31) / 32), dim3(32, 32), 0, s>>>(sums, (int32_t)grid.x, F, dbias);
+  if (sums) layer_bias_kernel<<<columns, dim3(32, 32), 0, s>>>(sums, (int32_t)grid.x, F, dbias);
   const cudaError_t e = cudaGetLastError();
   pool_free(partial, s);
   DG_CUDA(e);

@@ -57,66 +57,77 @@ __device__ __forceinline__ T warp_sum(T v) {
 }
 
 // K registers per lane hold a row of up to 32 K classes; K = 0 reads it twice.  stats[t] = (max, log of the sum
-// of exp(x - max)); partial[block] = (sum of the losses, rows that count; NaN after a bad index or label).
+// of exp(x - max)).  Each of `shares` (128 rows) leaves partial[share] = (sum of the losses, rows that count; NaN after
+// a bad index or label).  Without memory for them (partial null) one block takes all shares and writes the result.
 template <int K>
 __global__ void __launch_bounds__(kLossBlock)
     loss_fwd_kernel(const float* __restrict__ logits, int64_t n, int32_t C, const int64_t* __restrict__ index,
                     int64_t count, const int64_t* __restrict__ labels, float2* __restrict__ stats,
-                    double2* __restrict__ partial) {
+                    double2* __restrict__ partial, int64_t shares, float* __restrict__ result) {
   const int lane = threadIdx.x & 31, warp = threadIdx.x / 32;
-  const int64_t t0 = (int64_t)blockIdx.x * kRowsPerBlock + warp * kRowsPerWarp;
-  const Target mine = target_of(index, labels, lane < kRowsPerWarp ? t0 + lane : count, count, n, C);
-  const int64_t my_row = mine.row < 0 ? 0 : mine.row;
-  float my_max = 0.f, my_log = 0.f, my_target = 0.f;
-#pragma unroll 4
-  for (int j = 0; j < kRowsPerWarp; ++j) {
-    const float* x = logits + __shfl_sync(kAll, my_row, j) * C;
-    float m = -INFINITY, s = 0.f;
-    if constexpr (K > 0) {
-      float v[K > 0 ? K : 1];
-#pragma unroll
-      for (int k = 0; k < K; ++k) {
-        const int c = lane + 32 * k;
-        v[k] = c < C ? x[c] : -INFINITY;
-        m = m > v[k] || m != m ? m : v[k];
-      }
-      m = warp_max(m);
-#pragma unroll
-      for (int k = 0; k < K; ++k) s += lane + 32 * k < C ? expf(v[k] - m) : 0.f;
-    } else {
-      for (int c = lane; c < C; c += 32) m = m > x[c] || m != m ? m : x[c];
-      m = warp_max(m);
-      for (int c = lane; c < C; c += 32) s += expf(x[c] - m);
-    }
-    s = warp_sum(s);
-    if (lane == j) {
-      my_max = m;
-      my_log = logf(s);
-    }
-  }
-  if (lane < kRowsPerWarp && t0 + lane < count) {
-    my_target = logits[my_row * C + mine.label];
-    stats[t0 + lane] = make_float2(my_max, my_log);
-  }
-  double loss = mine.row >= 0 ? (double)((my_max - my_target) + my_log) : 0.0;
-  if (mine.bad) loss = NAN;
-  loss = warp_sum(loss);
-  const int rows = __popc(__ballot_sync(kAll, mine.row >= 0));
   __shared__ double losses[kLossBlock / 32];
   __shared__ int counts[kLossBlock / 32];
-  if (lane == 0) {
-    losses[warp] = loss;
-    counts[warp] = rows;
-  }
-  __syncthreads();
-  if (threadIdx.x == 0) {
-    double l = 0.0;
-    int r = 0;
-    for (int i = 0; i < kLossBlock / 32; ++i) {
-      l += losses[i];
-      r += counts[i];
+  double2 all = make_double2(0.0, 0.0);
+  for (int64_t share = blockIdx.x; share < shares; share += gridDim.x) {
+    const int64_t t0 = share * kRowsPerBlock + warp * kRowsPerWarp;
+    const Target mine = target_of(index, labels, lane < kRowsPerWarp ? t0 + lane : count, count, n, C);
+    const int64_t my_row = mine.row < 0 ? 0 : mine.row;
+    float my_max = 0.f, my_log = 0.f, my_target = 0.f;
+#pragma unroll 4
+    for (int j = 0; j < kRowsPerWarp; ++j) {
+      const float* x = logits + __shfl_sync(kAll, my_row, j) * C;
+      float m = -INFINITY, s = 0.f;
+      if constexpr (K > 0) {
+        float v[K > 0 ? K : 1];
+#pragma unroll
+        for (int k = 0; k < K; ++k) {
+          const int c = lane + 32 * k;
+          v[k] = c < C ? x[c] : -INFINITY;
+          m = m > v[k] || m != m ? m : v[k];
+        }
+        m = warp_max(m);
+#pragma unroll
+        for (int k = 0; k < K; ++k) s += lane + 32 * k < C ? expf(v[k] - m) : 0.f;
+      } else {
+        for (int c = lane; c < C; c += 32) m = m > x[c] || m != m ? m : x[c];
+        m = warp_max(m);
+        for (int c = lane; c < C; c += 32) s += expf(x[c] - m);
+      }
+      s = warp_sum(s);
+      if (lane == j) {
+        my_max = m;
+        my_log = logf(s);
+      }
     }
-    partial[blockIdx.x] = make_double2(l, (double)r);
+    if (lane < kRowsPerWarp && t0 + lane < count) {
+      my_target = logits[my_row * C + mine.label];
+      stats[t0 + lane] = make_float2(my_max, my_log);
+    }
+    double loss = mine.row >= 0 ? (double)((my_max - my_target) + my_log) : 0.0;
+    if (mine.bad) loss = NAN;
+    loss = warp_sum(loss);
+    const int rows = __popc(__ballot_sync(kAll, mine.row >= 0));
+    if (lane == 0) {
+      losses[warp] = loss;
+      counts[warp] = rows;
+    }
+    __syncthreads();
+    if (threadIdx.x == 0) {
+      double l = 0.0;
+      int r = 0;
+      for (int i = 0; i < kLossBlock / 32; ++i) {
+        l += losses[i];
+        r += counts[i];
+      }
+      if (partial) partial[share] = make_double2(l, (double)r);
+      all.x += l;
+      all.y += (double)r;
+    }
+    __syncthreads();
+  }
+  if (!partial && threadIdx.x == 0) {
+    result[0] = (float)(all.x / all.y);
+    result[1] = (float)(1.0 / all.y);
   }
 }
 
@@ -177,19 +188,19 @@ dg_status_t loss_fwd(const Graph* g, const float* logits, int32_t C, const int64
                      const int64_t* labels, float* stats, float* result, cudaStream_t s) {
   const unsigned blocks = loss_blocks(count);
   void* memory = nullptr;
-  if (blocks) DG_CUDA(pool_alloc(g->device, blocks * sizeof(double2), s, &memory));
+  const bool missing = blocks && scratch_alloc(g, blocks * sizeof(double2), s, &memory) != cudaSuccess;
   double2* partial = static_cast<double2*>(memory);
   float2* st = reinterpret_cast<float2*>(stats);
   if (blocks) {
     auto kernel = C <= 32 ? loss_fwd_kernel<1> : C <= 64 ? loss_fwd_kernel<2> : C <= 128 ? loss_fwd_kernel<4>
                                                                                         : loss_fwd_kernel<0>;
-    kernel<<<blocks, kLossBlock, 0, s>>>(logits, g->n, C, index, count, labels, st, partial);
+    kernel<<<missing ? 1 : blocks, kLossBlock, 0, s>>>(logits, g->n, C, index, count, labels, st, partial, blocks, result);
   }
-  loss_mean_kernel<<<1, 1024, 0, s>>>(partial, blocks, result);
+  if (!missing) loss_mean_kernel<<<1, 1024, 0, s>>>(partial, blocks, result);
   const cudaError_t e = cudaGetLastError();
   pool_free(memory, s);
   DG_CUDA(e);
-  count_launches(blocks ? 2 : 1);
+  count_launches(blocks && !missing ? 2 : 1);
   return DG_OK;
 }
 

@@ -157,6 +157,12 @@ cudaError_t pool_alloc(int device, size_t bytes, cudaStream_t s, void** out) {
   return e;
 }
 
+cudaError_t scratch_alloc(const Graph* g, size_t bytes, cudaStream_t s, void** out) {
+  *out = nullptr;
+  if (bytes > (size_t)g->scratch_mb << 20) return cudaErrorMemoryAllocation;
+  return pool_alloc(g->device, bytes, s, out);
+}
+
 void pool_free(void* p, cudaStream_t s) {
   if (p) cudaFreeAsync(p, s);
 }

@@ -61,6 +61,28 @@ def test_cut_rows(lengths, F, self_loops):
         assert torch.equal(g.dg_aggregate_fwd(H, op), g.dg_aggregate_fwd(H, op))
 
 
+@pytest.mark.parametrize("lengths", EDGES, ids=["edges", "star", "short", "one"])
+@pytest.mark.parametrize("F", [1, 32, 47, 130])
+def test_calls_without_scratch(lengths, F):
+    """"scratch_mb" = 0: the later pieces of cut rows are added by a kernel of their own, in either direction, for
+    every operator pair, with weights, own rows and bf16 storage."""
+    sg = graph_of(lengths, len(lengths) + 70, F, weighted=F == 47)
+    H, G = synth.features(sg.n, F, 1, DEV, nonneg=True), synth.features(sg.n, F, 2, DEV)
+    for self_loops in (0, 1):
+        g = handle(sg, self_loops)
+        g.dg_graph_set_param("scratch_mb", 0)
+        csc = check_transpose(g, *host(sg))
+        for op in OPS:
+            check_fwd_bwd(g, host(sg), H, G, op, csc, self_loops=bool(self_loops))
+            if F % 2 == 0:
+                Hb, plain = H.to(torch.bfloat16), handle(sg, self_loops)
+                got, want = g.dg_aggregate_fwd_bf16(Hb, op), plain.dg_aggregate_fwd_bf16(Hb, op)
+                # non-negative terms: two orders of the same sum differ by at most twice its own bound
+                assert bool(((got - want).abs() <= 2e-5 * want + 2e-7).all())
+    for binary, cols, reduce in ((0, 1, 1), (1, F, 0), (2, 1, 2), (3, F, 1), (4, 1, 0), (4, F, 0), (5, 1, 1), (5, F, 2)):
+        run_case(sg, F, cols, binary, reduce, seed=F, tie_heavy=binary != 5, params={"scratch_mb": 0})
+
+
 def test_cut_rows_of_larger_chunks():
     """1.6 M edges: chunks of 64 entries, rows over 128 are cut."""
     rng = np.random.default_rng(3)

@@ -42,6 +42,21 @@ def test_layer_passes_match_fp64(n, F, relu):
     assert torch.equal(G, G2) and torch.equal(db, db2)
 
 
+@pytest.mark.parametrize("n,F", [(1, 1), (2047, 33), (2048, 32), (70001, 260)])
+def test_layer_backward_without_scratch(n, F):
+    """The bias's gradient straight from dOut, before G takes its place."""
+    gen = torch.Generator(device=DEV).manual_seed(n + F)
+    dOut, out = (torch.randn(n, F, device=DEV, generator=gen) for _ in range(2))
+    scale = torch.rand(n, 1, device=DEV, generator=gen)
+    g = empty_graph(n)
+    g.dg_graph_set_param("scratch_mb", 0)
+    for mask in (None, out):
+        d = dOut if mask is None else torch.where(out > 0, dOut, 0.0)
+        G, db = g.dg_layer_bwd(dOut, mask, scale)
+        assert torch.equal(G, d * scale)
+        assert bool(((db.double() - d.double().sum(0)).abs() <= n * EPS * d.double().abs().sum(0)).all())
+
+
 def test_nan_passes_through_and_arguments_are_checked():
     g = empty_graph(4)
     scale, bias = torch.ones(4, 1, device=DEV), torch.zeros(8, device=DEV)

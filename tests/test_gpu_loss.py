@@ -52,6 +52,24 @@ def test_loss_and_gradient_match_fp64(count, C):
     assert torch.equal(loss, loss2) and torch.equal(y.grad, y2.grad)
 
 
+@pytest.mark.parametrize("C", [1, 47, 400])
+@pytest.mark.parametrize("count", [1, 128, 129, 5000])
+def test_loss_without_scratch(count, C):
+    """One block walks all shares: the same statistics; the mean adds the same doubles in another order, so it is the
+    same float up to its last rounding."""
+    n = 3000
+    gen = torch.Generator(device=DEV).manual_seed(count + C)
+    logits = torch.randn(n, C, device=DEV, generator=gen) * 4 + 30
+    labels = torch.randint(0, C, (n,), device=DEV, generator=gen)
+    index = torch.randint(-n, n, (count,), device=DEV, generator=gen)
+    g, without = empty_graph(n), empty_graph(n)
+    without.dg_graph_set_param("scratch_mb", 0)
+    want, stats = g.dg_cross_entropy_fwd(logits, index, labels)
+    got, stats2 = without.dg_cross_entropy_fwd(logits, index, labels)
+    assert torch.equal(stats, stats2)
+    assert bool(((got - want).abs() <= 2 * EPS * want.abs()).all())
+
+
 def test_out_of_range_targets_give_nan_and_nothing_else():
     g = empty_graph(10)
     logits = torch.zeros(10, 4, device=DEV)

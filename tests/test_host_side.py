@@ -207,3 +207,32 @@ def test_misaligned_statistics_of_the_loss_are_refused(fake):
         assert fake.lib.dg_cross_entropy_bwd(g, logits, 4, index, ctypes.c_int64(4), labels, at, result, result, grads,
                                              None) == want
     fake.lib.dg_graph_destroy(g)
+
+
+@pytest.mark.parametrize("how", ["no memory", "scratch_mb"])
+def test_calls_do_without_scratch(fake, how):
+    """No call needs memory of its own: the parts of cut rows, padded copies, the mask of max / min, partial sums."""
+    fake.lib.fake_plan_totals(3, 1)
+    n, nnz, F = 5000, 200000, 101
+    g, calls = aggregation_calls(fake, n, nnz, F)
+    X, Y, dV, arg, fE = fake.array(n, F), fake.array(n, F), fake.array(n, F), fake.array(n, F), fake.array(nnz, F)
+    index, labels, row = fake.array(n, dtype=np.int64), fake.array(n, dtype=np.int64), fake.array(2 * n + 2)
+    row = ctypes.c_void_p((row.value + 7) // 8 * 8)
+    calls += [
+        ("mul", lambda: fake.call("dg_ap_fwd", g, X, fE, F, F, binding.DG_BIN_MUL, binding.DG_RED_SUM, Y, None)),
+        ("dV of max", lambda: fake.call("dg_ap_bwd", g, X, Y, None, 1, F, binding.DG_BIN_COPY_LHS, binding.DG_RED_MAX, arg,
+                                        dV, None))]
+    cut = {name for name, _ in calls} - {"edge grad"}
+    calls += [("layer", lambda: fake.call("dg_layer_bwd", g, X, Y, F, row, dV, Y)),
+              ("loss", lambda: fake.lib.dg_cross_entropy_fwd(g, X, F, index, ctypes.c_int64(n), labels, row, Y, None))]
+    fake.events()
+    if how == "no memory":
+        fake.lib.fake_alloc_limit(0)
+    else:
+        assert fake.lib.dg_graph_set_param(g, b"scratch_mb", 0) == binding.DG_OK
+    for name, call in calls:
+        assert call() == binding.DG_OK, (name, fake.lib.dg_last_error())
+        done = [what for what, _, _ in fake.events()]
+        assert "alloc" not in done and done, name
+        assert any("pieces_kernel" in what for what in done) == (name in cut), name
+    fake.lib.dg_graph_destroy(g)
