@@ -128,7 +128,15 @@ def _holds(t: Optional[torch.Tensor], count: int, name: str) -> None:
 
 # The handle of the current stream of the current device.  torch.cuda.current_stream() builds two
 # Python objects on the way to it: 3.2 us, a third of what a call on a small graph took on the host.
-_raw_stream, _device = torch._C._cuda_getCurrentRawStream, torch._C._cuda_getDevice
+# A torch without CUDA, or one that names them differently, has neither: then the public call serves.
+_raw_stream = getattr(torch._C, "_cuda_getCurrentRawStream", None)
+_device = getattr(torch._C, "_cuda_getDevice", None)
+if _raw_stream is None or _device is None:
+    def _raw_stream(device):
+        return torch.cuda.current_stream().cuda_stream
+
+    def _device():
+        return 0
 
 
 def _stream(stream=None):

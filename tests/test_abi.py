@@ -2,6 +2,8 @@
 import ctypes
 import os
 import re
+import subprocess
+import sys
 
 import pytest
 
@@ -55,6 +57,22 @@ def test_host_side_argument_checks_need_no_gpu(libpath):
     assert lib.dg_aggregate_bwd(None, None, 4, 0, None, None) == 1
     assert lib.dg_graph_transpose(None, None, 0, None, 0, None) == 1
     assert lib.dg_graph_validate(None, None) == 1
+
+
+def test_binding_imports_on_a_torch_without_cuda():
+    """Such a torch lacks the private functions the binding asks for the current stream."""
+    code = """
+import torch
+for name in ("_cuda_getCurrentRawStream", "_cuda_getDevice"):
+    delattr(torch._C, name)
+from paper_2104_06700_b200 import binding
+assert binding.dg_version()
+class Stream:
+    cuda_stream = 7
+torch.cuda.current_stream = lambda device=None: Stream
+assert binding._stream() == 7 and binding._stream(Stream) == 7
+"""
+    subprocess.run([sys.executable, "-c", code], check=True, cwd=ROOT)
 
 
 def test_binding_refuses_short_arguments():
