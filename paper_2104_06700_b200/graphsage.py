@@ -149,6 +149,22 @@ def aggregate(graph: "binding.Graph", H: torch.Tensor, op: int = binding.DG_OP_S
     return _Aggregate.apply(H, graph, op, bf16, row_scale, edge_w)
 
 
+def _gcn(graph: "binding.Graph", M: torch.Tensor, inv_deg1: torch.Tensor, bf16: bool) -> torch.Tensor:
+    """(sum of the neighbours' rows + own row) / (in-degree + 1), operation by operation."""
+    total = aggregate(graph, M, binding.DG_OP_SUM, bf16)
+    return (total if graph.dg_graph_get_param("self_loops") else total + M) * inv_deg1
+
+
+def _is_plain(lin: torch.nn.Module) -> bool:
+    """Whether calling ``lin`` would compute x W^T + b from its parameters and do nothing else."""
+    hooks = torch.nn.modules.module
+    return (type(lin) is torch.nn.Linear and lin.bias is not None and "forward" not in lin.__dict__
+            and not (lin._forward_hooks or lin._forward_pre_hooks or lin._backward_hooks or lin._backward_pre_hooks
+                     or hooks._global_forward_hooks or hooks._global_forward_pre_hooks
+                     or hooks._global_backward_hooks or hooks._global_backward_pre_hooks)
+            and not torch.is_autocast_enabled())
+
+
 class GraphSAGE(torch.nn.Module):
     """`dims` = [in, hidden, ..., classes]; one Linear per layer.
 
@@ -157,6 +173,10 @@ class GraphSAGE(torch.nn.Module):
     aggregate the narrower matrix.  Same function up to fp32 rounding, less aggregation work
     (602 -> 256 columns on the first Reddit-like layer); off by default because the paper
     aggregates first (its Table 8 counts the aggregation at the layers' input widths).
+
+    A layer runs as one autograd function on its Linear's parameters; where that Linear has hooks, no bias,
+    another type (a parametrization, a module put in its place) or runs under autocast, the module itself is
+    called between the aggregation and the activation.
     """
 
     def __init__(self, graph: "binding.Graph", dims: Sequence[int], project_first: bool = False,
@@ -180,10 +200,20 @@ class GraphSAGE(torch.nn.Module):
         for i, lin in enumerate(self.lin):
             project = self.project_first and lin.out_features < lin.in_features
             relu = i + 1 < len(self.lin)
-            width = lin.out_features if project else lin.in_features
-            H = _GcnLayer.apply(H, lin.weight, lin.bias, self.graph, self.inv_deg1, relu, project,
-                                self.bf16_aggregate and width % 2 == 0)
+            if _is_plain(lin):
+                width = lin.out_features if project else lin.in_features
+                H = _GcnLayer.apply(H, lin.weight, lin.bias, self.graph, self.inv_deg1, relu, project,
+                                    self.bf16_aggregate and width % 2 == 0)
+                continue
+            if project:
+                H = self._aggregated(torch.nn.functional.linear(H, lin.weight)) + lin.bias
+            else:
+                H = lin(self._aggregated(H))
+            H = torch.relu(H) if relu else H
         return H
+
+    def _aggregated(self, M: torch.Tensor) -> torch.Tensor:
+        return _gcn(self.graph, M, self.inv_deg1, self.bf16_aggregate and M.shape[1] % 2 == 0)
 
 
 def make_epoch(model: GraphSAGE, X: torch.Tensor, labels: torch.Tensor, train_idx: torch.Tensor,

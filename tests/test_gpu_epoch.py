@@ -147,3 +147,70 @@ def test_learnable_edge_weights_gradient_and_refresh(op):
             w -= 0.05 * w.grad
             w.grad = None
         g.dg_graph_update_weights()
+
+
+@pytest.mark.parametrize("fused", [False, True])
+def test_layers_call_a_linear_that_is_more_than_its_parameters(fused):
+    """Hooks, parametrizations, a missing bias and modules in a Linear's place take part in forward and backward."""
+    sg = synth.make("tiny", weighted=False)
+    g = make_graph(sg)
+    g.dg_graph_set_param("self_loops", int(fused))
+    g.dg_graph_transpose()
+    X = synth.features(sg.n, 24, 3, DEV)
+    dims = [24, 16, 16, 5]
+    G = synth.features(sg.n, 5, 4, DEV)
+
+    class Doubled(torch.nn.Linear):
+        def forward(self, x):
+            return 2.0 * super().forward(x)
+
+    class Halved(torch.nn.Module):
+        def forward(self, W):
+            return 0.5 * W
+
+    def changed(kind, model):
+        """Changes the middle layer; the weight and bias it has in effect."""
+        lin = model.lin[1]
+        if kind == "hook":
+            lin.register_forward_hook(lambda module, args, out: 2.0 * out)
+            return 2.0 * lin.weight.detach(), 2.0 * lin.bias.detach()
+        if kind == "pre-hook":
+            lin.register_forward_pre_hook(lambda module, args: (2.0 * args[0],))
+            return 2.0 * lin.weight.detach(), lin.bias.detach()
+        if kind == "parametrization":
+            torch.nn.utils.parametrize.register_parametrization(lin, "weight", Halved())
+            return lin.weight.detach(), lin.bias.detach()
+        if kind == "module":
+            model.lin[1] = Doubled(16, 16).to(DEV)
+            return 2.0 * model.lin[1].weight.detach(), 2.0 * model.lin[1].bias.detach()
+        model.lin[1] = torch.nn.Linear(16, 16, bias=False).to(DEV)
+        return model.lin[1].weight.detach(), torch.zeros(16, device=DEV)
+
+    for kind in ("hook", "pre-hook", "parametrization", "module", "no bias"):
+        torch.manual_seed(0)
+        model = graphsage.GraphSAGE(g, dims, fused_aggregator=fused).to(DEV)
+        weights = [l.weight.detach().double() for l in model.lin]
+        biases = [l.bias.detach().double() for l in model.lin]
+        weights[1], biases[1] = (t.double() for t in changed(kind, model))
+        x = X.clone().requires_grad_(True)
+        out = model(x)
+        (out * G).sum().backward()
+        xr = X.double().requires_grad_(True)
+        want = reference_forward(sg, xr, weights, biases)
+        (want * G.double()).sum().backward()
+        for got, ref in ((out.detach(), want.detach()), (x.grad, xr.grad)):
+            assert float((got.double() - ref).abs().max()) <= 1e-4 * float(ref.abs().max()), kind
+
+
+def test_a_layer_under_autocast_gives_what_its_linear_gives():
+    sg = synth.make("tiny", weighted=False)
+    g = make_graph(sg)
+    g.dg_graph_transpose()
+    model = graphsage.GraphSAGE(g, [24, 5]).to(DEV)
+    X = synth.features(sg.n, 24, 3, DEV)
+    with torch.autocast("cuda", torch.bfloat16):
+        out = model(X)
+    assert out.dtype == torch.bfloat16
+    want = reference_forward(sg, X, [model.lin[0].weight], [model.lin[0].bias])
+    # operands and result rounded to bf16: 2^-9 each of the terms, 24 of them
+    assert float((out.double() - want).abs().max()) <= 24 * 3 * 2.0 ** -9 * float(X.abs().max())
