@@ -102,14 +102,20 @@ class _GcnLayer(torch.autograd.Function):
             X = _with_own_row(graph, M, bf16, False)
             Z = X @ weight.t()
         out = graph.dg_layer_fwd(Z, inv_deg1, bias.contiguous(), relu)
-        ctx.graph, ctx.project, ctx.bf16 = graph, project, bf16
-        ctx.save_for_backward(X, weight, inv_deg1, out if relu else None)
+        ctx.graph, ctx.relu, ctx.project, ctx.bf16 = graph, relu, project, bf16
+        # M is the layer's input (another layer's output, which that one keeps) and costs no memory
+        ctx.save_for_backward(X, weight, inv_deg1, out if relu else None, M, bias)
         return out
 
     @staticmethod
     def backward(ctx, dOut: torch.Tensor):
-        X, weight, inv_deg1, out = ctx.saved_tensors
+        X, weight, inv_deg1, out, M, bias = ctx.saved_tensors
         graph, needs = ctx.graph, ctx.needs_input_grad
+        if torch.is_grad_enabled():     # create_graph: the gradients are differentiated in their turn
+            again = _layer_by_operations(M, weight, bias, graph, inv_deg1, ctx.relu, ctx.project, ctx.bf16)
+            inputs = [t for t, need in zip((M, weight, bias), needs) if need]
+            grads = iter(torch.autograd.grad(again, inputs, dOut, create_graph=True))
+            return (*[next(grads) if need else None for need in needs[:3]], None, None, None, None, None)
         G, db = graph.dg_layer_bwd(dOut.contiguous(), out, inv_deg1)
         if ctx.project and (needs[0] or needs[1]):
             G = _with_own_row(graph, G, ctx.bf16, True)
@@ -153,6 +159,15 @@ def _gcn(graph: "binding.Graph", M: torch.Tensor, inv_deg1: torch.Tensor, bf16: 
     """(sum of the neighbours' rows + own row) / (in-degree + 1), operation by operation."""
     total = aggregate(graph, M, binding.DG_OP_SUM, bf16)
     return (total if graph.dg_graph_get_param("self_loops") else total + M) * inv_deg1
+
+
+def _layer_by_operations(M, weight, bias, graph, inv_deg1, relu: bool, project: bool, bf16: bool):
+    """What _GcnLayer computes, from operations that autograd knows."""
+    if project:
+        out = _gcn(graph, M @ weight.t(), inv_deg1, bf16) + bias
+    else:
+        out = torch.nn.functional.linear(_gcn(graph, M, inv_deg1, bf16), weight, bias)
+    return torch.relu(out) if relu else out
 
 
 def _is_plain(lin: torch.nn.Module) -> bool:

@@ -214,3 +214,24 @@ def test_a_layer_under_autocast_gives_what_its_linear_gives():
     want = reference_forward(sg, X, [model.lin[0].weight], [model.lin[0].bias])
     # operands and result rounded to bf16: 2^-9 each of the terms, 24 of them
     assert float((out.double() - want).abs().max()) <= 24 * 3 * 2.0 ** -9 * float(X.abs().max())
+
+
+def test_gradients_of_a_layer_can_be_differentiated():
+    """A gradient penalty on the weights of a one-layer model (its input needs no gradient), against fp64."""
+    sg = synth.make("tiny", weighted=False)
+    g = make_graph(sg)
+    g.dg_graph_transpose()
+    torch.manual_seed(0)
+    model = graphsage.GraphSAGE(g, [24, 5]).to(DEV)
+    X = synth.features(sg.n, 24, 3, DEV)
+    labels = torch.randint(0, 5, (sg.n,), device=DEV)
+
+    def penalty(logits, params):
+        loss = torch.nn.functional.cross_entropy(logits, labels)
+        return sum((d * d).sum() for d in torch.autograd.grad(loss, params, create_graph=True))
+
+    got = torch.autograd.grad(penalty(model(X), list(model.parameters())), list(model.parameters()))
+    W, b = (p.detach().double().requires_grad_(True) for p in model.parameters())
+    want = torch.autograd.grad(penalty(reference_forward(sg, X, [W], [b]), [W, b]), [W, b])
+    for x, y in zip(got, want):
+        assert float((x.double() - y).abs().max()) <= 1e-4 * float(y.abs().max())
