@@ -25,7 +25,7 @@ def reference_forward(sg, X, weights, biases):
     return H
 
 
-@pytest.mark.parametrize("fused", [False, "table", "row_scale"])
+@pytest.mark.parametrize("fused", [False, True])
 @pytest.mark.parametrize("project_first", [False, True])
 @pytest.mark.parametrize("dims", [[64, 32, 7], [20, 16, 16, 5]])
 def test_epoch_loss_and_gradients_match_torch_reference(dims, project_first, fused):
@@ -36,11 +36,7 @@ def test_epoch_loss_and_gradients_match_torch_reference(dims, project_first, fus
     g.dg_graph_transpose()
     torch.manual_seed(0)
     model = graphsage.GraphSAGE(g, dims, project_first=project_first,
-                                fused_aggregator=bool(fused)).to(DEV)
-    if fused == "table":
-        model.scaled_backward = True       # per-edge factors of the transpose
-    elif fused == "row_scale":
-        model.scaled_backward = False      # dOut scaled row by row, then the sum backward
+                                fused_aggregator=fused).to(DEV)
     X = synth.features(sg.n, dims[0], 3, DEV)
     labels = torch.randint(0, dims[-1], (sg.n,), device=DEV)
     train_idx = torch.arange(0, sg.n, 3, device=DEV)
@@ -235,3 +231,26 @@ def test_gradients_of_a_layer_can_be_differentiated():
     want = torch.autograd.grad(penalty(reference_forward(sg, X, [W], [b]), [W, b]), [W, b])
     for x, y in zip(got, want):
         assert float((x.double() - y).abs().max()) <= 1e-4 * float(y.abs().max())
+
+
+@pytest.mark.parametrize("bf16", [False, True])
+def test_both_backward_forms_of_the_mean_with_own_rows(bf16):
+    """aggregate(..., DG_OP_MEAN) on a handle with self loops: per-edge factors of the transposition, or dOut scaled row
+    by row and the sum's backward pass (row_scale)."""
+    sg = synth.make("tiny", weighted=False)
+    g = make_graph(sg)
+    g.dg_graph_set_param("self_loops", 1)
+    g.dg_graph_transpose()
+    X, G = synth.features(sg.n, 24, 3, DEV), synth.features(sg.n, 24, 4, DEV)
+    inv = 1.0 / ((sg.rowptr[1:] - sg.rowptr[:-1]).to(DEV).float() + 1.0).unsqueeze(1)
+    eye, zero = torch.eye(24, device=DEV), torch.zeros(24, device=DEV)
+    xr = X.double().requires_grad_(True)
+    want = reference_forward(sg, xr, [eye], [zero])
+    (want * G.double()).sum().backward()
+    tol = 2.0 ** -8 if bf16 else 1e-5
+    for scale in (None, inv):
+        x = X.clone().requires_grad_(True)
+        out = graphsage.aggregate(g, x, binding.DG_OP_MEAN, bf16, row_scale=scale)
+        (out * G).sum().backward()
+        for a, b in ((out.detach(), want.detach()), (x.grad, xr.grad)):
+            assert float((a.double() - b).abs().max()) <= tol * float(b.abs().max())
