@@ -27,6 +27,8 @@ __device__ float message_of(int bin, float x, float y) {
   }
 }
 
+constexpr int kGroup = 32;  // pieces that are added before they go to the total
+
 __global__ void __launch_bounds__(32) pieces_kernel(const PieceArgs a) {
   const int f = blockIdx.y * 32 + threadIdx.x;
   if (f >= a.F) return;
@@ -34,7 +36,7 @@ __global__ void __launch_bounds__(32) pieces_kernel(const PieceArgs a) {
   for (int i = blockIdx.x; i < cut_rows; i += gridDim.x) {
     const CutRow cut = a.cuts[i];
     const int64_t o = (int64_t)cut.row * a.F + f;
-    float total = 0.f;
+    float total = 0.f, group = 0.f;
     float best = a.red == kSum ? 0.f : a.out[o];
     int32_t at = a.red != kSum && a.arg_out ? a.arg_out[o] : 0;
     for (int c = cut.first; c < cut.first + cut.count; ++c) {
@@ -63,8 +65,13 @@ __global__ void __launch_bounds__(32) pieces_kernel(const PieceArgs a) {
           }
         }
       }
-      total += acc;
+      group += acc;
+      if ((c - cut.first) % kGroup == kGroup - 1) {
+        total += group;
+        group = 0.f;
+      }
     }
+    total += group;
     if (a.red != kSum && !a.gradient) {
       a.out[o] = best;
       if (a.arg_out) a.arg_out[o] = at;

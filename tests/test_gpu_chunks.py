@@ -83,6 +83,31 @@ def test_calls_without_scratch(lengths, F):
         run_case(sg, F, cols, binary, reduce, seed=F, tie_heavy=binary != 5, params={"scratch_mb": 0})
 
 
+def check_hub_of_equal_terms(params, F=64):
+    """A row of 4 M equal terms, whose partial sums round the same way: one chain over its 40 thousand pieces is off by
+    4e-5 of the sum.  The chains there are: 48 additions of a lane group, the groups, 32 slots, 170 totals of a warp, 8
+    warps; fewer than 265, each off by at most 2^-24 of the sum."""
+    n, hub = 1000, 4000000
+    rowptr = torch.arange(n + 1, device=DEV)
+    rowptr[8:] += hub - 1
+    nnz = int(rowptr[-1])
+    colidx = torch.arange(nnz, device=DEV).remainder(n).int()
+    g = binding.dg_graph_create(n, nnz, rowptr, colidx, None)
+    for name, value in params.items():
+        g.dg_graph_set_param(name, value)
+    for x in (0.1, 0.3, 0.9):
+        H = torch.full((n, F), x, device=DEV)
+        want = float(H[0, 0].double()) * hub
+        for got in (g.dg_aggregate_fwd(H, binding.DG_OP_SUM),
+                    g.dg_ap_fwd(H, torch.zeros(nnz, 1, device=DEV), binding.DG_BIN_ADD, binding.DG_RED_SUM)[0]):
+            assert float((got[7].double() - want).abs().max()) <= 265 * 2.0 ** -24 * want
+
+
+@pytest.mark.parametrize("params", [{}, {"scratch_mb": 0}], ids=["slots", "pieces"])
+def test_pieces_of_a_hub_are_not_one_chain(params):
+    check_hub_of_equal_terms(params)
+
+
 def test_cut_rows_of_larger_chunks():
     """1.6 M edges: chunks of 64 entries, rows over 128 are cut."""
     rng = np.random.default_rng(3)
