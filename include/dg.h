@@ -380,8 +380,8 @@ dg_status_t dg_aggregate_edge_grad(dg_graph_t g, const float* H, const float* dO
 
 /*
  * Tuning knobs (defaults come from the device's L2 size and SM count):
- *   "heavy_threshold"  rows longer than this may be cut into pieces for several warps (default:
- *                      twice the piece size chosen from the number of edges, 64 to 2048)
+ *   "heavy_threshold"  rows longer than this, and rows over 4096 entries, may be cut into pieces for several
+ *                      warps (default: twice the piece size chosen from the number of edges, 64 to 2048)
  *   "heavy_blocks_per_sm"  accepted in [0, 32]; no effect
  *   "slice_features"   features per pass over the graph (0 = choose from the L2 size; a value
  *                      that would need more than 65535 passes is widened)

@@ -108,6 +108,10 @@ def test_pieces_of_a_hub_are_not_one_chain(params):
     check_hub_of_equal_terms(params)
 
 
+def test_a_hub_is_cut_whatever_the_threshold():
+    check_hub_of_equal_terms({"heavy_threshold": 1 << 30})
+
+
 def test_cut_rows_of_larger_chunks():
     """1.6 M edges: chunks of 64 entries, rows over 128 are cut."""
     rng = np.random.default_rng(3)
