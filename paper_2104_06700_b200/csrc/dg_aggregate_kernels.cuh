@@ -486,6 +486,9 @@ __device__ __forceinline__ void ap_body(const ApArgs& a, const SelfArgs sa) {
 // of a lane's eight loads are in flight (forward + backward, kernels: 40 k edges, F = 256: 29.1 -> 21.3 us; 184 k,
 // F = 256, bf16: 27.2 -> 24.7; 619 k, F = 100: 42.7 -> 39.1 of two waves or more; but 125 k, F = 48, bf16:
 // 17.9 -> 20.6).  At eight waves the two are equal.
+// Three with four vectors per lane (only "slice_features" asks for such slices): the sums alone take up to 32 registers,
+// and 40 spill up to 0.7 KB (F = 602 in slices of 1024, bf16: 7.9 M edges 2507 us, so 881; 1.1 M 443 / 192; in slices of
+// 512, fp32: 1368 / 1182).
 template <typename E, int VEC, int G, int CPL, bool SCALED, bool SEG, int BLOCKS>
 __global__ void __launch_bounds__(kBlock, BLOCKS) ap_kernel(const ApArgs a) {
   cudaGridDependencySynchronize();            // the padded copy
@@ -505,15 +508,16 @@ template <typename E, int VEC, int G, int CPL, bool SCALED, bool SELF>
 dg_status_t launch_variant(const ApArgs& a, const SelfArgs& sa, int slices, cudaStream_t s) {
   const dim3 grid((unsigned)((a.chunk_count + kWarpsPerBlock - 1) / kWarpsPerBlock), (unsigned)slices);
   const bool overlap = a.overlap;
+  constexpr int kMany = CPL == 4 ? 3 : 6, kFew = CPL == 4 ? 3 : 4;
   if constexpr (SELF) {
-    auto kernel = a.seg_lo ? ap_kernel_self<E, VEC, G, CPL, SCALED, true, 6>
-                  : a.few_blocks ? ap_kernel_self<E, VEC, G, CPL, SCALED, false, 4>
-                                 : ap_kernel_self<E, VEC, G, CPL, SCALED, false, 6>;
+    auto kernel = a.seg_lo ? ap_kernel_self<E, VEC, G, CPL, SCALED, true, kMany>
+                  : a.few_blocks ? ap_kernel_self<E, VEC, G, CPL, SCALED, false, kFew>
+                                 : ap_kernel_self<E, VEC, G, CPL, SCALED, false, kMany>;
     DG_CUDA(launch_kernel(kernel, grid, kBlock, s, overlap, a, sa));
   } else {
-    auto kernel = a.seg_lo ? ap_kernel<E, VEC, G, CPL, SCALED, true, 6>
-                  : a.few_blocks ? ap_kernel<E, VEC, G, CPL, SCALED, false, 4>
-                                 : ap_kernel<E, VEC, G, CPL, SCALED, false, 6>;
+    auto kernel = a.seg_lo ? ap_kernel<E, VEC, G, CPL, SCALED, true, kMany>
+                  : a.few_blocks ? ap_kernel<E, VEC, G, CPL, SCALED, false, kFew>
+                                 : ap_kernel<E, VEC, G, CPL, SCALED, false, kMany>;
     DG_CUDA(launch_kernel(kernel, grid, kBlock, s, overlap, a));
   }
   count_launches(1);
