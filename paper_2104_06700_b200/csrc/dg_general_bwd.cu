@@ -45,7 +45,10 @@ __global__ void __launch_bounds__(kGenBlock, 4) general_dv_sum_kernel(const GenA
       const int e = e0 + j * NG + grp;
       const bool valid = kFullStep || e < cnt;
 #pragma unroll
-      for (int q = 0; q < VEC; ++q) x[j][q] = y[j][q] = 0.f;
+      for (int q = 0; q < VEC; ++q) {
+        x[j][q] = 0.f;
+        y[j][q] = BIN == kDiv ? 1.f : 0.f;  // absent edges: a division by zero takes a slow path
+      }
       const int32_t id = __shfl_sync(kAll, v, e & 31);
       if (valid) load_vec<VEC>(x[j], xlane + (int64_t)id * a.ldx);
       if (YM == kEdgeFull) {
@@ -313,10 +316,9 @@ __global__ void __launch_bounds__(kGenBlock, 4) general_dv_extremum_kernel(const
 
 // dE with full edge features: one value per (edge, feature).  The written rows, nnz * F floats in CSR
 // order, are the traffic: streaming stores leave L2 to the gathered rows.
-template <int BIN, int RED, int VEC>
+template <int BIN, int RED, int VEC, int U>
 __global__ void __launch_bounds__(kGenBlock) general_de_full_kernel(const GenArgs a) {
   constexpr bool kNeedsX = BIN == kMul || BIN == kDiv;
-  constexpr int U = 4;
   const int lane = threadIdx.x & 31;
   const int G = 1 << a.log_g, NG = 32 >> a.log_g;
   const int grp = lane >> a.log_g, c = lane & (G - 1);
@@ -338,7 +340,10 @@ __global__ void __launch_bounds__(kGenBlock) general_de_full_kernel(const GenArg
           for (int j = 0; j < U; ++j) {
             const int e = e0 + j * NG + grp;
 #pragma unroll
-            for (int q = 0; q < VEC; ++q) x[j][q] = y[j][q] = 0.f;
+            for (int q = 0; q < VEC; ++q) {
+              x[j][q] = 0.f;
+              y[j][q] = BIN == kDiv ? 1.f : 0.f;  // absent edges: a division by zero takes a slow path
+            }
             if (kNeedsX) {
               const int32_t id = __shfl_sync(kAll, u, e & 31);
               if (e < cnt) load_vec<VEC>(x[j], a.V + (int64_t)id * a.F + fl);
@@ -410,7 +415,8 @@ template <int BIN, int YM, int VEC>
 dg_status_t launch_dv_sum(const GenArgs& a, cudaStream_t s) {
   const dim3 grid = general_grid(a, VEC);
   if (a.log_g >= 3) general_dv_sum_kernel<BIN, YM, VEC, 4><<<grid, kGenBlock, 0, s>>>(a);
-  else general_dv_sum_kernel<BIN, YM, VEC, 2><<<grid, kGenBlock, 0, s>>>(a);
+  else if (a.log_g >= 1) general_dv_sum_kernel<BIN, YM, VEC, 2><<<grid, kGenBlock, 0, s>>>(a);
+  else general_dv_sum_kernel<BIN, YM, VEC, 1><<<grid, kGenBlock, 0, s>>>(a);  // a batch is one step
   return launched();
 }
 
@@ -458,11 +464,21 @@ dg_status_t dv_by_reducer(const GenArgs& a, int red, cudaStream_t s) {
   }
 }
 
+// A batch has 32 edges, which narrow groups cover in fewer steps: what is left over would only divide (gradients of
+// div / sum with full edge features, F = 4: 7.9 M edges 452 us with four steps and zero divisors, 199 so).
+template <int BIN, int RED, int VEC>
+void launch_de_full(const GenArgs& a, cudaStream_t s) {
+  const dim3 grid = general_grid(a, VEC);
+  if (a.log_g >= 2) general_de_full_kernel<BIN, RED, VEC, 4><<<grid, kGenBlock, 0, s>>>(a);
+  else if (a.log_g == 1) general_de_full_kernel<BIN, RED, VEC, 2><<<grid, kGenBlock, 0, s>>>(a);
+  else general_de_full_kernel<BIN, RED, VEC, 1><<<grid, kGenBlock, 0, s>>>(a);
+}
+
 template <int BIN, int RED>
 dg_status_t launch_de(const GenArgs& a, cudaStream_t s) {
   if (a.cols == 1) general_de_scalar_kernel<BIN, RED><<<chunk_blocks(a), kGenBlock, 0, s>>>(a);
-  else if (a.vec == 4) general_de_full_kernel<BIN, RED, 4><<<general_grid(a, 4), kGenBlock, 0, s>>>(a);
-  else general_de_full_kernel<BIN, RED, 1><<<general_grid(a, 1), kGenBlock, 0, s>>>(a);
+  else if (a.vec == 4) launch_de_full<BIN, RED, 4>(a, s);
+  else launch_de_full<BIN, RED, 1>(a, s);
   return launched();
 }
 
