@@ -24,9 +24,6 @@
 #define DG_AGGREGATE_KERNELS_CUH_
 #include "dg_internal.cuh"
 
-#ifndef DG_UM
-#define DG_UM 1
-#endif
 namespace dg {
 namespace {
 
@@ -72,14 +69,6 @@ __device__ __forceinline__ uint4 ldg_vec(const char* p, uint4) {
 // a 32-bit word holds two bf16 values: the low half is the element with the lower index
 __device__ __forceinline__ float bf_lo(uint32_t x) { return __uint_as_float(x << 16); }
 __device__ __forceinline__ float bf_hi(uint32_t x) { return __uint_as_float(x & 0xffff0000u); }
-// element i of a matrix stored as E
-template <typename E> __device__ __forceinline__ float ld_elem(const void* X, size_t i);
-template <> __device__ __forceinline__ float ld_elem<F32>(const void* X, size_t i) {
-  return __ldg(reinterpret_cast<const float*>(X) + i);
-}
-template <> __device__ __forceinline__ float ld_elem<BF16>(const void* X, size_t i) {
-  return __uint_as_float((uint32_t)__ldg(reinterpret_cast<const uint16_t*>(X) + i) << 16);
-}
 // 1 / (in-degree + 1) of vertex r, from the CSR row pointer
 __device__ __forceinline__ float self_factor(const int64_t* self_ptr, int64_t r) {
   return 1.0f / (float)(__ldg(self_ptr + r + 1) - __ldg(self_ptr + r) + 1);
@@ -485,7 +474,8 @@ __device__ __forceinline__ void ap_body(const ApArgs& a, const SelfArgs sa) {
 // registers) on grids of up to four waves of those: latency is the limit there, and with 40 registers not all
 // of a lane's eight loads are in flight (forward + backward, kernels: 40 k edges, F = 256: 29.1 -> 21.3 us; 184 k,
 // F = 256, bf16: 27.2 -> 24.7; 619 k, F = 100: 42.7 -> 39.1 of two waves or more; but 125 k, F = 48, bf16:
-// 17.9 -> 20.6).  At eight waves the two are equal.
+// 17.9 -> 20.6: a loss accepted for a rule on the grid alone; a bound below it, of one wave, would have given up the
+// 619 k case).  At eight waves the two are equal.
 // Three with four vectors per lane (only "slice_features" asks for such slices): the sums alone take up to 32 registers,
 // and 40 spill up to 0.7 KB (F = 602 in slices of 1024, bf16: 7.9 M edges 2507 us, so 881; 1.1 M 443 / 192; in slices of
 // 512, fp32: 1368 / 1182).

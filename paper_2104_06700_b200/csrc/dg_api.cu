@@ -66,7 +66,9 @@ static void free_owned(Graph* g) {
 // Rows up to twice a chunk stay whole: four times costs 2 to 15 % on the same graphs.  With the smallest
 // chunks rows up to kFewEdgesRow entries do: such a call is short against its launches, and the join of
 // cut rows is one more launch with scratch of its own, 4.5 us of host time and 3.5 us on the device (125 k
-// edges, rows up to 157, forward + backward: 31.4 us cut at 64, 20.5 whole).
+// edges, rows up to 157, forward + backward: 31.4 us cut at 64, 20.5 whole).  A compromise over graphs of 57 to 344 k
+// edges: rows of 20 to 300, F = 4 20.5 us at 160, 13.8 at 512; rows to 700, F = 16 27.6 / 21.0, F = 256 65.9 / 73.9;
+// power-law rows, F = 64 24.7 / 36.9; 300 rows of 100 to 1500, F = 64 26.9 / 32.4.
 // Rows over kLongestWhole entries are cut whatever the caller's threshold: a whole row is one warp's chain of fp32
 // additions (4 M entries, message add: relative error 1.4e-3 whole, 1.9e-7 in pieces; 2 M entries, F = 128: 197 and 1.3 ms).
 constexpr int64_t kMaxChunk = 1024, kMinChunk = 32, kChunksPerSm = 320, kRowCost = 8;

@@ -89,7 +89,6 @@ struct dg_graph {
   // set on a handle made by dg_graph_reorder: arrays inside the caller's reorder storage
   const int32_t* new_of_old = nullptr;   // n: new id of every old vertex
   const int32_t* reorder_pos = nullptr;  // nnz: old CSR position of every new position
-  bool degree_ordered = false;           // made by dg_graph_reorder with a hub-first order
 
   int device = 0;
   int sm_count = 148;
@@ -244,7 +243,7 @@ void transpose_sizes(int64_t n, int64_t nnz, bool weighted, size_t* csc_bytes,
                      size_t* scratch_bytes);
 dg_status_t transpose_run(Graph* g, void* csc, void* scratch, cudaStream_t s);
 dg_status_t refresh_csc_weights(Graph* g, cudaStream_t s);
-// dg_api.cu: what follows every transposition (heavy columns, the long-column count on its way)
+// dg_api.cu: what follows every transposition (the columns' plan, its totals on their way to the host)
 dg_status_t finish_transpose(Graph* g, cudaStream_t s);
 // the stable radix sort behind it, for other pre-processing steps (see dg_transpose.cu)
 struct SortPlan { int digit_bits; int passes; };
