@@ -16,11 +16,12 @@ training, where the graph is static over epochs); they are timed separately and 
 Beside the device-resident step the line carries: the roofline object of the slower of the two
 calls (compulsory bytes, DRAM traffic from the ncu captures, gather ceilings measured in the
 same run), the same step end to end from pinned host memory ("e2e"), the CPU oracle on a row
-sample ("cpu_baseline"), the time of one full-batch GraphSAGE epoch ("epoch"), and, in the
+sample ("cpu_baseline") and the time of one full-batch GraphSAGE epoch ("epoch_ms").  A second
+JSON object on stderr has the epoch's details and, in the
 default run on one GPU, "workloads": one record per workload shape of the paper's Table 2 at
 full size (the tiny graph, Reddit-like at both layer widths, Products-like, Proteins-like at
 three widths, Papers-like), each with forward and backward times, compulsory bytes, roofline
-fractions, its own clock record and a sampled CPU-oracle time.
+fractions, its own clock record and a sampled CPU-oracle time, "other_calls" and so on.
 
 N > 1 (under torchrun): the path has no exchange step and is not sharded, so every rank runs
 an independent replica of the same workload; the value is the units all ranks processed over
@@ -579,8 +580,8 @@ def extra_records(torch, binding, synth, name, g, sg, F, n_ref, peak, flush):
             ms = time_one(torch, bwd, 10, fl)
             out.append(rec("dg_ap_bwd (copylhs, max): dV", ms,
                            idx_bytes + sg.nnz * 4 + 3 * sg.n * F * 4,
-                           "gather over the CSC with an equality test on arg (dO and arg rows per "
-                           "edge), no atomics"))
+                           "mask of the selected edges over the CSR, then the selected dO over the "
+                           "CSC (arg compared per edge where the mask does not pay); no atomics"))
             del dV
     del arg
     if sg.nnz * F * 4 <= 24e9:
@@ -931,9 +932,7 @@ def main():
         traffic = None if t is None else t / per_call
     roofline = {
         "bound": "hbm",
-        "kernel": ("ap_kernel_r40" if ((weighted or (dom == "bwd" and op == "mean")) and F >= 64)
-                   or F <= 16 else "ap_kernel")
-                  + f" ({dom}: {per_call} launch(es) per dg_aggregate_{dom} call)",
+        "kernel": f"ap_kernel ({dom}: {per_call} launch(es) per dg_aggregate_{dom} call)",
         "achieved": achieved, "peak": peak, "unit": "GB/s", "frac": achieved / peak,
         "peak_kind": f"of {peak_kind}", "frac_of_nominal_8TBs": achieved / NOMINAL_HBM_GBS,
         "launches_per_call": per_call,
@@ -1157,13 +1156,14 @@ def main():
             "dtype": "f32" if not bf16 else "f32 sums over bf16-stored inputs", "data": "synthetic",
             "config": workload_config(args, sg, F, op, weighted, world, two_buffers),
             "roofline": roofline, "cpu_baseline": cpu, "e2e": e2e, "gpu_launches": launches,
-            "clocks": clocks, "epoch": epoch_info,
+            "clocks": clocks, "epoch_ms": epoch_info["ms_per_epoch"] if epoch_info else None,
             "ingest": {"graph_create_ms": create_ms, "transpose_ms": transpose_ms,
                        "transpose_edges_per_s": sg.nnz / (transpose_ms * 1e-3) if transpose_ms else None,
                        "reorder_ms": reorder_ms},
-            "workloads": workloads, "workloads_ingest": workloads_ingest,
-            "workloads_epoch": workloads_epoch, "other_calls": workloads_extras,
-        }))
+        }), flush=True)
+        # everything beside the headline, on stderr: a reader of the line need not take 20 KB with it
+        print(json.dumps({"epoch": epoch_info, "workloads": workloads, "workloads_ingest": workloads_ingest,
+                          "workloads_epoch": workloads_epoch, "other_calls": workloads_extras}), file=sys.stderr)
     if world > 1:
         dist.destroy_process_group()
 
