@@ -88,6 +88,22 @@ dg_status_t widen(const dg_graph* g, GenArgs* a, cudaStream_t s, void** copy) {
 // dV of max / min.  The mask of the selected edges (see dg_general_bwd.cu) is made and used for up to 256
 // features at a time, as many as fit kMaskMaxBytes: one 32-byte sector per edge holds 256 bits.
 constexpr size_t kMaskMaxBytes = (size_t)2 << 30;  // the pool keeps this much
+
+// Whether dV of max / min goes through the mask, or compares arg edge by edge.  The mask saves gathered rows but costs a
+// launch, scratch and a pass over the rows, so calls on fewer than kMaskMinEdges compare, unless
+// rows are short (124 k edges in rows of 4, F = 4: 18.5 / 20.6 us); and for 9 to 16 features its kernel has 16 lanes per
+// edge where the comparison has four.  The factors of mul / div make the comparison dearer.
+// Measured, us with / without the mask, copylhs: 57 k edges F = 16 18.5 / 9.5, F = 128 24.7 / 20.7; 158 k F = 64 20.6 /
+// 13.0, F = 602 92 / 86; 573 k F = 8 23.5 / 22.6, F = 32 36 / 27, F = 100 55 / 59; F = 16 at mean degree 4 309 / 458, 14.5
+// 732 / 714, 50 148 / 122, 110 125 / 92, 270 576 / 406.  mul with one column: 57 k F = 16 18.5 / 12.3, F = 64 22.6 / 26.7;
+// F = 16 at mean degree 14.5 908 / 1098, 50 962 / 1048, 84 49 / 38, 270 726 / 648.
+constexpr int64_t kMaskMinEdges = 1 << 17;
+bool mask_pays(const dg_graph* g, int32_t F, int32_t cols, int bin) {
+  const bool factors = bin == kMul || bin == kDiv;
+  if (factors && cols != 1) return true;
+  if (g->nnz < kMaskMinEdges) return g->nnz < 8 * g->n || (factors && F > 32);
+  return F <= 8 || F > 16 || g->nnz < (factors ? 64 : 24) * g->n;
+}
 dg_status_t extremum_dv(const dg_graph* g, GenArgs a, int bin, int red, cudaStream_t s) {
   const int blocks = g->split_csc && g->source_blocks > 1 ? (int)g->source_blocks : 1;
   int words = 1;
@@ -95,7 +111,7 @@ dg_status_t extremum_dv(const dg_graph* g, GenArgs a, int bin, int red, cudaStre
   while (words > 1 && (size_t)g->nnz * (size_t)words * 4 > kMaskMaxBytes) words /= 2;
   void* mask = nullptr;
   auto dv = [&](const GenArgs& p) { return launch_general_dv(p, bin, red, s); };
-  if (g->nnz == 0 || (size_t)g->nnz * (size_t)words * 4 > kMaskMaxBytes ||
+  if (g->nnz == 0 || !mask_pays(g, a.F, a.cols, bin) || (size_t)g->nnz * (size_t)words * 4 > kMaskMaxBytes ||
       scratch_alloc(g, (size_t)g->nnz * (size_t)words * 4, s, &mask) != cudaSuccess) {
     a.vec = vector_width(a.F, (uintptr_t)a.arg) == 4 ? 4 : 1;  // of arg; a lane has four features
     a.log_g = log_group((a.F + 3) / 4);

@@ -260,7 +260,7 @@ __global__ void __launch_bounds__(kGenBlock, 6) general_dv_mask_narrow_kernel(co
       [&](int r, int slot) { store_sum<1>(a, acc, r, slot, c, 1, G, grp); });
 }
 
-// The same without a mask (no memory for it): arg itself is compared, four features per lane.
+// The same without a mask (see mask_pays, or no memory for it): arg itself is compared, four features per lane.
 template <int BIN, int YM, int VEC>
 __global__ void __launch_bounds__(kGenBlock, 4) general_dv_extremum_kernel(const GenArgs a) {
   constexpr int U = 4;

@@ -1,6 +1,8 @@
 """Where the rows are shared out in chunks, long rows are cut, matrices are copied into padded rows, and
 the gradient of max / min goes through a bit mask: the sizes at which each of these changes its path,
 against the CPU oracle element by element, with the bounds of the other parity tests."""
+import threading
+
 import numpy as np
 import pytest
 import torch
@@ -163,6 +165,16 @@ def test_extremum_gradient_mask(F):
                  tie_heavy=binary != 5)
 
 
+@pytest.mark.parametrize("F", [1, 8, 9, 16, 17, 33, 129, 300])
+@pytest.mark.parametrize("degree", [9, 30, 70])
+def test_extremum_gradient_on_both_sides_of_its_rule(F, degree):
+    """The mask from 2^17 edges on, except for 9 to 16 features on longer rows; fewer edges compare arg (above)."""
+    sg = graph_of([5, 0, 33, 300, 1025, 2600, 0, 64] + [degree] * (270000 // degree), 270000 // degree + 20, F)
+    assert sg.nnz >= 1 << 17
+    for binary, cols in ((0, 1), (4, 1)):
+        run_case(sg, F, cols, binary, binding.DG_RED_MAX if F % 2 else binding.DG_RED_MIN, seed=F, tie_heavy=True)
+
+
 @pytest.mark.parametrize("nnz", [1, 3, 4, 5, 7, 8, 9, 4095, 4096, 4097, 12289])
 def test_csc_and_weight_refresh_remainders(nnz):
     """Four edges a thread in the refresh of the weights, eight in the column pointers, tiles of 4096."""
@@ -261,9 +273,8 @@ def test_positions_up_to_the_last(F):
     torch.cuda.empty_cache()
 
 
-def test_calls_on_two_streams_and_destroyed_handles():
-    """Scratch comes from a pool shared by handles, streams and threads; a destroyed handle's memory is not
-    reused while its kernels are queued."""
+def test_calls_on_two_streams():
+    """Scratch comes from a pool shared by handles and streams; each call's is its own."""
     sg = graph_of(EDGES[0] * 40, 1000, 7)
     G = synth.features(sg.n, 47, 3, DEV)
     g = handle(sg)
@@ -275,10 +286,48 @@ def test_calls_on_two_streams_and_destroyed_handles():
     for i in range(20):
         with torch.cuda.stream(streams[i % 2]):
             got.append(g.dg_aggregate_bwd(G, binding.DG_OP_MEAN))
-        if i % 5 == 4:
-            h = handle(sg)
-            h.dg_graph_transpose()
-            got.append(h.dg_aggregate_bwd(G, binding.DG_OP_MEAN))
-            del h
     torch.cuda.synchronize()
     assert all(torch.equal(x, want) for x in got)
+
+
+def test_a_destroyed_handle_keeps_its_memory_until_its_kernels_are_done():
+    """The short-lived handle works on a non-blocking stream behind a long queue and is destroyed at once; the plans of
+    handles made meanwhile by other threads would take its place."""
+    sg = graph_of(EDGES[0] * 40, 1000, 7)
+    other = graph_of([200] * 150, 1000, 8)
+    G = synth.features(sg.n, 47, 3, DEV)
+    keep = handle(sg)
+    keep.dg_graph_transpose()
+    want = keep.dg_aggregate_bwd(G, binding.DG_OP_MEAN)
+    torch.cuda.synchronize()
+    busy = torch.randn(4096, 4096, device=DEV)
+    side = torch.cuda.Stream()
+    failed = []
+
+    def make_handles():
+        try:
+            with torch.cuda.stream(torch.cuda.Stream()):
+                for _ in range(15):
+                    g = handle(other)
+                    g.dg_graph_transpose()
+                    g.dg_aggregate_bwd(G, binding.DG_OP_SUM)
+        except Exception as e:  # an assertion in a thread is not the test's
+            failed.append(e)
+
+    threads = [threading.Thread(target=make_handles) for _ in range(2)]
+    for t in threads:
+        t.start()
+    got = []
+    for _ in range(10):
+        h = handle(sg)
+        side.wait_stream(torch.cuda.current_stream())
+        with torch.cuda.stream(side):
+            h.dg_graph_transpose()
+            for _ in range(10):
+                busy = busy @ busy * 1e-3
+            got.append(h.dg_aggregate_bwd(G, binding.DG_OP_MEAN))
+        h.dg_graph_destroy()
+    for t in threads:
+        t.join()
+    torch.cuda.synchronize()
+    assert not failed and all(torch.equal(x, want) for x in got)
