@@ -10,9 +10,12 @@ namespace {
 // Adds the slots of every cut row to what the row's first chunk stored.  A block takes one row and 128
 // features; its 8 warps take every eighth slot, and their sums are added in warp order.  The traffic is
 // one row of F floats per chunk of up to 1024 gathered rows; the launch itself is most of the cost.
-// A warp adds kJoinChain slots before it adds to its total: a small graph's chunks are short, and a hub has tens of
-// thousands of them (4 M entries of a row, chunks of 96: relative error 1.0e-6 in one chain, 1.9e-7 so).
-constexpr int kJoinChain = 32;
+// HUB: a warp adds kJoinChain slots before it adds to its total.  A small graph's chunks are short, and a hub has tens of
+// thousands of them (4 M entries of a row, chunks of 96: relative error 1.0e-6 in one chain, 1.9e-7 so).  Compiled apart,
+// for plans with rows of over kJoinShare slots: the loops around the loop cost every short row half a microsecond (65 k
+// edges, F = 64, forward + backward 19.6 -> 20.5 us; 1.2 M, F = 47 75.6 -> 77.3).
+constexpr int kJoinChain = 32, kJoinShare = kJoinChain * kWarpsPerBlock;
+template <bool HUB>
 __global__ void __launch_bounds__(kBlock)
 join_kernel(const Chunk* __restrict__ chunks, const CutRow* __restrict__ cuts,
             const int32_t* __restrict__ totals, int32_t max_cuts, const float* __restrict__ partial, int32_t F,
@@ -25,9 +28,9 @@ join_kernel(const Chunk* __restrict__ chunks, const CutRow* __restrict__ cuts,
   for (int i = blockIdx.x; i < cut_rows; i += gridDim.x) {
     const CutRow cut = cuts[i];
     float total[4] = {0.f, 0.f, 0.f, 0.f};
-    for (int k0 = warp; k0 < cut.count; k0 += kWarpsPerBlock * kJoinChain) {
+    for (int k0 = warp; k0 < cut.count; k0 += kJoinShare) {
       float sum[4] = {0.f, 0.f, 0.f, 0.f};
-      const int k1 = min(cut.count, k0 + kWarpsPerBlock * kJoinChain);
+      const int k1 = HUB ? min(cut.count, k0 + kJoinShare) : cut.count;
       for (int k = k0; k < k1; k += kWarpsPerBlock) {
         const float* p = partial + (size_t)__ldg(&chunks[cut.first + k].slot) * (size_t)F;
 #pragma unroll
@@ -38,6 +41,7 @@ join_kernel(const Chunk* __restrict__ chunks, const CutRow* __restrict__ cuts,
       }
 #pragma unroll
       for (int j = 0; j < 4; ++j) total[j] += sum[j];
+      if (!HUB) break;
     }
 #pragma unroll
     for (int j = 0; j < 4; ++j) part[warp][32 * j + lane] = total[j];
@@ -101,7 +105,8 @@ dg_status_t join_cut_rows(const Graph* g, const Plan& plan, const float* partial
   int64_t blocks = plan.cut_rows >= 0 ? plan.cut_rows : plan.max_cuts;
   if (blocks > (int64_t)g->sm_count * 64) blocks = (int64_t)g->sm_count * 64;
   const dim3 grid((unsigned)blocks, (unsigned)((F + 127) / 128));
-  DG_CUDA(launch_kernel(join_kernel, grid, kBlock, s, true, (const Chunk*)plan.chunks, (const CutRow*)plan.cuts,
+  auto kernel = plan.most_pieces >= 0 && plan.most_pieces <= kJoinShare ? join_kernel<false> : join_kernel<true>;
+  DG_CUDA(launch_kernel(kernel, grid, kBlock, s, true, (const Chunk*)plan.chunks, (const CutRow*)plan.cuts,
                         (const int32_t*)plan.totals, (int32_t)plan.max_cuts, partial, F, Y));
   count_launches(1);
   return DG_OK;

@@ -97,7 +97,7 @@ static int64_t cut_threshold(const Graph* g) {
 }
 
 // Where the totals of the rows' (0) or the columns' (1) plan lie among the counters.
-static int totals_of(const Graph* g, int columns) { return kTotals + g->totals_set * kTotalsPerSet + 2 * columns; }
+static int totals_of(const Graph* g, int columns) { return kTotals + (2 * g->totals_set + columns) * kTotalsPerPlan; }
 
 // Takes the memory of both plans for the current chunk cost and threshold; on failure the plans are as they were.
 static dg_status_t reserve_plans(Graph* g) {
@@ -125,7 +125,7 @@ static dg_status_t reserve_plans(Graph* g) {
     // a row of m > threshold entries holds at most m / cost + 1 boundaries
     plan.max_slots = cuts ? g->nnz / cost + g->nnz / cut_threshold(g) + 1 : 0;
     if (plan.max_slots > count) plan.max_slots = count;
-    plan.slots = plan.cut_rows = cuts ? -1 : 0;
+    plan.slots = plan.cut_rows = plan.most_pieces = cuts ? -1 : 0;
   }
   return DG_OK;
 }
@@ -134,9 +134,11 @@ static dg_status_t plan_rows(Graph* g, cudaStream_t s) {
   return build_plan(g->rowptr, g->n, g->nnz, chunk_cost(g), row_cost(g), cut_threshold(g), g->row_plan, s);
 }
 
-static void take_row_totals(Graph* g) {
-  g->row_plan.slots = g->host->v[totals_of(g, 0)];
-  g->row_plan.cut_rows = g->host->v[totals_of(g, 0) + 1];
+static void take_totals(const Graph* g, int columns, Plan* plan) {
+  const int32_t* v = g->host->v + totals_of(g, columns);
+  plan->slots = v[0];
+  plan->cut_rows = v[1];
+  plan->most_pieces = v[2];
 }
 
 // What follows every transposition: the columns' plan, its totals sent to the host behind it (read by
@@ -146,9 +148,10 @@ dg_status_t finish_transpose(Graph* g, cudaStream_t s) {
                                      s))
     return st;
   if (g->col_plan.max_cuts == 0) return DG_OK;
-  g->col_plan.slots = g->col_plan.cut_rows = -1;
+  g->col_plan.slots = g->col_plan.cut_rows = g->col_plan.most_pieces = -1;
   const int at = totals_of(g, 1);
-  DG_CUDA(cudaMemcpyAsync(g->host->v + at, g->counters + at, 2 * sizeof(int32_t), cudaMemcpyDeviceToHost, s));
+  DG_CUDA(cudaMemcpyAsync(g->host->v + at, g->counters + at, kTotalsPerPlan * sizeof(int32_t),
+                          cudaMemcpyDeviceToHost, s));
   DG_CUDA(cudaEventRecord(g->col_totals_ready, s));
   return DG_OK;
 }
@@ -156,8 +159,7 @@ dg_status_t finish_transpose(Graph* g, cudaStream_t s) {
 const Plan& column_plan(Graph* g) {
   if (g->col_plan.slots < 0) {
     if (cudaEventQuery(g->col_totals_ready) == cudaSuccess) {
-      g->col_plan.slots = g->host->v[totals_of(g, 1)];
-      g->col_plan.cut_rows = g->host->v[totals_of(g, 1) + 1];
+      take_totals(g, 1, &g->col_plan);
     } else {
       (void)cudaGetLastError();  // "not ready" must not be mistaken for a failed launch later
     }
@@ -185,7 +187,7 @@ static dg_status_t replan(Graph* g, int64_t* knob, int64_t value) {
   dg_status_t st = reserve_plans(g);
   if (st == DG_OK) st = build_plans(g);
   if (st == DG_OK) {
-    take_row_totals(g);
+    take_totals(g, 0, &g->row_plan);
     pool_retire(g->device, before.plan_memory, before.plan_bytes);
     return DG_OK;
   }
@@ -355,7 +357,7 @@ dg_status_t dg_graph_create(int64_t n, int64_t nnz, const int64_t* rowptr,
   }
   if (st == DG_OK && g->host->v[kFlags]) st = malformed(g->host->v[kFlags]);
   if (st != DG_OK) { free_owned(g); delete g; return st; }
-  take_row_totals(g);
+  take_totals(g, 0, &g->row_plan);
   if (g->host->v[kUnsorted]) g->split_csr = nullptr;  // rows not sorted: no source blocking
   *out_graph = g;
   return DG_OK;

@@ -91,7 +91,7 @@ __global__ void __launch_bounds__(kGenBlock, 4) general_dv_sum_kernel(const GenA
 // is feature f_lo + 32 w + j's extremum (arg is read once, nnz * words * 4 bytes are written); then
 // general_dv_mask_kernel walks the CSC, reads the words of every edge, one random sector of 32 bytes, and of
 // dO only the values that are selected.
-// Bound by instruction issue and DRAM together (68 % and 58 % busy at F = 100): about 20 instructions per
+// Bound by instruction issue and DRAM together (55 % and 65 % busy at 31 M edges, F = 100): about 20 instructions per
 // edge with a selected feature, and a random sector per edge for its words beside the selected values.
 // Both kernels, B200: 31 M edges F = 100 3.71 -> 1.59 ms; 16 M edges, columns up to 10^5, F = 128
 // 4.28 -> 1.63 ms; 24 M edges F = 64 0.69 -> 0.41 ms; 5.7 M edges F = 602 5.73 -> 1.30 ms.

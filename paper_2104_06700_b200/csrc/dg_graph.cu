@@ -44,6 +44,7 @@ __global__ void plan_kernel(const int64_t* __restrict__ ptr, int64_t n, int64_t 
         out.slot = atomicAdd(totals + 0, 1);
         if (j == 0) {
           const int32_t i = atomicAdd(totals + 1, 1);
+          atomicMax(totals + 2, (int32_t)m);
           if (i < max_cuts) cuts[i] = CutRow{(int32_t)lo, (int32_t)c, (int32_t)m, 0};
         }
       }
@@ -144,7 +145,7 @@ dg_status_t build_split(const int64_t* ptr, const int32_t* idx, int64_t n, int64
 // The chunks of one direction (the arrays of `plan` are sized by its count); asynchronous.
 dg_status_t build_plan(const int64_t* ptr, int64_t n, int64_t nnz, int64_t chunk_cost, int64_t row_cost,
                        int64_t threshold, const Plan& plan, cudaStream_t s) {
-  DG_CUDA(cudaMemsetAsync(plan.totals, 0, 2 * sizeof(int32_t), s));
+  DG_CUDA(cudaMemsetAsync(plan.totals, 0, kTotalsPerPlan * sizeof(int32_t), s));
   plan_kernel<<<blocks_for(plan.count + 1), kBlock, 0, s>>>(ptr, n, nnz, chunk_cost, row_cost, threshold, plan.count,
                                                             plan.chunks, plan.cuts, plan.max_cuts,
                                                             plan.totals);

@@ -27,15 +27,15 @@ struct CutRow {
 struct Plan {
   Chunk* chunks = nullptr;    // count + 1 entries, the last one is (n, nnz)
   CutRow* cuts = nullptr;     // the cut rows, in any order
-  int32_t* totals = nullptr;  // device: [0] slots, [1] cut rows
+  int32_t* totals = nullptr;  // device: [0] slots, [1] cut rows, [2] most slots of a row
   int64_t count = 0;
   int64_t max_slots = 0, max_cuts = 0;  // bounds known from n and nnz alone
-  int32_t slots = -1, cut_rows = -1;    // the totals, or -1 while they are on their way to the host
+  int32_t slots = -1, cut_rows = -1, most_pieces = -1;  // the totals, or -1 while they are on their way to the host
 };
 
 // Device counters of a handle, and their order in the pinned copy.  There are two sets of plan totals, rows' then
 // columns', used in turn: until new plans are finished the old ones stay whole.
-enum { kFlags, kUnsorted, kTotals, kTotalsPerSet = 4, kCounters = kTotals + 2 * kTotalsPerSet };
+enum { kFlags, kUnsorted, kTotals, kTotalsPerPlan = 3, kCounters = kTotals + 4 * kTotalsPerPlan };
 struct HostCounters {
   int32_t v[kCounters];
 };

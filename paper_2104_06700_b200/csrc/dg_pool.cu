@@ -21,7 +21,7 @@ constexpr int kMaxDevices = 64;
 constexpr size_t kKeepInUse = (size_t)4 << 30;
 constexpr size_t kKeepIdle = (size_t)32 << 20;
 constexpr size_t kMaxPending = kKeepIdle;
-constexpr int kPinnedWords = 100;  // one page
+constexpr int kPinnedWords = 72;  // one page
 
 // A device block, or a handle's pinned counters, that queued work may still use.
 struct Retired {
