@@ -383,8 +383,9 @@ dg_status_t dg_aggregate_edge_grad(dg_graph_t g, const float* H, const float* dO
  *   "heavy_threshold"  rows longer than this, and rows over 4096 entries, may be cut into pieces for several
  *                      warps (default: twice the piece size chosen from the number of edges, 64 to 2048)
  *   "heavy_blocks_per_sm"  accepted in [0, 32]; no effect
- *   "slice_features"   features per pass over the graph (0 = choose from the L2 size; a value
- *                      that would need more than 65535 passes is widened)
+ *   "slice_features"   features per pass over the graph (0 = choose from F and the mean degree, and from the L2
+ *                      size where the call is cut into source blocks; a value that would need more than
+ *                      65535 passes is widened)
  *   "rows_per_block"   rows per thread block at the average row length (1..248, rounded up to a
  *                      multiple of 8: each of the 8 warps takes the edges of that many rows;
  *                      0 = 32 to 1024 edges per warp, from the number of edges)
