@@ -167,17 +167,23 @@ void count_launches(int64_t k);
 // launches is worth closing (forward + backward with copies and joins, 1.2 M edges, F = 47: 85 -> 75 us; with a
 // join, 65 k edges, F = 64: 20.5 -> 18.8 us).
 template <typename... P, typename... A>
-cudaError_t launch_kernel(void (*kernel)(P...), dim3 grid, int block, cudaStream_t s, bool overlap, const A&... args) {
+cudaError_t launch_kernel(void (*kernel)(P...), dim3 grid, int block, size_t smem, cudaStream_t s, bool overlap,
+                          const A&... args) {
   cudaLaunchAttribute attribute{};
   attribute.id = cudaLaunchAttributeProgrammaticStreamSerialization;
   attribute.val.programmaticStreamSerializationAllowed = 1;
   cudaLaunchConfig_t config{};
   config.gridDim = grid;
   config.blockDim = dim3((unsigned)block);
+  config.dynamicSmemBytes = smem;
   config.stream = s;
   config.attrs = &attribute;
   config.numAttrs = overlap ? 1 : 0;
   return cudaLaunchKernelEx(&config, kernel, args...);
+}
+template <typename... P, typename... A>
+cudaError_t launch_kernel(void (*kernel)(P...), dim3 grid, int block, cudaStream_t s, bool overlap, const A&... args) {
+  return launch_kernel(kernel, grid, block, (size_t)0, s, overlap, args...);
 }
 
 #define DG_CUDA(call)                                          \

@@ -7,12 +7,19 @@
 // three kernels and never makes one block wait for another:
 //   1. digit_histogram : per tile of kTile keys, the number of keys per digit -> hist[digit][tile]
 //   2. exclusive scan of hist (digit-major, so the scan yields global output offsets):
-//      scan_reduce -> scan_spine (one block) -> scan_apply
+//      scan_reduce -> scan_spine (one block) -> scan_apply, or scan_few
 //   3. digit_scatter   : ranks every key inside its tile in input order (ballots over the digit
 //      bits inside a warp, per-warp counters across rounds, a fixed pass across the warps), stages
 //      the tile sorted by digit in shared memory and writes each digit run to its global offset.
-// Stability of every step makes the final order (key, k) ascending.  After the last pass the
-// sorted keys give colptr by boundary detection, and perm gives rowidx_T and w_T by gathers.
+// Stability of every step makes the final order (key, k) ascending.
+//
+// The last pass of a transposition does not write the keys again: it counts the columns (the entries of a column lie
+// side by side in a sorted tile), and writes beside perm the row of every entry, which it finds in a table of 16 bytes per
+// 32 positions, and the row's factor.  That saves the passes that read the sorted keys, wrote (row, factor) pairs of 8 bytes
+// per edge and gathered them through perm, one random DRAM read per edge; the table of 124 M edges is 62 MB and its reads
+// hit L2.  Create and transposition, us before / after: 124 M edges, 2.4 M vertices 4670 / 3945; 81 M edges, 5.6 M vertices
+// 3758 / 2825; 115 M edges, 233 k vertices 4540 / 4000; 576 M edges 37100 / 34500; 65 k edges 138 / 131.  Rows carried through
+// the passes instead, with two passes of 11 bits or three of 8: 4150 and 4096.
 #include "dg_internal.cuh"
 
 namespace dg {
@@ -28,6 +35,14 @@ constexpr int kScanItems = 16;
 constexpr int kScanChunk = kScanBlock * kScanItems;
 constexpr unsigned kFull = 0xffffffffu;
 
+// The kernels of a sort follow one another closely (see launch_kernel): the next one's blocks come up while this one's last
+// run, and wait here for its end.  A small graph's ingest is the gaps between launches (create and transposition of 1.2 M
+// edges 179 -> 156 us, of 31 M 1308 -> 1277).
+__device__ __forceinline__ void overlap_begin() {
+  cudaGridDependencySynchronize();
+  cudaTriggerProgrammaticLaunchCompletion();
+}
+
 template <int BITS>
 __device__ __forceinline__ uint32_t digit_of(uint32_t key, int shift) {
   return (key >> shift) & ((1u << BITS) - 1u);
@@ -41,6 +56,7 @@ template <int BITS>
 __global__ void __launch_bounds__(kSortBlock)
 digit_histogram(const uint32_t* __restrict__ keys, int64_t count, int shift, int64_t tiles,
                 int vector_ok, uint32_t* __restrict__ hist) {
+  overlap_begin();
   constexpr int R = 1 << BITS;
   __shared__ uint32_t h[R];
   for (int d = threadIdx.x; d < R; d += kSortBlock) h[d] = 0;
@@ -70,8 +86,9 @@ digit_histogram(const uint32_t* __restrict__ keys, int64_t count, int shift, int
 }
 
 // ---- exclusive scan of a uint32 array of length m (in place), three kernels ----
+template <int THREADS>
 __device__ __forceinline__ uint32_t block_exclusive_scan(uint32_t v, uint32_t* total) {
-  __shared__ uint32_t warp_sums[kScanBlock / 32];
+  __shared__ uint32_t warp_sums[THREADS / 32];
   __shared__ uint32_t block_total;
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   uint32_t inc = v;
@@ -83,15 +100,15 @@ __device__ __forceinline__ uint32_t block_exclusive_scan(uint32_t v, uint32_t* t
   if (lane == 31) warp_sums[warp] = inc;
   __syncthreads();
   if (warp == 0) {
-    uint32_t w = lane < kScanBlock / 32 ? warp_sums[lane] : 0;
+    uint32_t w = lane < THREADS / 32 ? warp_sums[lane] : 0;
     uint32_t winc = w;
 #pragma unroll
     for (int d = 1; d < 32; d <<= 1) {
       const uint32_t t = __shfl_up_sync(kFull, winc, d);
       if (lane >= d) winc += t;
     }
-    if (lane < kScanBlock / 32) warp_sums[lane] = winc - w;
-    if (lane == kScanBlock / 32 - 1) block_total = winc;
+    if (lane < THREADS / 32) warp_sums[lane] = winc - w;
+    if (lane == THREADS / 32 - 1) block_total = winc;
   }
   __syncthreads();
   const uint32_t r = inc - v + warp_sums[warp];
@@ -102,31 +119,35 @@ __device__ __forceinline__ uint32_t block_exclusive_scan(uint32_t v, uint32_t* t
 
 __global__ void __launch_bounds__(kScanBlock)
 scan_reduce(const uint32_t* __restrict__ data, int64_t m, uint32_t* __restrict__ chunk_sums) {
+  overlap_begin();
   const int64_t base = (int64_t)blockIdx.x * kScanChunk + (int64_t)threadIdx.x * kScanItems;
   uint32_t s = 0;
 #pragma unroll
   for (int i = 0; i < kScanItems; ++i)
     if (base + i < m) s += data[base + i];
   uint32_t total;
-  block_exclusive_scan(s, &total);
+  block_exclusive_scan<kScanBlock>(s, &total);
   if (threadIdx.x == 0) chunk_sums[blockIdx.x] = total;
 }
 
+// `stride` words from one chunk's sum to the next
 __global__ void __launch_bounds__(kScanBlock)
-scan_spine(uint32_t* __restrict__ chunk_sums, int64_t chunks) {
+scan_spine(uint32_t* __restrict__ chunk_sums, int64_t stride, int64_t chunks) {
+  overlap_begin();
   uint32_t carry = 0;
   for (int64_t base = 0; base < chunks; base += kScanBlock) {
     const int64_t i = base + threadIdx.x;
-    const uint32_t v = i < chunks ? chunk_sums[i] : 0;
+    const uint32_t v = i < chunks ? chunk_sums[i * stride] : 0;
     uint32_t total;
-    const uint32_t ex = block_exclusive_scan(v, &total);
-    if (i < chunks) chunk_sums[i] = carry + ex;
+    const uint32_t ex = block_exclusive_scan<kScanBlock>(v, &total);
+    if (i < chunks) chunk_sums[i * stride] = carry + ex;
     carry += total;
   }
 }
 
 __global__ void __launch_bounds__(kScanBlock)
 scan_apply(uint32_t* __restrict__ data, int64_t m, const uint32_t* __restrict__ chunk_sums) {
+  overlap_begin();
   const int64_t base = (int64_t)blockIdx.x * kScanChunk + (int64_t)threadIdx.x * kScanItems;
   uint32_t v[kScanItems];
   uint32_t s = 0;
@@ -136,11 +157,147 @@ scan_apply(uint32_t* __restrict__ data, int64_t m, const uint32_t* __restrict__ 
     s += v[i];
   }
   uint32_t total;
-  uint32_t run = block_exclusive_scan(s, &total) + chunk_sums[blockIdx.x];
+  uint32_t run = block_exclusive_scan<kScanBlock>(s, &total) + chunk_sums[blockIdx.x];
 #pragma unroll
   for (int i = 0; i < kScanItems; ++i) {
     if (base + i < m) data[base + i] = run;
     run += v[i];
+  }
+}
+
+// The whole scan in one block: of up to kFewEntries, one launch instead of three (a second round of the block takes ten
+// microseconds).  PAIRS: `data` are the pairs below, and 64-bit sums take their place.
+constexpr int kFewThreads = 1024;
+constexpr int64_t kFewEntries = kFewThreads * kScanItems;
+template <bool PAIRS>
+__global__ void __launch_bounds__(kFewThreads) scan_few(uint32_t* __restrict__ data, int64_t m) {
+  overlap_begin();
+  const int base = threadIdx.x * kScanItems;
+  uint32_t v[kScanItems], s = 0;
+#pragma unroll
+  for (int i = 0; i < kScanItems; ++i) {
+    v[i] = base + i < m ? data[PAIRS ? 2 * (base + i) : base + i] : 0u;
+    s += v[i];
+  }
+  uint32_t total;
+  uint32_t run = block_exclusive_scan<kFewThreads>(s, &total);
+#pragma unroll
+  for (int i = 0; i < kScanItems; ++i) {
+    if (base + i < m) {
+      if (PAIRS) reinterpret_cast<int64_t*>(data)[base + i] = (int64_t)run;
+      else data[base + i] = run;
+    }
+    run += v[i];
+  }
+}
+
+// ---- the column pointers, from counts ----
+// While the edges are sorted, colptr holds a pair per column: x the entries counted so far, y the bits of the factor
+// 1/(in-degree + self) of the vertex.  Then it is scanned in place; the sum of a chunk of kScanChunk columns travels
+// in y of the chunk's first pair.
+__global__ void __launch_bounds__(256)
+columns_begin_kernel(const int64_t* __restrict__ rowptr, int64_t n, int self, uint2* __restrict__ columns) {
+  overlap_begin();
+  const int64_t v = (int64_t)blockIdx.x * 256 + threadIdx.x;
+  if (v > n) return;
+  float inv = 0.f;
+  if (v < n) inv = 1.0f / (float)(__ldg(rowptr + v + 1) - __ldg(rowptr + v) + self);
+  columns[v] = make_uint2(0u, __float_as_uint(inv));
+}
+
+__global__ void __launch_bounds__(kScanBlock)
+columns_reduce(uint2* __restrict__ columns, int64_t m) {
+  overlap_begin();
+  const int64_t chunk = (int64_t)blockIdx.x * kScanChunk;
+  uint32_t s = 0;
+#pragma unroll
+  for (int i = 0; i < kScanItems; ++i) {
+    const int64_t u = chunk + i * kScanBlock + threadIdx.x;
+    if (u < m) s += columns[u].x;
+  }
+  uint32_t total;
+  block_exclusive_scan<kScanBlock>(s, &total);
+  if (threadIdx.x == 0) columns[chunk].y = total;
+}
+
+__global__ void __launch_bounds__(kScanBlock)
+columns_apply(uint2* __restrict__ columns, int64_t m) {
+  overlap_begin();
+  const int64_t chunk = (int64_t)blockIdx.x * kScanChunk, base = chunk + (int64_t)threadIdx.x * kScanItems;
+  const uint32_t before = columns[chunk].y;  // read by all before the barriers below let anyone write it
+  uint32_t v[kScanItems], s = 0;
+#pragma unroll
+  for (int i = 0; i < kScanItems; ++i) {
+    v[i] = base + i < m ? columns[base + i].x : 0u;
+    s += v[i];
+  }
+  uint32_t total;
+  uint32_t run = before + block_exclusive_scan<kScanBlock>(s, &total);
+#pragma unroll
+  for (int i = 0; i < kScanItems; ++i) {
+    if (base + i < m) reinterpret_cast<int64_t*>(columns)[base + i] = (int64_t)run;
+    run += v[i];
+  }
+}
+
+// ---- the row of a position ----
+// table[b] for the positions 32 b ... 32 b + 31: x the row r of the first; y a bit for every other position that begins a
+// row, so that the row of position 32 b + i is r + the number of bits 1 ... i; bit 0: a row without entries lies between
+// them, and the count is wrong; z, w: the bits of the factors of r and r + 1, where most entries belong (one random
+// read instead of two).
+struct RowOf {
+  int64_t row;
+  bool known;       // `factor` is the row's
+  uint32_t factor;
+};
+__device__ __forceinline__ RowOf row_of(const uint4* __restrict__ table, const int64_t* __restrict__ rowptr, int64_t n,
+                                        int64_t nnz, uint32_t k, const uint4& block) {
+  if (!(block.y & 1u)) {
+    const int later = __popc(block.y & ((2u << (k & 31u)) - 1u));
+    return {(int64_t)block.x + later, later < 2, later ? block.w : block.z};
+  }
+  const int64_t b = (int64_t)(k >> 5) + 1;
+  int64_t lo = block.x, hi = 32 * b < nnz ? (int64_t)__ldg(&table[b].x) + 1 : n;  // the last row that begins at or before k
+  while (hi - lo > 1) {
+    const int64_t mid = (lo + hi) >> 1;
+    if (__ldg(rowptr + mid) <= (int64_t)k) lo = mid;
+    else hi = mid;
+  }
+  return {lo, false, 0u};
+}
+
+// A warp takes one chunk of the rows' plan (see Plan).  The bits are zero before.
+__global__ void __launch_bounds__(256)
+row_table_kernel(const Chunk* __restrict__ chunks, int32_t chunk_count, const int64_t* __restrict__ rowptr, int64_t n,
+                 const uint2* __restrict__ columns, uint4* __restrict__ table) {
+  overlap_begin();
+  const int lane = threadIdx.x & 31;
+  const int chunk = blockIdx.x * 8 + __shfl_sync(kFull, (int)(threadIdx.x >> 5), 0);
+  if (chunk >= chunk_count) return;
+  const int4 here = __ldg(reinterpret_cast<const int4*>(chunks) + chunk);
+  const int4 next = __ldg(reinterpret_cast<const int4*>(chunks) + chunk + 1);
+  const int nrows = here.z >= 0 ? 1 : next.x - here.x + (next.z >= 0 ? 1 : 0);
+  Position begin = 0, end = 0;
+  uint32_t factor = 0, following = 0;
+  if (lane < nrows) {
+    const int64_t r = here.x + lane;
+    const int64_t row_begin = __ldg(rowptr + r), row_end = __ldg(rowptr + r + 1);
+    begin = max((int)row_begin, here.y);
+    end = min((int)row_end, next.y);
+    factor = __ldg(&columns[r].y);
+    following = r + 1 < n ? __ldg(&columns[r + 1].y) : 0u;
+    if (row_begin < row_end && here.z < 0 && (row_begin & 31)) {  // a piece of a cut row begins no row
+      const bool after_empty = r > 0 && __ldg(rowptr + r - 1) == row_begin;
+      atomicOr(&table[row_begin >> 5].y, 1u << (row_begin & 31) | (after_empty ? 1u : 0u));
+    }
+  }
+  for (int i = 0; i < nrows; ++i) {
+    const Position lo = __shfl_sync(kFull, begin, i), hi = __shfl_sync(kFull, end, i);
+    const uint2 factors = make_uint2(__shfl_sync(kFull, factor, i), __shfl_sync(kFull, following, i));
+    for (Position b = ((lo + 31) >> 5) + lane; 32 * b < hi; b += 32) {
+      table[b].x = (uint32_t)(here.x + i);
+      *reinterpret_cast<uint2*>(&table[b].z) = factors;
+    }
   }
 }
 
@@ -167,11 +324,22 @@ __device__ __forceinline__ unsigned digit_peers(uint32_t d, bool valid) {
 // Four blocks per SM (64 registers a thread): the ranking is a chain of shared-memory and ballot latencies.
 // Values are read only when the keys have left their registers, and two places share one: nothing spills
 // (0.78 -> 0.68 ms per pass over 124 M pairs; three blocks at 80 registers 1.02, five at 48 0.73).
-template <int BITS>
+// With CSC the last pass of a transposition: twice the time of a plain pass (18.6 M edges 258 us, a plain one 111), for
+// the random reads of the table, four in flight per thread, and three arrays written instead of two.
+struct CscArgs {  // empty otherwise
+  const uint4* table;     // see row_of
+  const int64_t* rowptr;
+  int64_t n;
+  uint2* columns;         // see columns_begin_kernel
+  int32_t* rows_out;
+  float* scale_out;       // the factor of every entry's row, or nullptr
+};
+template <int BITS, bool CSC>
 __global__ void __launch_bounds__(kSortBlock, 4)
 digit_scatter(const uint32_t* __restrict__ keys_in, const uint32_t* __restrict__ vals_in,
               int64_t count, int shift, int64_t tiles, const uint32_t* __restrict__ offsets,
-              uint32_t* __restrict__ keys_out, uint32_t* __restrict__ vals_out) {
+              uint32_t* __restrict__ keys_out, uint32_t* __restrict__ vals_out, const CscArgs c) {
+  overlap_begin();
   constexpr int R = 1 << BITS;
   constexpr int DPT = R / kSortBlock;  // digits a thread owns (consecutive ones): 1 or 2
   // A warp ranks its 512 keys as two streams of 256 (rounds 0..7 and 8..15), each with its own
@@ -207,7 +375,7 @@ digit_scatter(const uint32_t* __restrict__ keys_in, const uint32_t* __restrict__
   // so (warp, round, lane) order is input order.
   uint32_t key[kItems];
   constexpr int kHalf = kItems / 2;
-  uint32_t place[kHalf];  // rank, later the place in the sorted tile: of key r low, of key r + kHalf high
+  uint32_t place[kHalf] = {};  // rank, later the place in the sorted tile: of key r low, of key r + kHalf high
   auto place_of = [&](int r) { return r < kHalf ? place[r] & 0xffffu : place[r - kHalf] >> 16; };
 #pragma unroll
   for (int r = 0; r < kItems; ++r) {
@@ -259,7 +427,7 @@ digit_scatter(const uint32_t* __restrict__ keys_in, const uint32_t* __restrict__
       mine += run;
     }
     uint32_t total;
-    uint32_t start = block_exclusive_scan(mine, &total);
+    uint32_t start = block_exclusive_scan<kSortBlock>(mine, &total);
 #pragma unroll
     for (int i = 0; i < DPT; ++i) {
       digit_base[threadIdx.x * DPT + i] = start;
@@ -290,7 +458,13 @@ digit_scatter(const uint32_t* __restrict__ keys_in, const uint32_t* __restrict__
       const uint32_t k = stage[i];
       const uint32_t d = digit_of<BITS>(k, shift);
       dst[j] = global_base[d] + ((uint32_t)i - digit_base[d]);
-      keys_out[dst[j]] = k;
+      if (!CSC) {
+        keys_out[dst[j]] = k;
+      } else if (k < (uint32_t)c.n) {  // an id outside the graph must not turn into a write outside the pairs
+        // a column's entries of this tile lie side by side: the two ends of the run make the count
+        if (i == 0 || stage[i - 1] != k) atomicAdd(&c.columns[k].x, 0u - (uint32_t)i);
+        if (i == tile_count - 1 || stage[i + 1] != k) atomicAdd(&c.columns[k].x, (uint32_t)i + 1u);
+      }
     }
   }
   __syncthreads();
@@ -302,10 +476,35 @@ digit_scatter(const uint32_t* __restrict__ keys_in, const uint32_t* __restrict__
     }
   }
   __syncthreads();
+  if (!CSC) {
 #pragma unroll
-  for (int j = 0; j < kItems; ++j) {
-    const int i = j * kSortBlock + threadIdx.x;
-    if (i < tile_count) vals_out[dst[j]] = stage[i];
+    for (int j = 0; j < kItems; ++j) {
+      const int i = j * kSortBlock + threadIdx.x;
+      if (i < tile_count) vals_out[dst[j]] = stage[i];
+    }
+    return;
+  }
+  constexpr int kAhead = 4;  // look-ups in flight
+#pragma unroll
+  for (int j0 = 0; j0 < kItems; j0 += kAhead) {
+    uint4 block[kAhead];
+#pragma unroll
+    for (int j = 0; j < kAhead; ++j) {
+      const int i = (j0 + j) * kSortBlock + threadIdx.x;
+      if (i < tile_count) block[j] = __ldg(c.table + (stage[i] >> 5));
+    }
+#pragma unroll
+    for (int j = 0; j < kAhead; ++j) {
+      const int i = (j0 + j) * kSortBlock + threadIdx.x;
+      if (i < tile_count) {
+        const uint32_t k = stage[i];
+        const RowOf at = row_of(c.table, c.rowptr, c.n, count, k, block[j]);
+        vals_out[dst[j0 + j]] = k;
+        c.rows_out[dst[j0 + j]] = (int32_t)at.row;
+        if (c.scale_out)
+          c.scale_out[dst[j0 + j]] = __uint_as_float(at.known ? at.factor : __ldcg(&c.columns[at.row].y));
+      }
+    }
   }
 }
 
@@ -373,35 +572,6 @@ __global__ void fill_long_gaps(const uint32_t* __restrict__ sorted, int64_t nnz,
   colptr[u] = lo;
 }
 
-// row_info[k] = (row r that holds CSR position k, bits of 1/(deg(r) + self)); self = 1 when the graph has
-// implicit self loops, else 0.  A warp takes one chunk of the rows' plan (see Plan) and writes its rows'
-// pairs over their entries: bound by the 8 bytes written per edge.  A search for the row of every eighth
-// position, and a walk from there, took 0.58 ms for 124 M edges, this 0.16.
-__global__ void __launch_bounds__(256)
-row_info_kernel(const Chunk* __restrict__ chunks, int32_t chunk_count, const int64_t* __restrict__ rowptr,
-                int self, uint2* __restrict__ row_info) {
-  const int lane = threadIdx.x & 31;
-  const int chunk = blockIdx.x * 8 + __shfl_sync(kFull, (int)(threadIdx.x >> 5), 0);
-  if (chunk >= chunk_count) return;
-  const int4 here = __ldg(reinterpret_cast<const int4*>(chunks) + chunk);
-  const int4 next = __ldg(reinterpret_cast<const int4*>(chunks) + chunk + 1);
-  const int nrows = here.z >= 0 ? 1 : next.x - here.x + (next.z >= 0 ? 1 : 0);
-  int end = next.y;
-  uint32_t inv = 0;
-  if (lane < nrows) {
-    const int64_t row_end = __ldg(rowptr + here.x + lane + 1);
-    end = min((int)row_end, next.y);
-    inv = __float_as_uint(1.0f / (float)(row_end - __ldg(rowptr + here.x + lane) + self));
-  }
-  Position p = here.y;
-  for (int i = 0; i < nrows; ++i) {
-    const Position hi = __shfl_sync(kFull, end, i);
-    const uint2 info = make_uint2((uint32_t)(here.x + i), __shfl_sync(kFull, inv, i));
-    for (Position k = p + lane; k < hi; k += 32) row_info[k] = info;
-    p = hi;
-  }
-}
-
 constexpr int kRowItems = 8;
 // out[k] = map[r] (or r) for the row r that holds position k.  A thread takes kRowItems consecutive
 // positions: one binary search for the first, then a galloping search forward from the previous row for
@@ -441,37 +611,14 @@ __global__ void expand_rows_kernel(const int64_t* __restrict__ rowptr, int64_t n
   }
 }
 
-// rowidx_T[q] = row of perm[q];  w_T[q] = edge_w[perm[q]];  mean_scale_T[q] = w_T[q] (1 if
-// unweighted) / (deg(row) + self), the factor of edge q in the backward pass of the mean, so that
-// the backward kernel streams it instead of gathering 1/deg.  Bound by the random reads, one of 8 bytes per
-// edge (two if weighted): 4-byte reads of the row alone and the degree from its row pointers, three random
-// reads, took 2.06 ms instead of 1.52 for 124 M edges; the row carried through the sort instead took 2.5 ms
-// more in the scatters.
-__global__ void gather_rows_and_weights(const uint32_t* __restrict__ perm, int64_t nnz,
-                                        const uint2* __restrict__ row_info,
-                                        const float* __restrict__ edge_w,
-                                        int32_t* __restrict__ rowidx_T, float* __restrict__ w_T,
-                                        float* __restrict__ mean_scale_T) {
-  const int64_t q = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-  if (q >= nnz) return;
-  const int64_t k = perm[q];
-  const uint2 info = __ldg(row_info + k);
-  rowidx_T[q] = (int32_t)info.x;
-  float w = 1.f;
-  if (edge_w) {
-    w = edge_w[k];
-    w_T[q] = w;
-  }
-  mean_scale_T[q] = w * __uint_as_float(info.y);
-}
-
-// After the caller changed edge_w in place (learnable edge weights): the two weight arrays of the
-// CSC again, from perm.  The in-degree comes from the CSR row pointer.  A thread takes four edges: their
+// The weight arrays of the CSC, from perm: the last step of a transposition, and again after the caller changed edge_w in
+// place (learnable edge weights).  The in-degree comes from the CSR row pointer.  A thread takes four edges: their
 // random reads are in flight together.
 __global__ void __launch_bounds__(256)
-regather_weights_kernel(const uint32_t* __restrict__ perm, int64_t nnz, const float* __restrict__ edge_w,
-                        const int32_t* __restrict__ rowidx_T, const int64_t* __restrict__ rowptr, int self,
-                        float* __restrict__ w_T, float* __restrict__ mean_scale_T) {
+gather_weights_kernel(const uint32_t* __restrict__ perm, int64_t nnz, const float* __restrict__ edge_w,
+                      const int32_t* __restrict__ rowidx_T, const int64_t* __restrict__ rowptr, int self,
+                      float* __restrict__ w_T, float* __restrict__ mean_scale_T) {
+  overlap_begin();
   const int64_t q0 = ((int64_t)blockIdx.x * 256 + threadIdx.x) * 4;
   if (q0 >= nnz) return;
   if (nnz - q0 >= 4) {  // the arrays of the CSC are 256-byte aligned
@@ -563,7 +710,8 @@ template <int BITS>
 static dg_status_t sort_passes_run(const uint32_t* keys_in, const uint32_t* vals_in, int64_t count,
                                    int passes, uint32_t* const keys_buf[2], uint32_t* vals_final,
                                    uint32_t* vals_tmp, uint32_t* hist,
-                                   uint32_t* sums, const uint32_t** sorted_keys, cudaStream_t s) {
+                                   uint32_t* sums, const uint32_t** sorted_keys, CscArgs* csc,
+                                   const Graph* g, cudaStream_t s) {
   const int64_t tiles = (count + kTile - 1) / kTile;
   const int64_t hist_len = tiles * (1 << BITS);
   const int64_t chunks = (hist_len + kScanChunk - 1) / kScanChunk;
@@ -573,19 +721,31 @@ static dg_status_t sort_passes_run(const uint32_t* keys_in, const uint32_t* vals
     // value buffers alternate so that the last pass lands in vals_final
     uint32_t* vals_out = ((passes - 1 - p) % 2 == 0) ? vals_final : vals_tmp;
     uint32_t* keys_out = keys_buf[p % 2];
-    digit_histogram<BITS><<<(unsigned)tiles, kSortBlock, 0, s>>>(keys_in, count, shift, tiles,
-                                                                 aligned16(keys_in), hist);
-    DG_CUDA(cudaGetLastError());
-    scan_reduce<<<(unsigned)chunks, kScanBlock, 0, s>>>(hist, hist_len, sums);
-    DG_CUDA(cudaGetLastError());
-    scan_spine<<<1, kScanBlock, 0, s>>>(sums, chunks);
-    DG_CUDA(cudaGetLastError());
-    scan_apply<<<(unsigned)chunks, kScanBlock, 0, s>>>(hist, hist_len, sums);
-    DG_CUDA(cudaGetLastError());
-    digit_scatter<BITS><<<(unsigned)tiles, kSortBlock, smem, s>>>(keys_in, vals_in, count, shift,
-                                                                  tiles, hist, keys_out, vals_out);
-    DG_CUDA(cudaGetLastError());
-    count_launches(5);
+    DG_CUDA(launch_kernel(digit_histogram<BITS>, dim3((unsigned)tiles), kSortBlock, s, true, keys_in, count, shift, tiles,
+                          aligned16(keys_in), hist));
+    if (hist_len <= kFewEntries) {
+      DG_CUDA(launch_kernel(scan_few<false>, dim3(1), kFewThreads, s, true, hist, hist_len));
+      count_launches(1);
+    } else {
+      const dim3 grid((unsigned)chunks);
+      DG_CUDA(launch_kernel(scan_reduce, grid, kScanBlock, s, true, hist, hist_len, sums));
+      DG_CUDA(launch_kernel(scan_spine, dim3(1), kScanBlock, s, true, sums, 1, chunks));
+      DG_CUDA(launch_kernel(scan_apply, grid, kScanBlock, s, true, hist, hist_len, sums));
+      count_launches(3);
+    }
+    if (csc && p == passes - 1) {
+      // no keys are written: their place takes the table of rows
+      uint4* table = reinterpret_cast<uint4*>(keys_out);
+      DG_CUDA(cudaMemsetAsync(table, 0, (size_t)((count + 31) / 32) * sizeof(uint4), s));
+      DG_CUDA(launch_kernel(row_table_kernel, dim3((unsigned)((g->row_plan.count + 7) / 8)), 256, s, true,
+                            g->row_plan.chunks, g->row_plan.count, g->rowptr, csc->n, csc->columns, table));
+      count_launches(1);
+      csc->table = table;
+    }
+    DG_CUDA(launch_kernel(csc && p == passes - 1 ? digit_scatter<BITS, true> : digit_scatter<BITS, false>,
+                          dim3((unsigned)tiles), kSortBlock, smem, s, true, keys_in, vals_in, count, shift, tiles, hist,
+                          keys_out, vals_out, csc ? *csc : CscArgs{}));
+    count_launches(2);
     keys_in = keys_out;
     vals_in = vals_out;
   }
@@ -597,15 +757,22 @@ static dg_status_t sort_passes_run(const uint32_t* keys_in, const uint32_t* vals
 // i is i".  keys_in is only read; the sorted keys end in one of keys_buf (reported through
 // *sorted_keys; keys_in may be keys_buf[1], which is first written by the second pass), the
 // sorted values in vals_final (vals_tmp is the other buffer of the ping-pong).
+static dg_status_t sort_run(const uint32_t* keys_in, const uint32_t* vals_in, int64_t count, SortPlan plan,
+                            uint32_t* const keys_buf[2], uint32_t* vals_final, uint32_t* vals_tmp, uint32_t* hist,
+                            uint32_t* sums, const uint32_t** sorted_keys, CscArgs* csc,
+                            const Graph* g, cudaStream_t s) {
+  if (plan.digit_bits == 9)
+    return sort_passes_run<9>(keys_in, vals_in, count, plan.passes, keys_buf, vals_final, vals_tmp,
+                              hist, sums, sorted_keys, csc, g, s);
+  return sort_passes_run<8>(keys_in, vals_in, count, plan.passes, keys_buf, vals_final, vals_tmp,
+                            hist, sums, sorted_keys, csc, g, s);
+}
 dg_status_t sort_pairs(const uint32_t* keys_in, const uint32_t* vals_in, int64_t count,
                        SortPlan plan, uint32_t* const keys_buf[2], uint32_t* vals_final,
                        uint32_t* vals_tmp, uint32_t* hist, uint32_t* sums,
                        const uint32_t** sorted_keys, cudaStream_t s) {
-  if (plan.digit_bits == 9)
-    return sort_passes_run<9>(keys_in, vals_in, count, plan.passes, keys_buf, vals_final, vals_tmp,
-                              hist, sums, sorted_keys, s);
-  return sort_passes_run<8>(keys_in, vals_in, count, plan.passes, keys_buf, vals_final, vals_tmp,
-                            hist, sums, sorted_keys, s);
+  return sort_run(keys_in, vals_in, count, plan, keys_buf, vals_final, vals_tmp, hist, sums, sorted_keys, nullptr,
+                  nullptr, s);
 }
 
 // ptr[u] = first position whose sorted key is >= u, for u = 0..n (ptr[n] = count)
@@ -641,10 +808,10 @@ void transpose_sizes(int64_t n, int64_t nnz, bool weighted, size_t* csc_bytes,
 
 dg_status_t refresh_csc_weights(Graph* g, cudaStream_t s) {
   if (g->nnz == 0 || !g->edge_w) return DG_OK;
-  regather_weights_kernel<<<(unsigned)((g->nnz + 1023) / 1024), 256, 0, s>>>(
-      reinterpret_cast<const uint32_t*>(g->perm), g->nnz, g->edge_w, g->rowidx_T, g->rowptr,
-      g->self_loops_in_csc ? 1 : 0, const_cast<float*>(g->w_T), const_cast<float*>(g->mean_scale_T));
-  DG_CUDA(cudaGetLastError());
+  DG_CUDA(launch_kernel(gather_weights_kernel, dim3((unsigned)((g->nnz + 1023) / 1024)), 256, s, true,
+                        reinterpret_cast<const uint32_t*>(g->perm), g->nnz, g->edge_w, g->rowidx_T, g->rowptr,
+                        g->self_loops_in_csc ? 1 : 0, const_cast<float*>(g->w_T),
+                        const_cast<float*>(g->mean_scale_T)));
   count_launches(1);
   return DG_OK;
 }
@@ -669,21 +836,25 @@ dg_status_t transpose_run(Graph* g, void* csc, void* scratch, cudaStream_t s) {
   if (nnz == 0) {
     DG_CUDA(cudaMemsetAsync(colptr, 0, (size_t)(n + 1) * 8, s));
   } else {
-    const uint32_t* keys_in = nullptr;
-    if (dg_status_t st = sort_pairs(reinterpret_cast<const uint32_t*>(g->colidx), nullptr, nnz,
-                                    sort_plan(n), keys_buf, perm, vals_tmp, hist, sums, &keys_in, s))
+    const SortPlan plan = sort_plan(n);
+    CscArgs c{nullptr, g->rowptr, n, reinterpret_cast<uint2*>(colptr), rowidx_T, weighted ? nullptr : mean_scale_T};
+    columns_begin_kernel<<<(unsigned)(n / 256 + 1), 256, 0, s>>>(g->rowptr, n, g->self_loops ? 1 : 0, c.columns);
+    DG_CUDA(cudaGetLastError());
+    count_launches(1);
+    const uint32_t* sorted = nullptr;
+    if (dg_status_t st = sort_run(reinterpret_cast<const uint32_t*>(g->colidx), nullptr, nnz, plan, keys_buf, perm,
+                                  vals_tmp, hist, sums, &sorted, &c, g, s))
       return st;
-    if (dg_status_t st = pointers_from_sorted_keys(keys_in, nnz, n, colptr, s)) return st;
-    // colptr has been derived from the sorted keys (stream order), so both key buffers, which
-    // are adjacent in the scratch, are free: they hold the nnz (row, 1/deg) pairs
-    uint2* row_info = reinterpret_cast<uint2*>(sb + L.keys_a_off);
-    row_info_kernel<<<(unsigned)((g->row_plan.count + 7) / 8), 256, 0, s>>>(
-        g->row_plan.chunks, (int32_t)g->row_plan.count, g->rowptr, g->self_loops ? 1 : 0, row_info);
-    DG_CUDA(cudaGetLastError());
-    gather_rows_and_weights<<<(unsigned)((nnz + 255) / 256), 256, 0, s>>>(perm, nnz, row_info, g->edge_w, rowidx_T,
-                                                                          w_T, mean_scale_T);
-    DG_CUDA(cudaGetLastError());
-    count_launches(2);
+    const unsigned chunks = (unsigned)(n / kScanChunk + 1);  // of n + 1 columns
+    if (n + 1 <= kFewEntries) {
+      DG_CUDA(launch_kernel(scan_few<true>, dim3(1), kFewThreads, s, true, reinterpret_cast<uint32_t*>(c.columns), n + 1));
+      count_launches(1);
+    } else {
+      DG_CUDA(launch_kernel(columns_reduce, dim3(chunks), kScanBlock, s, true, c.columns, n + 1));
+      DG_CUDA(launch_kernel(scan_spine, dim3(1), kScanBlock, s, true, &c.columns->y, 2 * kScanChunk, chunks));
+      DG_CUDA(launch_kernel(columns_apply, dim3(chunks), kScanBlock, s, true, c.columns, n + 1));
+      count_launches(3);
+    }
   }
   g->colptr = colptr;
   g->rowidx_T = rowidx_T;
@@ -691,6 +862,7 @@ dg_status_t transpose_run(Graph* g, void* csc, void* scratch, cudaStream_t s) {
   g->w_T = w_T;
   g->mean_scale_T = mean_scale_T;
   g->self_loops_in_csc = g->self_loops;
+  if (dg_status_t st = refresh_csc_weights(g, s)) return st;
   g->split_csc = nullptr;
   if (wants_split(n, nnz)) {
     // the columns come out of the stable sort ordered by row, so the check never fires here
