@@ -99,19 +99,38 @@ __global__ void __launch_bounds__(kGenBlock, 4) edge_grad_kernel(const EdgeGradA
       [](int, int) {});
 }
 
+// Lanes per edge.  Half of what covers the slice, so that a lane takes two vectors of a row: the shuffles (an id per
+// edge and load, and the butterfly) then serve twice the loads, and they share a pipe with them.  A quarter where that leaves
+// fewer lanes without a vector (25 vectors: 16 lanes; 43: 16, not 32).  us with lanes for all vectors / this rule: 39.6 M
+// edges, F = 64 778 / 631, 100 1398 / 1127, 172 2094 / 1660; 31 M edges (from DRAM), F = 64 1117 / 1187, 172 3323 / 2929;
+// but two vectors on one lane are slower (F = 8 331 / 379).
+int lanes_per_edge(int nvec) {
+  if (nvec <= 2) return nvec;
+  int half = 2, quarter = 4;
+  while (half < 32 && 2 * half < nvec) half *= 2;
+  while (quarter < 32 && 4 * quarter < nvec) quarter *= 2;
+  auto slots = [&](int lanes) { return (nvec + lanes - 1) / lanes * lanes; };
+  return quarter < half && slots(quarter) < slots(half) ? quarter : half;
+}
+
+template <int VEC, int G>
+dg_status_t launch_lanes(const EdgeGradArgs& a, cudaStream_t s) {
+  edge_grad_kernel<VEC, G><<<(unsigned)((a.walk.chunk_count + kGenWarps - 1) / kGenWarps), kGenBlock, 0, s>>>(a);
+  DG_CUDA(cudaGetLastError());
+  count_launches(1);
+  return DG_OK;
+}
+
 template <int VEC>
 dg_status_t launch_edge_grad(const EdgeGradArgs& a, cudaStream_t s) {
-  const unsigned grid = (unsigned)((a.walk.chunk_count + kGenWarps - 1) / kGenWarps);
-#define DG_EG_CASE(GG)                                                 \
-  if (a.nvec <= GG || GG == 32) {                                      \
-    edge_grad_kernel<VEC, GG><<<grid, kGenBlock, 0, s>>>(a);           \
-    DG_CUDA(cudaGetLastError());                                       \
-    count_launches(1);                                                 \
-    return DG_OK;                                                      \
+  switch (lanes_per_edge(a.nvec)) {
+    case 1: return launch_lanes<VEC, 1>(a, s);
+    case 2: return launch_lanes<VEC, 2>(a, s);
+    case 4: return launch_lanes<VEC, 4>(a, s);
+    case 8: return launch_lanes<VEC, 8>(a, s);
+    case 16: return launch_lanes<VEC, 16>(a, s);
+    default: return launch_lanes<VEC, 32>(a, s);
   }
-  DG_EG_CASE(1) DG_EG_CASE(2) DG_EG_CASE(4) DG_EG_CASE(8) DG_EG_CASE(16) DG_EG_CASE(32)
-#undef DG_EG_CASE
-  return DG_OK;
 }
 
 }  // namespace
