@@ -217,6 +217,24 @@ dg_status_t dg_layer_bwd(dg_graph_t g, const float* dOut, const float* out, int3
                          float* G, float* dbias, void* stream);
 
 /*
+ * The matrix products of such a layer on fp32 matrices, X n x K, W N x K, G n x N (n = the handle's vertices),
+ * to fp32 accuracy on the tensor cores.
+ *
+ *   fwd:         Y = X W^T (n x N); with row_scale and bias (each may be NULL) and `relu` the epilogue of
+ *                dg_layer_fwd follows: Y = act(row_scale[v] * Y + bias).
+ *   bwd_input:   dX = G W (n x K).
+ *   bwd_weight:  dW = G^T X (N x K), always summed in the same order.
+ * The result must not overlap an input.  bwd_weight without scratch ("scratch_mb" = 0) sums all rows in a few thread
+ * blocks: correct, and slow.  Asynchronous on `stream`.
+ */
+dg_status_t dg_linear_fwd(dg_graph_t g, const float* X, int32_t K, const float* W, int32_t N,
+                          const float* row_scale, const float* bias, int32_t relu, float* Y, void* stream);
+dg_status_t dg_linear_bwd_input(dg_graph_t g, const float* G, int32_t N, const float* W, int32_t K, float* dX,
+                                void* stream);
+dg_status_t dg_linear_bwd_weight(dg_graph_t g, const float* G, int32_t N, const float* X, int32_t K, float* dW,
+                                 void* stream);
+
+/*
  * Mean softmax cross-entropy of the rows index[0..count) of the n x C matrix `logits` against
  * labels[index[t]] (n labels; -100: the row does not count), and its gradient.
  *

@@ -30,6 +30,7 @@ EXPORTS = [
     "dg_graph_create", "dg_graph_destroy", "dg_graph_validate", "dg_graph_transpose_workspace",
     "dg_graph_transpose", "dg_graph_transpose_static", "dg_graph_update_weights", "dg_graph_get_csc", "dg_aggregate_fwd", "dg_aggregate_bwd",
     "dg_aggregate_fwd_self", "dg_aggregate_bwd_self", "dg_layer_fwd", "dg_layer_bwd",
+    "dg_linear_fwd", "dg_linear_bwd_input", "dg_linear_bwd_weight",
     "dg_cross_entropy_fwd", "dg_cross_entropy_bwd",
     "dg_aggregate_fwd_bf16", "dg_aggregate_bwd_bf16",
     "dg_ap_fwd", "dg_ap_bwd", "dg_aggregate_edge_grad",
@@ -74,6 +75,9 @@ def lib() -> ctypes.CDLL:
         L.dg_aggregate_bwd_self.argtypes = [p, p, i32, ctypes.c_int, p, p]
         L.dg_layer_fwd.argtypes = [p, p, i32, p, p, i32, p]
         L.dg_layer_bwd.argtypes = [p, p, p, i32, p, p, p, p]
+        L.dg_linear_fwd.argtypes = [p, p, i32, p, i32, p, p, i32, p, p]
+        L.dg_linear_bwd_input.argtypes = [p, p, i32, p, i32, p, p]
+        L.dg_linear_bwd_weight.argtypes = [p, p, i32, p, i32, p, p]
         L.dg_cross_entropy_fwd.argtypes = [p, p, i32, p, i64, p, p, p, p]
         L.dg_cross_entropy_bwd.argtypes = [p, p, i32, p, i64, p, p, p, p, p, p]
         L.dg_aggregate_fwd_bf16.argtypes = [p, p, i32, ctypes.c_int, p, p]
@@ -381,6 +385,43 @@ class Graph:
                                   _dev_ptr(G, torch.float32, "G"), _dev_ptr(dbias, torch.float32, "dbias"),
                                   _stream(stream)))
         return G, dbias
+
+    def dg_linear_fwd(self, X: torch.Tensor, W: torch.Tensor, row_scale: Optional[torch.Tensor] = None,
+                      bias: Optional[torch.Tensor] = None, relu: bool = False, stream=None) -> torch.Tensor:
+        """X W^T, or act(row_scale * (X W^T) + bias)."""
+        N, K = W.shape
+        _holds(X, self.n * K, "X")
+        if row_scale is not None:
+            _holds(row_scale, self.n, "row_scale")
+        if bias is not None:
+            _holds(bias, N, "bias")
+        Y = X.new_empty((self.n, N))
+        _check(lib().dg_linear_fwd(self._h, _dev_ptr(X, torch.float32, "X"), K, _dev_ptr(W, torch.float32, "W"), N,
+                                   _dev_ptr(row_scale, torch.float32, "row_scale"),
+                                   _dev_ptr(bias, torch.float32, "bias"), bool(relu),
+                                   _dev_ptr(Y, torch.float32, "Y"), _stream(stream)))
+        return Y
+
+    def dg_linear_bwd_input(self, G: torch.Tensor, W: torch.Tensor, stream=None) -> torch.Tensor:
+        """G W."""
+        N, K = W.shape
+        _holds(G, self.n * N, "G")
+        dX = G.new_empty((self.n, K))
+        _check(lib().dg_linear_bwd_input(self._h, _dev_ptr(G, torch.float32, "G"), N,
+                                         _dev_ptr(W, torch.float32, "W"), K, _dev_ptr(dX, torch.float32, "dX"),
+                                         _stream(stream)))
+        return dX
+
+    def dg_linear_bwd_weight(self, G: torch.Tensor, X: torch.Tensor, stream=None) -> torch.Tensor:
+        """G^T X."""
+        N, K = G.shape[1], X.shape[1]
+        _holds(G, self.n * N, "G")
+        _holds(X, self.n * K, "X")
+        dW = G.new_empty((N, K))
+        _check(lib().dg_linear_bwd_weight(self._h, _dev_ptr(G, torch.float32, "G"), N,
+                                          _dev_ptr(X, torch.float32, "X"), K, _dev_ptr(dW, torch.float32, "dW"),
+                                          _stream(stream)))
+        return dW
 
     def _loss_shapes(self, logits, index, labels) -> None:
         _holds(logits, self.n * logits.shape[1], "logits")

@@ -13,7 +13,7 @@ LIB_PATH = os.path.join(_HERE, "libdgagg.so")
 BUILD_DIR = os.path.join(_HERE, "_build")
 SOURCES = ["dg_api.cu", "dg_graph.cu", "dg_transpose.cu", "dg_aggregate.cu", "dg_aggregate_self.cu", "dg_pool.cu",
            "dg_static.cu", "dg_probe.cu", "dg_general.cu", "dg_general_fwd.cu", "dg_general_bwd.cu", "dg_edge_grad.cu",
-           "dg_layer.cu", "dg_loss.cu", "dg_pieces.cu", "dg_reorder.cu"]
+           "dg_layer.cu", "dg_linear.cu", "dg_loss.cu", "dg_pieces.cu", "dg_reorder.cu"]
 NVCC_FLAGS = ["-gencode", "arch=compute_100a,code=sm_100a", "-lineinfo", "-O3", "-std=c++17",
               "-Xcompiler", "-fPIC", "-Xcompiler", "-Wall", "--use_fast_math=false"]
 

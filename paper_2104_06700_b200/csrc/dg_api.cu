@@ -460,6 +460,49 @@ dg_status_t dg_layer_bwd(dg_graph_t g, const float* dOut, const float* out, int3
   return layer_bwd(g, dOut, out, F, row_scale, G, dbias, (cudaStream_t)stream);
 }
 
+// The inputs a and b and the result, with their numbers of elements.
+static dg_status_t check_linear(const Graph* g, int32_t N, int32_t K, const float* a, int64_t a_count, const float* b,
+                                int64_t b_count, const float* out, int64_t out_count) {
+  if (!g) return invalid("graph handle is NULL");
+  if (N < 1 || N > (1 << 20) || K < 1 || K > (1 << 20)) return invalid("N and K must be from 1 to 2^20");
+  if (g->n > ((int64_t)1 << 31) - 1024) {  // the kernel counts rows, up to a tile beyond the last, in 32 bits
+    set_error("the products take at most 2^31 - 1024 rows");
+    return DG_ERR_UNSUPPORTED;
+  }
+  if ((a_count > 0 && !a) || (b_count > 0 && !b) || (out_count > 0 && !out)) return invalid("a pointer is NULL");
+  if (overlaps(a, a_count * sizeof(float), out, out_count * sizeof(float)) ||
+      overlaps(b, b_count * sizeof(float), out, out_count * sizeof(float)))
+    return invalid("the result overlaps an input");
+  return DG_OK;
+}
+
+dg_status_t dg_linear_fwd(dg_graph_t g, const float* X, int32_t K, const float* W, int32_t N,
+                          const float* row_scale, const float* bias, int32_t relu, float* Y, void* stream) {
+  const int64_t n = g ? g->n : 0;
+  if (dg_status_t st = check_linear(g, N, K, X, n * K, W, (int64_t)N * K, Y, n * N)) return st;
+  if (n == 0) return DG_OK;
+  return linear_fwd(g, X, K, W, N, row_scale, bias, relu != 0, Y, (cudaStream_t)stream);
+}
+
+dg_status_t dg_linear_bwd_input(dg_graph_t g, const float* G, int32_t N, const float* W, int32_t K, float* dX,
+                                void* stream) {
+  const int64_t n = g ? g->n : 0;
+  if (dg_status_t st = check_linear(g, N, K, G, n * N, W, (int64_t)N * K, dX, n * K)) return st;
+  if (n == 0) return DG_OK;
+  return linear_bwd_input(g, G, N, W, K, dX, (cudaStream_t)stream);
+}
+
+dg_status_t dg_linear_bwd_weight(dg_graph_t g, const float* G, int32_t N, const float* X, int32_t K, float* dW,
+                                 void* stream) {
+  const int64_t n = g ? g->n : 0;
+  if (dg_status_t st = check_linear(g, N, K, G, n * N, X, n * K, dW, (int64_t)N * K)) return st;
+  if (n == 0) {
+    DG_CUDA(cudaMemsetAsync(dW, 0, (size_t)N * K * sizeof(float), (cudaStream_t)stream));
+    return DG_OK;
+  }
+  return linear_bwd_weight(g, G, N, X, K, dW, (cudaStream_t)stream);
+}
+
 static dg_status_t check_loss(const Graph* g, int32_t C, int64_t count, const void* stats, bool pointers) {
   if (!g) return invalid("graph handle is NULL");
   if (C < 1 || C > (1 << 20)) return invalid("C must be from 1 to 2^20");

@@ -237,6 +237,14 @@ dg_status_t layer_fwd(const Graph* g, float* Y, int32_t F, const float* scale, c
 dg_status_t layer_bwd(const Graph* g, const float* dOut, const float* out, int32_t F, const float* scale,
                       float* G, float* dbias, cudaStream_t s);
 
+// dg_linear.cu
+dg_status_t linear_fwd(const Graph* g, const float* X, int32_t K, const float* W, int32_t N, const float* scale,
+                       const float* bias, bool relu, float* Y, cudaStream_t s);
+dg_status_t linear_bwd_input(const Graph* g, const float* G, int32_t N, const float* W, int32_t K, float* dX,
+                             cudaStream_t s);
+dg_status_t linear_bwd_weight(const Graph* g, const float* G, int32_t N, const float* X, int32_t K, float* dW,
+                              cudaStream_t s);
+
 // dg_loss.cu
 dg_status_t loss_fwd(const Graph* g, const float* logits, int32_t C, const int64_t* index, int64_t count,
                      const int64_t* labels, float* stats, float* result, cudaStream_t s);

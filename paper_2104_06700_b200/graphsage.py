@@ -1,8 +1,8 @@
 """Full-batch GraphSAGE with the GCN aggregator (Section 5.1 of the paper, Models and
 Parameters), as the composite workload the epoch-time metric is quoted on.
 
-libdgagg runs the aggregation with the own row, the elementwise passes of a layer and the loss; the
-GEMMs and Adam are torch's.  Per layer  z_v = (sum_{u in N(v)} h_u + h_v) / (deg(v) + 1),
+libdgagg runs the aggregation with the own row, the matrix products of large layers, the elementwise passes
+of a layer and the loss; the products of small layers and Adam are torch's.  Per layer  z_v = (sum_{u in N(v)} h_u + h_v) / (deg(v) + 1),
 h'_v = act(z_v W + b)  (aggregate first, then the Linear: Table 8 of the paper lists the aggregation
 widths 100, 256, 256 for the 3-layer model, i.e. the layers' input widths), ReLU between layers, none
 after the last, softmax cross-entropy on a training mask, Adam.  The features need no gradient, so an
@@ -74,6 +74,16 @@ def _weight_grad(G: torch.Tensor, X: torch.Tensor) -> torch.Tensor:
     return dW.addmm_(G[m:].t(), X[m:]) if m < n else dW
 
 
+def _large(graph: "binding.Graph", weight: torch.Tensor) -> bool:
+    """Whether the library's products serve the layer.  From 2^29 multiplications on they are faster than torch's fp32
+    GEMMs in all three directions, if neither width is small: their tiles are 128 rows by whole steps of 16 columns.  us
+    library / torch, forward with its epilogue, gradient of the input, of the weights: 245 k rows of 256 x 256 186 / 660,
+    187 / 569, 267 / 594; of 256 x 47 160 / 198, 100 / 173, 173 / 166; 8 k of 256 x 256 23 / 31, 21 / 27, 31 / 36; but 100 k of
+    64 x 41 49 / 43, 39 / 29, 49 / 44; of 602 x 16 158 / 115, 160 / 94, 195 / 123."""
+    N, K = weight.shape
+    return min(N, K) >= 40 and graph.n * N * K >= 1 << 29
+
+
 def _with_own_row(graph: "binding.Graph", M: torch.Tensor, bf16: bool, transposed: bool) -> torch.Tensor:
     """(A + I) M, or with ``transposed`` (A^T + I) M.  bf16: the gathered rows are rounded; the own row too where
     the handle adds it itself."""
@@ -88,7 +98,8 @@ def _with_own_row(graph: "binding.Graph", M: torch.Tensor, bf16: bool, transpose
 class _GcnLayer(torch.autograd.Function):
     """One layer  act(D (A M + M) W^T + b),  D = diag(1 / (deg + 1)),  with the own row added inside the
     aggregation kernel.  D is applied after the GEMM, forward together with bias and ReLU, backward together
-    with the ReLU's mask and the sums of the bias: one elementwise pass over n x F each way (autograd's
+    with the ReLU's mask and the sums of the bias: one elementwise pass over n x F each way, none forward where the
+    library computes the product too (autograd's
     operations made two forward and three backward; 245 k vertices, 256 wide: 85 us a pass).
 
     ``project``: D ((A + I) (M W^T)) + b instead, the narrower product aggregated."""
@@ -97,11 +108,15 @@ class _GcnLayer(torch.autograd.Function):
     def forward(ctx, M, weight, bias, graph, inv_deg1, relu: bool, project: bool, bf16: bool):
         M = M.contiguous()
         if project:
-            Z, X = _with_own_row(graph, M @ weight.t(), bf16, False), M
+            X = M
+            Z = graph.dg_linear_fwd(M, weight.contiguous()) if _large(graph, weight) else M @ weight.t()
+            out = graph.dg_layer_fwd(_with_own_row(graph, Z, bf16, False), inv_deg1, bias.contiguous(), relu)
         else:
             X = _with_own_row(graph, M, bf16, False)
-            Z = X @ weight.t()
-        out = graph.dg_layer_fwd(Z, inv_deg1, bias.contiguous(), relu)
+            if _large(graph, weight):
+                out = graph.dg_linear_fwd(X, weight.contiguous(), inv_deg1, bias.contiguous(), relu)
+            else:
+                out = graph.dg_layer_fwd(X @ weight.t(), inv_deg1, bias.contiguous(), relu)
         ctx.graph, ctx.relu, ctx.project, ctx.bf16 = graph, relu, project, bf16
         # M is the layer's input (another layer's output, which that one keeps) and costs no memory
         ctx.save_for_backward(X, weight, inv_deg1, out if relu else None, M, bias)
@@ -119,10 +134,16 @@ class _GcnLayer(torch.autograd.Function):
         G, db = graph.dg_layer_bwd(dOut.contiguous(), out, inv_deg1)
         if ctx.project and (needs[0] or needs[1]):
             G = _with_own_row(graph, G, ctx.bf16, True)
-        dW = _weight_grad(G, X) if needs[1] else None
-        dM = None
+        large = _large(graph, weight)
+        dW = dM = None
+        if needs[1]:
+            # without scratch the library would sum all rows in a few blocks
+            if large and graph.dg_graph_get_param("scratch_mb"):
+                dW = graph.dg_linear_bwd_weight(G, X)
+            else:
+                dW = _weight_grad(G, X)
         if needs[0]:
-            dM = G @ weight
+            dM = graph.dg_linear_bwd_input(G, weight.contiguous()) if large else G @ weight
             if not ctx.project:
                 dM = _with_own_row(graph, dM, ctx.bf16, True)
         return dM, dW, db if needs[2] else None, None, None, None, None, None
