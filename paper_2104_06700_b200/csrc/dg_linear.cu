@@ -73,6 +73,7 @@ struct LinearArgs {
   int relu;
   float* out;               // slice s writes rows_a x rows_b at out + s * rows_a * rows_b
   int vector_out;
+  int linear_out;           // a tile's results are one stretch of memory that fits the staging tiles
 };
 
 __device__ __forceinline__ uint32_t smem_address(const void* p) { return (uint32_t)__cvta_generic_to_shared(p); }
@@ -277,6 +278,7 @@ __global__ void __launch_bounds__(kThreads, 1) linear_kernel(const LinearArgs a)
   __shared__ uint64_t done[2];     // the matrix instructions of a stage have finished
   __shared__ uint64_t arrived[2];  // a stage's chunk of the image has arrived
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  const int items = a.tiles_m * a.tiles_n * a.slices;
   const uint32_t filled0 = smem_address(filled), done0 = smem_address(done), arrived0 = smem_address(arrived);
   if (warp == kWarps) {
     asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], 512;" ::"r"(smem_address(&tmem_base))
@@ -296,7 +298,6 @@ __global__ void __launch_bounds__(kThreads, 1) linear_kernel(const LinearArgs a)
   __syncthreads();
   asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
   const uint32_t tmem = tmem_base;
-  const int items = a.tiles_m * a.tiles_n * a.slices;
   bool good = true;
   // Chunk j of the stream, counted over all tiles: its stage is j % 2, and it completes the phases of a barrier in turn.
   // A thread waits for every phase of a barrier, in order, before the next can complete.
@@ -376,9 +377,31 @@ __global__ void __launch_bounds__(kThreads, 1) linear_kernel(const LinearArgs a)
           warp < 6 ? smem + S::kTileAt + warp * kTileBytes
                    : warp < 12 ? smem + (j & 1) * operand_bytes(kM) + (warp - 6) * kTileBytes
                                : smem + S::kRingAt + slot * S::kRaw + (warp - 12) * kTileBytes);
+      if (a.linear_out) {
+        // Rows of a few columns that allow no vectors: written row by row they cost 20 cycles for every 16 numbers.
+        float* line = reinterpret_cast<float*>(smem + S::kTileAt);
+        const int N = a.rows_b;
+        float* mine = line + ((warp & 3) * 32 + lane) * N + c0;
+        const int cols = min(c1, N) - c0;  // at most 16
+        const float bias = a.bias && lane < cols ? __ldg(a.bias + c0 + lane) : 0.f;
+#pragma unroll
+        for (int i = 0; i < 16; ++i) {
+          const float x = i % 2 ? acc[i / 2].y : acc[i / 2].x;
+          const float y = max_nan(fmaf(x, s, __shfl_sync(0xffffffffu, bias, i)), least);
+          if (i < cols) mine[i] = y;
+        }
+        asm volatile("bar.sync 1, %0;" ::"n"(kWorkers) : "memory");
+        const int count = min(kM, a.rows_a - rt.m0) * N;
+        float* to = out + (int64_t)rt.m0 * N;  // 128 rows on from the matrix's start: aligned as that is
+        for (int i = 4 * threadIdx.x; i < count; i += 4 * kWorkers) {
+          if (i + 4 <= count) *reinterpret_cast<float4*>(to + i) = *reinterpret_cast<const float4*>(line + i);
+          else
+            for (int k = i; k < count; ++k) to[k] = line[k];
+        }
+      }
 #pragma unroll
       for (int b = 0; b < S::kColumns / 32; ++b) {
-        if (c0 + 32 * b >= c1) break;
+        if (c0 + 32 * b >= c1 || a.linear_out) break;
         const int n = rt.n0 + c0 + 32 * b, cols = min(min(32, c1 - c0 - 32 * b), a.rows_b - n);
         __syncwarp();
 #pragma unroll
@@ -393,8 +416,9 @@ __global__ void __launch_bounds__(kThreads, 1) linear_kernel(const LinearArgs a)
           if (a.bias && c < cols)
             bias = make_float4(__ldg(a.bias + n + c), __ldg(a.bias + n + c + 1), __ldg(a.bias + n + c + 2),
                                __ldg(a.bias + n + c + 3));
-#pragma unroll
-          for (int i = 0; i < 8; ++i) {
+          float* to = out + (int64_t)(row0 + (lane >> 3)) * a.rows_b + n + c;
+#pragma unroll 1
+          for (int i = 0; i < 8; ++i, to += 4 * (int64_t)a.rows_b) {
             const int r = 4 * i + (lane >> 3);
             const float sr = __shfl_sync(0xffffffffu, s, r);
             float4 y = *reinterpret_cast<const float4*>(tile + r * 32 + ((q ^ r) & 7) * 4);
@@ -402,12 +426,11 @@ __global__ void __launch_bounds__(kThreads, 1) linear_kernel(const LinearArgs a)
             y.y = max_nan(fmaf(y.y, sr, bias.y), least);
             y.z = max_nan(fmaf(y.z, sr, bias.z), least);
             y.w = max_nan(fmaf(y.w, sr, bias.w), least);
-            if (row0 + r < a.rows_a && c < cols)
-              *reinterpret_cast<float4*>(out + (int64_t)(row0 + r) * a.rows_b + n + c) = y;
+            if (row0 + r < a.rows_a && c < cols) *reinterpret_cast<float4*>(to) = y;
           }
         } else {
           const float bias = a.bias && lane < cols ? __ldg(a.bias + n + lane) : 0.f;
-#pragma unroll 4
+#pragma unroll 1
           for (int r = 0; r < 32; ++r) {
             const float sr = __shfl_sync(0xffffffffu, s, r);
             const float y = tile[r * 32 + ((lane >> 2 ^ r) & 7) * 4 + (lane & 3)];
@@ -581,6 +604,7 @@ void fill(LinearArgs* a) {
   a->vector_a = aligned_rows(a->A, a->lda, 4);
   a->vector_b = aligned_rows(a->B, a->ldb, 4);
   a->vector_out = aligned_rows(a->out, a->rows_b, 4);
+  a->linear_out = !a->vector_out && a->rows_b <= 48 && a->slices == 1 && aligned_rows(a->out, 4, 4);
 }
 
 // A layer's product with its weights as B: split first, where there is memory for it.

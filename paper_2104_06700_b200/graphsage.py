@@ -78,7 +78,7 @@ def _large(graph: "binding.Graph", weight: torch.Tensor) -> bool:
     """Whether the library's products serve the layer.  From 2^29 multiplications on they are faster than torch's fp32
     GEMMs in all three directions, if neither width is small: their tiles are 128 rows by whole steps of 16 columns.  us
     library / torch, forward with its epilogue, gradient of the input, of the weights: 245 k rows of 256 x 256 186 / 660,
-    187 / 569, 267 / 594; of 256 x 47 160 / 198, 100 / 173, 173 / 166; 8 k of 256 x 256 23 / 31, 21 / 27, 31 / 36; but 100 k of
+    187 / 569, 267 / 594; of 256 x 47 120 / 198, 100 / 173, 173 / 166; 8 k of 256 x 256 23 / 31, 21 / 27, 31 / 36; but 100 k of
     64 x 41 49 / 43, 39 / 29, 49 / 44; of 602 x 16 158 / 115, 160 / 94, 195 / 123."""
     N, K = weight.shape
     return min(N, K) >= 40 and graph.n * N * K >= 1 << 29
