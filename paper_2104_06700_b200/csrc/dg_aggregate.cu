@@ -228,6 +228,7 @@ dg_status_t aggregate_run(const Graph* g, const ApArgs& a0, const SelfArgs& sa0,
 
   const double budget = (double)g->l2_budget_bytes;
   const double avg_len = (double)g->nnz / (double)a.n;
+  a.long_rows = avg_len >= 24.0;
   const int64_t cap = 128LL * vec;
   int64_t slice;
   int nb = 1;
@@ -235,7 +236,7 @@ dg_status_t aggregate_run(const Graph* g, const ApArgs& a0, const SelfArgs& sa0,
     slice = g->slice_features < cap ? g->slice_features : cap;
     if (slice > a.F) slice = a.F;
   } else {
-    slice = avg_len >= 24.0 && 2 * a.F >= 96LL * vec ? 32LL * vec : 64LL * vec;
+    slice = a.long_rows && 2 * a.F >= 96LL * vec ? 32LL * vec : 64LL * vec;
     if (slice > a.F) slice = a.F;
   }
   if (g->source_blocks > 0) {

@@ -193,7 +193,7 @@ struct Shape {
   static constexpr int NG = 32 / G;  // edges one warp-wide load instruction covers
   // load steps in flight per lane (fewer when a step is several vectors wide), and no more
   // steps than one 32-edge batch holds
-  static constexpr int U0 = CPL == 1 ? 8 : (CPL == 2 ? 4 : (VEC <= 2 ? 4 : 2));
+  static constexpr int U0 = CPL == 1 ? 8 : (CPL == 2 ? 4 : (VEC <= 2 && CPL == 4 ? 4 : 2));
   static constexpr int U = (U0 * NG > 32) ? (32 / NG) : U0;
 };
 
@@ -555,6 +555,15 @@ dg_status_t dispatch_shape(const ApArgs& a, const SelfArgs& sa, int slices, cuda
   if (chunks <= 8) return launch_variant<E, VEC, 8, 1, SCALED, SELF>(a, sa, slices, s);
   if (chunks <= 16) return launch_variant<E, VEC, 16, 1, SCALED, SELF>(a, sa, slices, s);
   if (chunks <= 32) return launch_variant<E, VEC, 32, 1, SCALED, SELF>(a, sa, slices, s);
+  // 33 to 44 vectors in half a warp, three each: of 32 lanes with two each a third would idle.  us of the forward sum and
+  // the mean's backward pass, two / three each: F = 172, 1.2 M edges 78.6, 84.3 / 72.2, 74.6; 62 M 4612, 4834 / 4744, 4762;
+  // 7.9 M in rows of 420 368, 338 / 314, 317; F = 136 76.3, 81.5 / 69.2, 71.4; 360, 336 / 289, 279.  48 vectors are no faster,
+  // nor are rows of under 24 entries (14.5: F = 172 826, 1941 / 839, 1940).  The same with eight or four lanes for 17 to 24
+  // or 9 to 12 vectors: 0.83 to 1.28 of the time, faster only in long rows.
+  if constexpr (E::kBytes == 4 && VEC == 4) {
+    if (chunks > 32 && chunks <= 44 && a.long_rows)
+      return launch_variant<E, VEC, 16, 3, SCALED, SELF>(a, sa, slices, s);
+  }
   if (chunks <= 64) return launch_variant<E, VEC, 32, 2, SCALED, SELF>(a, sa, slices, s);
   return launch_variant<E, VEC, 32, 4, SCALED, SELF>(a, sa, slices, s);
 }

@@ -136,6 +136,7 @@ struct ApArgs {
   int32_t accumulate;         // source-blocked pass after the first: add to what Y holds
   int32_t overlap;            // host side: launch while the previous kernel (the copy) drains, see launch_kernel
   int32_t few_blocks;         // host side: the grid is small, see ap_kernel
+  int32_t long_rows;          // host side: the mean degree is 24 or more
   int32_t mean_factors;       // host side: w are the factors 1 / deg (+ 1) of the mean's backward pass alone
 };
 

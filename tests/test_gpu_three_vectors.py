@@ -1,0 +1,26 @@
+"""Slices of 33 to 44 vectors, where a lane takes three of them, and the widths beside them, on graphs with rows long
+enough for that: against the oracle, with weights, own rows, cut rows and padded copies."""
+import numpy as np
+import pytest
+
+from paper_2104_06700_b200 import binding, synth
+from parity_util import check_fwd_bwd, check_transpose
+from test_gpu_chunks import graph_of, handle, host
+
+pytestmark = pytest.mark.gpu
+DEV = "cuda"
+# rows around one and several pieces; mean degrees 24.2 and 23.8
+LENGTHS = [0, 1, 7, 8, 9, 31, 32, 33, 64, 65, 161, 300, 1025, 3, 2]
+
+
+@pytest.mark.parametrize("F", [128, 132, 136, 172, 176, 180, 171])
+@pytest.mark.parametrize("weighted,self_loops", [(False, 0), (True, 0), (False, 1)])
+@pytest.mark.parametrize("n", [72, 73])
+def test_three_vectors_per_lane(F, weighted, self_loops, n):
+    assert np.sum(LENGTHS) == 1741
+    sg = graph_of(LENGTHS, n, F, weighted)
+    g = handle(sg, self_loops)
+    csc = check_transpose(g, *host(sg))
+    H, G = synth.features(sg.n, F, 1, DEV), synth.features(sg.n, F, 2, DEV)
+    for op in (binding.DG_OP_SUM, binding.DG_OP_MEAN):
+        check_fwd_bwd(g, host(sg), H, G, op, csc, self_loops=bool(self_loops))
