@@ -99,18 +99,25 @@ __global__ void __launch_bounds__(kGenBlock, 4) edge_grad_kernel(const EdgeGradA
       [](int, int) {});
 }
 
-// Lanes per edge.  Half of what covers the slice, so that a lane takes two vectors of a row: the shuffles (an id per
-// edge and load, and the butterfly) then serve twice the loads, and they share a pipe with them.  A quarter where that leaves
-// fewer lanes without a vector (25 vectors: 16 lanes; 43: 16, not 32).  us with lanes for all vectors / this rule: 39.6 M
-// edges, F = 64 778 / 631, 100 1398 / 1127, 172 2094 / 1660; 31 M edges (from DRAM), F = 64 1117 / 1187, 172 3323 / 2929;
-// but two vectors on one lane are slower (F = 8 331 / 379).
-int lanes_per_edge(int nvec) {
-  if (nvec <= 2) return nvec;
-  int half = 2, quarter = 4;
-  while (half < 32 && 2 * half < nvec) half *= 2;
-  while (quarter < 32 && 4 * quarter < nvec) quarter *= 2;
-  auto slots = [&](int lanes) { return (nvec + lanes - 1) / lanes * lanes; };
-  return quarter < half && slots(quarter) < slots(half) ? quarter : half;
+// Lanes per edge.  Lanes for all vectors up to 32, or half of those: a lane then takes two vectors of a row, and the shuffles
+// (an id per edge and load, and the butterfly), which share a pipe with the loads, serve twice the loads.  us with all / half,
+// rows of 422 entries (L2), of 50 (376 MB), of 14.5 (306 MB and less):
+//    4 vectors   456 / 386   1626 / 1324   188 / 159; two lanes 380   1233   137: two lanes, for every length
+//    5           458 / 636   1762 / 2014   196 / 261: up to 8 otherwise all
+//   12           779 / 617   2839 / 2802   255 / 303: from 9 on half where a row has edges for the groups, 32
+//   16           774 / 628   2825 / 3011   254 / 324: 13 to 16 only where L2 keeps the matrix (36 entries, 77 MB: 325 / 335)
+//   32          1399 / 1139  5009 / 4866   360 / 386
+// Half of that again where fewer lanes are then without a vector: 12 vectors (four lanes 632, 2505), 20 (eight lanes 805,
+// 4115 against 1070, 4349), and for every length 43 (16 lanes against 32: 1649 / 2149, 7508 / 8509, 537 / 546).
+int lanes_per_edge(int nvec, double entries, bool resident) {
+  if (nvec == 4) return 2;
+  int lanes = 1;
+  while (lanes < 32 && lanes < nvec) lanes *= 2;
+  const bool half = entries >= 32.0 && nvec > 8 && (resident || nvec <= 12 || nvec > 16);
+  if (half && nvec <= 32) lanes /= 2;
+  auto slots = [&](int l) { return (nvec + l - 1) / l * l; };
+  if ((half || nvec > 32) && nvec <= 2 * lanes && slots(lanes / 2) < slots(lanes)) lanes /= 2;
+  return lanes;
 }
 
 template <int VEC, int G>
@@ -122,8 +129,8 @@ dg_status_t launch_lanes(const EdgeGradArgs& a, cudaStream_t s) {
 }
 
 template <int VEC>
-dg_status_t launch_edge_grad(const EdgeGradArgs& a, cudaStream_t s) {
-  switch (lanes_per_edge(a.nvec)) {
+dg_status_t launch_edge_grad(const EdgeGradArgs& a, double entries, bool resident, cudaStream_t s) {
+  switch (lanes_per_edge(a.nvec, entries, resident)) {
     case 1: return launch_lanes<VEC, 1>(a, s);
     case 2: return launch_lanes<VEC, 2>(a, s);
     case 4: return launch_lanes<VEC, 4>(a, s);
@@ -184,6 +191,8 @@ dg_status_t edge_grad_run(const Graph* g, const float* H, const float* dOut, int
     }
   }
   const int per = kFineBlocks / nb;
+  const double entries = (double)g->nnz / (double)g->n / nb; // of a row, in a launch
+  const bool resident = nb > 1 || (double)g->n * (double)a.ld * 4.0 <= (double)g->l2_budget_bytes;
   for (int j = 0; j < nb && st == DG_OK; ++j) {
     if (nb > 1) {
       a.walk.seg_lo = g->split_csr + (size_t)(j * per) * (size_t)g->n;
@@ -193,7 +202,9 @@ dg_status_t edge_grad_run(const Graph* g, const float* H, const float* dOut, int
       a.f_lo = (int32_t)f0;
       a.nvec = (int32_t)((width - f0 < slice ? width - f0 : slice) / vec);
       a.accumulate = f0 > 0;
-      st = vec == 4 ? launch_edge_grad<4>(a, s) : vec == 2 ? launch_edge_grad<2>(a, s) : launch_edge_grad<1>(a, s);
+      st = vec == 4   ? launch_edge_grad<4>(a, entries, resident, s)
+           : vec == 2 ? launch_edge_grad<2>(a, entries, resident, s)
+                      : launch_edge_grad<1>(a, entries, resident, s);
     }
   }
   pool_free(padded_h, s);

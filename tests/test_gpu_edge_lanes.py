@@ -27,3 +27,17 @@ def test_lanes_per_edge(tiny, F):
         ref, mag = oracle.edge_weight_grad(to_np(tiny.rowptr), to_np(tiny.colidx), to_np(H), to_np(G), op)
         assert_within_bound(to_np(dW), ref, mag, f"F = {F}")
         assert torch.equal(dW, g.dg_aggregate_edge_grad(H, G, op))
+
+
+# rows of 32 entries and more, where lanes are halved or not: 4, 8/9, 12/13, 16/17, 24/25, 32/33, 48/49 vectors
+@pytest.mark.parametrize("budget", [1, 64])
+@pytest.mark.parametrize("F", [4 * k for k in (4, 8, 9, 12, 13, 16, 17, 24, 25, 32, 33, 48, 49)] + [13, 26, 47])
+def test_lanes_per_edge_long_rows(F, budget):
+    sg = synth.tiny(seed=4, n=6000, nnz=210_000)
+    g = make_graph(sg)
+    g.dg_graph_set_param("l2_budget_mb", budget)  # 1 MB: the matrix counts as one that L2 does not keep
+    H, G = synth.features(sg.n, F, 1, DEV), synth.features(sg.n, F, 2, DEV)
+    dW = g.dg_aggregate_edge_grad(H, G, binding.DG_OP_MEAN)
+    ref, mag = oracle.edge_weight_grad(to_np(sg.rowptr), to_np(sg.colidx), to_np(H), to_np(G), binding.DG_OP_MEAN)
+    assert_within_bound(to_np(dW), ref, mag, f"F = {F}")
+    assert torch.equal(dW, g.dg_aggregate_edge_grad(H, G, binding.DG_OP_MEAN))
