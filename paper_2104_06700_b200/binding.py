@@ -130,6 +130,17 @@ def _holds(t: Optional[torch.Tensor], count: int, name: str) -> None:
         raise ValueError(f"{name} must hold {count} values, got {t.numel()}")
 
 
+def _is_matrix(t: torch.Tensor, rows: int, columns: int, name: str) -> None:
+    """A product is refused where its sizes do not fit: wider rows would be read as more of narrower ones."""
+    if tuple(t.shape) != (rows, columns):
+        raise ValueError(f"{name} must be {rows} x {columns}, got {' x '.join(map(str, t.shape))}")
+
+
+def _has(t: Optional[torch.Tensor], count: int, name: str) -> None:
+    if t is not None and t.numel() != count:
+        raise ValueError(f"{name} must have {count} values, got {t.numel()}")
+
+
 # The handle of the current stream of the current device.  torch.cuda.current_stream() builds two
 # Python objects on the way to it: 3.2 us, a third of what a call on a small graph took on the host.
 # A torch without CUDA, or one that names them differently, has neither: then the public call serves.
@@ -390,11 +401,9 @@ class Graph:
                       bias: Optional[torch.Tensor] = None, relu: bool = False, stream=None) -> torch.Tensor:
         """X W^T, or act(row_scale * (X W^T) + bias)."""
         N, K = W.shape
-        _holds(X, self.n * K, "X")
-        if row_scale is not None:
-            _holds(row_scale, self.n, "row_scale")
-        if bias is not None:
-            _holds(bias, N, "bias")
+        _is_matrix(X, self.n, K, "X")
+        _has(row_scale, self.n, "row_scale")
+        _has(bias, N, "bias")
         Y = X.new_empty((self.n, N))
         _check(lib().dg_linear_fwd(self._h, _dev_ptr(X, torch.float32, "X"), K, _dev_ptr(W, torch.float32, "W"), N,
                                    _dev_ptr(row_scale, torch.float32, "row_scale"),
@@ -405,7 +414,7 @@ class Graph:
     def dg_linear_bwd_input(self, G: torch.Tensor, W: torch.Tensor, stream=None) -> torch.Tensor:
         """G W."""
         N, K = W.shape
-        _holds(G, self.n * N, "G")
+        _is_matrix(G, self.n, N, "G")
         dX = G.new_empty((self.n, K))
         _check(lib().dg_linear_bwd_input(self._h, _dev_ptr(G, torch.float32, "G"), N,
                                          _dev_ptr(W, torch.float32, "W"), K, _dev_ptr(dX, torch.float32, "dX"),
@@ -415,8 +424,8 @@ class Graph:
     def dg_linear_bwd_weight(self, G: torch.Tensor, X: torch.Tensor, stream=None) -> torch.Tensor:
         """G^T X."""
         N, K = G.shape[1], X.shape[1]
-        _holds(G, self.n * N, "G")
-        _holds(X, self.n * K, "X")
+        _is_matrix(G, self.n, N, "G")
+        _is_matrix(X, self.n, K, "X")
         dW = G.new_empty((N, K))
         _check(lib().dg_linear_bwd_weight(self._h, _dev_ptr(G, torch.float32, "G"), N,
                                           _dev_ptr(X, torch.float32, "X"), K, _dev_ptr(dW, torch.float32, "dW"),

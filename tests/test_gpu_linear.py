@@ -83,6 +83,12 @@ def test_arguments_are_checked():
         g.dg_linear_fwd(X[1:], W)
     with pytest.raises(ValueError):
         g.dg_linear_bwd_weight(G[:, :4].contiguous(), X[1:])
+    wide = torch.zeros(40, 12, device=DEV)  # holds enough values for every operand
+    for call in (lambda: g.dg_linear_fwd(wide, W), lambda: g.dg_linear_fwd(X.view(8, 40), W),
+                 lambda: g.dg_linear_fwd(X, W, bias=wide[0]), lambda: g.dg_linear_fwd(X, W, scale.repeat(2, 1)),
+                 lambda: g.dg_linear_bwd_input(wide, W), lambda: g.dg_linear_bwd_weight(torch.zeros(41, 8, device=DEV), X)):
+        with pytest.raises(ValueError):
+            call()
     lib = binding.lib()
     assert lib.dg_linear_fwd(g._h, X.data_ptr(), 8, W.data_ptr(), 8, None, None, 0, X.data_ptr() + 16, None) \
         == binding.DG_ERR_INVALID_ARG
