@@ -224,8 +224,8 @@ dg_status_t dg_layer_bwd(dg_graph_t g, const float* dOut, const float* out, int3
  *                dg_layer_fwd follows: Y = act(row_scale[v] * Y + bias).
  *   bwd_input:   dX = G W (n x K).
  *   bwd_weight:  dW = G^T X (N x K), always summed in the same order.
- * The result must not overlap an input.  bwd_weight without scratch ("scratch_mb" = 0) sums all rows in a few thread
- * blocks: correct, and slow.  Asynchronous on `stream`.
+ * The result must not overlap an input.  bwd_weight sums slices of the rows in scratch, up to 9.3 MiB of it; with
+ * less memory it takes fewer slices and keeps fewer SMs busy, without any it sums all rows in a few thread blocks.  Asynchronous on `stream`.
  */
 dg_status_t dg_linear_fwd(dg_graph_t g, const float* X, int32_t K, const float* W, int32_t N,
                           const float* row_scale, const float* bias, int32_t relu, float* Y, void* stream);

@@ -684,11 +684,13 @@ dg_status_t linear_bwd_weight(const Graph* g, const float* G, int32_t N, const f
   int64_t slices = g->sm_count / tiles;
   const int64_t most = (g->n + 16 * kChunk - 1) / (16 * kChunk);
   if (slices > most) slices = most;
-  if (slices < 1) slices = 1;
+  // Fewer where the scratch holds fewer, down to one, which takes no memory.  245 k rows of 256 x 256: 37 slices 269 us,
+  // 20 481, 16 597, 8 1186, 4 2342, one 9317.
+  const int64_t slice_bytes = (int64_t)N * K * (int64_t)sizeof(float);
+  if (slices > (g->scratch_mb << 20) / slice_bytes) slices = (g->scratch_mb << 20) / slice_bytes;
   void* partial = nullptr;
-  if (slices > 1 &&
-      scratch_alloc(g, (size_t)slices * (size_t)N * (size_t)K * sizeof(float), s, &partial) != cudaSuccess)
-    slices = 1;
+  while (slices > 1 && scratch_alloc(g, (size_t)(slices * slice_bytes), s, &partial) != cudaSuccess) slices /= 2;
+  if (slices < 1) slices = 1;
   int64_t slice = (g->n + slices - 1) / slices;
   slice = (slice + kChunk - 1) / kChunk * kChunk;
   a.depth_slice = (int)(slice < g->n ? slice : g->n);

@@ -137,8 +137,9 @@ class _GcnLayer(torch.autograd.Function):
         large = _large(graph, weight)
         dW = dM = None
         if needs[1]:
-            # without scratch the library would sum all rows in a few blocks
-            if large and graph.dg_graph_get_param("scratch_mb"):
+            # with less scratch the library sums in so few blocks that torch's slices are as fast: 245 k rows of 256 x 256
+            # with 5 and 4 MiB 481 and 597 us, torch 594; of 602 x 256 with 5 MiB 1507, torch 1367
+            if large and graph.dg_graph_get_param("scratch_mb") >= 7:
                 dW = graph.dg_linear_bwd_weight(G, X)
             else:
                 dW = _weight_grad(G, X)

@@ -62,6 +62,20 @@ def test_products_without_scratch(n, K, N):
     check(n, K, N, scratch=False)
 
 
+@pytest.mark.parametrize("limit", [1, 2])
+def test_a_scratch_limit_costs_slices_and_not_all_of_them(limit):
+    n, K, N = 40000, 256, 100  # 37 slices of 100 KiB
+    X, W, G, scale, bias = operands(n, K, N)
+    g = empty_graph(n)
+    g.dg_graph_set_param("scratch_mb", limit)
+    g.dg_linear_bwd_weight(G, X)
+    before = binding.dg_kernel_launch_count()
+    dW = g.dg_linear_bwd_weight(G, X)
+    assert binding.dg_kernel_launch_count() - before == 2  # the products and the sum of the slices
+    want, size = G.double().t() @ X.double(), G.double().abs().t() @ X.double().abs()
+    assert bool(((dW.double() - want).abs() <= bound(n, 148, size)).all())
+
+
 def test_infinities_and_nan():
     """As torch's GEMM, element for element."""
     X, W, G, scale, bias = operands(700, 70, 50)
