@@ -416,6 +416,10 @@ dg_status_t dg_aggregate_edge_grad(dg_graph_t g, const float* H, const float* dO
  * Graph attribute (not a tuning knob: it changes the result):
  *   "self_loops"       0 (default) or 1: every vertex is its own in-neighbour with weight 1, see
  *                      dg_aggregate_fwd / dg_aggregate_bwd; set it before dg_graph_transpose
+ * Read only:
+ *   "expired_waits"    thread blocks of dg_linear_* that gave up a wait inside the kernel (seconds without progress;
+ *                      0 unless something is wrong) on the current device since the library was loaded.  Their results
+ *                      are NaN.  The call waits for the device.
  * Changing "heavy_threshold" or "rows_per_block" waits for the whole device, shares the rows out
  * anew and waits again: a rare, synchronous call.  CUDA graphs captured before it must not be launched
  * afterwards.  If it fails the handle is as it was.

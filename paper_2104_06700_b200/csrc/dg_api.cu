@@ -709,6 +709,7 @@ dg_status_t dg_graph_get_param(dg_graph_t g, const char* name, int64_t* value) {
   if (!strcmp(name, "self_loops")) { *value = g->self_loops; return DG_OK; }
   if (!strcmp(name, "scratch_mb")) { *value = g->scratch_mb; return DG_OK; }
   if (!strcmp(name, "heavy_blocks_per_sm")) { *value = g->heavy_blocks_per_sm; return DG_OK; }
+  if (!strcmp(name, "expired_waits")) return linear_expired(value);
   return invalid("unknown parameter name");
 }
 

@@ -245,6 +245,7 @@ dg_status_t linear_bwd_input(const Graph* g, const float* G, int32_t N, const fl
                              cudaStream_t s);
 dg_status_t linear_bwd_weight(const Graph* g, const float* G, int32_t N, const float* X, int32_t K, float* dW,
                               cudaStream_t s);
+dg_status_t linear_expired(int64_t* blocks);  // blocks that gave up a wait, on the current device
 
 // dg_loss.cu
 dg_status_t loss_fwd(const Graph* g, const float* logits, int32_t C, const int64_t* index, int64_t count,

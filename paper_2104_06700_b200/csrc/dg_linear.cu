@@ -30,6 +30,8 @@
 namespace dg {
 namespace {
 
+__device__ unsigned long long g_expired;  // blocks that gave up a wait
+
 constexpr int kWorkers = 512, kWarps = kWorkers / 32, kThreads = kWorkers + 128;
 constexpr int kM = 128;
 constexpr int kChunk = 32;                // products of a sum per chunk: two matrix instructions per pair of parts
@@ -84,15 +86,23 @@ __device__ __forceinline__ void mbarrier_init(uint32_t bar, int count) {
 __device__ __forceinline__ void mbarrier_arrive(uint32_t bar) {
   asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(bar) : "memory");
 }
-// Waits for the phase of that parity; gives up after a second or a few.
-__device__ __forceinline__ bool mbarrier_wait(uint32_t bar, uint32_t parity) {
-  for (int i = 0; i < 1 << 20; ++i) {
+// Waits for the phase of that parity.  Gives up after 2^22 tries, all but the first half a microsecond apart, or when
+// another thread of the block has (the word at `expired`, in shared memory).  A loop without the time: the workers have no
+// registers left for it.
+__device__ __forceinline__ bool mbarrier_wait(uint32_t bar, uint32_t parity, uint32_t expired) {
+#pragma unroll 1
+  for (int i = 0; i < 1 << 22; ++i) {
     uint32_t done;
     asm volatile(
         "{\n\t.reg .pred p;\n\tmbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2;\n\tselp.u32 %0, 1, 0, p;\n\t}"
         : "=r"(done) : "r"(bar), "r"(parity) : "memory");
     if (done) return true;
+    if (i < 256) continue;
+    asm volatile("ld.volatile.shared.u32 %0, [%1];" : "=r"(done) : "r"(expired) : "memory");
+    if (done) return false;
+    __nanosleep(500);
   }
+  asm volatile("st.volatile.shared.u32 [%0], %1;" ::"r"(expired), "r"(1) : "memory");
   return false;
 }
 
@@ -267,9 +277,21 @@ __device__ __forceinline__ Item item_of(const LinearArgs& a, int i) {
   return t;
 }
 
+// After a wait that ran out: the workers make the block's results NaN.
+template <int kN>
+__device__ __noinline__ void give_up(const LinearArgs& a) {
+  if (threadIdx.x == 0) atomicAdd(&g_expired, 1ull);
+  for (int i = blockIdx.x; i < a.tiles_m * a.tiles_n * a.slices; i += gridDim.x) {
+    const Item t = item_of<kN>(a, i);
+    float* out = a.out + ((int64_t)t.slice * a.rows_a + t.m0) * a.rows_b + t.n0;
+    for (int e = threadIdx.x; e < kM * kN; e += kWorkers)
+      if (t.m0 + e / kN < a.rows_a && t.n0 + e % kN < a.rows_b) out[(int64_t)(e / kN) * a.rows_b + e % kN] = NAN;
+  }
+}
+
 // SPLIT_B: B has been split before (a.image).
 template <bool ALONG_A, bool ALONG_B, bool SPLIT_B>
-__global__ void __launch_bounds__(kThreads, 1) linear_kernel(const LinearArgs a) {
+__global__ void __launch_bounds__(kThreads, 1) linear_kernel(const __grid_constant__ LinearArgs a) {
   using S = Shape<SPLIT_B>;
   constexpr int kN = S::kN;
   extern __shared__ __align__(128) unsigned char smem[];
@@ -277,6 +299,9 @@ __global__ void __launch_bounds__(kThreads, 1) linear_kernel(const LinearArgs a)
   __shared__ uint64_t filled[2];   // the workers have written a stage, and read the tensor memory that it will go to
   __shared__ uint64_t done[2];     // the matrix instructions of a stage have finished
   __shared__ uint64_t arrived[2];  // a stage's chunk of the image has arrived
+  __shared__ uint64_t idle;        // after a wait that ran out: no matrix instruction is in flight
+  __shared__ int expired;          // a wait has run out: nothing more is started, the block's results are NaN
+  __shared__ int never;            // stays 0
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   const int items = a.tiles_m * a.tiles_n * a.slices;
   const uint32_t filled0 = smem_address(filled), done0 = smem_address(done), arrived0 = smem_address(arrived);
@@ -292,6 +317,8 @@ __global__ void __launch_bounds__(kThreads, 1) linear_kernel(const LinearArgs a)
       mbarrier_init(done0 + 8 * i, 1);
       mbarrier_init(arrived0 + 8 * i, 1);
     }
+    mbarrier_init(smem_address(&idle), 1);
+    expired = never = 0;
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
   }
   asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
@@ -301,7 +328,9 @@ __global__ void __launch_bounds__(kThreads, 1) linear_kernel(const LinearArgs a)
   bool good = true;
   // Chunk j of the stream, counted over all tiles: its stage is j % 2, and it completes the phases of a barrier in turn.
   // A thread waits for every phase of a barrier, in order, before the next can complete.
-  auto wait_for = [&](uint32_t barriers, int j) { good = good && mbarrier_wait(barriers + 8 * (j & 1), j >> 1 & 1); };
+  auto wait_for = [&](uint32_t barriers, int j) {
+    good = good && mbarrier_wait(barriers + 8 * (j & 1), j >> 1 & 1, smem_address(&expired));
+  };
 
   // The launch gives every thread 96 registers; the workers, whose sums take 64, get 112 and the last four warps keep 24:
   // 512 x 112 + 128 x 24 = 60416 of 640 x 96 = 61440.  Spills would go to memory: no first-level cache is left.
@@ -357,10 +386,6 @@ __global__ void __launch_bounds__(kThreads, 1) linear_kernel(const LinearArgs a)
       }
       asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
       if (item < 0) return;
-      if (!good) {  // a wait ran out
-#pragma unroll
-        for (int i = 0; i < S::kColumns / 2; ++i) acc[i] = make_float2(NAN, NAN);
-      }
       const Item rt = item_of<kN>(a, item);
       const int row0 = rt.m0 + (warp & 3) * 32, m = row0 + lane;
       const float s = a.scale && m < a.rows_a ? __ldg(a.scale + m) : 1.f;
@@ -442,7 +467,7 @@ __global__ void __launch_bounds__(kThreads, 1) linear_kernel(const LinearArgs a)
       asm volatile("bar.sync 1, %0;" ::"n"(kWorkers) : "memory");
 #pragma unroll
       for (int i = 0; i < S::kColumns / 2; ++i) acc[i] = make_float2(0.f, 0.f);
-      if (!__any_sync(0xffffffffu, again) || !good) return;
+      if (!__any_sync(0xffffffffu, again)) return;
       // a sum held an infinity or a NaN: the warp's elements that are NaN once more, a lane each
       __syncwarp();
 #pragma unroll 1
@@ -494,7 +519,7 @@ __global__ void __launch_bounds__(kThreads, 1) linear_kernel(const LinearArgs a)
       if (lane == 0) {
         const uint64_t a0 = operand(smem_address(smem), group_stride(kM));
         int j = 0;
-        for (int i = blockIdx.x; i < items; i += gridDim.x) {
+        for (int i = blockIdx.x; i < items && good; i += gridDim.x) {
           const Item now = item_of<kN>(a, i);
           const int width = tile_width<kN>(a.rows_b, now.n0), strb = group_stride(width);
           const uint64_t b0 = operand(smem_address(smem + S::kB), strb);
@@ -506,6 +531,7 @@ __global__ void __launch_bounds__(kThreads, 1) linear_kernel(const LinearArgs a)
             const uint32_t d = tmem + (uint32_t)((j & 1) * kN);
             if (SPLIT_B) wait_for(arrived0, j);
             wait_for(filled0, j);
+            if (!good) break;  // who waits for this chunk gives up too
             asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
             constexpr int kPairs[6][2] = {{0, 2}, {2, 0}, {1, 1}, {0, 1}, {1, 0}, {0, 0}};
 #pragma unroll
@@ -519,26 +545,37 @@ __global__ void __launch_bounds__(kThreads, 1) linear_kernel(const LinearArgs a)
                          : "memory");
           }
         }
+        if (!good) {  // the instructions in flight end before the tensor memory is given back
+          asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(
+                           smem_address(&idle))
+                       : "memory");
+          mbarrier_wait(smem_address(&idle), 0, smem_address(&never));
+        }
       }
       __syncwarp();
     } else if (warp == kWarps + 1) {
       // ---- the image's copies, two chunks ahead; one lane works
       if (SPLIT_B && lane == 0) {
         int j = 0;
-        for (int i = blockIdx.x; i < items; i += gridDim.x) {
+        for (int i = blockIdx.x; i < items && good; i += gridDim.x) {
           const Item now = item_of<kN>(a, i);
           const uint32_t bytes = operand_bytes(tile_width<kN>(a.rows_b, now.n0));
           const unsigned char* from = a.image + (int64_t)(now.n0 / kN) * now.chunks * operand_bytes(kN);
           for (int left = now.chunks; left > 0; --left, ++j, from += bytes) {
             if (j >= 2) wait_for(done0, j - 2);
+            if (!good) break;
             bulk_copy(smem_address(smem + S::kB + (j & 1) * operand_bytes(kN)), from, bytes, arrived0 + 8 * (j & 1));
           }
         }
+        // the copies in flight have arrived before the block ends; their readers wait for them otherwise
+        for (int k = j > 2 ? j - 2 : 0; !good && k < j; ++k)
+          mbarrier_wait(arrived0 + 8 * (k & 1), k >> 1 & 1, smem_address(&never));
       }
       __syncwarp();
     }
   }
   __syncthreads();
+  if (warp < kWarps && expired) give_up<kN>(a);
   if (warp == kWarps)
     asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, 512;" ::"r"(tmem) : "memory");
 }
@@ -635,6 +672,14 @@ dg_status_t with_weights(const Graph* g, LinearArgs a, cudaStream_t s) {
 }
 
 }  // namespace
+
+dg_status_t linear_expired(int64_t* blocks) {
+  unsigned long long count = 0;
+  DG_CUDA(cudaDeviceSynchronize());
+  DG_CUDA(cudaMemcpyFromSymbol(&count, g_expired, sizeof(count)));
+  *blocks = (int64_t)count;
+  return DG_OK;
+}
 
 dg_status_t linear_fwd(const Graph* g, const float* X, int32_t K, const float* W, int32_t N, const float* scale,
                        const float* bias, bool relu, float* Y, cudaStream_t s) {

@@ -90,6 +90,17 @@ def test_infinities_and_nan():
         assert torch.equal(got[~finite].nan_to_num(9.0), want[~finite].nan_to_num(9.0))
 
 
+def test_no_wait_ran_out():
+    g = empty_graph(3000)
+    X, W, G, scale, bias = operands(3000, 300, 300)
+    g.dg_linear_fwd(X, W)
+    g.dg_linear_bwd_input(G, W)
+    g.dg_linear_bwd_weight(G, X)
+    assert g.dg_graph_get_param("expired_waits") == 0
+    with pytest.raises(binding.DgError):
+        g.dg_graph_set_param("expired_waits", 0)
+
+
 def test_arguments_are_checked():
     X, W, G, scale, bias = operands(40, 8, 8)
     g = empty_graph(40)
