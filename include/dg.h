@@ -224,6 +224,8 @@ dg_status_t dg_layer_bwd(dg_graph_t g, const float* dOut, const float* out, int3
  *                dg_layer_fwd follows: Y = act(row_scale[v] * Y + bias).
  *   bwd_input:   dX = G W (n x K).
  *   bwd_weight:  dW = G^T X (N x K), always summed in the same order.
+ * Infinities and NaN come out as in fp32; the 128 x 128 results around one that is not finite are formed again, which takes
+ * two to eight times as long as the products.
  * The result must not overlap an input.  bwd_weight sums slices of the rows in scratch, up to 9.3 MiB of it; with
  * less memory it takes fewer slices and keeps fewer SMs busy, without any it sums all rows in a few thread blocks.  Asynchronous on `stream`.
  */

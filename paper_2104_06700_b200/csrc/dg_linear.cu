@@ -9,7 +9,7 @@
 // |x||w|.  The tensor cores add in fp32, but need not round to nearest, so they only add kChunk products of a
 // sum at a time: every chunk's result is read from tensor memory and added to a register with an fp32 addition.
 // Infinities and NaN, whose parts are NaN, and sums that overflow give a NaN here: such an element is computed again
-// with fp32 multiply-adds (dot_again).  Error against 64-bit sums, 2-norms, this / torch's fp32 GEMM: 245 k x 256 times
+// with fp32 multiply-adds (sum_again).  Error against 64-bit sums, 2-norms, this / torch's fp32 GEMM: 245 k x 256 times
 // 256 x 256 8.5e-8 / 2.9e-7; summed over 245 k rows 2.2e-7 / 1.1e-6; 602 products 1.05e-7 / 4.4e-7; with two chunks to a sum in
 // tensor memory, small products behind large ones, 2.0e-7.
 //
@@ -244,16 +244,6 @@ __device__ __forceinline__ float element(const float* p, int64_t ld, int64_t r, 
   return __ldg(ALONG ? p + r * ld + k : p + k * ld + r);
 }
 
-// One element of a slice in plain fp32, for sums that hold an infinity or a NaN.
-template <bool ALONG_A, bool ALONG_B>
-__device__ __forceinline__ float dot_again(const LinearArgs& a, int m, int n, int k0, int k1) {
-  float s = 0.f;
-#pragma unroll 1
-  for (int k = k0; k < k1; ++k)
-    s = fmaf(element<ALONG_A>(a.A, a.lda, m, k), element<ALONG_B>(a.B, a.ldb, n, k), s);
-  return s;
-}
-
 // Columns of the tile at n0, in whole steps of 16.
 template <int N>
 __device__ __forceinline__ int tile_width(int columns, int n0) {
@@ -275,6 +265,91 @@ __device__ __forceinline__ Item item_of(const LinearArgs& a, int i) {
   t.k1 = a.depth - t.k0 > a.depth_slice ? t.k0 + a.depth_slice : a.depth;
   t.chunks = (t.k1 - t.k0 + kChunk - 1) / kChunk;
   return t;
+}
+
+__device__ __forceinline__ void sync_workers() { asm volatile("bar.sync 1, %0;" ::"n"(kWorkers) : "memory"); }
+__device__ __forceinline__ bool any_worker(bool mine) {
+  uint32_t any;
+  asm volatile("{\n\t.reg .pred p, q;\n\tsetp.ne.u32 p, %1, 0;\n\tbar.red.or.pred q, 1, %2, p;\n\tselp.u32 %0, 1, 0, q;\n\t}"
+               : "=r"(any) : "r"((uint32_t)mine), "n"(kWorkers) : "memory");
+  return any != 0;
+}
+
+// The results of the block that are NaN once more with fp32 multiply-adds, in the order of the sum: infinities and NaN,
+// and sums that overflow, come out as NaN above.  All workers take 128 columns of a tile at a time, eight rows and four
+// columns each, through shared memory, as the inputs may be NaN throughout.
+// 20 k x 256 x 256 of NaN, us: forward 252, gradient of the input 236, of the weights 117 (an element per lane 10031, 6411,
+// 3640; torch 79 and 92); 245 k 1726, 1609, 1163 (torch 581, 593).
+constexpr int kAgainDepth = 32, kAgainRow = kM + 4;
+template <bool ALONG_A, bool ALONG_B, int kN>
+__device__ __noinline__ void sum_again(const LinearArgs& a, float* space) {
+  constexpr int kLoads = kAgainDepth * kM / kWorkers, kStage = 2 * kAgainDepth * kAgainRow;
+  const int items = a.tiles_m * a.tiles_n * a.slices;
+  const int t = threadIdx.x, tr = t / 32 * 8, tc = t % 32 * 4;
+  for (int i = blockIdx.x; i < items; i += gridDim.x) {
+    const Item now = item_of<kN>(a, i);
+    float* out = a.out + (int64_t)now.slice * a.rows_a * a.rows_b;
+    for (int n0 = now.n0; n0 < min(now.n0 + kN, a.rows_b); n0 += kM) {
+      auto each = [&](auto f) {  // of the thread's results
+#pragma unroll
+        for (int p = 0; p < 8; ++p)
+#pragma unroll
+          for (int q = 0; q < 4; ++q) {
+            const int r = now.m0 + tr + p, n = n0 + tc + q;
+            if (r < a.rows_a && n < a.rows_b) f(p, q, r, n, out + (int64_t)r * a.rows_b + n);
+          }
+      };
+      bool nan = false;
+      each([&](int, int, int, int, float* y) { nan = nan || *y != *y; });
+      if (!any_worker(nan)) continue;
+      float xa[kLoads], xb[kLoads], sum[8][4] = {};
+      auto load = [&](int k) {
+#pragma unroll
+        for (int j = 0; j < kLoads; ++j) {
+          const int ka = k + (ALONG_A ? t % 32 : t / kM + 4 * j), ra = now.m0 + (ALONG_A ? t / 32 + 16 * j : t % kM);
+          const int kb = k + (ALONG_B ? t % 32 : t / kM + 4 * j), rb = n0 + (ALONG_B ? t / 32 + 16 * j : t % kM);
+          xa[j] = ra < a.rows_a && ka < now.k1 ? element<ALONG_A>(a.A, a.lda, ra, ka) : 0.f;
+          xb[j] = rb < a.rows_b && kb < now.k1 ? element<ALONG_B>(a.B, a.ldb, rb, kb) : 0.f;
+        }
+      };
+      auto store = [&](float* to) {
+#pragma unroll
+        for (int j = 0; j < kLoads; ++j) {
+          to[ALONG_A ? t % 32 * kAgainRow + t / 32 + 16 * j : (t / kM + 4 * j) * kAgainRow + t % kM] = xa[j];
+          to[kStage / 2 + (ALONG_B ? t % 32 * kAgainRow + t / 32 + 16 * j : (t / kM + 4 * j) * kAgainRow + t % kM)] = xb[j];
+        }
+      };
+      load(now.k0);
+      store(space);
+      sync_workers();
+      int stage = 0;
+#pragma unroll 1
+      for (int k = now.k0; k < now.k1; k += kAgainDepth, stage ^= 1) {
+        const bool more = k + kAgainDepth < now.k1;
+        if (more) load(k + kAgainDepth);
+        const float* from = space + stage * kStage;
+#pragma unroll 4
+        for (int kk = 0; kk < kAgainDepth; ++kk) {
+          const float* x = from + kk * kAgainRow + tr;
+          const float4 w = *reinterpret_cast<const float4*>(from + kStage / 2 + kk * kAgainRow + tc);
+#pragma unroll
+          for (int p = 0; p < 8; ++p) {
+            sum[p][0] = fmaf(x[p], w.x, sum[p][0]);
+            sum[p][1] = fmaf(x[p], w.y, sum[p][1]);
+            sum[p][2] = fmaf(x[p], w.z, sum[p][2]);
+            sum[p][3] = fmaf(x[p], w.w, sum[p][3]);
+          }
+        }
+        if (more) store(space + (stage ^ 1) * kStage);
+        sync_workers();
+      }
+      each([&](int p, int q, int r, int n, float* y) {
+        if (*y == *y) return;
+        const float z = fmaf(sum[p][q], a.scale ? __ldg(a.scale + r) : 1.f, a.bias ? __ldg(a.bias + n) : 0.f);
+        *y = max_nan(z, a.relu ? 0.f : -INFINITY);
+      });
+    }
+  }
 }
 
 // After a wait that ran out: the workers make the block's results NaN.
@@ -301,6 +376,7 @@ __global__ void __launch_bounds__(kThreads, 1) linear_kernel(const __grid_consta
   __shared__ uint64_t arrived[2];  // a stage's chunk of the image has arrived
   __shared__ uint64_t idle;        // after a wait that ran out: no matrix instruction is in flight
   __shared__ int expired;          // a wait has run out: nothing more is started, the block's results are NaN
+  __shared__ int again;            // a result has to be formed again
   __shared__ int never;            // stays 0
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   const int items = a.tiles_m * a.tiles_n * a.slices;
@@ -318,7 +394,7 @@ __global__ void __launch_bounds__(kThreads, 1) linear_kernel(const __grid_consta
       mbarrier_init(arrived0 + 8 * i, 1);
     }
     mbarrier_init(smem_address(&idle), 1);
-    expired = never = 0;
+    expired = never = again = 0;
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
   }
   asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
@@ -391,13 +467,17 @@ __global__ void __launch_bounds__(kThreads, 1) linear_kernel(const __grid_consta
       const float s = a.scale && m < a.rows_a ? __ldg(a.scale + m) : 1.f;
       float* out = a.out + (int64_t)rt.slice * a.rows_a * a.rows_b;
       const float least = a.relu ? 0.f : -INFINITY;  // act(y) = max(y, least), NaN stays NaN
-      float2 check = make_float2(0.f, 0.f);          // becomes NaN if a sum is
+      float2 check = make_float2(0.f, 0.f);          // becomes NaN if a sum is NaN or infinite
 #pragma unroll
       for (int i = 0; i < S::kColumns / 2; ++i) check = __ffma2_rn(acc[i], make_float2(0.f, 0.f), check);
-      const bool again = check.x + check.y != 0.f;
+      if (check.x + check.y != 0.f) {
+        again = 1;
+#pragma unroll
+        for (int i = 0; i < S::kColumns / 2; ++i) acc[i] = __ffma2_rn(acc[i], make_float2(0.f, 0.f), acc[i]);  // all NaN
+      }
       // The stage of chunk j and the slot split last are free until the next chunk: 32 x 32 numbers for every warp, so that
       // results leave in whole lines (in pieces of 32 bytes, from tiles of 8 columns, this took 11 000 cycles of 26 000 a tile).
-      asm volatile("bar.sync 1, %0;" ::"n"(kWorkers) : "memory");
+      sync_workers();
       float* tile = reinterpret_cast<float*>(
           warp < 6 ? smem + S::kTileAt + warp * kTileBytes
                    : warp < 12 ? smem + (j & 1) * operand_bytes(kM) + (warp - 6) * kTileBytes
@@ -415,7 +495,7 @@ __global__ void __launch_bounds__(kThreads, 1) linear_kernel(const __grid_consta
           const float y = max_nan(fmaf(x, s, __shfl_sync(0xffffffffu, bias, i)), least);
           if (i < cols) mine[i] = y;
         }
-        asm volatile("bar.sync 1, %0;" ::"n"(kWorkers) : "memory");
+        sync_workers();
         const int count = min(kM, a.rows_a - rt.m0) * N;
         float* to = out + (int64_t)rt.m0 * N;  // 128 rows on from the matrix's start: aligned as that is
         for (int i = 4 * threadIdx.x; i < count; i += 4 * kWorkers) {
@@ -464,23 +544,9 @@ __global__ void __launch_bounds__(kThreads, 1) linear_kernel(const __grid_consta
           }
         }
       }
-      asm volatile("bar.sync 1, %0;" ::"n"(kWorkers) : "memory");
+      sync_workers();
 #pragma unroll
       for (int i = 0; i < S::kColumns / 2; ++i) acc[i] = make_float2(0.f, 0.f);
-      if (!__any_sync(0xffffffffu, again)) return;
-      // a sum held an infinity or a NaN: the warp's elements that are NaN once more, a lane each
-      __syncwarp();
-#pragma unroll 1
-      for (int r = row0; r < min(row0 + 32, a.rows_a); ++r) {
-#pragma unroll 1
-        for (int n = rt.n0 + c0 + lane; n < min(rt.n0 + c1, a.rows_b); n += 32) {
-          float* p = out + (int64_t)r * a.rows_b + n;
-          if (*p == *p) continue;
-          float y = dot_again<ALONG_A, ALONG_B>(a, r, n, rt.k0, rt.k1);
-          y = fmaf(y, a.scale ? __ldg(a.scale + r) : 1.f, a.bias ? __ldg(a.bias + n) : 0.f);
-          *p = max_nan(y, least);
-        }
-      }
     };
 
     for (int i = 0; i < S::kRing - 1; ++i) ring_next();
@@ -492,7 +558,7 @@ __global__ void __launch_bounds__(kThreads, 1) linear_kernel(const __grid_consta
         asm volatile("cp.async.wait_group %0;" ::"n"(S::kRing - 2) : "memory");  // this thread's part of chunk j is there
         // A thread splits what others copied, of its warp or of any; and they are done with the slot that is filled next.
         if (SPLIT_B && ALONG_A) __syncwarp();
-        else asm volatile("bar.sync 1, %0;" ::"n"(kWorkers) : "memory");
+        else sync_workers();
         ring_next();
         // The stage is free: the chunk before the last, which had it, has been drained.
         unsigned char* pa = smem + (j & 1) * operand_bytes(kM);
@@ -512,6 +578,8 @@ __global__ void __launch_bounds__(kThreads, 1) linear_kernel(const __grid_consta
     }
     if (j > 0) drain(j - 1, slot, before, finished);  // nothing is in the ring any more
     asm volatile("cp.async.wait_all;" ::: "memory");
+    sync_workers();
+    if (again) sum_again<ALONG_A, ALONG_B, kN>(a, reinterpret_cast<float*>(smem));
     } else {
     asm volatile("setmaxnreg.dec.sync.aligned.u32 24;");
     if (warp == kWarps) {

@@ -62,6 +62,65 @@ def test_products_without_scratch(n, K, N):
     check(n, K, N, scratch=False)
 
 
+def same_as_torch(got, want):
+    """Where torch's result is infinite or NaN, the same; finite elsewhere."""
+    finite = want.isfinite()
+    assert torch.equal(got.isfinite(), finite)
+    assert torch.equal(got[~finite].nan_to_num(9.0), want[~finite].nan_to_num(9.0))
+
+
+# several tiles a block, a part-filled one among them, one and two passes of 128 columns
+@pytest.mark.parametrize("n,K,N", [(20000, 100, 256), (20011, 260, 300), (20011, 256, 47)])
+@pytest.mark.parametrize("kind", ["some", "all"])
+def test_infinities_and_nan_in_many_tiles(n, K, N, kind):
+    X, W, G, scale, bias = operands(n, K, N)
+    if kind == "all":
+        X.fill_(float("nan"))
+        G[:, 3] = float("nan")
+    else:
+        X[n // 2:n // 2 + 200], X[n - 1, 0], X[3, K - 1] = float("nan"), float("inf"), -float("inf")
+        G[5, N - 1], W[7, 7] = float("inf"), float("-inf")
+    g = empty_graph(n)
+    same_as_torch(g.dg_linear_fwd(X, W), X @ W.t())
+    same_as_torch(g.dg_linear_fwd(X, W, scale, bias, True), (X @ W.t() * scale + bias).relu())
+    same_as_torch(g.dg_linear_bwd_input(G, W), G @ W)
+    same_as_torch(g.dg_linear_bwd_weight(G, X), G.t() @ X)
+
+
+def test_sums_that_overflow():
+    """Finite where the sum of the absolute products is, whatever the order."""
+    X, W, G, scale, bias = operands(2000, 100, 60)
+    X, W = X * 2.0 ** 62, W * 2.0 ** 60
+    want, size = X.double() @ W.double().t(), X.double().abs() @ W.double().abs().t()
+    fits = size < 3.0e38
+    assert 0.05 < float(fits.double().mean()) < 0.5
+    got = empty_graph(2000).dg_linear_fwd(X, W).double()
+    assert bool(((got - want).abs() <= bound(100, 1, size))[fits].all())
+
+
+def test_nan_costs_no_more_than_plain_arithmetic():
+    """A diverged model's epochs end.  The factor is 3 to 8; an element at a time it was over 100."""
+    n = 20000
+    X, W, G, scale, bias = operands(n, 256, 256)
+    g = empty_graph(n)
+    nan = torch.full_like(X, float("nan"))
+
+    def time(call):
+        best = float("inf")
+        for _ in range(5):
+            a, b = (torch.cuda.Event(enable_timing=True) for _ in range(2))
+            a.record()
+            call()
+            b.record()
+            b.synchronize()
+            best = min(best, a.elapsed_time(b))
+        return best
+
+    for call in (lambda x: g.dg_linear_fwd(x, W), lambda x: g.dg_linear_bwd_input(x, W),
+                 lambda x: g.dg_linear_bwd_weight(x, x)):
+        assert time(lambda: call(nan)) < 40 * time(lambda: call(X))
+
+
 @pytest.mark.parametrize("limit", [1, 2])
 def test_a_scratch_limit_costs_slices_and_not_all_of_them(limit):
     n, K, N = 40000, 256, 100  # 37 slices of 100 KiB
