@@ -3,15 +3,20 @@
 //   backward  dX = G W                  n x N times N x K
 //             dW = G^T X                n rows reduced to N x K
 //
-// Arithmetic.  An fp32 number is the exact sum of three bf16 numbers, x = x0 + x1 + x2 (x0 truncated, x1 and x2
-// rounded; 8 bits each).  Of the nine products of two such sums the six that matter are formed by the tensor cores,
-// each exact, (0,2) (2,0) (1,1) (0,1) (1,0) (0,0) in this order, smallest first; what is left out is below 2^-24 of
-// |x||w|.  The tensor cores add in fp32, but need not round to nearest, so they only add kChunk products of a
-// sum at a time: every chunk's result is read from tensor memory and added to a register with an fp32 addition.
+// Arithmetic.  An fp32 number is the exact sum of three bf16 numbers, x = x0 + 2^-8 x1 + 2^-16 x2, each rounded from
+// what the ones before leave: for every finite number, as the parts are held scaled up (unscaled, x2 of |x| < 2^-110 would fall
+// below bf16's smallest).  Of the nine products of two such sums the six that matter are formed by the tensor cores, each
+// exact, (0,2) (2,0) (1,1) (0,1) (1,0) (0,0) in this order, smallest first; the sum so far is scaled by 2^-8 where the parts'
+// places add up to one less.  What is left out is at most 0.98 of 2^-24 |x||w|, 0.09 in the mean square.  The
+// tensor cores add in fp32, but cut off where fp32 arithmetic rounds, so they only add kChunk products of a sum at a
+// time: every chunk's result is read from tensor memory and added to a register with an fp32 addition.
 // Infinities and NaN, whose parts are NaN, and sums that overflow give a NaN here: such an element is computed again
-// with fp32 multiply-adds (sum_again).  Error against 64-bit sums, 2-norms, this / torch's fp32 GEMM: 245 k x 256 times
-// 256 x 256 8.5e-8 / 2.9e-7; summed over 245 k rows 2.2e-7 / 1.1e-6; 602 products 1.05e-7 / 4.4e-7; with two chunks to a sum in
-// tensor memory, small products behind large ones, 2.0e-7.
+// with fp32 multiply-adds (sum_again).
+// Errors against 64-bit sums, 2-norms, this / torch's fp32 GEMM: 245 k x 256 times 256 x 256 8.0e-8 / 2.9e-7, ReLU'd 7.7e-8 /
+// 2.0e-7; summed over 245 k rows 2.8e-7 / 7.9e-7; 602 products 1.04e-7 / 4.5e-7; operands of 2^-126 7.8e-8 / 2.9e-7.  Rows with
+// one to three numbers that are not 0, where the cut-off shows, 4.5e-8 to 5.6e-8 / 2.5e-8 to 3.6e-8, eight 6.5e-8 / 5.4e-8, sixteen
+// 7.1e-8 / 7.4e-8.  Adding the (0,0) products apart from the others, so that their sum with the rest is an fp32 addition, gave
+// 2.6e-8 for one number and took 231 us instead of 199 (all eight products above 2^-32: 2.53e-8, 254 us).
 //
 // Shape of the kernel.  A block computes 128 x up to 256 elements at a time, one block per SM.  The fp32 operands arrive in a
 // ring of chunks in shared memory, by asynchronous copies (loads to registers need a place in the first-level cache,
@@ -41,6 +46,7 @@ constexpr int kGroups = kChunk / 8;       // 16-byte groups of a row of a part
 __host__ __device__ constexpr int group_stride(int rows) { return rows * 16 + 32; }
 __host__ __device__ constexpr int operand_bytes(int rows) { return 3 * kGroups * group_stride(rows); }
 constexpr int kTileBytes = 32 * 32 * 4;  // of a warp's staging tile
+constexpr int kPartBits = 8;             // a part is held as 2^kPartBits times what it is to the part before
 
 // Columns of a tile, and shared memory: two stages of operands, the ring of fp32 chunks, and staging tiles of the first
 // six warps; the others' lie in a stage of A and a slot of the ring that are free when a tile of results is written.
@@ -128,13 +134,21 @@ __device__ __forceinline__ uint64_t operand(uint32_t address, int stride) {
   return (uint64_t)((address >> 4) & 0x3fff) | (uint64_t)(stride >> 4) << 16 | (uint64_t)(128 >> 4) << 32 |
          (uint64_t)1 << 46;
 }
-// D[128 x n] (+)= A[128 x 16] B[n x 16]^T, bf16 in, fp32 out
+// D[128 x n] = A[128 x 16] B[n x 16]^T + D 2^-SHIFT, or without D; bf16 in, fp32 out
+template <int SHIFT>
 __device__ __forceinline__ void mma(uint32_t d, uint64_t a, uint64_t b, uint32_t shape, bool add) {
-  asm volatile(
-      "{\n\t.reg .pred p;\n\tsetp.ne.u32 p, %4, 0;\n\t"
-      "tcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, p;\n\t}" ::"r"(d), "l"(a), "l"(b), "r"(shape),
-      "r"((uint32_t)add)
-      : "memory");
+  if constexpr (SHIFT == 0)
+    asm volatile(
+        "{\n\t.reg .pred p;\n\tsetp.ne.u32 p, %4, 0;\n\t"
+        "tcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, p;\n\t}" ::"r"(d), "l"(a), "l"(b), "r"(shape),
+        "r"((uint32_t)add)
+        : "memory");
+  else
+    asm volatile(
+        "{\n\t.reg .pred p;\n\tsetp.ne.u32 p, %4, 0;\n\t"
+        "tcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, p, %5;\n\t}" ::"r"(d), "l"(a), "l"(b), "r"(shape),
+        "r"((uint32_t)add), "n"(SHIFT)
+        : "memory");
 }
 
 // 16 columns of this warp's 32 lanes of tensor memory (32 at a time spill: seventeen warps have 96 registers)
@@ -163,19 +177,19 @@ __device__ __forceinline__ uint32_t round_pair(float lo, float hi) {
 }
 // Splits eight numbers of a row and writes the parts at `to` and every kGroups * stride bytes on.
 __device__ __forceinline__ void put(unsigned char* to, int stride, const float (&x)[8]) {
+  constexpr float kUp = 1 << kPartBits;  // exact: what is left is at most 2^-kPartBits of the number
   uint32_t p[3][4];
 #pragma unroll
   for (int i = 0; i < 4; ++i) {
-    const float a = x[2 * i], b = x[2 * i + 1];
-    const uint32_t ua = __float_as_uint(a), ub = __float_as_uint(b);
-    p[0][i] = __byte_perm(ua, ub, 0x7632);
-    // exact subtractions, two in an instruction
-    const float2 r = __ffma2_rn(make_float2(__uint_as_float(ua & 0xffff0000u), __uint_as_float(ub & 0xffff0000u)),
-                                make_float2(-1.f, -1.f), make_float2(a, b));
-    p[1][i] = round_pair(r.x, r.y);
-    const float2 q = __ffma2_rn(make_float2(__uint_as_float(p[1][i] << 16), __uint_as_float(p[1][i] & 0xffff0000u)),
-                                make_float2(-1.f, -1.f), r);
-    p[2][i] = round_pair(q.x, q.y);
+    // exact but for the roundings to bf16, of which the last is exact too; two in an instruction
+    float2 r = make_float2(x[2 * i], x[2 * i + 1]);
+#pragma unroll
+    for (int t = 0; t < 3; ++t) {
+      p[t][i] = round_pair(r.x, r.y);
+      r = __ffma2_rn(make_float2(__uint_as_float(p[t][i] << 16), __uint_as_float(p[t][i] & 0xffff0000u)),
+                     make_float2(-1.f, -1.f), r);
+      r = __fmul2_rn(r, make_float2(kUp, kUp));
+    }
   }
 #pragma unroll
   for (int t = 0; t < 3; ++t)
@@ -605,9 +619,13 @@ __global__ void __launch_bounds__(kThreads, 1) linear_kernel(const __grid_consta
 #pragma unroll
             for (int p = 0; p < 6; ++p)
 #pragma unroll
-              for (int k = 0; k < kChunk / 16; ++k)
-                mma(d, da + (kPairs[p][0] * kGroups + 2 * k) * (group_stride(kM) >> 4),
-                    db + (kPairs[p][1] * kGroups + 2 * k) * (uint32_t)(strb >> 4), shape, p + k > 0);
+              for (int k = 0; k < kChunk / 16; ++k) {
+                const uint64_t pa = da + (kPairs[p][0] * kGroups + 2 * k) * (group_stride(kM) >> 4);
+                const uint64_t qb = db + (kPairs[p][1] * kGroups + 2 * k) * (uint32_t)(strb >> 4);
+                const bool scaled = p > 0 && k == 0 && kPairs[p][0] + kPairs[p][1] < kPairs[p - 1][0] + kPairs[p - 1][1];
+                if (scaled) mma<kPartBits>(d, pa, qb, shape, true);
+                else mma<0>(d, pa, qb, shape, p + k > 0);
+              }
             asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(
                              done0 + 8 * (j & 1))
                          : "memory");

@@ -12,9 +12,17 @@ EPS = 2.0 ** -24
 
 
 def bound(depth, slices, magnitude):
-    """Per chunk of 32 products: 12 tensor-core additions, each off by at most 2 EPS of the partial sum, and 4 EPS of what
-    the split leaves out; then an fp32 addition per chunk and per slice."""
-    return (28 + (depth + 31) // 32 + slices) * EPS * magnitude
+    """Per chunk of 32 products: two tensor-core additions of products of the first parts and ten of 2^-8 of those and less,
+    each off by at most 2 EPS of the partial sum, and EPS of what the split leaves out: 5.2 EPS; then an fp32 addition per
+    chunk and per slice of the sum."""
+    return (6 + (depth + 31) // 32 + slices) * EPS * magnitude
+
+
+def slices_of(n, K, N):
+    """(slices of the rows that the weights' gradient is summed in, their length)"""
+    sms = torch.cuda.get_device_properties(0).multi_processor_count
+    slices = max(1, min(sms // ((N + 127) // 128 * ((K + 127) // 128)), (n + 511) // 512))
+    return slices, -(-n // slices)
 
 
 def operands(n, K, N, offset=0):
@@ -40,7 +48,8 @@ def check(n, K, N, offset=0, scratch=True):
     dX = g.dg_linear_bwd_input(G, W).double()
     assert bool(((dX - Gd @ Wd).abs() <= bound(N, 1, Gd.abs() @ Wd.abs())).all())
     dW = g.dg_linear_bwd_weight(G, X)
-    assert bool(((dW.double() - Gd.t() @ Xd).abs() <= bound(n, 148, Gd.abs().t() @ Xd.abs())).all())
+    slices, length = slices_of(n, K, N) if scratch else (1, n)
+    assert bool(((dW.double() - Gd.t() @ Xd).abs() <= bound(length, slices, Gd.abs().t() @ Xd.abs())).all())
     assert torch.equal(dW, g.dg_linear_bwd_weight(G, X))
 
 
@@ -60,6 +69,61 @@ def test_misaligned_matrices(n, K, N, offset):
 @pytest.mark.parametrize("n,K,N", [(129, 33, 17), (1500, 260, 130)])
 def test_products_without_scratch(n, K, N):
     check(n, K, N, scratch=False)
+
+
+def without_one(X, W, p, q):
+    """X W^T less the products of X's part p and W's part q."""
+    def part(x, which):
+        for t in range(which + 1):
+            piece = x.to(torch.bfloat16).float()
+            x = (x - piece) * 256
+        return piece.double() * 2.0 ** (-8 * which)
+
+    return X.double() @ W.double().t() - part(X, p) @ part(W, q).t()
+
+
+@pytest.mark.parametrize("nonzeros", [1, 2, 3, 16, 256])
+def test_rows_of_few_numbers(nonzeros):
+    """Their sums have no other rounding errors to hide a product that is left out."""
+    n, K, N = 2000, 256, 256
+    X, W, G, scale, bias = operands(n, K, N)
+    G = G.contiguous()
+    X = X * torch.zeros_like(X).scatter_(1, torch.rand_like(X).topk(nonzeros, 1).indices, 1.0)
+    G = G * (X != 0)
+    g = empty_graph(n)
+    chunks = min(nonzeros, 8)
+    for A, B, got in ((X, W, g.dg_linear_fwd(X, W)), (G, W.t().contiguous(), g.dg_linear_bwd_input(G, W))):
+        want, size = A.double() @ B.double().t(), A.double().abs() @ B.double().abs().t()
+        limit = (6 + chunks) * EPS * size
+        assert bool(((got.double() - want).abs() <= limit).all())
+        for p, q in ((0, 0), (0, 1), (1, 0), (1, 1), (0, 2), (2, 0)):  # the limit tells each of the six products
+            assert nonzeros > 16 or bool(((without_one(A, B, p, q) - want).abs() > limit).any())
+    dW, want, size = g.dg_linear_bwd_weight(G, X), G.double().t() @ X.double(), G.double().abs().t() @ X.double().abs()
+    slices, length = slices_of(n, K, N)
+    assert bool(((dW.double() - want).abs() <= bound(length, slices, size)).all())
+
+
+def norm_error(got, want):
+    return float((got.double() - want).norm() / want.norm())
+
+
+@pytest.mark.parametrize("kind", ["normal", "one sign"] + [f"2^{e}" for e in (-100, -115, -122, -126)])
+def test_errors_are_below_those_of_fp32_sums(kind):
+    """2-norms against those of torch's fp32 products, in sums of 256 and of 20000; half of them at least where numbers have
+    both signs.  Small operands against large ones: bf16 parts of fp32's smallest numbers."""
+    n, K, N = 20000, 256, 256
+    X, W, G, scale, bias = operands(n, K, N)
+    if kind == "one sign":
+        X, W, G = X.abs(), W.abs(), G.abs()
+    elif kind != "normal":
+        X = X * 2.0 ** int(kind[2:])
+        G, W = G * 2.0 ** 60, W * 2.0 ** 60
+    g = empty_graph(n)
+    part = 1.0 if kind == "one sign" else 0.5
+    for got, fp32, want in ((g.dg_linear_fwd(X, W), X @ W.t(), X.double() @ W.double().t()),
+                            (g.dg_linear_bwd_input(G, W), G @ W, G.double() @ W.double()),
+                            (g.dg_linear_bwd_weight(G, X), G.t() @ X, G.double().t() @ X.double())):
+        assert norm_error(got, want) <= part * norm_error(fp32, want)
 
 
 def same_as_torch(got, want):
@@ -132,7 +196,8 @@ def test_a_scratch_limit_costs_slices_and_not_all_of_them(limit):
     dW = g.dg_linear_bwd_weight(G, X)
     assert binding.dg_kernel_launch_count() - before == 2  # the products and the sum of the slices
     want, size = G.double().t() @ X.double(), G.double().abs().t() @ X.double().abs()
-    assert bool(((dW.double() - want).abs() <= bound(n, 148, size)).all())
+    slices = limit * 2 ** 20 // (K * N * 4)
+    assert bool(((dW.double() - want).abs() <= bound(-(-n // slices), slices, size)).all())
 
 
 def test_infinities_and_nan():
