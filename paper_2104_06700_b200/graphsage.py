@@ -79,9 +79,13 @@ def _large(graph: "binding.Graph", weight: torch.Tensor) -> bool:
     GEMMs in all three directions, if neither width is small: their tiles are 128 rows by whole steps of 16 columns.  us
     library / torch, forward with its epilogue, gradient of the input, of the weights: 245 k rows of 256 x 256 186 / 660,
     187 / 569, 267 / 594; of 256 x 47 120 / 198, 100 / 173, 173 / 166; 8 k of 256 x 256 23 / 31, 21 / 27, 31 / 36; but 100 k of
-    64 x 41 49 / 43, 39 / 29, 49 / 44; of 602 x 16 158 / 115, 160 / 94, 195 / 123."""
+    64 x 41 49 / 43, 39 / 29, 49 / 44; of 602 x 16 158 / 115, 160 / 94, 195 / 123.
+
+    A caller who allowed torch TF32 products (set_float32_matmul_precision, allow_tf32) keeps them: us
+    library / TF32, 245 k rows of 256 x 256 194 / 168, 194 / 85, 267 / 101."""
     N, K = weight.shape
-    return min(N, K) >= 40 and graph.n * N * K >= 1 << 29
+    return (min(N, K) >= 40 and graph.n * N * K >= 1 << 29
+            and torch.backends.cuda.matmul.fp32_precision in ("none", "ieee"))
 
 
 def _with_own_row(graph: "binding.Graph", M: torch.Tensor, bf16: bool, transposed: bool) -> torch.Tensor:

@@ -4,7 +4,7 @@ from types import SimpleNamespace
 import pytest
 import torch
 
-from paper_2104_06700_b200 import graphsage, synth
+from paper_2104_06700_b200 import binding, graphsage, synth
 from parity_util import make_graph
 
 pytestmark = pytest.mark.gpu
@@ -32,3 +32,27 @@ def test_features_of_another_width_are_refused(dims, project_first, n):
             model(X)
         with torch.no_grad(), pytest.raises((RuntimeError, ValueError)):
             model(X)
+
+
+@pytest.fixture
+def tf32():
+    torch.set_float32_matmul_precision("high")
+    yield
+    torch.set_float32_matmul_precision("highest")
+
+
+def test_a_caller_who_asked_for_tf32_keeps_it(tf32):
+    n, dims = 8192 + 5, [256, 256]
+    g = make_graph(random_graph(n))
+    g.dg_graph_transpose()
+    model = graphsage.GraphSAGE(g, dims).to(DEV)
+    X, dOut = synth.features(n, 256, 1, DEV).requires_grad_(True), synth.features(n, 256, 2, DEV)
+    W, b = (p.detach() for p in model.parameters())
+    out = model(X)
+    out.backward(dOut)
+    Z = g.dg_aggregate_fwd_self(X.detach(), binding.DG_OP_SUM)
+    assert torch.equal(out, g.dg_layer_fwd(Z @ W.t(), model.inv_deg1, b, False))
+    G, _ = g.dg_layer_bwd(dOut, None, model.inv_deg1)
+    assert torch.equal(X.grad, g.dg_aggregate_bwd_self(G @ W, binding.DG_OP_SUM))
+    torch.set_float32_matmul_precision("highest")
+    assert not torch.equal(out, model(X))
