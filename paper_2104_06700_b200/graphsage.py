@@ -74,18 +74,29 @@ def _weight_grad(G: torch.Tensor, X: torch.Tensor) -> torch.Tensor:
     return dW.addmm_(G[m:].t(), X[m:]) if m < n else dW
 
 
-def _large(graph: "binding.Graph", weight: torch.Tensor) -> bool:
-    """Whether the library's products serve the layer.  From 2^29 multiplications on they are faster than torch's fp32
-    GEMMs in all three directions, if neither width is small: their tiles are 128 rows by whole steps of 16 columns.  us
-    library / torch, forward with its epilogue, gradient of the input, of the weights: 245 k rows of 256 x 256 186 / 660,
-    187 / 569, 267 / 594; of 256 x 47 120 / 198, 100 / 173, 173 / 166; 8 k of 256 x 256 23 / 31, 21 / 27, 31 / 36; but 100 k of
-    64 x 41 49 / 43, 39 / 29, 49 / 44; of 602 x 16 158 / 115, 160 / 94, 195 / 123.
+def _by_library(graph: "binding.Graph", weight: torch.Tensor):
+    """Which products of a layer the library computes, and not torch's fp32 GEMMs: forward, gradient of the input, of the
+    weights.  From 2^29 multiplications on it is faster, if neither width is small: tiles are 128 rows by whole steps of 16
+    columns.  us library / torch, forward with its epilogue, gradients: 245 k rows of 256 x 256 189 / 660, 191 / 569, 267 / 594; of
+    256 x 47 123 / 198, 103 / 173, -; 8 k of 256 x 256 23 / 31, 21 / 27, 31 / 36; but 100 k of 64 x 41 49 / 43, 39 / 29, 49 / 44;
+    of 602 x 16 158 / 115, 160 / 94, 195 / 123.  Of the large ones torch keeps
+      - those that fill few SMs: 4096 rows of 602 to 256 columns 40 / 36, 39 / 32; 8192 23 / 31;
+      - gradients of narrow inputs, which have no epilogue to save: 245 k rows to 64 columns from 41 75 / 62, 100 k from 100
+        45 / 39, from 602 171 / 156; and of wide ones from rows that allow no vectors: 33 k from 41 to 602 71 / 65;
+      - gradients of weights of which one side is mostly padding to 128 and the other takes more than one tile, 245 k rows:
+        47 x 256 174 / 165, 602 x 47 508 / 432 (47 x 128 99 / 117), or both are read number by number: 47 x 47 115 / 106;
+        and those with little scratch, summed in few blocks: 256 x 256 with 5 and 4 MiB 481 and 597 / 594, 602 x 256 with 5 1507 / 1367.
 
     A caller who allowed torch TF32 products (set_float32_matmul_precision, allow_tf32) keeps them: us
     library / TF32, 245 k rows of 256 x 256 194 / 168, 194 / 85, 267 / 101."""
     N, K = weight.shape
-    return (min(N, K) >= 40 and graph.n * N * K >= 1 << 29
-            and torch.backends.cuda.matmul.fp32_precision in ("none", "ieee"))
+    if (min(N, K) < 40 or graph.n * N * K < 1 << 29
+            or torch.backends.cuda.matmul.fp32_precision not in ("none", "ieee")):
+        return False, False, False
+    small, big, tiles = min(N, K), max(N, K), (graph.n + 127) // 128
+    return (tiles * ((N + 255) // 256) >= 64,
+            tiles * ((K + 255) // 256) >= 64 and K > 64 and (N % 4 == 0 or K <= 256),
+            (small > 64 or big <= 128 and (N % 4 == 0 or K % 4 == 0)) and graph.dg_graph_get_param("scratch_mb") >= 7)
 
 
 def _with_own_row(graph: "binding.Graph", M: torch.Tensor, bf16: bool, transposed: bool) -> torch.Tensor:
@@ -113,11 +124,12 @@ class _GcnLayer(torch.autograd.Function):
         M = M.contiguous()
         if project:
             X = M
-            Z = graph.dg_linear_fwd(M, weight.contiguous()) if _large(graph, weight) else M @ weight.t()
+            large = _by_library(graph, weight)[0]
+            Z = graph.dg_linear_fwd(M, weight.contiguous()) if large else M @ weight.t()
             out = graph.dg_layer_fwd(_with_own_row(graph, Z, bf16, False), inv_deg1, bias.contiguous(), relu)
         else:
             X = _with_own_row(graph, M, bf16, False)
-            if _large(graph, weight):
+            if _by_library(graph, weight)[0]:
                 out = graph.dg_linear_fwd(X, weight.contiguous(), inv_deg1, bias.contiguous(), relu)
             else:
                 out = graph.dg_layer_fwd(X @ weight.t(), inv_deg1, bias.contiguous(), relu)
@@ -138,17 +150,12 @@ class _GcnLayer(torch.autograd.Function):
         G, db = graph.dg_layer_bwd(dOut.contiguous(), out, inv_deg1)
         if ctx.project and (needs[0] or needs[1]):
             G = _with_own_row(graph, G, ctx.bf16, True)
-        large = _large(graph, weight)
+        _, input_grad, weight_grad = _by_library(graph, weight)
         dW = dM = None
         if needs[1]:
-            # with less scratch the library sums in so few blocks that torch's slices are as fast: 245 k rows of 256 x 256
-            # with 5 and 4 MiB 481 and 597 us, torch 594; of 602 x 256 with 5 MiB 1507, torch 1367
-            if large and graph.dg_graph_get_param("scratch_mb") >= 7:
-                dW = graph.dg_linear_bwd_weight(G, X)
-            else:
-                dW = _weight_grad(G, X)
+            dW = graph.dg_linear_bwd_weight(G, X) if weight_grad else _weight_grad(G, X)
         if needs[0]:
-            dM = graph.dg_linear_bwd_input(G, weight.contiguous()) if large else G @ weight
+            dM = graph.dg_linear_bwd_input(G, weight.contiguous()) if input_grad else G @ weight
             if not ctx.project:
                 dM = _with_own_row(graph, dM, ctx.bf16, True)
         return dM, dW, db if needs[2] else None, None, None, None, None, None
