@@ -55,7 +55,9 @@ def check(n, K, N, offset=0, scratch=True):
 
 @pytest.mark.parametrize("n,K,N", [(1, 1, 1), (127, 31, 15), (128, 32, 16), (129, 33, 17), (513, 64, 47), (300, 100, 127),
                                    (640, 128, 128), (257, 129, 129), (1000, 255, 255), (511, 256, 256), (512, 257, 257),
-                                   (700, 602, 41), (150, 41, 602), (40000, 100, 256)])
+                                   (700, 602, 41), (150, 41, 602), (40000, 100, 256),
+                                   # blocks with several tiles: of two widths, of rows that leave as one stretch
+                                   (20011, 64, 257), (20011, 300, 300), (40000, 256, 47), (40100, 41, 41), (20011, 48, 45)])
 def test_products_match_fp64(n, K, N):
     check(n, K, N)
 
@@ -66,7 +68,7 @@ def test_misaligned_matrices(n, K, N, offset):
     check(n, K, N, offset)
 
 
-@pytest.mark.parametrize("n,K,N", [(129, 33, 17), (1500, 260, 130)])
+@pytest.mark.parametrize("n,K,N", [(129, 33, 17), (1500, 260, 130), (20011, 64, 257), (40000, 100, 47)])
 def test_products_without_scratch(n, K, N):
     check(n, K, N, scratch=False)
 
