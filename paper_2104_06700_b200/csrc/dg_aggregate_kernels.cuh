@@ -140,6 +140,24 @@ __device__ __forceinline__ void fma(float4& a, float s, const float4& v) {
   a.x = fmaf(s, v.x, a.x); a.y = fmaf(s, v.y, a.y);
   a.z = fmaf(s, v.z, a.z); a.w = fmaf(s, v.w, a.w);
 }
+// A scaled edge with G lanes.  Two lanes (rows of 16 numbers at most) load an edge's ids and factors as often as its
+// numbers and are not bound by issue: there pairs of operations only cost registers (49 M edges, F = 16, bf16, the mean's
+// backward pass 446 us with them, 436 without; F = 64 955, 1003).
+template <int G, typename A, typename V>
+__device__ __forceinline__ void fma_edge(A& a, float s, const V& v) {
+  fma(a, s, v);
+}
+template <int G>
+__device__ __forceinline__ void fma_edge(f8& a, float s, const uint4& v) {
+  if constexpr (G == 2) {
+    a.lo.x = fmaf(s, bf_lo(v.x), a.lo.x); a.lo.y = fmaf(s, bf_hi(v.x), a.lo.y);
+    a.lo.z = fmaf(s, bf_lo(v.y), a.lo.z); a.lo.w = fmaf(s, bf_hi(v.y), a.lo.w);
+    a.hi.x = fmaf(s, bf_lo(v.z), a.hi.x); a.hi.y = fmaf(s, bf_hi(v.z), a.hi.y);
+    a.hi.z = fmaf(s, bf_lo(v.w), a.hi.z); a.hi.w = fmaf(s, bf_hi(v.w), a.hi.w);
+  } else {
+    fma(a, s, v);
+  }
+}
 __device__ __forceinline__ void scale(float& a, float s) { a *= s; }
 __device__ __forceinline__ void scale(float2& a, float s) { a.x *= s; a.y *= s; }
 __device__ __forceinline__ void scale(float4& a, float s) { a.x *= s; a.y *= s; a.z *= s; a.w *= s; }
@@ -198,9 +216,9 @@ struct Shape {
 };
 
 // Adds the edges held in lanes [s, e) of the current batch (cur_u / cur_s: one edge per lane)
-// into acc.  Lane group `grp` takes edges s+grp, s+grp+NG, ...  Full steps of U*NG edges run
-// without predicates; the ragged end runs once with predicated loads.  xrow[c] is the address
-// of this lane's c-th vector inside row 0 of X.
+// into acc.  Lane group `grp` takes edges s+grp, s+grp+NG, ..., with kIds (below) U neighbouring ones of every full
+// step.  Full steps of U*NG edges run without predicates; the ragged end runs once with predicated loads.  xrow[c]
+// is the address of this lane's c-th vector inside row 0 of X.
 template <typename E, int VEC, int G, int CPL, bool SCALED, bool STAGE>
 __device__ __forceinline__ void add_edges(const char* const (&xrow)[CPL], uint32_t row_bytes,
                                           int32_t cur_u, float cur_s, int s, int e, int grp,
@@ -269,7 +287,7 @@ __device__ __forceinline__ void add_edges(const char* const (&xrow)[CPL], uint32
       if (SCALED) sj = kLate ? __shfl_sync(kFull, cur_s, p + j * NG + grp) : sc[j];
 #pragma unroll
       for (int c = 0; c < CPL; ++c) {
-        if (SCALED) fma(acc[c], sj, v[j][c]);
+        if (SCALED) fma_edge<G>(acc[c], sj, v[j][c]);
         else add(acc[c], v[j][c]);
       }
     }
@@ -294,7 +312,7 @@ __device__ __forceinline__ void add_edges(const char* const (&xrow)[CPL], uint32
       if (SCALED && src >= e) sj = 0.f;  // lanes past the batch hold neutral factors, not NaNs
 #pragma unroll
       for (int c = 0; c < CPL; ++c) {
-        if (SCALED) fma(acc[c], sj, v[j][c]);
+        if (SCALED) fma_edge<G>(acc[c], sj, v[j][c]);
         else add(acc[c], v[j][c]);
       }
     }
