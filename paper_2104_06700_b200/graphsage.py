@@ -87,10 +87,10 @@ def _by_library(graph: "binding.Graph", weight: torch.Tensor):
         47 x 256 174 / 165, 602 x 47 508 / 432 (47 x 128 99 / 117), or both are read number by number: 47 x 47 115 / 106;
         and those with little scratch, summed in few blocks: 256 x 256 with 5 and 4 MiB 481 and 597 / 594, 602 x 256 with 5 1507 / 1367.
 
-    A caller who allowed torch TF32 products (set_float32_matmul_precision, allow_tf32) keeps them: us
+    The library's calls take widths of up to 2^20.  A caller who allowed torch TF32 products (set_float32_matmul_precision, allow_tf32) keeps them: us
     library / TF32, 245 k rows of 256 x 256 194 / 168, 194 / 85, 267 / 101."""
     N, K = weight.shape
-    if (min(N, K) < 40 or graph.n * N * K < 1 << 29
+    if (min(N, K) < 40 or max(N, K) > 1 << 20 or graph.n * N * K < 1 << 29
             or torch.backends.cuda.matmul.fp32_precision not in ("none", "ieee")):
         return False, False, False
     small, big, tiles = min(N, K), max(N, K), (graph.n + 127) // 128
