@@ -89,8 +89,10 @@ def _by_library(graph: "binding.Graph", weight: torch.Tensor):
 
     The library's calls take widths of up to 2^20.  A caller who allowed torch TF32 products (set_float32_matmul_precision, allow_tf32) keeps them: us
     library / TF32, 245 k rows of 256 x 256 194 / 168, 194 / 85, 267 / 101."""
+    if graph.n * weight.numel() < 1 << 29:      # first: a small graph's epoch is host time
+        return False, False, False
     N, K = weight.shape
-    if (min(N, K) < 40 or max(N, K) > 1 << 20 or graph.n * N * K < 1 << 29
+    if (min(N, K) < 40 or max(N, K) > 1 << 20
             or torch.backends.cuda.matmul.fp32_precision not in ("none", "ieee")):
         return False, False, False
     small, big, tiles = min(N, K), max(N, K), (graph.n + 127) // 128
