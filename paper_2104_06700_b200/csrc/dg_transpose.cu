@@ -362,7 +362,7 @@ struct CscArgs {  // empty otherwise
   int64_t n;
   uint2* columns;         // see columns_begin_kernel
   int32_t* rows_out;
-  float* scale_out;       // the factor of every entry's row, or nullptr
+  float* scale_out;       // the factor of every entry's row
 };
 template <int BITS, bool CSC>
 __global__ void __launch_bounds__(kSortBlock, 4)
@@ -531,8 +531,7 @@ digit_scatter(const uint32_t* __restrict__ keys_in, const uint32_t* __restrict__
         const RowOf at = row_of(c.table, c.rowptr, c.n, count, k, block[j]);
         vals_out[dst[j0 + j]] = k;
         c.rows_out[dst[j0 + j]] = (int32_t)at.row;
-        if (c.scale_out)
-          c.scale_out[dst[j0 + j]] = __uint_as_float(at.known ? at.factor : __ldcg(&c.columns[at.row].y));
+        c.scale_out[dst[j0 + j]] = __uint_as_float(at.known ? at.factor : __ldcg(&c.columns[at.row].y));
       }
     }
   }
@@ -641,9 +640,13 @@ __global__ void expand_rows_kernel(const int64_t* __restrict__ rowptr, int64_t n
   }
 }
 
-// The weight arrays of the CSC, from perm: the last step of a transposition, and again after the caller changed edge_w in
-// place (learnable edge weights).  The in-degree comes from the CSR row pointer.  A thread takes four edges: their
-// random reads are in flight together.
+// The weight arrays of the CSC, from perm: the last step of a transposition, whose last pass has written the factors
+// (TABULATED), and again after the caller changed edge_w in place (learnable edge weights), when mean_scale_T holds
+// products and the in-degree comes from the CSR row pointer.  A thread takes four edges: their random reads are in
+// flight together.  Transposition of weighted graphs, us, degrees from the row pointers / tabulated: 11.5 M edges 499 / 460,
+// 39.6 M 1490 / 1345, 79 M 3083 / 2893, 124 M 5226 / 5157.  Weights read in the last sort pass instead, whose few warps wait
+// for them: 39.6 M 1790, 79 M 3829.
+template <bool TABULATED>
 __global__ void __launch_bounds__(256)
 gather_weights_kernel(const uint32_t* __restrict__ perm, int64_t nnz, const float* __restrict__ edge_w,
                       const int32_t* __restrict__ rowidx_T, const int64_t* __restrict__ rowptr, int self,
@@ -652,14 +655,19 @@ gather_weights_kernel(const uint32_t* __restrict__ perm, int64_t nnz, const floa
   const int64_t q0 = ((int64_t)blockIdx.x * 256 + threadIdx.x) * 4;
   if (q0 >= nnz) return;
   if (nnz - q0 >= 4) {  // the arrays of the CSC are 256-byte aligned
-    const int4 v = *reinterpret_cast<const int4*>(rowidx_T + q0);
     const uint4 k = *reinterpret_cast<const uint4*>(perm + q0);
     const float w[4] = {__ldg(edge_w + k.x), __ldg(edge_w + k.y), __ldg(edge_w + k.z), __ldg(edge_w + k.w)};
-    const int32_t r[4] = {v.x, v.y, v.z, v.w};
     float t[4];
+    if (TABULATED) {
+      const float4 f = *reinterpret_cast<const float4*>(mean_scale_T + q0);
+      t[0] = w[0] * f.x; t[1] = w[1] * f.y; t[2] = w[2] * f.z; t[3] = w[3] * f.w;
+    } else {
+      const int4 v = *reinterpret_cast<const int4*>(rowidx_T + q0);
+      const int32_t r[4] = {v.x, v.y, v.z, v.w};
 #pragma unroll
-    for (int i = 0; i < 4; ++i)
-      t[i] = w[i] * (1.0f / (float)(__ldg(rowptr + r[i] + 1) - __ldg(rowptr + r[i]) + self));
+      for (int i = 0; i < 4; ++i)
+        t[i] = w[i] * (1.0f / (float)(__ldg(rowptr + r[i] + 1) - __ldg(rowptr + r[i]) + self));
+    }
     *reinterpret_cast<float4*>(w_T + q0) = make_float4(w[0], w[1], w[2], w[3]);
     *reinterpret_cast<float4*>(mean_scale_T + q0) = make_float4(t[0], t[1], t[2], t[3]);
     return;
@@ -668,7 +676,8 @@ gather_weights_kernel(const uint32_t* __restrict__ perm, int64_t nnz, const floa
     const float w = edge_w[perm[q]];
     const int64_t v = rowidx_T[q];
     w_T[q] = w;
-    mean_scale_T[q] = w * (1.0f / (float)(__ldg(rowptr + v + 1) - __ldg(rowptr + v) + self));
+    mean_scale_T[q] =
+        w * (TABULATED ? mean_scale_T[q] : 1.0f / (float)(__ldg(rowptr + v + 1) - __ldg(rowptr + v) + self));
   }
 }
 
@@ -836,15 +845,17 @@ void transpose_sizes(int64_t n, int64_t nnz, bool weighted, size_t* csc_bytes,
   *scratch_bytes = L.scratch_bytes;
 }
 
-dg_status_t refresh_csc_weights(Graph* g, cudaStream_t s) {
+static dg_status_t gather_weights(Graph* g, bool tabulated, cudaStream_t s) {
   if (g->nnz == 0 || !g->edge_w) return DG_OK;
-  DG_CUDA(launch_kernel(gather_weights_kernel, dim3((unsigned)((g->nnz + 1023) / 1024)), 256, s, true,
+  DG_CUDA(launch_kernel(tabulated ? gather_weights_kernel<true> : gather_weights_kernel<false>,
+                        dim3((unsigned)((g->nnz + 1023) / 1024)), 256, s, true,
                         reinterpret_cast<const uint32_t*>(g->perm), g->nnz, g->edge_w, g->rowidx_T, g->rowptr,
                         g->self_loops_in_csc ? 1 : 0, const_cast<float*>(g->w_T),
                         const_cast<float*>(g->mean_scale_T)));
   count_launches(1);
   return DG_OK;
 }
+dg_status_t refresh_csc_weights(Graph* g, cudaStream_t s) { return gather_weights(g, false, s); }
 
 dg_status_t transpose_run(Graph* g, void* csc, void* scratch, cudaStream_t s) {
   const int64_t n = g->n, nnz = g->nnz;
@@ -867,7 +878,7 @@ dg_status_t transpose_run(Graph* g, void* csc, void* scratch, cudaStream_t s) {
     DG_CUDA(cudaMemsetAsync(colptr, 0, (size_t)(n + 1) * 8, s));
   } else {
     const SortPlan plan = sort_plan(n);
-    CscArgs c{nullptr, g->rowptr, n, reinterpret_cast<uint2*>(colptr), rowidx_T, weighted ? nullptr : mean_scale_T};
+    CscArgs c{nullptr, g->rowptr, n, reinterpret_cast<uint2*>(colptr), rowidx_T, mean_scale_T};
     columns_begin_kernel<<<(unsigned)(n / 256 + 1), 256, 0, s>>>(g->rowptr, n, g->self_loops ? 1 : 0, c.columns);
     DG_CUDA(cudaGetLastError());
     count_launches(1);
@@ -892,7 +903,7 @@ dg_status_t transpose_run(Graph* g, void* csc, void* scratch, cudaStream_t s) {
   g->w_T = w_T;
   g->mean_scale_T = mean_scale_T;
   g->self_loops_in_csc = g->self_loops;
-  if (dg_status_t st = refresh_csc_weights(g, s)) return st;
+  if (dg_status_t st = gather_weights(g, true, s)) return st;
   g->split_csc = nullptr;
   if (wants_split(n, nnz)) {
     // the columns come out of the stable sort ordered by row, so the check never fires here
