@@ -26,10 +26,11 @@
 // before to their sums and split the next.  The stream of chunks runs over tile borders.  The weights are split once, by a
 // kernel of their own, and arrive as one bulk copy per chunk, asked for by an eighteenth warp.
 //
-// What bounds it, per tile of 128 x 256 and K = 256: the tensor cores, 12 300 cycles at their full rate of the 27 000 it
-// takes; the rest is the epilogue and the chunks' chain of barriers.  245 k x 256 x 256: 186 us with the epilogue, of
-// 84 at that rate and 77 for the bytes; torch's SIMT GEMM and an elementwise pass 660.  The gradient of the weights is bound by
-// shared memory, which takes every number in, splits it and feeds it out (2300 cycles a chunk of 768 of the tensor cores).
+// What bounds it, per tile of 128 x 256 and K = 256: the tensor cores, 12 300 cycles at their nominal rate of the 27 000 it
+// takes; the rest is the epilogue and the chunks' chain of barriers.  245 k x 256 x 256: 189 us with the epilogue, of
+// 117 for six bf16 products at the measured rate of 1640 TFLOP/s and 77 for the bytes; torch's SIMT GEMM and an elementwise
+// pass 660.  The gradient of the weights is bound by shared memory, which takes every number in, splits it and feeds it out
+// (2300 cycles a chunk of 768 of the tensor cores).
 #include "dg_internal.cuh"
 
 namespace dg {
