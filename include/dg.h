@@ -219,7 +219,7 @@ dg_status_t dg_layer_bwd(dg_graph_t g, const float* dOut, const float* out, int3
 /*
  * The matrix products of such a layer on fp32 matrices, X n x K, W N x K, G n x N (n = the handle's vertices),
  * to fp32 accuracy on the tensor cores: for all finite numbers the 2-norm errors of sums of sixteen numbers (that are not 0)
- * and more are below those of fp32 arithmetic, of fewer up to 1.8 times those.
+ * and more are below those of the same sum in fp32 arithmetic, term by term; of fewer up to 1.8 times those.
  *
  *   fwd:         Y = X W^T (n x N); with row_scale and bias (each may be NULL) and `relu` the epilogue of
  *                dg_layer_fwd follows: Y = act(row_scale[v] * Y + bias).
